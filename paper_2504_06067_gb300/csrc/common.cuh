@@ -2,8 +2,11 @@
 //
 // Layout of one run in HBM (n2 = 2N merged population, ld = n2 rounded up
 // to a multiple of 256, NW = ld / 32 bit-mask words):
-//   X     n2 x d  FP32 row-major   parents rows [0,N), children rows [N,2N)
-//   F     ld x m  FP32 row-major   rows >= n2 are NaN padding (never dominate)
+//   X     n2 x d  FP32 row-major   decision vectors; rows never move: pcan, pold, cslot
+//                                  and fslot say which row holds which individual
+//   F     ld x m  FP32 row-major   merged objectives (parents, then children); rows >= n2
+//                                  are NaN padding (never dominate)
+//   PF    N x m   FP32             the parents' objectives between generations
 //   Fp    ld x m  FP32             F in bucket order of f_0 (perm: position -> index)
 //   Dom   NW x ld u32              bit (i mod 32) of Dom[i/32][j] = "i dominates j",
 //                                  i, j positions in bucket order
@@ -71,7 +74,7 @@ struct Ctrl {
     int32_t nT;              // |S u F_l| (association set)
     int32_t Lstar;           // niche level threshold L*
     int32_t rlev;            // refs taken at level L*
-    int32_t nsel;            // selected count written by the compaction
+    int32_t nsel;            // selected count
     int32_t overflow;        // association candidate-list overflows (slow path taken)
     int32_t recheck_miss;    // debug: association misses found by the full FP64 recheck
     int32_t nlarge;          // references whose partial take needs the block-wide select
@@ -91,7 +94,6 @@ struct Ctrl {
     uint32_t thr_done;       // completion ticket of the sort's threshold histogram blocks
     uint32_t omin[NSGA3_FAST_M], omax[NSGA3_FAST_M];  // objective ranges (order-preserving uint)
     float thr[NSGA3_FAST_M][SORT_LMAX];               // level thresholds of the sort keys (m <= 10)
-    uint32_t cmp_done;       // completion ticket of the compaction blocks
     uint32_t zmin[NSGA3_MAX_M];  // ideal point as order-preserving uint of FP32
     double zstar[NSGA3_MAX_M];   // ideal point (FP64, +0.0 for zero)
     double a[NSGA3_MAX_M];       // intercepts
@@ -119,12 +121,22 @@ struct RunView {
     uint64_t seed;
     float eta_c, eta_m, p_c, p_m;
     Ctrl* ctrl;
+    // Decision vectors stay in the row they were written to: a generation
+    // that copied the selected rows moved 4 N d floats (82 of 1,870 us at
+    // m = 10, N = 100,000, d = 200).  pcan and fslot split the 2N rows: the
+    // parents' and the free ones, which the next children take.  The
+    // variation copies pcan to pold, fslot to cslot and PF into F, so that
+    // the end of the generation can write pcan, fslot and PF in place.
     float* X;          // n2 x d
     float* F;          // ld x m
+    float* PF;         // N x m  parents' objectives
     int32_t* rank;     // parents' ranks (N), used by the tournament
-    float* Xtmp;       // N x d gather target
-    float* Ftmp;       // N x m
-    int32_t* ranktmp;  // N
+    int32_t* pcan;     // N  row of parent p
+    int32_t* fslot;    // N  rows that hold no parent
+    int32_t* pold;     // N  row of merged individual i < N (the parents of the last variation)
+    int32_t* cslot;    // N  row of merged individual N + c (the children of the last variation)
+    float* Xtmp;       // N x d staging of get / set calls on pageable host memory
+    int32_t* bsum;     // selected individuals per 1,024 merged ones
     uint32_t* Dom;     // NW x ld
     int32_t* cnt;      // ld   remaining dominator counts
     int32_t* rank2;    // ld   merged ranks (original order)

@@ -5,7 +5,7 @@
 // kernel nodes:
 //   vary+eval -> reset -> sort -> dominance -> peel (one cooperative launch,
 //   every front) -> post-peel -> ideal, extremes+solve, prep, scan, level,
-//   bucket, pick -> compaction -> gather -> gen++
+//   bucket, pick -> mark -> gather, gen++
 // The niching kernels return at once when |S| + |F_l| == N.  A replay never
 // returns to the host.
 #include <cstdarg>
@@ -103,7 +103,7 @@ int select_launches(const nsga3_ctx* ctx)
     const int m = ctx->m;
     // m <= 10: + the sort's level thresholds, the dominance build's boxes and tile plan;
     // - three association kernels with few reference directions (one fused kernel)
-    return 18 + (m > NSGA3_FAST_M ? 5 : 3) + (m > NSGA3_WARP_M ? 1 : 0) + (ctx->v.dom_ks > 1 ? 1 : 0) -
+    return 19 + (m > NSGA3_FAST_M ? 5 : 3) + (m > NSGA3_WARP_M ? 1 : 0) + (ctx->v.dom_ks > 1 ? 1 : 0) -
            (assoc_small(ctx->v) ? 3 : 0);
 }
 // the softmax-simplex objective's dot-product kernel (m > 10)
@@ -118,8 +118,9 @@ int variation_launches(const nsga3_ctx* ctx)
 }
 int generation_launches(const nsga3_ctx* ctx)
 {
-    // the selection without its finite check, + variation, gather, commit
-    return select_launches(ctx) - 1 + variation_launches(ctx) + 2;
+    // the selection without its finite check, + variation; m > 10: + the
+    // objectives of the next population
+    return select_launches(ctx) - 1 + variation_launches(ctx) + (ctx->m > NSGA3_FAST_M ? 1 : 0);
 }
 
 nsga3_status fail(nsga3_ctx* c, nsga3_status s, const char* fmt, ...)
@@ -223,7 +224,7 @@ nsga3_status record_selection(nsga3_ctx* ctx, const RunView& v, cudaStream_t s,
     CK(launch_pick(v, s));
     st = record_event(ctx, s, EV_NICHE, events);
     if (st) return st;
-    CK(launch_compact(v, s));
+    CK(launch_mark(v, s));
     return NSGA3_OK;
 }
 
@@ -271,7 +272,7 @@ nsga3_status eager_selection(nsga3_ctx* ctx, const RunView& v, cudaStream_t s, b
     }
     st = record_event(ctx, s, EV_NICHE, true);
     if (st) return st;
-    CK(launch_compact(v, s));
+    CK(launch_mark(v, s));
     return NSGA3_OK;
 }
 
@@ -297,6 +298,7 @@ nsga3_status build_graphs(nsga3_ctx* ctx)
     nsga3_status st = record_event(ctx, ctx->cap, EV_START, true);
     if (!st) st = record_event(ctx, ctx->cap, EV_VARY, true);
     if (!st) st = record_selection(ctx, ctx->vs, ctx->cap, true, true);
+    if (!st && launch_select_out(ctx->vs, ctx->cap) != cudaSuccess) st = fail(ctx, NSGA3_ECUDA, "launch failed");
     if (!st) st = record_event(ctx, ctx->cap, EV_END, true);
     {
         cudaError_t e = cudaStreamEndCapture(ctx->cap, &g);
@@ -483,8 +485,12 @@ nsga3_status setup_alloc(nsga3_ctx* ctx)
     AL(v.F, (size_t)ld * m);
     AL(v.rank, N);
     AL(v.Xtmp, (size_t)N * d);
-    AL(v.Ftmp, (size_t)N * m);
-    AL(v.ranktmp, N);
+    AL(v.PF, (size_t)N * m);
+    AL(v.pcan, N);
+    AL(v.fslot, N);
+    AL(v.pold, N);
+    AL(v.cslot, N);
+    AL(v.bsum, (NW + 31) / 32);
     AL(v.Dom, v.streaming ? (size_t)1 : (size_t)NW * ld);
     AL(v.cnt, ld);
     AL(v.rank2, ld);
@@ -642,6 +648,8 @@ nsga3_status setup(nsga3_ctx* ctx)
     CK(cudaMemsetAsync(v.rank, 0, (size_t)N * sizeof(int32_t), s));
     CK(cudaMemsetAsync(v.X, 0, (size_t)n2 * d * sizeof(float), s));
     CK(cudaMemsetAsync(v.F, 0, (size_t)ld * m * sizeof(float), s));
+    CK(cudaMemsetAsync(v.PF, 0, (size_t)N * m * sizeof(float), s));
+    CK(launch_slots_init(v, s));
     CK(cudaMemsetAsync(ctx->vs.F, 0, (size_t)ld * m * sizeof(float), s));
     CK(cudaMemsetAsync(v.pi, 0xff, (size_t)ld * sizeof(int32_t), s));
     CK(cudaMemsetAsync(v.dist, 0, (size_t)ld * sizeof(double), s));
@@ -740,6 +748,33 @@ nsga3_status device_status(nsga3_ctx* ctx, cudaStream_t s, bool clear)
         CK(cudaStreamSynchronize(s));
     }
     return (nsga3_status)st;
+}
+
+// Whether kernels of this context's device can use p directly: device
+// memory of that device (or, with pinned, page-locked host memory).
+bool on_device(const nsga3_ctx* ctx, const void* p, bool pinned)
+{
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    if (a.type == cudaMemoryTypeDevice) return a.device == ctx->device && a.devicePointer == p;
+    return pinned && a.type == cudaMemoryTypeHost && a.devicePointer == p;
+}
+
+// Rows idx[0..N) of X to dst (any): written by the kernel where it can reach
+// dst, through the staging rows otherwise (the copy to pageable memory
+// returns when it is done, so the staging rows are free again).
+nsga3_status rows_out(nsga3_ctx* ctx, const int32_t* idx, float* dst, cudaStream_t s)
+{
+    if (on_device(ctx, dst, true)) {
+        CK(launch_rows_out(ctx->v, idx, dst, s));
+        return NSGA3_OK;
+    }
+    CK(launch_rows_out(ctx->v, idx, ctx->v.Xtmp, s));
+    CK(cudaMemcpyAsync(dst, ctx->v.Xtmp, (size_t)ctx->N * ctx->d * sizeof(float), cudaMemcpyDefault, s));
+    return NSGA3_OK;
 }
 
 // Checks the arguments of a context and fills its sizes (no device work).
@@ -1028,6 +1063,7 @@ nsga3_status nsga3_select(nsga3_ctx* ctx, const float* objs, int32_t* ranks, int
         nsga3_status st = record_event(ctx, s, EV_START, true);
         if (!st) st = record_event(ctx, s, EV_VARY, true);
         if (!st) st = eager_selection(ctx, ctx->vs, s, true);
+        if (!st) CK(launch_select_out(ctx->vs, s));
         if (!st) st = record_event(ctx, s, EV_END, true);
         if (st) return st;
     } else {
@@ -1146,8 +1182,11 @@ nsga3_status nsga3_get_population(nsga3_ctx* ctx, float* X, float* F, int32_t* r
 {
     if (!ctx) return fail(ctx, NSGA3_EINVAL, "null context");
     cudaStream_t s = (cudaStream_t)stream;
-    if (X) CK(cudaMemcpyAsync(X, ctx->v.X, (size_t)ctx->N * ctx->d * sizeof(float), cudaMemcpyDefault, s));
-    if (F) CK(cudaMemcpyAsync(F, ctx->v.F, (size_t)ctx->N * ctx->m * sizeof(float), cudaMemcpyDefault, s));
+    if (X) {
+        nsga3_status st = rows_out(ctx, ctx->v.pcan, X, s);
+        if (st) return st;
+    }
+    if (F) CK(cudaMemcpyAsync(F, ctx->v.PF, (size_t)ctx->N * ctx->m * sizeof(float), cudaMemcpyDefault, s));
     if (rank) CK(cudaMemcpyAsync(rank, ctx->v.rank, (size_t)ctx->N * sizeof(int32_t), cudaMemcpyDefault, s));
     return NSGA3_OK;
 }
@@ -1157,8 +1196,15 @@ nsga3_status nsga3_set_population(nsga3_ctx* ctx, const float* X, const float* F
 {
     if (!ctx) return fail(ctx, NSGA3_EINVAL, "null context");
     cudaStream_t s = (cudaStream_t)stream;
-    if (X) CK(cudaMemcpyAsync(ctx->v.X, X, (size_t)ctx->N * ctx->d * sizeof(float), cudaMemcpyDefault, s));
-    if (F) CK(cudaMemcpyAsync(ctx->v.F, F, (size_t)ctx->N * ctx->m * sizeof(float), cudaMemcpyDefault, s));
+    if (X) {
+        const float* src = X;
+        if (!on_device(ctx, X, false)) {
+            CK(cudaMemcpyAsync(ctx->v.Xtmp, X, (size_t)ctx->N * ctx->d * sizeof(float), cudaMemcpyDefault, s));
+            src = ctx->v.Xtmp;
+        }
+        CK(launch_rows_in(ctx->v, src, s));
+    }
+    if (F) CK(cudaMemcpyAsync(ctx->v.PF, F, (size_t)ctx->N * ctx->m * sizeof(float), cudaMemcpyDefault, s));
     if (rank) CK(cudaMemcpyAsync(ctx->v.rank, rank, (size_t)ctx->N * sizeof(int32_t), cudaMemcpyDefault, s));
     return NSGA3_OK;
 }
@@ -1168,7 +1214,10 @@ nsga3_status nsga3_get_children(nsga3_ctx* ctx, float* X, float* F, void* stream
     if (!ctx) return fail(ctx, NSGA3_EINVAL, "null context");
     cudaStream_t s = (cudaStream_t)stream;
     const size_t N = ctx->N;
-    if (X) CK(cudaMemcpyAsync(X, ctx->v.X + N * ctx->d, N * ctx->d * sizeof(float), cudaMemcpyDefault, s));
+    if (X) {
+        nsga3_status st = rows_out(ctx, ctx->v.cslot, X, s);
+        if (st) return st;
+    }
     if (F) CK(cudaMemcpyAsync(F, ctx->v.F + N * ctx->m, N * ctx->m * sizeof(float), cudaMemcpyDefault, s));
     return NSGA3_OK;
 }
@@ -1351,9 +1400,8 @@ nsga3_status nsga3_last_launches(nsga3_ctx* ctx, int32_t* launches)
     CK(cudaDeviceSynchronize());
     // reset, 3 sort, dominance, peel (every pass), 10 niching (the first
     // also writes the ranks back; the others return at once when no niching
-    // is needed; one or two more for m > 10), compaction (+ finite check
-    // for a selection; + variation, objective, gather, commit for a
-    // generation)
+    // is needed; one or two more for m > 10), mark, gather (+ finite check
+    // for a selection; + variation, objective for a generation)
     *launches = (ctx->last_kind == 1) ? select_launches(ctx) : generation_launches(ctx);
     return NSGA3_OK;
 }

@@ -28,8 +28,13 @@ __global__ void k_kp_init(RunView v)
     if (e >= (long long)v.N * v.d) return;
     const int i = (int)(e / v.d), var = (int)(e - (long long)i * v.d);
     const U4 r = philox((uint32_t)i * (uint32_t)v.d + (uint32_t)var, 0u, RNG_INIT, 0u, v.seed);
-    v.X[e] = u01(r.x) < 0.5f ? 1.0f : 0.0f;
-    if (var == 0) v.rank[i] = 0;
+    const int slot = v.pold[i];
+    v.X[(size_t)slot * v.d + var] = u01(r.x) < 0.5f ? 1.0f : 0.0f;
+    if (var == 0) {
+        v.rank[i] = 0;
+        v.pcan[i] = slot;
+        v.fslot[i] = v.cslot[i];
+    }
 }
 
 __global__ void k_kp_vary(RunView v)
@@ -44,13 +49,21 @@ __global__ void k_kp_vary(RunView v)
     const U4 cx = philox((uint32_t)q, gen, RNG_TOURNAMENT, 1u, v.seed);
     const uint32_t a1 = bounded(t.x, N), b1 = bounded(t.y, N);
     const uint32_t a2 = bounded(t.z, N), b2 = bounded(t.w, N);
-    const uint32_t p1 = v.rank[b1] < v.rank[a1] ? b1 : a1;
-    const uint32_t p2 = v.rank[b2] < v.rank[a2] ? b2 : a2;
+    const int ra1 = v.pcan[a1], rb1 = v.pcan[b1], ra2 = v.pcan[a2], rb2 = v.pcan[b2];
+    const size_t p1 = v.rank[b1] < v.rank[a1] ? rb1 : ra1;
+    const size_t p2 = v.rank[b2] < v.rank[a2] ? rb2 : ra2;
     const bool cross = u01(cx.x) < v.p_c;
-    float* x0 = v.X + (size_t)(N + 2 * q) * d;
-    float* x1 = v.X + (size_t)(N + 2 * q + 1) * d;
+    const int f0 = v.fslot[2 * q], f1 = v.fslot[2 * q + 1];
+    float* x0 = v.X + (size_t)f0 * d;
+    float* x1 = v.X + (size_t)f1 * d;
+    // the pair's share of the merged state (as merge_pair of k_problem.cu)
+    if (lane < 2) {
+        v.pold[2 * q + lane] = v.pcan[2 * q + lane];
+        v.cslot[2 * q + lane] = lane ? f1 : f0;
+    }
+    if (lane < 2 * v.m) v.F[(size_t)2 * q * v.m + lane] = v.PF[(size_t)2 * q * v.m + lane];  // 2 m <= 20
     for (int var = lane; var < d; var += 32) {
-        float c1 = v.X[(size_t)p1 * d + var], c2 = v.X[(size_t)p2 * d + var];
+        float c1 = v.X[p1 * d + var], c2 = v.X[p2 * d + var];
         const uint32_t ctr = (uint32_t)q * (uint32_t)d + (uint32_t)var;
         const U4 s = philox(ctr, gen, RNG_SBX, 0u, v.seed);
         if (cross && u01(s.x) < 0.5f) {
@@ -68,15 +81,15 @@ __global__ void k_kp_vary(RunView v)
 
 constexpr int KB = 256;  // threads per block of k_kp_eval (8 individuals)
 
-// Repair and objectives of rows [row0, row0 + n).  A warp owns a row.
-__global__ void __launch_bounds__(KB) k_kp_eval(RunView v, int row0, int n)
+// Repair and objectives of n rows of X (rows_of), into Fout.  A warp owns a row.
+__global__ void __launch_bounds__(KB) k_kp_eval(RunView v, const int32_t* rows_of, float* Fout, int n)
 {
     const int lane = lane_id();
     const int r = (blockIdx.x * KB + threadIdx.x) >> 5;
     if (r >= n) return;
     if (read_status(v.ctrl)) return;
     const int m = v.m, d = v.d;
-    float* x = v.X + (size_t)(row0 + r) * d;
+    float* x = v.X + (size_t)rows_of[r] * d;
     // loads and excess per knapsack (integers; sums below 2^31 by the
     // limits checked at creation)
     int excess[NSGA3_FAST_M];
@@ -128,7 +141,7 @@ __global__ void __launch_bounds__(KB) k_kp_eval(RunView v, int row0, int n)
         for (int e = lane; e < d; e += 32)
             if (x[e] == 0.0f) s += __ldg(&v.kp_p[(size_t)j * d + e]);
         s = warp_sum(s);
-        if (lane == 0) v.F[(size_t)(row0 + r) * m + j] = (float)s;
+        if (lane == 0) Fout[(size_t)r * m + j] = (float)s;
     }
 }
 
@@ -140,7 +153,7 @@ cudaError_t launch_kp_init(const RunView& v, cudaStream_t s)
     k_kp_init<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(v);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_kp_eval<<<(unsigned)((v.N + KB / 32 - 1) / (KB / 32)), KB, 0, s>>>(v, 0, v.N);
+    k_kp_eval<<<(unsigned)((v.N + KB / 32 - 1) / (KB / 32)), KB, 0, s>>>(v, v.pold, v.PF, v.N);
     return cudaGetLastError();
 }
 
@@ -150,6 +163,6 @@ cudaError_t launch_kp_vary_eval(const RunView& v, cudaStream_t s)
     k_kp_vary<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(v);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_kp_eval<<<(unsigned)((v.N + KB / 32 - 1) / (KB / 32)), KB, 0, s>>>(v, v.N, v.N);
+    k_kp_eval<<<(unsigned)((v.N + KB / 32 - 1) / (KB / 32)), KB, 0, s>>>(v, v.cslot, v.F + (size_t)v.N * v.m, v.N);
     return cudaGetLastError();
 }

@@ -14,7 +14,7 @@
 //   of that block < p_m mutates child 2q with u = word 0 of
 //   Philox(q*d+v, gen, 3, 0); word 1 of that block < p_m mutates child 2q+1
 //   with u = its word 2 (two Philox blocks per pair and variable).
-//   Children go to rows N + 2q and N + 2q + 1.  FP32 arithmetic.
+//   Children 2q and 2q + 1 go to the rows fslot[2q], fslot[2q + 1].  FP32 arithmetic.
 // Objective (the softmax-simplex family): k = m - 1,
 //   g = sum_{v >= k} (x_v - 0.5)^2, f_j = (1 + g) softmax(W x[0:k])_j,
 //   evaluated in FP64 (sums left to right) and rounded to FP32; for m > 10
@@ -68,7 +68,7 @@ __global__ void k_refdirs(int m, int p1, int p2, double tau, int w1, int w, doub
     for (int q = 0; q < M4; ++q) Zh[(size_t)t * M4 + q] = q < m ? __double2float_rn(__ddiv_rn(z[q], n)) : 0.0f;
 }
 
-// Objective of rows [row0, row0 + n): a block covers R = obj_rows(m) rows.
+// Objective of n rows of X into Fout: a block covers R = obj_rows(m) rows.
 //   g = sum_{v >= m-1} (x_v - 0.5)^2: each term is formed exactly as a
 //   float-float value (x - 0.5 by Fast2Sum, the square by an FMA product
 //   error) and the terms are added in float-float (TwoSum) by a warp per row
@@ -111,7 +111,8 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e)
 constexpr int RB = 4;     // rows per CTA
 constexpr int DT = 128;   // objectives per CTA
 
-__global__ void __launch_bounds__(DT) k_obj_dot(RunView v, int row0, int n)
+// (row r of the n is row rows[r] of X, here and in k_objective)
+__global__ void __launch_bounds__(DT) k_obj_dot(RunView v, const int32_t* rows_of, int n)
 {
     extern __shared__ float xs[];  // RB x k
     const int m = v.m, d = v.d, k = m - 1;
@@ -119,7 +120,7 @@ __global__ void __launch_bounds__(DT) k_obj_dot(RunView v, int row0, int n)
     const int rows = min(RB, n - base);
     for (int e = threadIdx.x; e < RB * k; e += DT) {
         const int r = e / k, c = e - r * k;
-        xs[e] = r < rows ? v.X[(size_t)(row0 + base + r) * d + c] : 0.0f;
+        xs[e] = r < rows ? v.X[(size_t)rows_of[base + r] * d + c] : 0.0f;
     }
     __syncthreads();
     const int j = blockIdx.y * DT + threadIdx.x;
@@ -152,7 +153,7 @@ __global__ void __launch_bounds__(DT) k_obj_dot(RunView v, int row0, int n)
         }
 }
 
-__global__ void __launch_bounds__(OT) k_objective(RunView v, int row0, int n, int R)
+__global__ void __launch_bounds__(OT) k_objective(RunView v, const int32_t* rows_of, float* Fout, int n, int R)
 {
     extern __shared__ double sobj[];
     double* sg = sobj;        // R
@@ -164,7 +165,7 @@ __global__ void __launch_bounds__(OT) k_objective(RunView v, int row0, int n, in
     for (int rr = warp; rr < R; rr += OT / 32) {
         float sh = 0.0f, sl = 0.0f;
         if (base + rr < n) {
-            const float* x = v.X + (size_t)(row0 + base + rr) * d;
+            const float* x = v.X + (size_t)rows_of[base + rr] * d;
             for (int e = k + lane; e < d; e += 32) {
                 const float xv = x[e];
                 const float th = __fsub_rn(xv, 0.5f);
@@ -196,7 +197,7 @@ __global__ void __launch_bounds__(OT) k_objective(RunView v, int row0, int n, in
             se[idx] = v.fprime[(size_t)(base + rr) * m + j];
             continue;
         }
-        const float* x = v.X + (size_t)(row0 + base + rr) * d;
+        const float* x = v.X + (size_t)rows_of[base + rr] * d;
         double a = 0.0;
         for (int e = 0; e < k; ++e) a = __dadd_rn(a, __dmul_rn((double)v.Wobj[j * k + e], (double)x[e]));
         se[idx] = exp(a);
@@ -212,7 +213,7 @@ __global__ void __launch_bounds__(OT) k_objective(RunView v, int row0, int n, in
         const int rr = idx / m, j = idx - rr * m;
         if (base + rr >= n) continue;
         const double f = __dmul_rn(__dadd_rn(1.0, sg[rr]), __ddiv_rn(se[idx], sden[rr]));
-        v.F[(size_t)(row0 + base + rr) * m + j] = __double2float_rn(f);
+        Fout[(size_t)(base + rr) * m + j] = __double2float_rn(f);
     }
 }
 
@@ -222,12 +223,17 @@ __global__ void k_init(RunView v)
     const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (i >= v.N) return;
     const int lane = lane_id();
-    float* xrow = v.X + (size_t)i * v.d;
+    const int slot = v.pold[i];  // as a population set by the caller (k_rows_in)
+    float* xrow = v.X + (size_t)slot * v.d;
     for (int e = lane; e < v.d; e += 32) {
         U4 r = philox((uint32_t)i * (uint32_t)v.d + (uint32_t)e, 0u, RNG_INIT, 0u, v.seed);
         xrow[e] = u01(r.x);
     }
-    if (lane == 0) v.rank[i] = 0;
+    if (lane == 0) {
+        v.rank[i] = 0;
+        v.pcan[i] = slot;
+        v.fslot[i] = v.cslot[i];
+    }
 }
 
 // Bounded polynomial mutation (Deb and Goyal): y + dq with
@@ -250,6 +256,18 @@ __device__ __forceinline__ float pm_mutate(float y, float u, float eta_m)
     return fminf(fmaxf(y, 0.0f), 1.0f);
 }
 
+// The pair's share of the state that the end of the generation overwrites:
+// rows of the merged individuals and the parents' objectives.
+__device__ __forceinline__ void merge_pair(const RunView& v, int q)
+{
+    const int lane = lane_id();
+    if (lane < 2) {
+        v.pold[2 * q + lane] = v.pcan[2 * q + lane];
+        v.cslot[2 * q + lane] = v.fslot[2 * q + lane];
+    }
+    for (int e = lane; e < 2 * v.m; e += 32) v.F[(size_t)2 * q * v.m + e] = v.PF[(size_t)2 * q * v.m + e];
+}
+
 // Variation of one pair (one warp, lanes over the variables): binary
 // tournament on rank (first drawn wins ties), SBX with per-variable
 // crossover and child swap, polynomial mutation, clip to [0, 1].  Calls
@@ -265,12 +283,14 @@ __device__ __forceinline__ void vary_pair(const RunView& v, int q, uint32_t gen,
     const U4 cx = philox((uint32_t)q, gen, RNG_TOURNAMENT, 1u, v.seed);
     const uint32_t a1 = bounded(t.x, N), b1 = bounded(t.y, N);
     const uint32_t a2 = bounded(t.z, N), b2 = bounded(t.w, N);
-    const uint32_t p1 = v.rank[b1] < v.rank[a1] ? b1 : a1;
-    const uint32_t p2 = v.rank[b2] < v.rank[a2] ? b2 : a2;
+    // the rows of all four drawn parents are read beside their ranks
+    const int ra1 = v.pcan[a1], rb1 = v.pcan[b1], ra2 = v.pcan[a2], rb2 = v.pcan[b2];
+    const size_t p1 = v.rank[b1] < v.rank[a1] ? rb1 : ra1;
+    const size_t p2 = v.rank[b2] < v.rank[a2] ? rb2 : ra2;
     const bool cross = u01(cx.x) < v.p_c;
     const float e = 1.0f / (v.eta_c + 1.0f);
     for (int var = lane; var < d; var += 32) {
-        const float y1 = v.X[(size_t)p1 * d + var], y2 = v.X[(size_t)p2 * d + var];
+        const float y1 = v.X[p1 * d + var], y2 = v.X[p2 * d + var];
         float c1 = y1, c2 = y2;
         const U4 sb = philox((uint32_t)q * (uint32_t)d + (uint32_t)var, gen, RNG_SBX, 0u, v.seed);
         if (cross && u01(sb.y) < 0.5f) {
@@ -304,8 +324,9 @@ __global__ void k_vary(RunView v)
     if (q >= v.N / 2) return;
     if (read_status(v.ctrl)) return;
     const uint32_t gen = v.ctrl->gen;
-    float* x0 = v.X + (size_t)(v.N + 2 * q) * v.d;
-    float* x1 = v.X + (size_t)(v.N + 2 * q + 1) * v.d;
+    float* x0 = v.X + (size_t)v.fslot[2 * q] * v.d;
+    float* x1 = v.X + (size_t)v.fslot[2 * q + 1] * v.d;
+    merge_pair(v, q);
     vary_pair(v, q, gen, [&](int var, float c1, float c2) {
         x0[var] = c1;
         x1[var] = c2;
@@ -352,8 +373,9 @@ __global__ void __launch_bounds__(256) k_vary_eval(RunView v)
     const int lane = lane_id();
     const uint32_t gen = v.ctrl->gen;
     const int N = v.N;
-    float* x0 = v.X + (size_t)(N + 2 * q) * v.d;
-    float* x1 = v.X + (size_t)(N + 2 * q + 1) * v.d;
+    float* x0 = v.X + (size_t)v.fslot[2 * q] * v.d;
+    float* x1 = v.X + (size_t)v.fslot[2 * q + 1] * v.d;
+    merge_pair(v, q);
     float gh0 = 0.0f, gl0 = 0.0f, gh1 = 0.0f, gl1 = 0.0f;
     float xk0 = 0.0f, xk1 = 0.0f;
     vary_pair(v, q, gen, [&](int var, float c1, float c2) {
@@ -424,11 +446,11 @@ __global__ void __launch_bounds__(256) k_vary_eval(RunView v)
     }
 }
 
-cudaError_t launch_obj_dot(const RunView& v, int row0, int n, cudaStream_t s)
+cudaError_t launch_obj_dot(const RunView& v, const int32_t* rows_of, int n, cudaStream_t s)
 {
     if (!v.Wt) return cudaErrorInvalidValue;
     const size_t sm = (size_t)RB * (v.m - 1) * sizeof(float);
-    k_obj_dot<<<dim3((n + RB - 1) / RB, (v.m + DT - 1) / DT), DT, sm, s>>>(v, row0, n);
+    k_obj_dot<<<dim3((n + RB - 1) / RB, (v.m + DT - 1) / DT), DT, sm, s>>>(v, rows_of, n);
     return cudaGetLastError();
 }
 
@@ -456,11 +478,11 @@ cudaError_t launch_init(const RunView& v, cudaStream_t s)
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (v.m > NSGA3_FAST_M) {
-        e = launch_obj_dot(v, 0, v.N, s);
+        e = launch_obj_dot(v, v.pold, v.N, s);
         if (e != cudaSuccess) return e;
     }
     const int R = obj_rows(v.m);
-    k_objective<<<(v.N + R - 1) / R, OT, obj_smem(v.m), s>>>(v, 0, v.N, R);
+    k_objective<<<(v.N + R - 1) / R, OT, obj_smem(v.m), s>>>(v, v.pold, v.PF, v.N, R);
     return cudaGetLastError();
 }
 
@@ -486,9 +508,9 @@ cudaError_t launch_vary_eval(const RunView& v, cudaStream_t s)
     k_vary<<<blocks, 256, 0, s>>>(v);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    e = launch_obj_dot(v, v.N, v.N, s);
+    e = launch_obj_dot(v, v.cslot, v.N, s);
     if (e != cudaSuccess) return e;
     const int R = obj_rows(v.m);
-    k_objective<<<(v.N + R - 1) / R, OT, obj_smem(v.m), s>>>(v, v.N, v.N, R);
+    k_objective<<<(v.N + R - 1) / R, OT, obj_smem(v.m), s>>>(v, v.cslot, v.F + (size_t)v.N * v.m, v.N, R);
     return cudaGetLastError();
 }

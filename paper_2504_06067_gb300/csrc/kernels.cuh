@@ -56,8 +56,15 @@ cudaError_t launch_pick(const RunView& v, cudaStream_t s);
 // self-test of the block-wide selection of the smallest keys (one CTA)
 cudaError_t launch_select_probe(const unsigned long long* keys, int n, int need, uint32_t* marks,
                                 unsigned* paths, cudaStream_t s);
-cudaError_t launch_compact(const RunView& v, cudaStream_t s);
+// masks and counts of the selected individuals, then their indices (a
+// selection) or the next population and the generation counter
+cudaError_t launch_mark(const RunView& v, cudaStream_t s);
+cudaError_t launch_select_out(const RunView& v, cudaStream_t s);
 cudaError_t launch_gather(const RunView& v, cudaStream_t s);
+// rows of X to dst (row r of dst = row idx[r] of X), and back
+cudaError_t launch_rows_out(const RunView& v, const int32_t* idx, float* dst, cudaStream_t s);
+cudaError_t launch_rows_in(const RunView& v, const float* src, cudaStream_t s);
+cudaError_t launch_slots_init(const RunView& v, cudaStream_t s);
 
 // issue-rate probe of the dominance test's FADD / LOP3 mix (k_probe.cu)
 double issue_probe_instructions(int blocks, int iters);
