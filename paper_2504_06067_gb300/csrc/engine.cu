@@ -64,6 +64,7 @@ struct nsga3_ctx {
     unsigned ev_mask = 0; // bit e set: event e is recorded (opts.phase_timing; eager: all)
     std::string err;
     unsigned long long serial = 0;  // creation serial (g_ctx_serial)
+    bool small = false;             // selections and generations run in one cluster (k_small.cu)
     bool shared_gpu = false;        // runs side by side with others (RunView::shared_gpu)
     // batched graph cache: the graphs hold the device buffers of every run in
     // the list, so they are keyed by the runs' creation serials (a pointer of
@@ -98,8 +99,27 @@ bool assoc_tile_wanted(int m)
     return m >= 7;
 }
 
+// Small populations take one launch of one cluster (k_small.cu) instead of
+// the 20 kernels of the general path.  Not with options that belong to the
+// general path's kernels: timed phases, launch shapes, the FP64 recheck, a
+// forced association.
+bool small_wanted(const nsga3_ctx* ctx)
+{
+    const nsga3_opts& o = ctx->opts;
+    return ctx->m <= NSGA3_FAST_M && ctx->n2 <= SMALL_N2 && ctx->w <= SMALL_W && !ctx->eager && ctx->ev_mask == 0u &&
+           !o.debug_recheck_all && o.dom_ctas_per_sm == 0 && o.peel_ctas_per_sm == 0 && !getenv("NSGA3_ASSOC");
+}
+
+// ... and the variation inside that launch while its N d / 2 pair-variables
+// are few; above, the whole chip varies faster in a launch of its own
+bool small_varies(const nsga3_ctx* ctx)
+{
+    return ctx->v.problem == 0 && (long long)ctx->N * ctx->d <= 16384;
+}
+
 int select_launches(const nsga3_ctx* ctx)
 {
+    if (ctx->small) return 1;
     const int m = ctx->m;
     // m <= 10: + the sort's level thresholds, the dominance build's boxes and tile plan;
     // - three association kernels with few reference directions (one fused kernel)
@@ -118,6 +138,7 @@ int variation_launches(const nsga3_ctx* ctx)
 }
 int generation_launches(const nsga3_ctx* ctx)
 {
+    if (ctx->small) return small_varies(ctx) ? 1 : 1 + variation_launches(ctx);
     // the selection without its finite check, + variation; m > 10: + the
     // objectives of the next population
     return select_launches(ctx) - 1 + variation_launches(ctx) + (ctx->m > NSGA3_FAST_M ? 1 : 0);
@@ -230,6 +251,12 @@ nsga3_status record_selection(nsga3_ctx* ctx, const RunView& v, cudaStream_t s,
 
 nsga3_status record_generation(nsga3_ctx* ctx, cudaStream_t s, bool events)
 {
+    if (ctx->small) {
+        const bool varies = small_varies(ctx);
+        if (!varies) CK(launch_vary_eval(ctx->v, s));
+        CK(launch_small(ctx->v, varies ? 1 : 2, nullptr, ctx->v.rank2, ctx->v.sel, s));
+        return NSGA3_OK;
+    }
     nsga3_status st = record_event(ctx, s, EV_START, events);
     if (st) return st;
     CK(launch_vary_eval(ctx->v, s));
@@ -291,7 +318,7 @@ nsga3_status eager_generation(nsga3_ctx* ctx, cudaStream_t s)
 
 nsga3_status build_graphs(nsga3_ctx* ctx)
 {
-    if (ctx->eager) return NSGA3_OK;
+    if (ctx->eager || ctx->small) return NSGA3_OK;
     cudaGraph_t g = nullptr;
     // selection graph
     CK(cudaStreamBeginCapture(ctx->cap, cudaStreamCaptureModeRelaxed));
@@ -733,6 +760,7 @@ nsga3_status init_attributes(nsga3_ctx* ctx)
     CK(assoc_init_attributes());
     CK(norm_init_attributes());
     CK(dom_init_attributes());
+    CK(small_init_attributes());
     g_attr_done = true;
     return NSGA3_OK;
 }
@@ -856,6 +884,7 @@ nsga3_status ctx_create(int m, int d, int N, int ref_divisions, const nsga3_opts
         ctx->ev_mask = (ctx->eager || pt == 2) ? (1u << EV_COUNT) - 1u
                        : pt == 1               ? (1u << EV_RESET) | (1u << EV_DOM) | (1u << EV_PEEL)
                                                : 0u;
+        ctx->small = small_wanted(ctx);
         if (cudaGetDevice(&ctx->device) != cudaSuccess ||
             cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess) {
             cudaGetLastError();
@@ -1058,6 +1087,17 @@ nsga3_status nsga3_select(nsga3_ctx* ctx, const float* objs, int32_t* ranks, int
 {
     if (!ctx || !objs || !ranks || !selected) return fail(ctx, NSGA3_EINVAL, "null argument");
     cudaStream_t s = (cudaStream_t)stream;
+    if (ctx->small) {
+        // device buffers are read and written by the launch itself
+        const bool of = on_device(ctx, objs, false), ok = on_device(ctx, ranks, false), os = on_device(ctx, selected, false);
+        if (!of) CK(cudaMemcpyAsync(ctx->vs.F, objs, (size_t)ctx->n2 * ctx->m * sizeof(float), cudaMemcpyDefault, s));
+        CK(launch_small(ctx->vs, 0, of ? objs : ctx->vs.F, ok ? ranks : ctx->vs.rank2, os ? selected : ctx->vs.sel, s));
+        if (!ok) CK(cudaMemcpyAsync(ranks, ctx->vs.rank2, (size_t)ctx->n2 * sizeof(int32_t), cudaMemcpyDefault, s));
+        if (!os) CK(cudaMemcpyAsync(selected, ctx->vs.sel, (size_t)ctx->N * sizeof(int32_t), cudaMemcpyDefault, s));
+        ctx->host_launches += select_launches(ctx);
+        ctx->last_kind = 1;
+        return NSGA3_OK;
+    }
     CK(cudaMemcpyAsync(ctx->vs.F, objs, (size_t)ctx->n2 * ctx->m * sizeof(float), cudaMemcpyDefault, s));
     if (ctx->eager) {
         nsga3_status st = record_event(ctx, s, EV_START, true);
@@ -1104,6 +1144,9 @@ nsga3_status nsga3_step(nsga3_ctx* ctx, void* stream)
     if (!ctx->has_obj) return fail(ctx, NSGA3_ESTATE, "context has no objective (opts.W or the knapsack arrays were NULL)");
     if (ctx->eager) {
         nsga3_status st = eager_generation(ctx, (cudaStream_t)stream);
+        if (st) return st;
+    } else if (ctx->small) {
+        nsga3_status st = record_generation(ctx, (cudaStream_t)stream, false);
         if (st) return st;
     } else {
         CK(cudaGraphLaunch(ctx->gx_step, (cudaStream_t)stream));

@@ -35,6 +35,7 @@
 // A point whose candidate list overflows is rescanned in FP64 over all
 // references by a whole CTA (k_assoc_slow), as is every point in debug mode.
 // m > 10: no pruning (k_assoc_scan_gen), the same band and FP64 kernels.
+#include "associate.cuh"
 #include "kernels.cuh"
 
 namespace {
@@ -43,20 +44,7 @@ constexpr int AB = 256;   // threads per CTA (8 warps, one point per warp)
 constexpr int LC = 64;    // candidate slots per warp
 constexpr float EPS = 1e-5f;
 
-__device__ __forceinline__ double perp_dist(const double* fp, double nf, const double* Zj, double nzj,
-                                            int m)
-{
-    if (nf == 0.0) return 0.0;
-    double dot = 0.0;
-    for (int q = 0; q < m; ++q) dot = __dadd_rn(dot, __dmul_rn(fp[q], Zj[q]));
-    const double den = __dmul_rn(nf, nzj);
-    const double cth = __ddiv_rn(dot, den);
-    double one_m = __dsub_rn(1.0, __dmul_rn(cth, cth));
-    if (one_m < 0.0) one_m = 0.0;
-    return __dmul_rn(nf, __dsqrt_rn(one_m));
-}
-
-// the same for a run-time m with both rows in memory: sixteen loads of
+// perp_dist for a run-time m with both rows in memory: sixteen loads of
 // each row in flight
 __device__ __forceinline__ double perp_dist_mem(const double* fp, double nf, const double* Zj, double nzj,
                                                 int m)

@@ -17,6 +17,7 @@
 // j -> word 0 of Philox(j, gen, 4, 0), member i -> word 0 of
 // Philox(i, gen, 5, 0); ties go to the lower index.
 #include "kernels.cuh"
+#include "niche.cuh"
 
 namespace {
 
@@ -25,16 +26,6 @@ constexpr int LCAP = 4096;  // niche levels resolved by the shared histogram
 constexpr int EXACT = 1024; // candidates ranked pairwise in the last select phase
 constexpr int CKCAP = 4096; // level-L* reference keys staged in shared memory
 constexpr int RRCAP = 12288; // references whose (rho, rho') are staged in shared memory
-
-__device__ __forceinline__ uint32_t mem_prio(uint64_t seed, uint32_t gen, int i)
-{
-    return philox((uint32_t)i, gen, RNG_MEMPRIO, 0u, seed).x;
-}
-
-__device__ __forceinline__ unsigned long long ref_key(uint64_t seed, uint32_t gen, int j)
-{
-    return ((unsigned long long)philox((uint32_t)j, gen, RNG_REFPRIO, 0u, seed).x << 32) | (unsigned)j;
-}
 
 // ------------------------------------------------ block-wide helpers -------
 __device__ int block_sum(int x, int* scratch)
@@ -52,36 +43,6 @@ __device__ int block_sum(int x, int* scratch)
     t = scratch[32];
     __syncthreads();
     return t;
-}
-
-// exclusive scan of one value per thread; returns the prefix, *total the sum
-__device__ int block_excl_scan(int x, int* scratch, int* total)
-{
-    const int lane = lane_id(), warp = threadIdx.x >> 5;
-    int inc = x;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        int y = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += y;
-    }
-    if (lane == 31) scratch[warp] = inc;
-    __syncthreads();
-    if (warp == 0) {
-        int v = (lane < (int)(blockDim.x >> 5)) ? scratch[lane] : 0;
-        int vi = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            int y = __shfl_up_sync(0xffffffffu, vi, o);
-            if (lane >= o) vi += y;
-        }
-        scratch[lane] = vi - v;
-        if (lane == 31) scratch[32] = vi;
-    }
-    __syncthreads();
-    const int res = scratch[warp] + inc - x;
-    *total = scratch[32];
-    __syncthreads();
-    return res;
 }
 
 // Exclusive scan of a[0..n) into out[0..n] (out[n] = total) by one block:

@@ -14,6 +14,14 @@ cudaError_t launch_nan_pad(const RunView& v, cudaStream_t s);
 // variation + objective (Alg. 1, crossover and mutation; Sec. III-A)
 cudaError_t launch_vary_eval(const RunView& v, cudaStream_t s);
 
+// one selection or generation in one cluster (k_small.cu); mode 0: objectives
+// F in, ranks and indices out; 1: a whole generation; 2: a generation whose
+// variation has run
+#define SMALL_N2 2048  // merged individuals at most
+#define SMALL_W 2048   // reference directions at most
+cudaError_t launch_small(const RunView& v, int mode, const float* F, int32_t* ranks, int32_t* sel, cudaStream_t s);
+cudaError_t small_init_attributes();
+
 // selection (Alg. 1 sort / Alg. 2)
 // 0-1 knapsack workload (k_knapsack.cu): bits + repair + objectives
 cudaError_t launch_kp_init(const RunView& v, cudaStream_t s);
