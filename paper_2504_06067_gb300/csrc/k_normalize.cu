@@ -74,56 +74,47 @@ __device__ __forceinline__ double zstar_of(const Ctrl* c, int q)
 }
 
 // Ideal point, E b = 1 (solve_rows), a = 1 / b and the nadir fallback; one
-// warp, lane r on row r.  M <= NSGA3_FAST_M: m = M; M = NSGA3_WARP_M: any
-// m <= 32 at run time (rows and columns >= m are never touched).
-template <int M>
-__device__ void solve_intercepts(const RunView& v, Ctrl* c, const int* ext, const double* nad)
+// warp, lane r on row r, m <= 32.  A: m x (m + 1) values of shared memory.
+__device__ __noinline__ void solve_intercepts(const RunView& v, Ctrl* c, const int* ext, const double* nad, double* A)
 {
-    const int m = (M <= NSGA3_FAST_M) ? M : v.m;
+    const int m = v.m;
     const int lane = lane_id();
-    double zs[M];
-#pragma unroll
-    for (int q = 0; q < M; ++q) zs[q] = q < m ? zstar_of(c, q) : 0.0;
-    if (lane == 0) {
-#pragma unroll
-        for (int q = 0; q < M; ++q)
-            if (q < m) {
-                c->zstar[q] = zs[q];
-                c->ext[q] = ext[q];
-            }
-    }
-    bool ok = true;
-    const int ncand = v.n2 + ((v.norm_history && c->hvalid) ? m : 0);
-#pragma unroll
-    for (int q = 0; q < M; ++q)
-        if (q < m && (ext[q] < 0 || ext[q] >= ncand)) ok = false;
-    double A[M];
-    float evec[M];  // this lane's extreme vector (a merged point or a remembered one)
     const bool row = lane < m;
-    const int er = row ? ext[lane] : 0;
-#pragma unroll
-    for (int q = 0; q < M; ++q) {
-        const bool in = ok && row && q < m;
-        evec[q] = in ? (er < v.n2 ? v.F[(size_t)er * m + q] : v.he[(er - v.n2) * m + q]) : 0.0f;
-        A[q] = in ? __dsub_rn((double)evec[q], zs[q]) : 0.0;
+    const double z = row ? zstar_of(c, lane) : 0.0;
+    if (row) {
+        c->zstar[lane] = z;
+        c->ext[lane] = ext[lane];
     }
+    const int ncand = v.n2 + ((v.norm_history && c->hvalid) ? m : 0);
+    const int er = row ? ext[lane] : 0;
+    const bool ok0 = __all_sync(0xffffffffu, er >= 0 && er < ncand);
+    // this lane's extreme vector (a merged point or a remembered one)
+    const float* ev = er < v.n2 ? v.F + (size_t)er * m : v.he + (size_t)(er - v.n2) * m;
+#pragma unroll 4
+    for (int q = 0; q < m; ++q) {
+        const double zq = __shfl_sync(0xffffffffu, z, q);
+        if (row) A[lane * (m + 1) + q] = ok0 ? __dsub_rn((double)ev[q], zq) : 0.0;
+    }
+    if (row) A[lane * (m + 1) + m] = 1.0;
     double a = 0.0;
-    ok = solve_rows<M>(m, A, ok, a);
-    if (lane < m) {
-        if (!ok) a = (nad[lane] == 0.0) ? 1.0 : nad[lane];
+    const bool ok = solve_rows(m, A, ok0, a);
+    if (row) {
+        if (!ok) a = sf64::is_zero(nad[lane]) ? 1.0 : nad[lane];
         c->a[lane] = a;
     }
     if (lane == 0) c->fallback = ok ? 0 : 1;
     if (v.norm_history) {
-        // the ideal and the extreme vectors become the history (every lane
-        // read its remembered row above, before these writes)
+        // the ideal and the extreme vectors become the history; every lane
+        // reads its remembered row before any is replaced
+        if (row) c->hz[lane] = z;
         __syncwarp();
-        if (lane < m) {
-            c->hz[lane] = zs[lane];
-#pragma unroll
-            for (int q = 0; q < M; ++q)
-                if (q < m) v.he[lane * m + q] = evec[q];
-        }
+#pragma unroll 1
+        for (int q = 0; q < m; ++q)
+            if (row) A[lane * (m + 1) + q] = ok0 ? (double)ev[q] : 0.0;  // A is free again
+        __syncwarp();
+#pragma unroll 1
+        for (int q = 0; q < m; ++q)
+            if (row) v.he[lane * m + q] = (float)A[lane * (m + 1) + q];
         if (lane == 0) c->hvalid = 1;
     }
 }
@@ -139,6 +130,7 @@ __global__ void __launch_bounds__(EB) k_norm_extreme(RunView v)
     __shared__ unsigned s_ticket;
     __shared__ int f_ext[NSGA3_FAST_M];
     __shared__ double f_nad[NSGA3_FAST_M];
+    __shared__ double s_A[M * (M + 1)];
     Ctrl* c = v.ctrl;
     if (skip_niche(c)) return;
     constexpr int m = M;
@@ -290,7 +282,7 @@ __global__ void __launch_bounds__(EB) k_norm_extreme(RunView v)
     __syncthreads();
     if (warp == 0) {
         if (lane == 0) c->ext_done = 0u;
-        solve_intercepts<M>(v, c, f_ext, f_nad);
+        solve_intercepts(v, c, f_ext, f_nad, s_A);
     }
 }
 
@@ -486,6 +478,7 @@ __global__ void __launch_bounds__(256) k_ext_reduce(RunView v, int parts)
     __shared__ unsigned s_ticket;
     __shared__ int f_ext[NSGA3_WARP_M];
     __shared__ double f_nad[NSGA3_WARP_M];
+    __shared__ double s_A[NSGA3_WARP_M * (NSGA3_WARP_M + 1)];
     Ctrl* c = v.ctrl;
     if (skip_niche(c)) return;
     const int m = v.m, lane = lane_id();
@@ -533,7 +526,7 @@ __global__ void __launch_bounds__(256) k_ext_reduce(RunView v, int parts)
     }
     __syncthreads();
     if (threadIdx.x == 0) c->ext_done = 0u;
-    if (threadIdx.x < 32) solve_intercepts<NSGA3_WARP_M>(v, c, f_ext, f_nad);
+    if (threadIdx.x < 32) solve_intercepts(v, c, f_ext, f_nad, s_A);
 }
 
 // m > NSGA3_WARP_M: the elimination of the warp solver spread over a

@@ -58,6 +58,14 @@ __device__ __forceinline__ void st_peer(uint32_t a, unsigned long long x)
     asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(a), "l"(x) : "memory");
 }
 
+// FP32 pairs: two differences in one instruction, each rounded once
+__device__ __forceinline__ void sub2(unsigned long long a, unsigned long long b, uint32_t& lo, uint32_t& hi)
+{
+    unsigned long long d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "l"(d));
+}
+
 // Dynamic shared memory: byte offsets of the arrays for a population.
 struct SmallLayout {
     int wpc, colsP;  // words and columns per CTA
@@ -102,11 +110,60 @@ struct SmallShared {
     int rank[SCOLS], pos[SCOLS], flag[SCOLS], mem[SCOLS];
     double z[NSGA3_FAST_M], a[NSGA3_FAST_M], nad[NSGA3_FAST_M];
     float evec[NSGA3_FAST_M][NSGA3_FAST_M];
+    sf64::Divisor da[NSGA3_FAST_M];  // the intercepts as divisors
+    double A[NSGA3_FAST_M * (NSGA3_FAST_M + 1)];
+    float z32[NSGA3_FAST_M], ia32[NSGA3_FAST_M];
     int ext[NSGA3_FAST_M];
     int scratch[40];
     unsigned long long key[SKEYS];
     int fs, nc, novf, Lstar, bin, before, nkey, fallback;
 };
+
+// Dominance words of the owned columns, NC columns (colsP / NC apart) per
+// thread and row word: a row's objectives come by broadcast loads, whose rate
+// bounds the loop, so one load serves two columns where they come in pairs.
+// The OR of the differences f_j - f_i has its sign bit set iff some f_i > f_j
+// and is zero only for equal vectors (differences are never -0.0): i
+// dominates j iff it is positive.
+template <int M, int NC>
+__device__ __forceinline__ void dominance_words(const float* Fs, uint32_t* dom, int n2, int c0, int colsP)
+{
+    constexpr int MP = (M + 1) & ~1;
+    const int NWs = (n2 + 31) / 32, half = colsP / NC;
+    for (int t = threadIdx.x; t < NWs * half; t += ST) {
+        const int I = t / half, cl = t - I * half;
+        const int nr = min(32, n2 - I * 32);
+        unsigned long long pj[NC][MP / 2];
+        uint32_t word[NC];
+#pragma unroll
+        for (int u = 0; u < NC; ++u) {
+            const float* fj = Fs + min(c0 + cl + u * half, n2 - 1) * MP;
+#pragma unroll
+            for (int h = 0; h < MP / 2; ++h) pj[u][h] = reinterpret_cast<const unsigned long long*>(fj)[h];
+            word[u] = 0u;
+        }
+        const unsigned long long* fr = reinterpret_cast<const unsigned long long*>(Fs + I * 32 * MP);
+#pragma unroll 4
+        for (int k = nr - 1; k >= 0; --k) {
+            unsigned long long fi[MP / 2];
+#pragma unroll
+            for (int h = 0; h < MP / 2; ++h) fi[h] = fr[k * (MP / 2) + h];
+#pragma unroll
+            for (int u = 0; u < NC; ++u) {
+                uint32_t acc = 0u;
+#pragma unroll
+                for (int h = 0; h < MP / 2; ++h) {
+                    uint32_t lo, hi;
+                    sub2(pj[u][h], fi[h], lo, hi);
+                    acc |= lo | hi;
+                }
+                word[u] = __funnelshift_l(0u - acc, word[u], 1);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < NC; ++u) dom[I * colsP + cl + u * half] = word[u];
+    }
+}
 
 // Selects (mode 0: objectives Fin, ranks and indices out) or steps (mode 1:
 // variation too; mode 2: the merged individuals are in v.F already).
@@ -151,6 +208,8 @@ __global__ void __launch_bounds__(ST, 1) k_small(RunView v, int mode, int C, con
             bad |= mode == 0 && !isfinite(x);
             Fs[p * MP + q] = x + 0.0f;  // -0.0 as +0.0
         }
+    if (M & 1)  // the pad of an odd row
+        for (int p = tid; p < n2; p += ST) Fs[p * MP + M] = 0.0f;
     if (tid < NWs) {
         const int lo = tid * 32;
         sh.rem[tid] = lo + 32 <= n2 ? 0xffffffffu : (1u << (n2 - lo)) - 1u;
@@ -168,28 +227,10 @@ __global__ void __launch_bounds__(ST, 1) k_small(RunView v, int mode, int C, con
     }
 
     // ---- dominance: word I of column j = rows 32 I .. 32 I + 31 that dominate j
-    for (int t = tid; t < NWs * colsP; t += ST) {
-        const int I = t / colsP, cl = t - I * colsP;
-        const int j = min(c0 + cl, n2 - 1);
-        const int nr = min(32, n2 - I * 32);
-        float fj[M];
-#pragma unroll
-        for (int q = 0; q < M; ++q) fj[q] = Fs[j * MP + q];
-        const float* fr = Fs + I * 32 * MP;
-        uint32_t word = 0u;
-#pragma unroll 4
-        for (int k = nr - 1; k >= 0; --k) {
-            uint32_t oa = 0u, ob = 0u;  // signs: some f_i > f_j, some f_j > f_i
-#pragma unroll
-            for (int q = 0; q < M; ++q) {
-                const float fi = fr[k * MP + q];
-                oa |= __float_as_uint(fj[q] - fi);
-                ob |= __float_as_uint(fi - fj[q]);
-            }
-            word = __funnelshift_l(ob & ~oa, word, 1);
-        }
-        dom[t] = word;
-    }
+    if (wpc & 1)
+        dominance_words<M, 1>(Fs, dom, n2, c0, colsP);
+    else
+        dominance_words<M, 2>(Fs, dom, n2, c0, colsP);
     __syncthreads();
 
     // ---- fronts: an unranked column without an unranked dominator is ranked
@@ -304,8 +345,13 @@ __global__ void __launch_bounds__(ST, 1) k_small(RunView v, int mode, int C, con
                     m2 = kr;
                 }
             }
-            const unsigned long long k1 = okey(__ddiv_rn(__longlong_as_double((long long)m1), 1e-6));
-            const unsigned long long k2 = okey(__ddiv_rn(__longlong_as_double((long long)m2), 1e-6));
+            const sf64::Divisor micro = sf64::divisor(1e-6);
+            unsigned long long k1, k2 = m1;
+#pragma unroll 1
+            for (int h = 0; h < 2; ++h) {  // (one copy of the division's code)
+                k1 = k2;
+                k2 = okey(sf64::div(__longlong_as_double((long long)(h ? m2 : m1)), micro));
+            }
 #pragma unroll
             for (int q = 0; q < M; ++q) {
                 const unsigned long long other = q == r1 ? k2 : k1, kq = okey(ft[q]);
@@ -377,19 +423,25 @@ __global__ void __launch_bounds__(ST, 1) k_small(RunView v, int mode, int C, con
                 sh.nad[lane] = __longlong_as_double((long long)n);
             }
             __syncwarp();
-            double A[M];
             const int er = sh.ext[lane < M ? lane : 0];
-            const bool okr = er >= 0 && er < n2 + (hist ? M : 0);
-            bool ok = __all_sync(0xffffffffu, okr);
-#pragma unroll
-            for (int q = 0; q < M; ++q) {
-                const float x = ok && lane < M ? (er < n2 ? Fs[er * MP + q] : v.he[(er - n2) * M + q]) : 0.0f;
-                if (lane < M) sh.evec[lane][q] = x;
-                A[q] = ok && lane < M ? __dsub_rn((double)x, sh.z[q]) : 0.0;
+            bool ok = __all_sync(0xffffffffu, er >= 0 && er < n2 + (hist ? M : 0));
+#pragma unroll 1
+            for (int e = lane; e < M * M; e += 32) {
+                const int r = e / M, q = e - r * M, x = sh.ext[r];
+                const float f = !ok ? 0.0f : x < n2 ? Fs[x * MP + q] : v.he[(x - n2) * M + q];
+                sh.evec[r][q] = f;
+                sh.A[r * (M + 1) + q] = ok ? __dsub_rn((double)f, sh.z[q]) : 0.0;
             }
+            if (lane < M) sh.A[lane * (M + 1) + M] = 1.0;
             double a = 0.0;
-            ok = solve_rows<M>(M, A, ok, a);
-            if (lane < M) sh.a[lane] = ok ? a : sh.nad[lane] == 0.0 ? 1.0 : sh.nad[lane];
+            ok = solve_rows(M, sh.A, ok, a);
+            if (lane < M) {
+                const double al = ok ? a : sf64::is_zero(sh.nad[lane]) ? 1.0 : sh.nad[lane];
+                sh.a[lane] = al;
+                sh.da[lane] = sf64::divisor(al);
+                sh.z32[lane] = (float)sh.z[lane];
+                sh.ia32[lane] = __frcp_rn((float)al);
+            }
             if (lane == 0) sh.fallback = ok ? 0 : 1;
         }
         // ---- association of the owned members
@@ -411,26 +463,32 @@ __global__ void __launch_bounds__(ST, 1) k_small(RunView v, int mode, int C, con
         float* us = reinterpret_cast<float*>(bj + colsP);                    // colsP x M
         for (int e = tid; e < nm * M; e += ST) {
             const int p = e / M, q = e - p * M;
-            fp[e] = __ddiv_rn(__dsub_rn((double)Fs[(c0 + sh.mem[p]) * MP + q], sh.z[q]), sh.a[q]);
+            fp[e] = sf64::div(__dsub_rn((double)Fs[(c0 + sh.mem[p]) * MP + q], sh.z[q]), sh.da[q]);
         }
         __syncthreads();
         for (int p = tid; p < nm; p += ST) {
             double ss = 0.0;
 #pragma unroll
             for (int q = 0; q < M; ++q) ss = __dadd_rn(ss, __dmul_rn(fp[p * M + q], fp[p * M + q]));
-            const double x = __dsqrt_rn(ss);
+            const double x = sf64::sqrt_rn(ss);
+            const bool zero = sf64::is_zero(x);
             nf[p] = x;
-            const double inv = x > 0.0 ? 1.0 / x : 0.0;
+            float u[M];
+            if (!unit32<M>(Fs + (c0 + sh.mem[p]) * MP, sh.z32, sh.ia32, u)) {
+                const double inv = zero ? 0.0 : 1.0 / x;
 #pragma unroll
-            for (int q = 0; q < M; ++q) us[p * M + q] = __double2float_rn(fp[p * M + q] * inv);
+                for (int q = 0; q < M; ++q) u[q] = __double2float_rn(fp[p * M + q] * inv);
+            }
+#pragma unroll
+            for (int q = 0; q < M; ++q) us[p * M + q] = u[q];
             // |f'| = 0: every distance is 0, the first direction
-            bd[p] = x == 0.0 ? 0ull : ~0ull;
-            bj[p] = x == 0.0 ? 0 : 0x7fffffff;
+            bd[p] = zero ? 0ull : ~0ull;
+            bj[p] = zero ? 0 : 0x7fffffff;
         }
         __syncthreads();
         // FP32 cosines, a lane per direction, four members per warp pass;
         // each lane keeps its best direction and its second-best cosine
-        const float band = 2.0f * (float)(M + 4) * 5.9604644775390625e-08f + 1e-12f;
+        const float band = cos_band<M>();
         const int cap = colsP * SCAND;
         for (int p0 = warp * 4; p0 < nm; p0 += SWARPS * 4) {
             float u[4][M], b1[4], b2[4];
@@ -815,7 +873,7 @@ __global__ void __launch_bounds__(ST, 1) k_small(RunView v, int mode, int C, con
 int small_ctas(int n2)
 {
     const int NWs = (n2 + 31) / 32;
-    if (NWs > 8 * SCOLS / 32) return 16;
+    if (NWs > 16) return 16;
     return NWs > 4 ? 8 : NWs > 2 ? 4 : NWs > 1 ? 2 : 1;
 }
 

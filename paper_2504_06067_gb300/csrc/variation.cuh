@@ -56,15 +56,16 @@ __device__ __forceinline__ void vary_pair(const RunView& v, int q, uint32_t gen,
 {
     const int lane = lane_id();
     const int N = v.N, d = v.d;
-    const U4 t = philox((uint32_t)q, gen, RNG_TOURNAMENT, 0u, v.seed);
-    const U4 cx = philox((uint32_t)q, gen, RNG_TOURNAMENT, 1u, v.seed);
-    const uint32_t a1 = bounded(t.x, N), b1 = bounded(t.y, N);
-    const uint32_t a2 = bounded(t.z, N), b2 = bounded(t.w, N);
+    // the pair's two blocks by odd and even lanes at once
+    const U4 t = philox((uint32_t)q, gen, RNG_TOURNAMENT, (uint32_t)lane & 1u, v.seed);
+    const uint32_t a1 = bounded(__shfl_sync(0xffffffffu, t.x, 0), N), b1 = bounded(__shfl_sync(0xffffffffu, t.y, 0), N);
+    const uint32_t a2 = bounded(__shfl_sync(0xffffffffu, t.z, 0), N), b2 = bounded(__shfl_sync(0xffffffffu, t.w, 0), N);
+    const uint32_t cx = __shfl_sync(0xffffffffu, t.x, 1);
     // the rows of all four drawn parents are read beside their ranks
     const int ra1 = v.pcan[a1], rb1 = v.pcan[b1], ra2 = v.pcan[a2], rb2 = v.pcan[b2];
     const size_t p1 = v.rank[b1] < v.rank[a1] ? rb1 : ra1;
     const size_t p2 = v.rank[b2] < v.rank[a2] ? rb2 : ra2;
-    const bool cross = u01(cx.x) < v.p_c;
+    const bool cross = u01(cx) < v.p_c;
     const float e = 1.0f / (v.eta_c + 1.0f);
     for (int var = lane; var < d; var += 32) {
         const float y1 = v.X[p1 * d + var], y2 = v.X[p2 * d + var];
@@ -88,8 +89,16 @@ __device__ __forceinline__ void vary_pair(const RunView& v, int q, uint32_t gen,
         }
         const bool mut0 = u01(sb.w) < v.p_m;
         const U4 pm = philox((uint32_t)q * (uint32_t)d + (uint32_t)var, gen, RNG_PM, 0u, v.seed);
-        if (mut0) c1 = pm_mutate(c1, u01(pm.x), v.eta_m);
-        if (u01(pm.y) < v.p_m) c2 = pm_mutate(c2, u01(pm.z), v.eta_m);
+        const bool mut1 = u01(pm.y) < v.p_m;
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h)  // one copy of the mutation's code
+            if (h ? mut1 : mut0) {
+                const float y = pm_mutate(h ? c2 : c1, u01(h ? pm.z : pm.x), v.eta_m);
+                if (h)
+                    c2 = y;
+                else
+                    c1 = y;
+            }
         out(var, c1, c2);
     }
 }
