@@ -24,8 +24,6 @@
 #define NSGA3_TILE 256          // column tile of the dominance build; ld % 256 == 0
 #define NSGA3_PEEL_COLS 128     // columns per peel chunk (4 per lane, 32 lanes)
 #define SORT_NB 4096            // sort keys of the f_0 bucket order (m > 10)
-#define SORT_KMAX 65536         // largest number of sort keys (m <= 10: 2^kbits keys)
-#define SORT_QB 1024            // histogram bins per objective for the level thresholds
 #define SORT_LMAX 7             // level thresholds per objective (3 bits of level)
 
 // Capacity paths of the niching kernels (Ctrl::npath, reported by
@@ -89,10 +87,7 @@ struct Ctrl {
     int32_t ncand;           // association candidates written by the scan
     int32_t nslow;           // points sent to the full FP64 association scan
     uint32_t ext_done;       // completion ticket of the extreme-point blocks
-    uint32_t sort_done;      // completion ticket of the bucket histogram
     uint32_t f0lo, f0hi;     // range of f_0 as order-preserving uint
-    uint32_t thr_done;       // completion ticket of the sort's threshold histogram blocks
-    uint32_t omin[NSGA3_FAST_M], omax[NSGA3_FAST_M];  // objective ranges (order-preserving uint)
     float thr[NSGA3_FAST_M][SORT_LMAX];               // level thresholds of the sort keys (m <= 10)
     uint32_t zmin[NSGA3_MAX_M];  // ideal point as order-preserving uint of FP32
     double zstar[NSGA3_MAX_M];   // ideal point (FP64, +0.0 for zero)
@@ -145,10 +140,11 @@ struct RunView {
     uint32_t* skey;    // ld   sort key of each position (0xffffffff for padding)
     uint32_t* pkey;    // n2   sort key of each point (original order)
     float* Fp;         // ld x m objectives in bucket order, -0.0 as +0.0, NaN padding
-    int32_t* bcnt;     // nkeys + 1 key counts, then offsets / cursors
+    int32_t* bcnt;     // nkeys key counts
+    int32_t* bcur;     // nkeys points of a key placed so far
+    int32_t* bgrp;     // nkeys / 32 counts of groups of keys
     int kbits;         // bits of a sort key (nkeys = 2^kbits)
     int lbits;         // bits of level per objective in a sort key (m <= 10)
-    int32_t* qhist;    // m x SORT_QB objective histograms (level thresholds)
     float* bbox;       // NW x 2 M4: per 32-position block min, then max of each objective
     uint32_t* bkey;    // NW x 2: per block smallest, largest sort key
     uint8_t* dnz;      // NW x NB8 bits: Dom block (I, J) has a nonzero word (m <= 10, matrix);

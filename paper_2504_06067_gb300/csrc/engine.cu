@@ -77,10 +77,6 @@ struct nsga3_ctx {
 
 namespace {
 
-// kernels of one selection / one generation: m > 10 adds five (ideal point,
-// extreme-point keys and reduction, |f'|, candidate distances), m > 32 the
-// cooperative elimination, and a split dominance build (few tiles) its
-// finishing kernel
 // Association of more than ASSOC_SMALL_W directions (m <= 10): the tiled
 // scan (every FP32 cosine at the FMA rate) or the pruned scan (cone bounds
 // per block of 32 directions).  Both give the same association.  The cone
@@ -117,14 +113,17 @@ bool small_varies(const nsga3_ctx* ctx)
     return ctx->v.problem == 0 && (long long)ctx->N * ctx->d <= 16384;
 }
 
+// Kernels of one selection / one generation; m > 10: with the ideal point,
+// extreme-point keys and reduction, |f'| and candidate distances, m > 32 the
+// cooperative elimination, and a split dominance build (few tiles) its
+// finishing kernel.
 int select_launches(const nsga3_ctx* ctx)
 {
     if (ctx->small) return 1;
     const int m = ctx->m;
-    // m <= 10: + the sort's level thresholds, the dominance build's boxes and tile plan;
-    // - three association kernels with few reference directions (one fused kernel)
-    return 19 + (m > NSGA3_FAST_M ? 5 : 3) + (m > NSGA3_WARP_M ? 1 : 0) + (ctx->v.dom_ks > 1 ? 1 : 0) -
-           (assoc_small(ctx->v) ? 3 : 0);
+    // three association kernels fewer with few reference directions (one fused kernel)
+    if (m <= NSGA3_FAST_M) return 19 - (assoc_small(ctx->v) ? 3 : 0);
+    return 24 + (m > NSGA3_WARP_M ? 1 : 0) + (ctx->v.dom_ks > 1 ? 1 : 0);
 }
 // the softmax-simplex objective's dot-product kernel (m > 10)
 int objective_dot_launches(const nsga3_ctx* ctx) { return ctx->m > NSGA3_FAST_M && ctx->v.problem == 0 ? 1 : 0; }
@@ -139,9 +138,9 @@ int variation_launches(const nsga3_ctx* ctx)
 int generation_launches(const nsga3_ctx* ctx)
 {
     if (ctx->small) return small_varies(ctx) ? 1 : 1 + variation_launches(ctx);
-    // the selection without its finite check, + variation; m > 10: + the
-    // objectives of the next population
-    return select_launches(ctx) - 1 + variation_launches(ctx) + (ctx->m > NSGA3_FAST_M ? 1 : 0);
+    // the selection and the variation (m > 10: without the finite check's
+    // launch, with one for the objectives of the next population)
+    return select_launches(ctx) + variation_launches(ctx);
 }
 
 nsga3_status fail(nsga3_ctx* c, nsga3_status s, const char* fmt, ...)
@@ -222,8 +221,7 @@ nsga3_status record_event(nsga3_ctx* ctx, cudaStream_t s, int which, bool events
 nsga3_status record_selection(nsga3_ctx* ctx, const RunView& v, cudaStream_t s,
                               bool check_finite, bool events)
 {
-    CK(launch_sel_reset(v, s));
-    if (check_finite) CK(launch_check_finite(v, s));
+    CK(launch_front(v, ctx->num_sms, check_finite, s));
     CK(launch_sort(v, ctx->num_sms, s));
     nsga3_status st = record_event(ctx, s, EV_RESET, events);
     if (st) return st;
@@ -273,8 +271,7 @@ nsga3_status record_generation(nsga3_ctx* ctx, cudaStream_t s, bool events)
 // needed.  For tools and debugging that want direct launches.
 nsga3_status eager_selection(nsga3_ctx* ctx, const RunView& v, cudaStream_t s, bool check_finite)
 {
-    CK(launch_sel_reset(v, s));
-    if (check_finite) CK(launch_check_finite(v, s));
+    CK(launch_front(v, ctx->num_sms, check_finite, s));
     CK(launch_sort(v, ctx->num_sms, s));
     nsga3_status st = record_event(ctx, s, EV_RESET, true);
     if (st) return st;
@@ -539,10 +536,11 @@ nsga3_status setup_alloc(nsga3_ctx* ctx)
         v.lbits = 0;
         v.kbits = 12;
     }
-    AL(v.bcnt, (1 << v.kbits) + 1);
+    AL(v.bcnt, 1 << v.kbits);
+    AL(v.bcur, 1 << v.kbits);
+    AL(v.bgrp, (1 << v.kbits) / 32);
     v.NB8 = (NW + 7) / 8;
     if (m <= NSGA3_FAST_M) {
-        AL(v.qhist, (size_t)m * SORT_QB);
         AL(v.bbox, (size_t)NW * 2 * M4);
         AL(v.bkey, (size_t)NW * 2);
         const size_t T = (size_t)ld / NSGA3_TILE;

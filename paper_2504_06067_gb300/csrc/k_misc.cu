@@ -1,81 +1,9 @@
-// k_misc.cu -- per-selection reset, boundary check of the objectives, the
+// k_misc.cu -- boundary check of the objectives (m > 10), the
 // selected indices and the next population (Alg. 2 last line: P_{t+1} = rows
 // with rank < l after selection), and copies of populations in and out.
 #include "kernels.cuh"
 
 namespace {
-
-__global__ void k_sel_reset(RunView v)
-{
-    const int tid = blockIdx.x * blockDim.x + threadIdx.x;
-    const int stride = gridDim.x * blockDim.x;
-    for (int j = tid; j < v.ld; j += stride) {
-        v.cnt[j] = 0;
-        v.rank2[j] = -1;
-        v.srank[j] = -1;
-    }
-    for (int b = tid; b <= (1 << v.kbits); b += stride) v.bcnt[b] = 0;
-    if (v.qhist)
-        for (int b = tid; b < v.m * SORT_QB; b += stride) v.qhist[b] = 0;
-    if (v.dnz) {
-        // the block bitmap starts empty: only tiles with block pairs to test write bytes
-        const long long nb = (long long)v.NW * v.NB8;  // 8 T^2 bytes, T = ld / 256
-        uint2* z = reinterpret_cast<uint2*>(v.dnz);
-        for (long long e = tid; e < nb / 8; e += stride) z[e] = make_uint2(0u, 0u);
-    }
-    for (int wd = tid; wd < v.NW; wd += stride) {
-        const int lo = wd * 32;
-        uint32_t m = 0u;
-        if (lo + 32 <= v.n2)
-            m = 0xffffffffu;
-        else if (lo < v.n2)
-            m = (1u << (v.n2 - lo)) - 1u;
-        v.rem[wd] = m;
-        v.selmask[wd] = 0u;
-    }
-    for (int j = tid; j < v.w; j += stride) {
-        v.rho[j] = 0;
-        v.rhop[j] = 0;
-        v.cursor[j] = 0;
-    }
-    if (tid == 0) {
-        Ctrl* c = v.ctrl;
-        c->sbar = 0u;
-        c->pbar = 0ull;
-        c->prel = 0ull;
-        c->cum = 0;
-        c->l = -1;
-        c->nS = 0;
-        c->K = 0;
-        c->nFl = 0;
-        c->need_niche = 0;
-        c->fallback = 0;
-        c->passes = 0;
-        c->nT = 0;
-        c->Lstar = -1;
-        c->rlev = 0;
-        c->nsel = 0;
-        c->nlarge = 0;
-        c->npath = 0u;
-        c->ntile = 0;
-        for (int t = 0; t < 8; ++t) c->domstat[t] = 0ull;
-        c->peel_rows = 0u;
-        c->ncand = 0;
-        c->nslow = 0;
-        c->ext_done = 0u;
-        c->sort_done = 0u;
-        c->f0lo = 0xffffffffu;
-        c->f0hi = 0u;
-        c->thr_done = 0u;
-        for (int q = 0; q < NSGA3_FAST_M; ++q) {
-            c->omin[q] = 0xffffffffu;
-            c->omax[q] = 0u;
-        }
-        c->overflow = 0;
-        c->recheck_miss = 0;
-        for (int q = 0; q < v.m; ++q) c->zmin[q] = 0xffffffffu;
-    }
-}
 
 __global__ void k_check_finite(RunView v)
 {
@@ -271,15 +199,6 @@ __global__ void k_wait_probe(RunView v)
 cudaError_t launch_wait_probe(const RunView& v, cudaStream_t s)
 {
     k_wait_probe<<<1, 32, 0, s>>>(v);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_sel_reset(const RunView& v, cudaStream_t s)
-{
-    int n = v.ld > v.w ? v.ld : v.w;
-    int blocks = (n + 255) / 256;
-    if (blocks > 2048) blocks = 2048;
-    k_sel_reset<<<blocks, 256, 0, s>>>(v);
     return cudaGetLastError();
 }
 

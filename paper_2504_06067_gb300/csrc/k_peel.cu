@@ -53,14 +53,9 @@ __global__ void __launch_bounds__(PEEL_THREADS, STREAM ? 1 : 2) k_peel(RunView v
                 my_rank = __ldcg(&v.srank[j0 + tid]);
                 my_cnt = __ldcg(&v.cnt[j0 + tid]);
             }
-            // Dominators of a column have a sort key <= its key (k_sort.cu).  Keys
-            // are non-decreasing in position order and bcnt[b] is the end of key b,
-            // so the positions that can dominate this chunk end at bcnt[key of its
-            // last column].
-            const int jl = min(j0 + NSGA3_PEEL_COLS, v.n2) - 1;
-            int lim = 0;
-            if (jl >= j0) lim = (v.bcnt[v.skey[jl]] + 31) >> 5;
-            if (lim > v.NW) lim = v.NW;
+            // dominators of a column have a sort key <= its key: the chunk's row
+            // blocks end with its last column's key (k_sort.cu)
+            const int lim = j0 < v.n2 ? min((int)v.chunk_lim[chunk], v.NW) : 0;
 
             uint32_t rw = (tid < NSGA3_PEEL_COLS / 32) ? __ldcg(&v.rem[j0 / 32 + tid]) : 0u;
             const int any_rem = __syncthreads_or(rw != 0u);

@@ -16,25 +16,33 @@
 // ties and order inside a key do not matter: every pair that can dominate is
 // still tested exactly.
 // The thresholds (and, for m > 10, the f_0 range of the buckets) come from a
-// fixed sample of at most 8,192 points, every (n2 / 8,192)-th: they only
+// fixed sample of evenly spaced points (512; 8,192 for the range): they only
 // steer how well the blocks prune, and a value outside the sample's range
 // still gets a monotone key (levels count thresholds, buckets are clamped).
-//   k_sort_range    per-objective min / max of the sample (order-preserving atomics)
-//   k_sort_thr      per-objective histograms of the sample over [min, max] in
-//                   the order-preserving integer space (about equal steps of
-//                   relative size); the last CTA turns them into thresholds
-//   k_sort_hist     every point's key (kept in pkey) and the key histogram;
-//                   the last CTA turns it into offsets
-//   k_sort_scatter  perm[pos] = i, skey[pos] = key, Fp = F in key order
-//                   with -0.0 written as +0.0
+//   k_front         (m <= 10) the selection's reset and finite check, and per
+//                   objective one CTA that sorts its sampled values and takes
+//                   the quantiles: 4.4 us in place of the reset, the check,
+//                   the range and the histogram kernels (23 of 227 us at
+//                   m = 5, N = 10,628; 34 us at m = 10, N = 100,000)
+//   k_sort_range    (m > 10) min / max of f_0 over the sample
+//   k_sort_hist     every point's key (kept in pkey), key counts and counts of
+//                   groups of 32 keys
+//   k_sort_scatter  each CTA scans the group counts (nkeys / 32 of them) and a
+//                   point adds the counts before its key in its group, instead
+//                   of one last CTA scanning every key (both kernels 58 us for
+//                   65,536 keys and 200,000 points; now 28);
+//                   perm[pos] = i, skey[pos] = key, Fp = F in key order with
+//                   -0.0 written as +0.0; row limits of the peel's chunks
 #include "kernels.cuh"
 
 namespace {
 
 constexpr int SB = 1024;
-constexpr int SAMPLE = 8192;  // points that set the thresholds and the f_0 range
+constexpr int SAMPLE = 8192;  // points that set the f_0 range
+constexpr int FS = 512;       // points that set the level thresholds
+constexpr int KGROUP = 32;    // keys per group of the counting sort
 
-// stride of the threshold sample
+// stride of that sample
 __device__ __forceinline__ int sample_stride(int n2) { return n2 > SAMPLE ? (n2 + SAMPLE - 1) / SAMPLE : 1; }
 
 __device__ __forceinline__ int bucket_of(float f, float lo, float scale, int nb)
@@ -83,181 +91,191 @@ __device__ __forceinline__ uint32_t key_of(const RunView& v, const Ctrl* c, cons
     return key >> (lb * m - v.kbits);
 }
 
-// m <= 10: min / max of every objective; above, of f_0
+// m > 10: min / max of the sampled f_0
 __global__ void __launch_bounds__(SB) k_sort_range(RunView v)
 {
-    __shared__ uint32_t smin[NSGA3_FAST_M], smax[NSGA3_FAST_M];
     Ctrl* c = v.ctrl;
     if (read_status(c)) return;
-    const int m = v.m, mr = m <= NSGA3_FAST_M ? m : 1;
-    if (threadIdx.x < NSGA3_FAST_M) {
-        smin[threadIdx.x] = 0xffffffffu;
-        smax[threadIdx.x] = 0u;
-    }
-    __syncthreads();
-    uint32_t lo[NSGA3_FAST_M], hi[NSGA3_FAST_M];
-#pragma unroll
-    for (int q = 0; q < NSGA3_FAST_M; ++q) {
-        lo[q] = 0xffffffffu;
-        hi[q] = 0u;
-    }
+    uint32_t lo = 0xffffffffu, hi = 0u;
     const int st = sample_stride(v.n2);
     for (int i = (blockIdx.x * SB + threadIdx.x) * st; i < v.n2; i += gridDim.x * SB * st) {
-        const float* f = v.F + (size_t)i * m;
-#pragma unroll
-        for (int q = 0; q < NSGA3_FAST_M; ++q)
-            if (q < mr) {
-                const uint32_t o = f2ord(f[q] + 0.0f);
-                lo[q] = min(lo[q], o);
-                hi[q] = max(hi[q], o);
-            }
+        const uint32_t o = f2ord(v.F[(size_t)i * v.m] + 0.0f);
+        lo = min(lo, o);
+        hi = max(hi, o);
     }
-#pragma unroll
-    for (int q = 0; q < NSGA3_FAST_M; ++q)
-        if (q < mr) {
-            const uint32_t a = __reduce_min_sync(0xffffffffu, lo[q]), b = __reduce_max_sync(0xffffffffu, hi[q]);
-            if (lane_id() == 0) {
-                atomicMin(&smin[q], a);
-                atomicMax(&smax[q], b);
-            }
-        }
-    __syncthreads();
-    if (threadIdx.x < mr) {
-        atomicMin(&c->omin[threadIdx.x], smin[threadIdx.x]);
-        atomicMax(&c->omax[threadIdx.x], smax[threadIdx.x]);
-        if (threadIdx.x == 0) {
-            atomicMin(&c->f0lo, smin[0]);
-            atomicMax(&c->f0hi, smax[0]);
-        }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if (lane_id() == 0) {
+        atomicMin(&c->f0lo, lo);
+        atomicMax(&c->f0hi, hi);
     }
 }
 
-// bin of an order-preserving value o in [omin, omin + span) (span >= 1)
-__device__ __forceinline__ int qbin(uint32_t o, uint32_t omin, unsigned long long span)
+// The per-selection reset by the threads [t0, t0 + stride, ...) of a launch
+__device__ __forceinline__ void sel_reset(const RunView& v, int tid, int stride)
 {
-    return (int)(((unsigned long long)(o - omin) * SORT_QB) / span);
-}
-
-// m <= 10: level thresholds.  Bin e of objective q holds the values whose
-// order-preserving codes o satisfy floor((o - omin) QB / span) = e; the
-// threshold of level k + 1 is the largest value of the first bin whose
-// cumulative count reaches (k + 1) n2 / L.
-__global__ void __launch_bounds__(SB) k_sort_thr(RunView v)
-{
-    __shared__ int h[NSGA3_FAST_M * SORT_QB];
-    __shared__ unsigned ticket;
+    for (int j = tid; j < v.ld; j += stride) {
+        v.cnt[j] = 0;
+        v.rank2[j] = -1;
+        v.srank[j] = -1;
+    }
+    const int nk = 1 << v.kbits;
+    for (int b = tid; b < nk; b += stride) {
+        v.bcnt[b] = 0;
+        v.bcur[b] = 0;
+    }
+    for (int b = tid; b < nk / KGROUP; b += stride) v.bgrp[b] = 0;
+    if (v.dnz) {
+        // the block bitmap starts empty: only tiles with block pairs to test write bytes
+        const long long nb = (long long)v.NW * v.NB8;  // 8 T^2 bytes, T = ld / 256
+        uint2* z = reinterpret_cast<uint2*>(v.dnz);
+        for (long long e = tid; e < nb / 8; e += stride) z[e] = make_uint2(0u, 0u);
+    }
+    for (int wd = tid; wd < v.NW; wd += stride) {
+        const int lo = wd * 32;
+        uint32_t m = 0u;
+        if (lo + 32 <= v.n2)
+            m = 0xffffffffu;
+        else if (lo < v.n2)
+            m = (1u << (v.n2 - lo)) - 1u;
+        v.rem[wd] = m;
+        v.selmask[wd] = 0u;
+    }
+    for (int j = tid; j < v.w; j += stride) {
+        v.rho[j] = 0;
+        v.rhop[j] = 0;
+        v.cursor[j] = 0;
+    }
     Ctrl* c = v.ctrl;
-    if (read_status(c)) return;
-    const int m = v.m;
-    for (int b = threadIdx.x; b < m * SORT_QB; b += SB) h[b] = 0;
-    __syncthreads();
-    uint32_t omin[NSGA3_FAST_M];
-    unsigned long long span[NSGA3_FAST_M];
-#pragma unroll
-    for (int q = 0; q < NSGA3_FAST_M; ++q) {
-        omin[q] = q < m ? c->omin[q] : 0u;
-        span[q] = q < m ? (unsigned long long)(c->omax[q] - omin[q]) + 1ull : 1ull;
-    }
-    const int st = sample_stride(v.n2);
-    for (int i = (blockIdx.x * SB + threadIdx.x) * st; i < v.n2; i += gridDim.x * SB * st) {
-        const float* f = v.F + (size_t)i * m;
-#pragma unroll
-        for (int q = 0; q < NSGA3_FAST_M; ++q)
-            if (q < m) atomicAdd(&h[q * SORT_QB + qbin(f2ord(f[q] + 0.0f), omin[q], span[q])], 1);
-    }
-    __syncthreads();
-    for (int b = threadIdx.x; b < m * SORT_QB; b += SB)
-        if (h[b]) atomicAdd(&v.qhist[b], h[b]);
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) ticket = atomicAdd(&c->thr_done, 1u);
-    __syncthreads();
-    if (ticket != gridDim.x - 1) return;
-    __threadfence();
-    // last CTA: warp q scans objective q's bins (32 per lane)
-    const int lane = lane_id(), warp = threadIdx.x >> 5;
-    if (warp >= m) return;
-    const int q = warp, L = 1 << v.lbits;
-    constexpr int PER = SORT_QB / 32;
-    int loc[PER];
-    int s = 0;
-#pragma unroll
-    for (int t = 0; t < PER; ++t) {
-        loc[t] = __ldcg(&v.qhist[q * SORT_QB + lane * PER + t]);
-        s += loc[t];
-    }
-    int inc = s;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += y;
-    }
-    const int before = inc - s;
-    const int ns = (v.n2 + sample_stride(v.n2) - 1) / sample_stride(v.n2);  // points sampled
-    for (int k = 0; k + 1 < L; ++k) {
-        const long long target = ((long long)(k + 1) * ns + L - 1) / L;  // ceil((k + 1) ns / L)
-        int e = -1;
-        if (before < target && target <= inc) {
-            int run = before;
-            for (int t = 0; t < PER; ++t) {
-                run += loc[t];
-                if (run >= target) {
-                    e = lane * PER + t;
-                    break;
-                }
-            }
-        }
-        const unsigned who = __ballot_sync(0xffffffffu, e >= 0);
-        const int eb = __shfl_sync(0xffffffffu, e, who ? __ffs(who) - 1 : 0);
-        if (lane == 0) {
-            // largest code of bin eb: omin + ceil((eb + 1) span / QB) - 1
-            const unsigned long long hiw = ((unsigned long long)(eb + 1) * span[q] + SORT_QB - 1) / SORT_QB;
-            c->thr[q][k] = who ? ord2f(omin[q] + (uint32_t)(hiw - 1ull)) : ord2f(omin[q] + (uint32_t)(span[q] - 1ull));
-        }
+    if (tid < v.m) c->zmin[tid] = 0xffffffffu;
+    if (tid < 8) c->domstat[tid] = 0ull;
+    if (tid == 0) {
+        c->sbar = 0u;
+        c->pbar = 0ull;
+        c->prel = 0ull;
+        c->cum = 0;
+        c->l = -1;
+        c->nS = 0;
+        c->K = 0;
+        c->nFl = 0;
+        c->need_niche = 0;
+        c->fallback = 0;
+        c->passes = 0;
+        c->nT = 0;
+        c->Lstar = -1;
+        c->rlev = 0;
+        c->nsel = 0;
+        c->nlarge = 0;
+        c->npath = 0u;
+        c->ntile = 0;
+        c->peel_rows = 0u;
+        c->ncand = 0;
+        c->nslow = 0;
+        c->ext_done = 0u;
+        c->f0lo = 0xffffffffu;
+        c->f0hi = 0u;
+        c->overflow = 0;
+        c->recheck_miss = 0;
     }
 }
 
+__global__ void __launch_bounds__(256) k_sel_reset(RunView v)
+{
+    sel_reset(v, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+}
+
+// m <= 10.  CTA q < m: level thresholds of objective q.  A thread holds one
+// sampled value (order-preserving code); a bitonic sort, exchanges within a
+// warp by shuffles, wider ones through shared memory (10 of the 45 steps);
+// the threshold of level k + 1 is the smallest sampled value with at least
+// (k + 1) / L of the sample at or below it.  (Ranking each value by counting
+// the smaller ones took 11 us; a sample of 1,024 values 7.2.)  The other CTAs
+// reset the selection's buffers and (check != 0) look for non-finite
+// objectives.
+__global__ void __launch_bounds__(FS) k_front(RunView v, int check)
+{
+    Ctrl* c = v.ctrl;
+    const int tid = threadIdx.x;
+    if ((int)blockIdx.x >= v.m) {
+        const int t = ((int)blockIdx.x - v.m) * FS + tid, stride = ((int)gridDim.x - v.m) * FS;
+        sel_reset(v, t, stride);
+        if (check) {
+            const long long n = (long long)v.n2 * v.m;
+            bool bad = false;
+            for (long long e = t; e < n; e += stride) bad |= !isfinite(v.F[e]);
+            if (__any_sync(0xffffffffu, bad) && lane_id() == 0) set_status(c, DEV_ENONFINITE);
+        }
+        return;
+    }
+    __shared__ uint32_t x[2][FS];  // two buffers: one barrier per exchange
+    int buf = 0;
+    const int q = blockIdx.x, ns = min(v.n2, FS);
+    uint32_t a = 0xffffffffu;
+    if (tid < ns) a = f2ord(v.F[(size_t)((long long)tid * v.n2 / ns) * v.m + q] + 0.0f);
+#pragma unroll 1
+    for (int k = 2; k <= FS; k <<= 1) {
+        const bool up = (tid & k) == 0;  // this run's direction
+#pragma unroll 1
+        for (int o = k >> 1; o >= 32; o >>= 1) {
+            x[buf][tid] = a;
+            __syncthreads();
+            const uint32_t b = x[buf][tid ^ o];
+            buf ^= 1;
+            a = (((tid & o) == 0) == up) ? min(a, b) : max(a, b);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const uint32_t b = __shfl_xor_sync(0xffffffffu, a, o);
+            const uint32_t y = (((tid & o) == 0) == up) ? min(a, b) : max(a, b);
+            a = o < k ? y : a;
+        }
+    }
+    const int L = 1 << v.lbits;
+    // thread t holds the t-th smallest: rank t + 1 = ceil((k + 1) ns / L) sets threshold k
+    for (int k = 0; k + 1 < L; ++k)
+        if (tid + 1 == ((k + 1) * ns + L - 1) / L) c->thr[q][k] = ord2f(a);
+}
+
+// (the group counts of a CTA's points meet in shared memory first: most
+// points of a converged population share a few groups)
 __global__ void __launch_bounds__(SB) k_sort_hist(RunView v)
 {
-    __shared__ int scratch[40];
-    __shared__ unsigned ticket;
+    extern __shared__ int gcnt[];  // nkeys / KGROUP
     __shared__ float thr[NSGA3_FAST_M][SORT_LMAX];
     Ctrl* c = v.ctrl;
     if (read_status(c)) return;
-    if (threadIdx.x < NSGA3_FAST_M * SORT_LMAX)
-        thr[threadIdx.x / SORT_LMAX][threadIdx.x % SORT_LMAX] = c->thr[threadIdx.x / SORT_LMAX][threadIdx.x % SORT_LMAX];
+    if (v.m <= NSGA3_FAST_M) {
+        if (threadIdx.x < NSGA3_FAST_M * SORT_LMAX)
+            thr[threadIdx.x / SORT_LMAX][threadIdx.x % SORT_LMAX] = c->thr[threadIdx.x / SORT_LMAX][threadIdx.x % SORT_LMAX];
+    }
+    const int ng = (1 << v.kbits) / KGROUP;
+    for (int g = threadIdx.x; g < ng; g += SB) gcnt[g] = 0;
     __syncthreads();
-    for (int i = blockIdx.x * SB + threadIdx.x; i < v.n2; i += gridDim.x * SB) {
+    const int i = blockIdx.x * SB + threadIdx.x;
+    if (i < v.n2) {
         const uint32_t key = key_of(v, c, thr, i);
         v.pkey[i] = key;
         atomicAdd(&v.bcnt[key], 1);
+        atomicAdd(&gcnt[key / KGROUP], 1);
     }
-    __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) ticket = atomicAdd(&c->sort_done, 1u);
+    for (int g = threadIdx.x; g < ng; g += SB)
+        if (gcnt[g]) atomicAdd(&v.bgrp[g], gcnt[g]);
+}
+
+constexpr int TB = 512;  // threads of the scatter's CTAs
+
+// positions before key group g, for every group: an exclusive scan of the
+// group counts in shared memory (each CTA for itself)
+__device__ __forceinline__ void scan_groups(const RunView& v, int* off, int* scratch)
+{
+    const int ng = (1 << v.kbits) / KGROUP, per = (ng + TB - 1) / TB;
+    const int tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
+    for (int g = tid; g < ng; g += TB) off[g] = v.bgrp[g];
     __syncthreads();
-    if (ticket != gridDim.x - 1) return;
-    // last CTA: exclusive scan of the counts, a contiguous run per thread
-    __threadfence();
-    const int nk = 1 << v.kbits;  // >= 256: a multiple of 4, at most 2^16
-    const int per = ((nk + SB - 1) / SB + 3) & ~3;  // <= 64
-    const int b0 = min(nk, (int)threadIdx.x * per), b1 = min(nk, b0 + per);
-    // the thread's run read in batches of 8 vectors, each batch's loads
-    // issued before their first use
-    constexpr int RUN4 = ((1 << 16) / SB + 3) / 4, BAT = 8;
+    const int lo = min(ng, tid * per), hi = min(ng, lo + per);
     int s = 0;
-#pragma unroll
-    for (int h = 0; h < RUN4; h += BAT) {
-        int4 xs[BAT];
-#pragma unroll
-        for (int t = 0; t < BAT; ++t) {
-            const int b = b0 + 4 * (h + t);
-            xs[t] = b < b1 ? __ldcg(reinterpret_cast<const int4*>(v.bcnt + b)) : make_int4(0, 0, 0, 0);
-        }
-#pragma unroll
-        for (int t = 0; t < BAT; ++t) s += xs[t].x + xs[t].y + xs[t].z + xs[t].w;
-    }
-    const int lane = lane_id(), warp = threadIdx.x >> 5;
+    for (int g = lo; g < hi; ++g) s += off[g];
     int inc = s;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -266,71 +284,92 @@ __global__ void __launch_bounds__(SB) k_sort_hist(RunView v)
     }
     if (lane == 31) scratch[warp] = inc;
     __syncthreads();
-    if (warp == 0) {
-        const int x = scratch[lane];
-        int xi = x;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, xi, o);
-            if (lane >= o) xi += y;
-        }
-        scratch[lane] = xi - x;
+    int run = inc - s;
+    for (int t = 0; t < warp; ++t) run += scratch[t];
+    for (int g = lo; g < hi; ++g) {
+        const int x = off[g];
+        off[g] = run;
+        run += x;
     }
     __syncthreads();
-    int run = scratch[warp] + inc - s;
+}
+
+// Position of a point of key b, and where the positions of key b end: the
+// group's offset, the counts before b in the group (whole 16-byte loads) and
+// the order in which the key's points arrive.
+__device__ __forceinline__ int place(const RunView& v, const int* off, uint32_t b, int& end)
+{
+    const int g0 = (int)(b & ~(uint32_t)(KGROUP - 1));
+    int at = off[b / KGROUP], own = 0;
 #pragma unroll
-    for (int h = 0; h < RUN4; h += BAT) {
-        int4 xs[BAT];
+    for (int e = 0; e < KGROUP; e += 4) {
+        if (g0 + e > (int)b) break;
+        const int4 x = *reinterpret_cast<const int4*>(v.bcnt + g0 + e);
+        const int y[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
-        for (int t = 0; t < BAT; ++t) {
-            const int b = b0 + 4 * (h + t);
-            xs[t] = b < b1 ? __ldcg(reinterpret_cast<const int4*>(v.bcnt + b)) : make_int4(0, 0, 0, 0);
-        }
-#pragma unroll
-        for (int t = 0; t < BAT; ++t) {
-            const int4 x = xs[t];
-            int4 y;
-            y.x = run;
-            y.y = run + x.x;
-            y.z = y.y + x.y;
-            y.w = y.z + x.z;
-            run = y.w + x.w;
-            const int b = b0 + 4 * (h + t);
-            if (b < b1) *reinterpret_cast<int4*>(v.bcnt + b) = y;
+        for (int t = 0; t < 4; ++t) {
+            at += g0 + e + t < (int)b ? y[t] : 0;
+            own = g0 + e + t == (int)b ? y[t] : own;
         }
     }
-    if (threadIdx.x == 0) c->sort_done = 0u;
+    end = at + own;
+    return at + atomicAdd(&v.bcur[b], 1);
 }
 
-__global__ void __launch_bounds__(256) k_sort_scatter(RunView v)
+// dominators of a column have a key <= its key: the peel's chunk of columns
+// reads row blocks up to the end of its last column's key
+__device__ __forceinline__ void chunk_limit(const RunView& v, int pos, int end)
 {
-    Ctrl* c = v.ctrl;
-    if (read_status(c)) return;
-    const int i = blockIdx.x * 256 + threadIdx.x;
-    if (i >= v.n2) return;
-    const int m = v.m;
-    const uint32_t b = v.pkey[i];
-    const int pos = atomicAdd(&v.bcnt[b], 1);
-    v.perm[pos] = i;
-    v.skey[pos] = (uint32_t)b;
-    for (int q = 0; q < m; ++q) v.Fp[(size_t)pos * m + q] = v.F[(size_t)i * m + q] + 0.0f;
+    if ((pos & (NSGA3_PEEL_COLS - 1)) == NSGA3_PEEL_COLS - 1 || pos == v.n2 - 1)
+        v.chunk_lim[pos / NSGA3_PEEL_COLS] = (uint32_t)((end + 31) >> 5);
 }
 
-// m > NSGA3_FAST_M: a warp per point (lane 0 takes the position, the lanes
-// copy the row)
-__global__ void __launch_bounds__(256) k_sort_scatter_rows(RunView v)
+__global__ void __launch_bounds__(TB) k_sort_scatter(RunView v)
 {
+    extern __shared__ int goff[];  // nkeys / KGROUP
+    __shared__ int scratch[TB / 32];
+    __shared__ int spos[TB];
     Ctrl* c = v.ctrl;
     if (read_status(c)) return;
-    const int i = (blockIdx.x * 256 + threadIdx.x) >> 5;
+    scan_groups(v, goff, scratch);
+    const int m = v.m, i0 = blockIdx.x * TB, i = i0 + threadIdx.x;
+    if (i < v.n2) {
+        const uint32_t b = v.pkey[i];
+        int end;
+        const int pos = place(v, goff, b, end);
+        v.perm[pos] = i;
+        v.skey[pos] = b;
+        chunk_limit(v, pos, end);
+        spos[threadIdx.x] = pos;
+    }
+    __syncthreads();
+    // rows, consecutive threads on consecutive values
+    const int ne = min(TB, v.n2 - i0) * m;
+    for (int e = threadIdx.x; e < ne; e += TB) {
+        const int r = e / m;
+        v.Fp[(size_t)spos[r] * m + (e - r * m)] = v.F[(size_t)i0 * m + e] + 0.0f;
+    }
+}
+
+// m > NSGA3_FAST_M: a warp per point copies its row
+__global__ void __launch_bounds__(TB) k_sort_scatter_rows(RunView v)
+{
+    extern __shared__ int goff[];
+    __shared__ int scratch[TB / 32];
+    Ctrl* c = v.ctrl;
+    if (read_status(c)) return;
+    scan_groups(v, goff, scratch);
+    const int i = (blockIdx.x * TB + threadIdx.x) >> 5;
     if (i >= v.n2) return;
     const int lane = lane_id(), m = v.m;
     int pos = 0;
     if (lane == 0) {
         const uint32_t b = v.pkey[i];
-        pos = atomicAdd(&v.bcnt[b], 1);
+        int end;
+        pos = place(v, goff, b, end);
         v.perm[pos] = i;
-        v.skey[pos] = (uint32_t)b;
+        v.skey[pos] = b;
+        chunk_limit(v, pos, end);
     }
     pos = __shfl_sync(0xffffffffu, pos, 0);
     for (int q = lane; q < m; q += 32) v.Fp[(size_t)pos * m + q] = v.F[(size_t)i * m + q] + 0.0f;
@@ -338,24 +377,39 @@ __global__ void __launch_bounds__(256) k_sort_scatter_rows(RunView v)
 
 }  // namespace
 
+cudaError_t launch_front(const RunView& v, int num_sms, bool check, cudaStream_t s)
+{
+    if (v.m > NSGA3_FAST_M) {
+        const int n = v.ld > v.w ? v.ld : v.w;
+        int blocks = (n + 255) / 256;
+        if (blocks > 2048) blocks = 2048;
+        k_sel_reset<<<blocks, 256, 0, s>>>(v);
+        const cudaError_t e = cudaGetLastError();
+        return e != cudaSuccess || !check ? e : launch_check_finite(v, s);
+    }
+    long long n = (long long)v.n2 * v.m;  // at least a few elements per thread
+    int blocks = (int)((n + 4 * FS - 1) / (4 * FS));
+    if (blocks > 4 * num_sms) blocks = 4 * num_sms;
+    k_front<<<v.m + blocks, FS, 0, s>>>(v, check ? 1 : 0);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_sort(const RunView& v, int num_sms, cudaStream_t s)
 {
-    int blocks = (v.n2 + SB - 1) / SB;
-    if (blocks > num_sms) blocks = num_sms;
-    k_sort_range<<<blocks, SB, 0, s>>>(v);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    if (v.m <= NSGA3_FAST_M) {
-        k_sort_thr<<<blocks, SB, 0, s>>>(v);
-        e = cudaGetLastError();
+    if (v.m > NSGA3_FAST_M) {
+        int blocks = (v.n2 + SB - 1) / SB;
+        if (blocks > num_sms) blocks = num_sms;
+        k_sort_range<<<blocks, SB, 0, s>>>(v);
+        const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    k_sort_hist<<<blocks, SB, 0, s>>>(v);
-    e = cudaGetLastError();
+    const size_t sm = (size_t)((1 << v.kbits) / KGROUP) * sizeof(int);
+    k_sort_hist<<<(v.n2 + SB - 1) / SB, SB, sm, s>>>(v);
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (v.m > NSGA3_FAST_M)
-        k_sort_scatter_rows<<<(unsigned)(((long long)v.n2 * 32 + 255) / 256), 256, 0, s>>>(v);
+        k_sort_scatter_rows<<<(unsigned)(((long long)v.n2 * 32 + TB - 1) / TB), TB, sm, s>>>(v);
     else
-        k_sort_scatter<<<(v.n2 + 255) / 256, 256, 0, s>>>(v);
+        k_sort_scatter<<<(v.n2 + TB - 1) / TB, TB, sm, s>>>(v);
     return cudaGetLastError();
 }

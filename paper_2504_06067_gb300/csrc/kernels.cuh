@@ -26,7 +26,8 @@ cudaError_t small_init_attributes();
 // 0-1 knapsack workload (k_knapsack.cu): bits + repair + objectives
 cudaError_t launch_kp_init(const RunView& v, cudaStream_t s);
 cudaError_t launch_kp_vary_eval(const RunView& v, cudaStream_t s);
-cudaError_t launch_sel_reset(const RunView& v, cudaStream_t s);
+// reset of the selection's buffers, level thresholds (m <= 10), finite check
+cudaError_t launch_front(const RunView& v, int num_sms, bool check, cudaStream_t s);
 // the device-wait self-test (nsga3_wait_probe)
 cudaError_t launch_wait_probe(const RunView& v, cudaStream_t s);
 cudaError_t launch_check_finite(const RunView& v, cudaStream_t s);
