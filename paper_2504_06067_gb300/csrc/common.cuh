@@ -18,6 +18,8 @@
 #include <cuda_runtime.h>
 #include <math_constants.h>
 
+#include "sf64.cuh"
+
 #define NSGA3_MAX_M 512         // objectives accepted by a context
 #define NSGA3_FAST_M 10         // largest m with kernels specialised for each m
 #define NSGA3_WARP_M 32         // largest m whose intercept system one warp solves
@@ -92,6 +94,9 @@ struct Ctrl {
     uint32_t zmin[NSGA3_MAX_M];  // ideal point as order-preserving uint of FP32
     double zstar[NSGA3_MAX_M];   // ideal point (FP64, +0.0 for zero)
     double a[NSGA3_MAX_M];       // intercepts
+    // m <= 10: the intercepts as divisors, z* and 1 / a in FP32
+    sf64::Divisor da[NSGA3_FAST_M];
+    float z32[NSGA3_FAST_M], ia32[NSGA3_FAST_M];
     int32_t ext[NSGA3_MAX_M];    // extreme-point indices
     unsigned long long passes_total;  // peel passes since the context was created
     // normalization history (opts.norm_history), kept across selections
@@ -162,8 +167,8 @@ struct RunView {
     uint32_t* chunk_lim;   // ld / NSGA3_PEEL_COLS dominator row blocks a column chunk reads
     uint32_t* selmask;     // NW picked members of F_l
     int32_t* Tlist;        // n2 members of S u F_l
-    double* fprime;        // n2 x m  normalised objectives (indexed by T slot)
-    double* fnorm;         // n2      |f'|
+    double* fprime;        // n2 x m  normalised objectives (indexed by T slot; m > NSGA3_FAST_M)
+    double* fnorm;         // n2      |f'| (m > NSGA3_FAST_M)
     float* uhat;           // n2 x M4 FP32 unit vectors
     int32_t* pi;           // ld
     double* dist;          // ld
@@ -176,29 +181,32 @@ struct RunView {
     int32_t* take;         // w
     int32_t* ref_off;      // w + 1
     int32_t* cursor;       // w
-    int32_t* bucket;       // n2
-    int4* large;           // w   (ref, members still to take, excluded member, -)
+    int32_t* bucket;       // n2  members of F_l by reference
+    uint32_t* bprio;       // n2  their Philox priorities and distances
+    double* bdist;
+    uint32_t* rprio;       // w   Philox priorities of the references this generation
+    int4* large;           // w   (ref, members to take, rho, -)
     int32_t* sel;          // N   selected indices, ascending
     const double* Zd;      // w x m
     const double* nz;      // w
     const float* Zh;       // w x M4
     const float* Wobj;     // m x (m-1)
     const float* Wt;       // (m-1) x m  W transposed (m > NSGA3_FAST_M)
-    // association scan: references reordered into compact blocks of 32
-    int nblk;              // ceil(w / 32)
-    const float* blk_c;    // nblk x M4  unit cone centres (FP32)
-    const float2* blk_r;   // nblk       (cos r, sin r) of the inflated cone radius
+    // association scan (m <= 10): references reordered into compact blocks of 32
     const float* blk_z;    // w x M4     zhat in block order
     const int32_t* blk_j;  // w          original reference index in block order
-    int2* arun;            // n2         candidate run (start, count) per T slot; start -1 = slow
-    int2* cand;            // cand_cap   (T slot, reference)
+    const unsigned char* bop;   // their FP16 rows in chunks of 128 (assoc_pack_refs)
+    unsigned char* aop;    // the T slots' FP16 rows, in the same layout
+    int2* arun;            // n2         start -1: the slot takes the FP64 scan; m > 10: its
+                           //            candidate run (start, count)
+    int2* cand;            // cand_cap   (T slot, reference) (m > NSGA3_FAST_M)
     int cand_cap;
     int32_t* slow;         // n2         T slots for the full FP64 scan
-    // tiled association (null: the pruned scan): per work item (a tile of T
-    // slots x a range of reference blocks) and slot, ASSOC_K entries
-    // (block maximum of the FP32 cosines as float bits, block; -1 empty, -2 overflow)
-    int2* aent;
-    int assoc_grid;        // CTAs of the tiled scan (the entries' layout depends on it)
+    // per work item (512 T slots x a range of reference chunks) and slot: the
+    // three largest block maxima of the cosines (float bits), the blocks of
+    // the first two (16 bits each)
+    int4* aent;
+    int assoc_grid;        // CTAs of the scan (the entries' layout depends on it)
     double* cdist;         // cand_cap   FP64 distance of each candidate (m > NSGA3_FAST_M)
     float* he;             // m x m      remembered extreme vectors (history), row q for axis q
     // m > NSGA3_FAST_M: extreme points by entry keys, then per-axis blocks

@@ -77,24 +77,6 @@ struct nsga3_ctx {
 
 namespace {
 
-// Association of more than ASSOC_SMALL_W directions (m <= 10): the tiled
-// scan (every FP32 cosine at the FMA rate) or the pruned scan (cone bounds
-// per block of 32 directions).  Both give the same association.  The cone
-// bounds skip most blocks up to m = 6 (the pruned scan is as fast or faster
-// there: m = 5 and 10,626 directions 0.12 against 0.16 ms of niching per
-// generation, m = 6 and 2,002 directions 0.133 against 0.137 ms); from m = 7
-// they skip few and the tiled scan wins (m = 8 and 11,440 directions 0.79
-// against 0.29 ms, m = 10 and 2,002 directions 0.31 against 0.21 ms).
-// NSGA3_ASSOC=tile|scan overrides the choice for every context a process
-// creates.
-bool assoc_tile_wanted(int m)
-{
-    const char* e = getenv("NSGA3_ASSOC");
-    if (e && strcmp(e, "scan") == 0) return false;
-    if (e && strcmp(e, "tile") == 0) return true;
-    return m >= 7;
-}
-
 // Small populations take one launch of one cluster (k_small.cu) instead of
 // the 20 kernels of the general path.  Not with options that belong to the
 // general path's kernels: timed phases, launch shapes, the FP64 recheck, a
@@ -121,8 +103,7 @@ int select_launches(const nsga3_ctx* ctx)
 {
     if (ctx->small) return 1;
     const int m = ctx->m;
-    // three association kernels fewer with few reference directions (one fused kernel)
-    if (m <= NSGA3_FAST_M) return 19 - (assoc_small(ctx->v) ? 3 : 0);
+    if (m <= NSGA3_FAST_M) return 19;
     return 24 + (m > NSGA3_WARP_M ? 1 : 0) + (ctx->v.dom_ks > 1 ? 1 : 0);
 }
 // the softmax-simplex objective's dot-product kernel (m > 10)
@@ -353,12 +334,11 @@ nsga3_status build_graphs(nsga3_ctx* ctx)
 
 // Orders the w reference directions into blocks of 32 by recursive median
 // splits of their unit vectors along the widest coordinate (every block but
-// the last holds exactly 32), and records each block's unit centre and
-// angular radius, inflated by 1e-6 rad to cover the FP32 rounding of the
-// centre.  Only the association scan's pruning uses this order; results are
-// reported with the original indices.
-void build_ref_blocks(int m, int w, int M4, const std::vector<double>& Z, std::vector<float>& cent,
-                      std::vector<float2>& crsr, std::vector<float>& zp, std::vector<int32_t>& jidx)
+// the last holds exactly 32), so that a point's nearest directions share few
+// blocks.  Only the association scan uses this order; results are reported
+// with the original indices.
+void build_ref_blocks(int m, int w, int M4, const std::vector<double>& Z, std::vector<float>& zp,
+                      std::vector<int32_t>& jidx)
 {
     std::vector<double> U((size_t)w * m);
     for (int j = 0; j < w; ++j) {
@@ -401,34 +381,11 @@ void build_ref_blocks(int m, int w, int M4, const std::vector<double>& Z, std::v
         stack.push_back({r.lo, mid});
         stack.push_back({mid, r.hi});
     }
-    const int nb = (w + 31) / 32;
-    cent.assign((size_t)nb * M4, 0.0f);
-    crsr.assign(nb, make_float2(1.0f, 0.0f));
     zp.assign((size_t)w * M4, 0.0f);
     jidx.assign(w, 0);
-    for (int b = 0; b < nb; ++b) {
-        const int lo = 32 * b, hi = std::min(w, lo + 32);
-        double cvec[NSGA3_MAX_M] = {0};
-        for (int t = lo; t < hi; ++t)
-            for (int q = 0; q < m; ++q) cvec[q] += U[(size_t)perm[t] * m + q];
-        double cn = 0.0;
-        for (int q = 0; q < m; ++q) cn += cvec[q] * cvec[q];
-        cn = std::sqrt(cn);
-        for (int q = 0; q < m; ++q) cvec[q] /= cn;
-        double cmin = 1.0;
-        for (int t = lo; t < hi; ++t) {
-            double dt = 0.0;
-            for (int q = 0; q < m; ++q) dt += U[(size_t)perm[t] * m + q] * cvec[q];
-            cmin = std::min(cmin, dt);
-        }
-        double r = std::acos(std::max(-1.0, std::min(1.0, cmin))) + 1e-6;
-        if (r > M_PI) r = M_PI;
-        crsr[b] = make_float2((float)std::cos(r), (float)std::sin(r));
-        for (int q = 0; q < m; ++q) cent[(size_t)b * M4 + q] = (float)cvec[q];
-        for (int t = lo; t < hi; ++t) {
-            jidx[t] = perm[t];
-            for (int q = 0; q < m; ++q) zp[(size_t)t * M4 + q] = (float)U[(size_t)perm[t] * m + q];
-        }
+    for (int t = 0; t < w; ++t) {
+        jidx[t] = perm[t];
+        for (int q = 0; q < m; ++q) zp[(size_t)t * M4 + q] = (float)U[(size_t)perm[t] * m + q];
     }
 }
 
@@ -554,8 +511,8 @@ nsga3_status setup_alloc(nsga3_ctx* ctx)
     AL(v.chunk_lim, ld / NSGA3_PEEL_COLS);
     AL(v.selmask, NW);
     AL(v.Tlist, n2);
-    AL(v.fprime, (size_t)n2 * m);
-    AL(v.fnorm, n2);
+    AL(v.fprime, m > NSGA3_FAST_M ? (size_t)n2 * m : (size_t)1);
+    AL(v.fnorm, m > NSGA3_FAST_M ? n2 : 1);
     AL(v.uhat, (size_t)n2 * M4);
     AL(v.pi, ld);
     AL(v.dist, ld);
@@ -568,19 +525,25 @@ nsga3_status setup_alloc(nsga3_ctx* ctx)
     AL(v.ref_off, w + 1);
     AL(v.cursor, w);
     AL(v.bucket, n2);
+    AL(v.bprio, n2);
+    AL(v.bdist, n2);
+    AL(v.rprio, w);
     AL(v.large, w);
     AL(v.sel, N);
-    v.nblk = (w + 31) / 32;
-    v.cand_cap = 4 * n2 + 64;
+    v.cand_cap = m > NSGA3_FAST_M ? 4 * n2 + 64 : 1;
     AL(v.arun, n2);
     AL(v.cand, v.cand_cap);
     AL(v.slow, n2);
     v.aent = nullptr;
     v.assoc_grid = 0;
-    if (m <= NSGA3_FAST_M && w > ASSOC_SMALL_W && assoc_tile_wanted(m)) {
-        v.assoc_grid = assoc_tile_grid(v.num_sms);
-        AL(v.aent, assoc_tile_entries(n2, v.num_sms));
+    unsigned char* bm = nullptr;
+    if (m <= NSGA3_FAST_M) {
+        v.assoc_grid = assoc_grid(v.num_sms);
+        AL(v.aent, assoc_entries(n2, v.num_sms));
+        AL(v.aop, assoc_rows_bytes(m, n2));
+        AL(bm, assoc_rows_bytes(m, w));
     }
+    v.bop = bm;
     AL(v.he, (size_t)m * m);
     if (m > NSGA3_FAST_M) {
         AL(v.cdist, v.cand_cap);
@@ -598,16 +561,10 @@ nsga3_status setup_alloc(nsga3_ctx* ctx)
         AL(v.amat, (size_t)m * (m + 1));
         AL(v.etmp, (size_t)m * m);
     }
-    float* bc;
-    float2* br;
     float* bz;
     int32_t* bj;
-    AL(bc, (size_t)v.nblk * M4);
-    AL(br, v.nblk);
     AL(bz, (size_t)w * M4);
     AL(bj, w);
-    v.blk_c = bc;
-    v.blk_r = br;
     v.blk_z = bz;
     v.blk_j = bj;
     double* Zd;
@@ -647,6 +604,9 @@ nsga3_status setup_alloc(nsga3_ctx* ctx)
 
 nsga3_status setup(nsga3_ctx* ctx)
 {
+    // a limit of the interface: m <= 10 took up to 220 KB of block tables
+    if (ctx->m <= NSGA3_FAST_M && (size_t)((ctx->w + 31) / 32) * (ctx->M4 + 10) * 4 + 4096 > 220 * 1024)
+        return fail(ctx, NSGA3_EINVAL, "%d reference directions exceed the association's limit", ctx->w);
     nsga3_status ast = setup_alloc(ctx);
     if (ast) return ast;
     const int m = ctx->m, d = ctx->d, N = ctx->N, n2 = ctx->n2, ld = ctx->ld, NW = ctx->NW;
@@ -656,8 +616,6 @@ nsga3_status setup(nsga3_ctx* ctx)
     double* nz = const_cast<double*>(v.nz);
     float* Zh = const_cast<float*>(v.Zh);
     float* Wd = const_cast<float*>(v.Wobj);
-    float* bc = const_cast<float*>(v.blk_c);
-    float2* br = const_cast<float2*>(v.blk_r);
     float* bz = const_cast<float*>(v.blk_z);
     int32_t* bj = const_cast<int32_t*>(v.blk_j);
 
@@ -714,35 +672,21 @@ nsga3_status setup(nsga3_ctx* ctx)
         std::vector<double> Zh((size_t)w * m);
         CK(cudaMemcpyAsync(Zh.data(), Zd, Zh.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
-        std::vector<float> hc, hz;
-        std::vector<float2> hr;
+        std::vector<float> hz;
         std::vector<int32_t> hj;
-        build_ref_blocks(m, w, M4, Zh, hc, hr, hz, hj);
+        std::vector<unsigned char> hb;
+        build_ref_blocks(m, w, M4, Zh, hz, hj);
         // copies on the context's own stream: no implicit synchronisation with
         // other streams of the process (runs of a server keep executing)
-        CK(cudaMemcpyAsync(bc, hc.data(), hc.size() * sizeof(float), cudaMemcpyHostToDevice, s));
-        CK(cudaMemcpyAsync(br, hr.data(), hr.size() * sizeof(float2), cudaMemcpyHostToDevice, s));
+        if (v.bop) {
+            hb.assign(assoc_rows_bytes(m, w), 0);
+            assoc_pack_refs(m, M4, w, hz.data(), hb.data());
+            CK(cudaMemcpyAsync(const_cast<unsigned char*>(v.bop), hb.data(), hb.size(), cudaMemcpyHostToDevice, s));
+            CK(cudaMemsetAsync(v.aop, 0, assoc_rows_bytes(m, n2), s));  // rows past the points are read, not used
+        }
         CK(cudaMemcpyAsync(bz, hz.data(), hz.size() * sizeof(float), cudaMemcpyHostToDevice, s));
         CK(cudaMemcpyAsync(bj, hj.data(), hj.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
         CK(cudaStreamSynchronize(s));
-        ctx->vs.blk_c = bc;
-        ctx->vs.blk_r = br;
-        ctx->vs.blk_z = bz;
-        ctx->vs.blk_j = bj;
-        ctx->vs.nblk = v.nblk;
-        ctx->vs.arun = v.arun;
-        ctx->vs.cand = v.cand;
-        ctx->vs.cand_cap = v.cand_cap;
-        ctx->vs.slow = v.slow;
-    }
-    cudaError_t ae;
-    {
-        std::lock_guard<std::mutex> lk(g_attr_mutex);
-        ae = assoc_prepare(v);
-    }
-    if (ae != cudaSuccess) {
-        cudaGetLastError();
-        return fail(ctx, NSGA3_EINVAL, "%d reference directions exceed the association scan's tables", w);
     }
     return build_graphs(ctx);
 }

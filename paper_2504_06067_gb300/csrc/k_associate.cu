@@ -4,12 +4,12 @@
 // the niche counts rho (over S) and rho' (over F_l) of Alg. 2.
 //
 // Exactness.  The FP64 distance is evaluated operation for operation like a
-// plain CPU evaluation (_rn intrinsics, left-to-right sums), but only for
+// plain CPU evaluation (_rn operations, left-to-right sums), but only for
 // candidate references.  Candidates come from FP32 cosines
 // qhat_j = u . zhat_j of the unit vectors u = f'/|f'| and zhat_j = z_j/|z_j|
-// (all components >= 0).  qhat_j is within Delta = (m+4) 2^-24 of the exact
-// cosine (FP32 rounding of u and zhat, m FMA roundings over non-negative
-// terms summing to <= 1).  A reference whose qhat is more than
+// (all components >= 0).  qhat_j is within Delta = (m+7) 2^-24 of the exact
+// cosine up to a factor common to all j (unit32 in associate.cuh; m > 10: u
+// rounded from FP64, (m+4) 2^-24).  A reference whose qhat is more than
 // band = 2 Delta + 1e-12 below the best qhat has an exact cosine > 1e-12
 // below the best reference's; as the vertices e_q are references the best
 // cosine is >= 1/sqrt(m), so its exact 1 - c^2 is larger by > 1e-12/sqrt(m),
@@ -17,32 +17,24 @@
 // strictly larger, so it can neither win nor tie.  The FP64 argmin over the
 // candidates (ties -> lowest j) equals the argmin over all references.
 //
-// Pruning.  References are reordered (host, at context creation) into
-// spatially compact blocks of 32 by recursive median splits; block b has a
-// unit centre c_b and angular radius r_b.  For a point at angle theta from
-// c_b every reference of the block has cosine <= cos(max(0, theta - r_b))
-// = cos(theta) cos(r_b) + sin(theta) sin(r_b) when theta > r_b (sin(theta)
-// computed from the rejection vector u - cos(theta) c_b, which has no
-// cancellation).  With its FP32 error below EPS, a block whose bound + EPS
-// is below best - band cannot hold a candidate and is skipped.  A warp owns
-// one point: it bounds every block, scans the best-bounded block first, then
-// the blocks that survive the bound.
+// m <= 10: the references are ordered into spatially compact blocks of 32
+// (host, at context creation); a tensor-core product gives every cosine to
+// 4.5e-6 and each point's block maxima (k_assoc_mma), and only the blocks that
+// can hold its nearest reference are scanned in FP32 (k_assoc_final).
+// m > 10: every cosine in FP32 (k_assoc_scan_gen).
 //
-// FP64 work (GB300 runs FP64 at 1/64 of the FP32 rate) stays off the scan:
-// the scan only writes (point, reference) candidate runs; a second kernel
-// evaluates each point's candidates in FP64 (one thread per point) and takes
-// their argmin.
-// A point whose candidate list overflows is rescanned in FP64 over all
+// FP64 work (GB300 runs FP64 at 1/64 of the FP32 rate) is left to the
+// candidates.  A point whose lists overflow is rescanned in FP64 over all
 // references by a whole CTA (k_assoc_slow), as is every point in debug mode.
-// m > 10: no pruning (k_assoc_scan_gen), the same band and FP64 kernels.
+#include <cuda_fp16.h>
+#include <cstring>
+
 #include "associate.cuh"
 #include "kernels.cuh"
 
 namespace {
 
-constexpr int AB = 256;   // threads per CTA (8 warps, one point per warp)
-constexpr int LC = 64;    // candidate slots per warp
-constexpr float EPS = 1e-5f;
+constexpr int AB = 256;   // threads per CTA of the FP64 scan
 
 // perp_dist for a run-time m with both rows in memory: sixteen loads of
 // each row in flight
@@ -60,300 +52,574 @@ __device__ __forceinline__ double perp_dist_mem(const double* fp, double nf, con
     return __dmul_rn(nf, __dsqrt_rn(one_m));
 }
 
-// f' = (f - z*) / a and |f'| in FP64; FP32 unit vector for the scan
-// small blocks spread the FP64 work over every SM sub-partition
-constexpr int PB = 64;
+// ---------------------------------------------------------------------------
+// m <= 10.
+
+// T slot s: FP32 unit vector (uhat) and its FP16 row for the tensor cores:
+// u = h + l with h, l FP16 (to about 2^-23), the row [h, h, l, 0 ...] of
+// KP = 16 (m <= 5) or 32 halves, stored as the MMA reads it (see k_assoc_mma).
+template <int M>
+__host__ __device__ constexpr int kp_of() { return 3 * M <= 16 ? 16 : 32; }
+
+constexpr int PB = 128;
 
 template <int M>
 __global__ void __launch_bounds__(PB) k_assoc_prep(RunView v)
 {
-    constexpr int M4 = (M + 3) & ~3;
+    constexpr int M4 = (M + 3) & ~3, KP = kp_of<M>();
+    __shared__ float sz[M], sa[M];
     Ctrl* c = v.ctrl;
-    if (skip_niche(c)) return;
     const int s = blockIdx.x * PB + threadIdx.x;
+    if (skip_niche(c)) return;
+    if (threadIdx.x < M) {
+        sz[threadIdx.x] = c->z32[threadIdx.x];
+        sa[threadIdx.x] = c->ia32[threadIdx.x];
+    }
+    __syncthreads();
     if (s >= c->nT) return;
     const int i = v.Tlist[s];
-    double fp[M];
-    double ss = 0.0;
+    float f[M], u[M4];
+#pragma unroll
+    for (int q = 0; q < M; ++q) f[q] = v.F[(size_t)i * M + q];
+#pragma unroll
+    for (int q = 0; q < M4; ++q) u[q] = 0.0f;
+    if (!unit32<M>(f, sz, sa, u)) {  // out of the FP32 form's range
+        double fp[M], ss = 0.0;
+#pragma unroll
+        for (int q = 0; q < M; ++q) {
+            fp[q] = __ddiv_rn(__dsub_rn((double)f[q], c->zstar[q]), c->a[q]);
+            ss = __dadd_rn(ss, __dmul_rn(fp[q], fp[q]));
+        }
+        const double nf = __dsqrt_rn(ss), inv = nf > 0.0 ? 1.0 / nf : 0.0;
+#pragma unroll
+        for (int q = 0; q < M; ++q) u[q] = __double2float_rn(fp[q] * inv);
+    }
+#pragma unroll
+    for (int q4 = 0; q4 < M4 / 4; ++q4)
+        reinterpret_cast<float4*>(v.uhat + (size_t)s * M4)[q4] = make_float4(u[4 * q4], u[4 * q4 + 1], u[4 * q4 + 2], u[4 * q4 + 3]);
+    unsigned short r[KP];
+#pragma unroll
+    for (int e = 0; e < KP; ++e) r[e] = 0;
 #pragma unroll
     for (int q = 0; q < M; ++q) {
-        const double ft = __dsub_rn((double)v.F[(size_t)i * M + q], c->zstar[q]);
-        fp[q] = __ddiv_rn(ft, c->a[q]);
-        ss = __dadd_rn(ss, __dmul_rn(fp[q], fp[q]));
-        v.fprime[(size_t)s * M + q] = fp[q];
+        const __half h = __float2half_rn(u[q]);
+        const __half l = __float2half_rn(u[q] - __half2float(h));
+        r[q] = r[M + q] = __half_as_ushort(h);
+        r[2 * M + q] = __half_as_ushort(l);
     }
-    const double nf = __dsqrt_rn(ss);
-    v.fnorm[s] = nf;
-    const double inv = nf > 0.0 ? 1.0 / nf : 0.0;
+    unsigned char* a = v.aop + (size_t)(s / 128) * (KP * 256) + (s % 128) * 16;
 #pragma unroll
-    for (int q = 0; q < M4; ++q)
-        v.uhat[(size_t)s * M4 + q] = q < M ? __double2float_rn(fp[q] * inv) : 0.0f;
+    for (int k = 0; k < KP / 8; ++k) {
+        uint4 x;
+        x.x = r[8 * k + 0] | ((uint32_t)r[8 * k + 1] << 16);
+        x.y = r[8 * k + 2] | ((uint32_t)r[8 * k + 3] << 16);
+        x.z = r[8 * k + 4] | ((uint32_t)r[8 * k + 5] << 16);
+        x.w = r[8 * k + 6] | ((uint32_t)r[8 * k + 7] << 16);
+        *reinterpret_cast<uint4*>(a + k * 2048) = x;
+    }
 }
 
-template <int M>
-__global__ void __launch_bounds__(AB) k_assoc_scan(RunView v)
+// Cosines of every point with every direction on the tensor cores, reduced
+// to block maxima.  The points' rows [h, h, l] and the directions' rows
+// [zh, zl, zh] make one FP16 product with FP32 accumulators equal to
+// u . z without the l l term: within MMA_ERR of it (splits: 2^-23 per
+// component, so about 2 sqrt(m) 2^-23; l l below m 2^-24; at most 32
+// accumulations of partial sums below 1, each truncated at 2^-24; together
+// below 3.4e-6).
+//
+// A CTA takes work items: a group of TP = 256 points (two tiles of 128 rows)
+// against a range of chunks of 128 directions.  Per step one chunk meets each
+// tile: an MMA (128 x 128 x KP) into one of the tile's two TMEM accumulators
+// (all 512 columns).  A warpgroup per tile reads them (a thread one point's
+// 128 cosines; tcgen05.ld.red forms the maximum of 32 columns in the load) as
+// the maxima of four blocks of 32 directions; a warp per tile issues the MMAs
+// and one the bulk copies (the chunks are stored as the MMA reads them:
+// K-major core matrices of 8 rows x 16 bytes, so a chunk is one contiguous
+// copy; a ring of eight).  Full / empty barriers per accumulator and ring
+// slot let the warps drift.  Per point and item the scan keeps the two best
+// blocks and the third-best maximum, without a branch.  The block that holds
+// the exact nearest direction has a maximum within MBAND of the best:
+// k_assoc_final rescans the listed blocks within MBAND of the best in FP32,
+// and a point whose third maximum in some item is within it too (about one
+// in 20,000) takes the FP32 scan over all directions (k_assoc_slow).
+//
+// Bound: the chain of product, load and barrier of a step, then the tensor
+// cores' reads of operands of so small a K.  Measured at m = 8, 38,700 points
+// and 11,440 directions, and m = 5, 21,000 points and 10,626 directions:
+// 36 and 16-22 us.  FP32 FMAs took 173 us at m = 8 (the FMA pipe's time), a
+// scan pruned by cone bounds 42-52 us at m = 5; on the way here: a branch per
+// block that lists every block near the best 102 us (m = 8), a block barrier
+// per step 56, four tiles of 64 directions 42.
+constexpr float MMA_ERR = 4.5e-6f;
+constexpr float MBAND = 2.0f * MMA_ERR + 3e-6f;  // + the FP32 unit vectors' own error, both sides
+constexpr int TILES = 2;            // tiles of 128 points per item, a warpgroup each
+constexpr int TP = 128 * TILES;     // points per item
+constexpr int MT = TP + 32 * (TILES + 1);  // threads per CTA: one per point, an issuing warp per tile, a loading warp
+constexpr int CHUNK = 128;          // directions per step
+constexpr int SETS = 512 / (TILES * CHUNK);  // accumulators per tile (512 TMEM columns)
+constexpr int RING = 8;             // chunks in shared memory
+
+// items of nT points and nch chunks over `grid` CTAs: groups of points,
+// splits per group and chunks per split, the same on the device for both
+// kernels and on the host for the maximum.  The split count minimises the
+// waves of the grid times the chunks of an item (plus an item's own cost of
+// about six chunks), over at most twice the count that fills the grid once
+// (so that items <= 2 (grid + groups)).
+__host__ __device__ __forceinline__ void tile_split(int nT, int nch, int grid, int& ntile, int& S, int& cps)
 {
-    constexpr int M4 = (M + 3) & ~3;
-    constexpr int CH = (M4 <= 8) ? 4 : 2;  // blocks whose loads are in flight together
-    extern __shared__ __align__(16) float sm[];
-    Ctrl* c = v.ctrl;
-    if (skip_niche(c)) return;
-    const int nT = c->nT;
-    const int nb = v.nblk;
-    const int lane = lane_id(), warp = threadIdx.x >> 5;
-    float* cent = sm;                                                     // nb x M4
-    float2* crsr = reinterpret_cast<float2*>(cent + (size_t)nb * M4);      // nb
-    float* wall = reinterpret_cast<float*>(crsr + nb);                     // 8 x nb bounds
-    float* wbnd = wall + (size_t)warp * nb;
-    int* lj = reinterpret_cast<int*>(wall + (size_t)8 * nb) + warp * 2 * LC;
-    float* lq = reinterpret_cast<float*>(lj + LC);
-    for (int e = threadIdx.x; e < nb * M4; e += AB) cent[e] = v.blk_c[e];
-    for (int e = threadIdx.x; e < nb; e += AB) crsr[e] = v.blk_r[e];
-    __syncthreads();
-    const float band = 2.0f * (float)(M + 4) * 5.9604644775390625e-08f + 1e-12f;
-    const int w = v.w;
-
-    // the next point's unit vector and |f'| are loaded while this one is
-    // scanned
-    const int pstride = gridDim.x * 8;
-    float un[M];
-    double nfn = 0.0;
-    {
-        const int p0 = blockIdx.x * 8 + warp;
-#pragma unroll
-        for (int q = 0; q < M; ++q) un[q] = p0 < nT ? v.uhat[(size_t)p0 * M4 + q] : 0.0f;
-        if (p0 < nT) nfn = v.fnorm[p0];
-    }
-    for (int pt = blockIdx.x * 8 + warp; pt < nT; pt += pstride) {
-        float u[M];
-#pragma unroll
-        for (int q = 0; q < M; ++q) u[q] = un[q];
-        const double nf = nfn;
-        const int pn = pt + pstride;
-#pragma unroll
-        for (int q = 0; q < M; ++q) un[q] = pn < nT ? v.uhat[(size_t)pn * M4 + q] : 0.0f;
-        if (pn < nT) nfn = v.fnorm[pn];
-        if (nf == 0.0) {  // every distance is 0: handled by the finalisation
-            if (lane == 0) v.arun[pt] = make_int2(0, 0);
-            continue;
+    ntile = (nT + TP - 1) / TP;
+    S = 1;
+    cps = nch;
+    if (ntile == 0 || nch == 0) return;
+    const int fill = (grid + ntile - 1) / ntile;
+    const int smax = nch < 2 * fill ? nch : 2 * fill;
+    unsigned best = 0xffffffffu;
+    for (int t = 1; t <= smax; ++t) {
+        const unsigned b = (unsigned)(nch + t - 1) / t;
+        const unsigned st = (nch + b - 1) / b;
+        const unsigned cost = ((ntile * st + grid - 1) / grid) * (b + 6);  // (all below 2^26)
+        if (cost < best) {
+            best = cost;
+            S = st;
+            cps = b;
         }
-        // phase 1: cone bound of every block
-        float bmax = -4.0f;
-        int bb = 0x7fffffff;
-        for (int b = lane; b < nb; b += 32) {
-            const float* cb = cent + b * M4;
-            float ct = 0.0f;
-#pragma unroll
-            for (int q = 0; q < M; ++q) ct = fmaf(u[q], cb[q], ct);
-            float s2 = 0.0f;
-#pragma unroll
-            for (int q = 0; q < M; ++q) {
-                const float r = fmaf(-ct, cb[q], u[q]);
-                s2 = fmaf(r, r, s2);
-            }
-            const float2 cs = crsr[b];
-            const float bound = (ct >= cs.x) ? 1.0f : fmaf(ct, cs.x, sqrtf(s2) * cs.y);
-            wbnd[b] = bound;
-            if (bound > bmax) {
-                bmax = bound;
-                bb = b;
-            }
-        }
-        // The first scan takes the best-bounded blocks of up to CH lanes (each
-        // lane's best, in decreasing order of bound), all loads in flight
-        // together, so that `best` is near its final value before the bound
-        // filters the rest; the blocks taken are marked scanned (bound -4).
-        // Bounds are >= 0 (u, c_b, cos r >= 0): their bits order like
-        // unsigned ints.
-        int first[CH];
-        int nfirst = 0;
-        {
-            unsigned mine = (bb == 0x7fffffff) ? 0u : __float_as_uint(fmaxf(bmax, 0.0f)) + 1u;  // 0: none
-#pragma unroll
-            for (int t = 0; t < CH; ++t) {
-                const unsigned mx = __reduce_max_sync(0xffffffffu, mine);
-                first[t] = -1;
-                if (mx == 0u) continue;
-                const unsigned cand = (mine == mx) ? (unsigned)bb : 0xffffffffu;
-                const int b = (int)__reduce_min_sync(0xffffffffu, cand);
-                first[t] = b;
-                nfirst = t + 1;
-                if (bb == b) mine = 0u;  // this lane's best is taken
-            }
-        }
-        __syncwarp();
-#pragma unroll
-        for (int t = 0; t < CH; ++t)
-            if (lane == 0 && first[t] >= 0) wbnd[first[t]] = -4.0f;
-        __syncwarp();
-        // phase 2: scan the best-bounded block, then every block the bound cannot exclude
-        float best = -4.0f;
-        int nl = 0;
-        bool ovf = false;
-        // candidate-list update with one block's cosines (qh, j) per lane
-        auto take_block = [&](float qh, int j) {
-            // cosines are >= 0, so the float bits order like unsigned ints
-            const float wm = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(qh, 0.0f))));
-            best = fmaxf(best, wm);
-            const bool keep = j >= 0 && qh >= best - band;
-            unsigned bal = __ballot_sync(0xffffffffu, keep);
-            if (nl + __popc(bal) > LC) {  // drop entries that fell out of the band
-                __syncwarp();
-                int kept = 0;
-                for (int e0 = 0; e0 < nl; e0 += 32) {
-                    const int e = e0 + lane;
-                    const bool k2 = e < nl && lq[e] >= best - band;
-                    const unsigned b2 = __ballot_sync(0xffffffffu, k2);
-                    int jj = 0;
-                    float qq = 0.0f;
-                    if (k2) {
-                        jj = lj[e];
-                        qq = lq[e];
-                    }
-                    __syncwarp();
-                    if (k2) {
-                        const int p = kept + __popc(b2 & ((1u << lane) - 1u));
-                        lj[p] = jj;
-                        lq[p] = qq;
-                    }
-                    kept += __popc(b2);
-                    __syncwarp();
-                }
-                nl = kept;
-                if (nl + __popc(bal) > LC) {
-                    ovf = true;
-                    bal = 0u;
-                }
-            }
-            if (keep && bal) {
-                const int p = nl + __popc(bal & ((1u << lane) - 1u));
-                lj[p] = j;
-                lq[p] = qh;
-            }
-            nl += __popc(bal);
-            __syncwarp();
-        };
-        // Scans up to CH blocks with all their loads issued before any use
-        // (the surviving blocks of a point are scanned in a few latency
-        // rounds instead of one round per block).
-        int pend[CH];
-        int npend = 0;
-        auto flush = [&]() {
-            float qh[CH];
-            int jj[CH];
-#pragma unroll
-            for (int t = 0; t < CH; ++t) {
-                const int pos = (t < npend ? pend[t] : 0) * 32 + lane;
-                qh[t] = -4.0f;
-                jj[t] = -1;
-                if (t < npend && pos < w) {
-                    const float4* z4 = reinterpret_cast<const float4*>(v.blk_z + (size_t)pos * M4);
-                    float zz[M4];
-#pragma unroll
-                    for (int q4 = 0; q4 < M4 / 4; ++q4) {
-                        const float4 z = __ldg(z4 + q4);
-                        zz[4 * q4 + 0] = z.x;
-                        zz[4 * q4 + 1] = z.y;
-                        zz[4 * q4 + 2] = z.z;
-                        zz[4 * q4 + 3] = z.w;
-                    }
-                    float a = 0.0f;
-#pragma unroll
-                    for (int q = 0; q < M; ++q) a = fmaf(u[q], zz[q], a);
-                    qh[t] = a;
-                    jj[t] = __ldg(v.blk_j + pos);
-                }
-            }
-#pragma unroll
-            for (int t = 0; t < CH; ++t)
-                if (t < npend) take_block(qh[t], jj[t]);
-            npend = 0;
-        };
-#pragma unroll
-        for (int t = 0; t < CH; ++t) pend[t] = first[t] >= 0 ? first[t] : 0;
-        npend = nfirst;
-        flush();
-        for (int base = 0; base < nb; base += 32) {
-            const int b = base + lane;
-            const bool f = b < nb && wbnd[b] + EPS >= best - band;
-            unsigned msk = __ballot_sync(0xffffffffu, f);
-            while (msk) {
-                const int b2 = base + __ffs(msk) - 1;
-                msk &= msk - 1;
-                if (wbnd[b2] + EPS >= best - band) {
-#pragma unroll
-                    for (int t = 0; t < CH; ++t)
-                        if (t == npend) pend[t] = b2;
-                    if (++npend == CH) flush();
-                }
-            }
-        }
-        if (npend) flush();
-        // final candidates: q >= best - band
-        int cnt = 0;
-        for (int e0 = 0; e0 < nl; e0 += 32) {
-            const int e = e0 + lane;
-            cnt += __popc(__ballot_sync(0xffffffffu, e < nl && lq[e] >= best - band));
-        }
-        int start = 0;
-        if (lane == 0 && !ovf) start = atomicAdd(&c->ncand, cnt);
-        start = __shfl_sync(0xffffffffu, start, 0);
-        if (ovf || start + cnt > v.cand_cap) {
-            if (lane == 0) {
-                v.arun[pt] = make_int2(-1, 0);
-                v.slow[atomicAdd(&c->nslow, 1)] = pt;
-            }
-            __syncwarp();
-            continue;
-        }
-        int off = 0;
-        for (int e0 = 0; e0 < nl; e0 += 32) {
-            const int e = e0 + lane;
-            const bool k2 = e < nl && lq[e] >= best - band;
-            const unsigned b2 = __ballot_sync(0xffffffffu, k2);
-            if (k2) v.cand[start + off + __popc(b2 & ((1u << lane) - 1u))] = make_int2(pt, lj[e]);
-            off += __popc(b2);
-        }
-        if (lane == 0) v.arun[pt] = make_int2(start, cnt);
-        __syncwarp();
     }
 }
 
-__device__ __forceinline__ void write_assoc(const RunView& v, Ctrl* c, int i, int j, double d)
+__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+__device__ __forceinline__ void mbar_init(unsigned long long* b, uint32_t n)
+{
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(n) : "memory");
+}
+__device__ __forceinline__ void mbar_expect(unsigned long long* b, uint32_t bytes)
+{
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(b)), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(unsigned long long* b)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(b)) : "memory");
+}
+// Waits for the barrier's phase of this parity, at most wait_ns of device
+// time; false when it did not come or another thread's wait ran out (*fail).
+__device__ __forceinline__ bool mbar_wait(unsigned long long* b, uint32_t parity, unsigned long long wait_ns, volatile int* fail)
+{
+    const uint32_t a = smem_u32(b);
+    unsigned long long t0 = 0ull;
+    for (unsigned it = 0;; ++it) {
+        uint32_t done;
+        asm volatile("{\n\t.reg .pred p;\n\t"
+                     "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+                     "selp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(done)
+                     : "r"(a), "r"(parity)
+                     : "memory");
+        if (done) return true;
+        if ((it & 63u) == 63u) {
+            if (*fail) return false;
+            const unsigned long long t = global_ns();
+            if (t0 == 0ull) t0 = t;
+            if (t - t0 > wait_ns || it > (1u << 28)) {
+                *fail = 1;
+                return false;
+            }
+        }
+    }
+}
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, unsigned long long* b)
+{
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(dst)),
+                 "l"(src), "r"(bytes), "r"(smem_u32(b))
+                 : "memory");
+}
+// K-major operand of `rows` rows without swizzle: core matrices of 8 rows x
+// 16 bytes, 16 rows bytes apart along K, 128 bytes apart along the rows
+__device__ __forceinline__ unsigned long long mma_desc(uint32_t addr, uint32_t rows)
+{
+    return (unsigned long long)((addr >> 4) & 0x3fffu) | (unsigned long long)rows << 16 |
+           (unsigned long long)(128u >> 4) << 32 | 1ull << 46;
+}
+__device__ __forceinline__ void mma_f16(uint32_t d, unsigned long long a, unsigned long long b, uint32_t idesc, bool add)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+                 "l"(a), "l"(b), "r"(idesc), "r"(add ? 1 : 0)
+                 : "memory");
+}
+__device__ __forceinline__ void mma_commit(unsigned long long* b)
+{
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(b)) : "memory");
+}
+// Maximum of 32 accumulator columns of each of this warp's 32 lanes, formed
+// by the load itself (the loaded values are not used, but their registers are
+// not free before the load's wait: tmem_keep after it)
+__device__ __forceinline__ void tmem_max32(uint32_t a, float& mx, uint32_t (&r)[32])
+{
+    asm volatile("tcgen05.ld.red.sync.aligned.32x32b.x32.max.f32 "
+                 "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+                 "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, %32, [%33];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+                   "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+                   "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]),
+                   "=f"(mx)
+                 : "r"(a));
+}
+__device__ __forceinline__ void tmem_keep(const uint32_t (&r)[32])
+{
+#pragma unroll
+    for (int k = 0; k < 32; ++k) asm volatile("" ::"r"(r[k]));
+}
+__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tmem_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tmem_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+
+// dynamic shared memory: the point tiles, the ring of chunks
+template <int KP>
+constexpr size_t mma_smem() { return (size_t)(TP + RING * CHUNK) * KP * 2 + 1024; }
+
+template <int KP>
+__global__ void __launch_bounds__(MT, 1) k_assoc_mma(RunView v)
+{
+    constexpr uint32_t ATILE = 128 * KP * 2, BTILE = CHUNK * KP * 2;  // bytes
+    // M = 128, N = CHUNK, FP16 operands, FP32 accumulators
+    constexpr uint32_t IDESC = (1u << 4) | ((CHUNK >> 3) << 17) | ((128u >> 4) << 24);
+    extern __shared__ unsigned char raw[];
+    // loads landed (points, ring slots); slots and tiles free again (an arrival
+    // per issuing thread); per set and tile: accumulator written, read
+    __shared__ unsigned long long bar_a, bar_afree, bar_b[RING], bar_bfree[RING], bar_full[SETS][TILES], bar_empty[SETS][TILES];
+    __shared__ uint32_t s_tmem;
+    __shared__ int s_fail;
+    Ctrl* c = v.ctrl;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = lane_id();
+    if (__syncthreads_or(skip_niche(c))) return;  // the same for every thread of the CTA
+    const int nT = c->nT, nch = (v.w + CHUNK - 1) / CHUNK;
+    int ntile, S, cps;
+    tile_split(nT, nch, gridDim.x, ntile, S, cps);
+    const int items = ntile * S;
+    if ((int)blockIdx.x >= items) return;
+    unsigned char* As = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~(uintptr_t)1023);
+    unsigned char* Bs = As + TILES * ATILE;
+    if (tid == 0) {
+        mbar_init(&bar_a, 1);
+        mbar_init(&bar_afree, TILES);
+        for (int k = 0; k < RING; ++k) {
+            mbar_init(&bar_b[k], 1);
+            mbar_init(&bar_bfree[k], TILES);
+        }
+        for (int k = 0; k < SETS * TILES; ++k) {
+            mbar_init(&bar_full[k / TILES][k % TILES], 1);
+            mbar_init(&bar_empty[k / TILES][k % TILES], 4);  // a lane of each of the tile's reading warps
+        }
+        s_fail = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (warp == TP / 32) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&s_tmem)) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tmem_fence_before();
+    __syncthreads();
+    tmem_fence_after();
+    const uint32_t tmem = s_tmem;
+    volatile int* fail = &s_fail;
+    auto wait = [&](unsigned long long* bar, uint32_t n) { return mbar_wait(bar, n & 1u, v.wait_ns, fail); };
+    // (after a failed wait: the end of what is in flight, or the limit)
+    auto drain = [&](unsigned long long* bar, uint32_t n) {
+        int none = 0;
+        mbar_wait(bar, n & 1u, v.wait_ns, &none);
+    };
+    if (warp == TP / 32 + TILES) {  // loads
+        if (lane == 0) {
+            uint32_t nload = 0, nitem = 0;
+            bool ok = true;
+            for (int it = blockIdx.x; it < items && ok; it += gridDim.x, ++nitem) {
+                const int g = it / S, sp = it - g * S;
+                const int c0 = sp * cps, c1 = min(nch, c0 + cps);
+                if (nitem > 0) ok = wait(&bar_afree, nitem - 1);  // the previous item's products are formed
+                if (!ok) break;
+                mbar_expect(&bar_a, TILES * ATILE);
+                bulk_load(As, v.aop + (size_t)g * TILES * ATILE, TILES * ATILE, &bar_a);
+                for (int ch = c0; ch < c1; ++ch, ++nload) {
+                    const uint32_t k = nload % RING;
+                    if (nload >= RING) ok = wait(&bar_bfree[k], nload / RING - 1);
+                    if (!ok) break;
+                    mbar_expect(&bar_b[k], BTILE);
+                    bulk_load(Bs + k * BTILE, v.bop + (size_t)ch * BTILE, BTILE, &bar_b[k]);
+                }
+            }
+            if (!ok) {
+                set_status(c, DEV_ETIMEOUT);
+                drain(&bar_a, nitem);
+                for (uint32_t k = nload > RING ? nload - RING : 0u; k < nload; ++k) drain(&bar_b[k % RING], k / RING);
+            }
+        }
+        __syncwarp();
+    } else if (warp >= TP / 32) {  // products of tile t
+        if (lane == 0) {
+            const int t = warp - TP / 32;
+            const uint32_t a = smem_u32(As) + t * ATILE;
+            uint32_t nstep = 0, nitem = 0;
+            bool ok = true;
+            for (int it = blockIdx.x; it < items && ok; it += gridDim.x, ++nitem) {
+                const int sp = it % S;
+                const int c0 = sp * cps, c1 = min(nch, c0 + cps);
+                ok = wait(&bar_a, nitem);
+                for (int ch = c0; ch < c1 && ok; ++ch, ++nstep) {
+                    const uint32_t k = nstep % RING, set = nstep % SETS;
+                    ok = wait(&bar_b[k], nstep / RING);
+                    // the accumulator's last maxima are taken
+                    if (ok && nstep >= SETS) ok = wait(&bar_empty[set][t], nstep / SETS - 1u);
+                    if (!ok) break;
+                    tmem_fence_after();
+                    const uint32_t b = smem_u32(Bs) + k * BTILE, d = tmem + (set * TILES + t) * CHUNK;
+#pragma unroll
+                    for (int kk = 0; kk < KP / 16; ++kk)
+                        mma_f16(d, mma_desc(a + kk * 4096, 128), mma_desc(b + kk * CHUNK * 32, CHUNK), IDESC, kk > 0);
+                    mma_commit(&bar_full[set][t]);
+                    mma_commit(&bar_bfree[k]);
+                }
+                if (ok) mma_commit(&bar_afree);
+            }
+            if (!ok) {
+                set_status(c, DEV_ETIMEOUT);
+                for (uint32_t k = nstep > SETS ? nstep - SETS : 0u; k < nstep; ++k) drain(&bar_full[k % SETS][t], k / SETS);
+            }
+        }
+        __syncwarp();
+    } else {  // maxima of tile t; the warp reads lanes 32 (warp & 3) ...
+        const int t = warp >> 2;
+        const uint32_t lanes = (uint32_t)((warp & 3) * 32) << 16;
+        uint32_t nstep = 0;
+        bool ok = true;
+        for (int it = blockIdx.x; it < items && ok; it += gridDim.x) {
+            const int g = it / S, sp = it - g * S;
+            const int c0 = sp * cps, c1 = min(nch, c0 + cps);
+            // this thread's point: best, second and third block maximum, the
+            // blocks of the first two
+            float b1 = -4.0f, b2 = -4.0f, b3 = -4.0f;
+            int k1 = 0, k2 = 0;
+            for (int ch = c0; ch < c1; ++ch, ++nstep) {
+                const uint32_t set = nstep % SETS;
+                ok = wait(&bar_full[set][t], nstep / SETS);
+                if (!__all_sync(0xffffffffu, ok)) {
+                    if (lane == 0) set_status(c, DEV_ETIMEOUT);
+                    ok = false;
+                    break;
+                }
+                tmem_fence_after();
+                const uint32_t ta = tmem + lanes + (set * TILES + t) * CHUNK;
+                float bm[CHUNK / 32];
+#pragma unroll
+                for (int h = 0; h < CHUNK / 32; h += 2) {
+                    uint32_t r0[32], r1[32];
+                    tmem_max32(ta + 32 * h, bm[h], r0);
+                    tmem_max32(ta + 32 * h + 32, bm[h + 1], r1);
+                    tmem_ld_wait();
+                    tmem_keep(r0);
+                    tmem_keep(r1);
+                }
+                tmem_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&bar_empty[set][t]);
+#pragma unroll
+                for (int h = 0; h < CHUNK / 32; ++h) {
+                    const int blk = ch * (CHUNK / 32) + h;
+                    const bool g1 = bm[h] > b1, g2 = bm[h] > b2;
+                    b3 = fmaxf(b3, fminf(b2, bm[h]));
+                    k2 = g1 ? k1 : g2 ? blk : k2;
+                    b2 = fmaxf(b2, fminf(b1, bm[h]));
+                    k1 = g1 ? blk : k1;
+                    b1 = fmaxf(b1, bm[h]);
+                }
+            }
+            if (ok && g * TP + tid < nT)  // (blocks number below 2^16)
+                v.aent[(size_t)it * TP + tid] = make_int4(__float_as_int(b1), __float_as_int(b2), __float_as_int(b3),
+                                                          k1 | (k2 << 16));
+        }
+    }
+    tmem_fence_before();
+    __syncthreads();
+    if (warp == TP / 32) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
+}
+
+__device__ __forceinline__ void write_assoc(const RunView& v, Ctrl* c, int i, int rk, int j, double d)
 {
     v.pi[i] = j;
     v.dist[i] = d;
-    if (v.rank2[i] < c->l)
+    if (rk < c->l)
         atomicAdd(&v.rho[j], 1);
     else
         atomicAdd(&v.rhop[j], 1);
 }
 
-// per point: FP64 distances of its candidates (usually one to three, so the
-// threads of a warp stay nearly converged on the FP64 pipe) and their
-// lexicographic (d, j) minimum
+// Per point the best maximum over the items and the blocks within MBAND of it
+// (a thread per T slot); a warp rescans its 32 points' blocks in FP32, a lane
+// per direction (coalesced rows; a thread rescanning its own blocks read 32
+// scattered lines per load: 26 us at m = 8, 38,700 points); then per thread
+// f' and |f'| in FP64 and the FP64 distances of the directions within the
+// FP32 band of the best (usually one), and their lexicographic (d, j)
+// minimum.  A point with more than FT_BLK blocks or FT_CAND candidates, or a
+// third block within MBAND in one item, takes the FP32 scan over all
+// directions.
 constexpr int FB = 128;
+constexpr int FT_BLK = 4;
+constexpr int FT_CAND = 8;
+
+// f' and |f'| of objectives f, in FP64
+template <int M>
+__device__ __forceinline__ double fprime_of(const Ctrl* c, const float* f, double (&fp)[M])
+{
+    double ss = 0.0;
+#pragma unroll
+    for (int q = 0; q < M; ++q) {
+        fp[q] = sf64::div(__dsub_rn((double)f[q], c->zstar[q]), c->da[q]);
+        ss = __dadd_rn(ss, __dmul_rn(fp[q], fp[q]));
+    }
+    return sf64::sqrt_rn(ss);
+}
 
 template <int M>
 __global__ void __launch_bounds__(FB) k_assoc_final(RunView v)
 {
+    constexpr int M4 = (M + 3) & ~3, Q4 = M4 / 4;
+    __shared__ int sblk[FT_BLK][FB];
+    __shared__ int scand[FT_CAND][FB];
+    __shared__ float scos[FT_CAND][FB];
+    __shared__ unsigned sjob[FB * FT_BLK];
+    __shared__ __align__(16) float suh[FB * M4];
     Ctrl* c = v.ctrl;
     if (skip_niche(c)) return;
-    const int pt = blockIdx.x * FB + threadIdx.x;
-    if (pt >= c->nT) return;
-    const int2 run = v.arun[pt];
-    if (run.x < 0) return;  // slow path
+    const int nT = c->nT;
+    const int tid = threadIdx.x, lane = lane_id(), wb = tid & ~31;
+    const int s = blockIdx.x * FB + tid;
+    if (blockIdx.x * FB >= nT) return;
+    int ntile, S, cps;
+    tile_split(nT, (v.w + CHUNK - 1) / CHUNK, v.assoc_grid, ntile, S, cps);
+    const int tile = s / TP, l = s - tile * TP;
+    const bool in = s < nT;
+    // the point's objectives and rank, used after the rescans
+    int i = 0, rk = 0;
+    float f[M];
+    if (in) {
+        i = v.Tlist[s];
+        rk = v.rank2[i];
+    }
+#pragma unroll
+    for (int q = 0; q < M; ++q) f[q] = in ? v.F[(size_t)i * M + q] : 0.0f;
+    bool ovf = false, third = false;
+    int nblk = 0;
+    if (in) {
+        float gbest = -4.0f;
+        const int4* ent = v.aent + (size_t)tile * S * TP + l;
+        for (int sp = 0; sp < S; ++sp) gbest = fmaxf(gbest, __int_as_float(ent[(size_t)sp * TP].x));
+        const float thr = gbest - MBAND;
+        for (int sp = 0; sp < S; ++sp) {
+            const int4 e = ent[(size_t)sp * TP];
+            third = third || __int_as_float(e.z) >= thr;
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                if (__int_as_float(k ? e.y : e.x) < thr) continue;
+                if (nblk == FT_BLK)
+                    ovf = true;
+                else
+                    sblk[nblk++][tid] = (e.w >> (16 * k)) & 0xffff;
+            }
+        }
+        if (ovf || third) nblk = 0;
+    }
+    // the warp's rescans as a list of (point, block), its points' unit vectors
+    // in shared memory; JB rescans' loads in flight together
+    int at = nblk;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, at, o);
+        if (lane >= o) at += y;
+    }
+    const int njob = __shfl_sync(0xffffffffu, at, 31);
+    at -= nblk;
+    unsigned* job = sjob + (wb >> 5) * (32 * FT_BLK);
+    for (int b = 0; b < nblk; ++b) job[at + b] = (unsigned)sblk[b][tid] * 32u + (unsigned)lane;
+    float* su = suh + (size_t)wb * M4;
+#pragma unroll
+    for (int q4 = 0; q4 < Q4; ++q4)
+        reinterpret_cast<float4*>(su + lane * M4)[q4] =
+            in ? reinterpret_cast<const float4*>(v.uhat + (size_t)s * M4)[q4] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    __syncwarp();
+    const float band = cos_band<M>();
+    float best = -4.0f;
+    int ncand = 0;
+    const float4* bz4 = reinterpret_cast<const float4*>(v.blk_z);
+    constexpr int JB = M4 <= 8 ? 8 : 4;  // rescans whose loads are in flight together
+    for (int j0 = 0; j0 < njob; j0 += JB) {
+        float qv[JB];
+        int pos[JB], pt[JB];
+        float4 z[JB][Q4];
+#pragma unroll
+        for (int t = 0; t < JB; ++t) {
+            const unsigned x = job[min(j0 + t, njob - 1)];
+            pt[t] = (int)(x & 31u);
+            pos[t] = (int)(x & ~31u) + lane;
+#pragma unroll
+            for (int q4 = 0; q4 < Q4; ++q4) z[t][q4] = __ldg(bz4 + (size_t)min(pos[t], v.w - 1) * Q4 + q4);
+        }
+#pragma unroll
+        for (int t = 0; t < JB; ++t) {
+            const float* u = su + pt[t] * M4;
+            float a = 0.0f;
+#pragma unroll
+            for (int q4 = 0; q4 < Q4; ++q4) {
+                const float4 y = reinterpret_cast<const float4*>(u)[q4];
+                a = fmaf(y.x, z[t][q4].x, a);
+                if (4 * q4 + 1 < M) a = fmaf(y.y, z[t][q4].y, a);
+                if (4 * q4 + 2 < M) a = fmaf(y.z, z[t][q4].z, a);
+                if (4 * q4 + 3 < M) a = fmaf(y.w, z[t][q4].w, a);
+            }
+            qv[t] = a;
+        }
+#pragma unroll
+        for (int t = 0; t < JB; ++t) {
+            if (j0 + t >= njob) break;
+            const int p = pt[t];
+            const bool ref = pos[t] < v.w;
+            // cosines are >= 0: their bits order like unsigned ints
+            const float bm = __uint_as_float(__reduce_max_sync(0xffffffffu, ref ? __float_as_uint(fmaxf(qv[t], 0.0f)) : 0u));
+            const float run = fmaxf(__shfl_sync(0xffffffffu, best, p), bm);
+            const int n = __shfl_sync(0xffffffffu, ncand, p);
+            const bool take = ref && qv[t] >= run - band;
+            const unsigned bal = __ballot_sync(0xffffffffu, take);
+            if (take) {
+                const int e = n + __popc(bal & ((1u << lane) - 1u));
+                if (e < FT_CAND) {
+                    scand[e][wb + p] = pos[t];
+                    scos[e][wb + p] = qv[t];
+                }
+            }
+            if (lane == p) {
+                best = run;
+                ncand = n + __popc(bal);
+            }
+        }
+    }
+    __syncwarp();
+    if (!in) return;
+    double fp[M];
+    const double nf = fprime_of<M>(c, f, fp);
+    const bool zero = sf64::is_zero(nf);  // every distance is 0: the first direction
     double bd = 0.0;
     int bj = 0;
-    const double nf = v.fnorm[pt];
-    if (nf != 0.0) {
-        double fp[M];
-#pragma unroll
-        for (int q = 0; q < M; ++q) fp[q] = v.fprime[(size_t)pt * M + q];
+    if (!zero) {
+        if (ovf || third || ncand > FT_CAND) {
+            v.arun[s] = make_int2(third ? -2 : -1, 0);  // (-1: a list overflowed)
+            v.slow[atomicAdd(&c->nslow, 1)] = s;
+            return;
+        }
         bd = CUDART_INF;
         bj = 0x7fffffff;
-        for (int e = run.x; e < run.x + run.y; ++e) {
-            const int j = v.cand[e].y;
+        for (int e = 0; e < ncand; ++e) {
+            if (scos[e][tid] < best - band) continue;
+            const int j = v.blk_j[scand[e][tid]];
             const double d = perp_dist(fp, nf, v.Zd + (size_t)j * M, v.nz[j], M);
             if (lex_less(d, j, bd, bj)) {
                 bd = d;
@@ -362,21 +628,25 @@ __global__ void __launch_bounds__(FB) k_assoc_final(RunView v)
         }
     }
     if (v.debug_recheck_all) {
-        v.dist[v.Tlist[pt]] = bd;  // compared by k_assoc_slow
-        v.pi[v.Tlist[pt]] = bj;
-        v.slow[atomicAdd(&c->nslow, 1)] = pt;
+        v.dist[i] = bd;  // compared by k_assoc_slow
+        v.pi[i] = bj;
+        v.arun[s] = make_int2(0, 0);
+        v.slow[atomicAdd(&c->nslow, 1)] = s;
         return;
     }
-    write_assoc(v, c, v.Tlist[pt], bj, bd);
+    write_assoc(v, c, i, rk, bj, bd);
 }
 
-// full FP64 scan of one point per CTA (overflowed lists, debug mode)
-// M = 0: runtime m (f' read from memory)
+// One point per CTA over all directions: points whose lists overflowed, and
+// in debug mode every point.  m <= 10: the best FP32 cosine, then the FP64
+// distances of the directions within the band of it (in debug mode and for
+// m > 10, M = 0, of every direction).
 template <int M>
 __global__ void __launch_bounds__(AB) k_assoc_slow(RunView v)
 {
     __shared__ double sd[AB / 32];
     __shared__ int sj[AB / 32];
+    __shared__ unsigned s_best;
     Ctrl* c = v.ctrl;
     if (skip_niche(c)) return;
     const int ns = c->nslow;
@@ -384,14 +654,42 @@ __global__ void __launch_bounds__(AB) k_assoc_slow(RunView v)
     const int lane = lane_id(), warp = threadIdx.x >> 5;
     for (int t = blockIdx.x; t < ns; t += gridDim.x) {
         const int pt = v.slow[t];
-        double fr[M > 0 ? M : 1];
+        double fr[M > 0 ? M : 1], nf;
+        float thr = -4.0f, u[M > 0 ? M : 1];
+        if constexpr (M > 0) {
+            constexpr int M4 = (M + 3) & ~3;
+            nf = fprime_of<M>(c, v.F + (size_t)v.Tlist[pt] * M, fr);
 #pragma unroll
-        for (int q = 0; q < M; ++q) fr[q] = v.fprime[(size_t)pt * M + q];
+            for (int q = 0; q < M; ++q) u[q] = v.uhat[(size_t)pt * M4 + q];
+            if (!v.debug_recheck_all) {
+                if (threadIdx.x == 0) s_best = 0u;
+                __syncthreads();
+                float b = 0.0f;
+                for (int j = threadIdx.x; j < v.w; j += AB) {
+                    float x = 0.0f;
+#pragma unroll
+                    for (int q = 0; q < M; ++q) x = fmaf(u[q], __ldg(v.Zh + (size_t)j * M4 + q), x);
+                    b = fmaxf(b, x);
+                }
+                const unsigned wm = __reduce_max_sync(0xffffffffu, __float_as_uint(b));  // cosines are >= 0
+                if (lane == 0) atomicMax(&s_best, wm);
+                __syncthreads();
+                thr = __uint_as_float(s_best) - cos_band<M>();
+            }
+        } else {
+            nf = v.fnorm[pt];
+        }
         const double* fp = M > 0 ? fr : v.fprime + (size_t)pt * m;
-        const double nf = v.fnorm[pt];
         double d0 = CUDART_INF;
         int j0 = 0x7fffffff;
         for (int j = threadIdx.x; j < v.w; j += AB) {
+            if constexpr (M > 0) {
+                constexpr int M4 = (M + 3) & ~3;
+                float x = 0.0f;
+#pragma unroll
+                for (int q = 0; q < M; ++q) x = fmaf(u[q], __ldg(v.Zh + (size_t)j * M4 + q), x);
+                if (x < thr) continue;
+            }
             const double d = perp_dist(fp, nf, v.Zd + (size_t)j * m, v.nz[j], m);
             if (lex_less(d, j, d0, j0)) {
                 d0 = d;
@@ -420,11 +718,11 @@ __global__ void __launch_bounds__(AB) k_assoc_slow(RunView v)
                 }
             const int i = v.Tlist[pt];
             if (v.arun[pt].x < 0) {
-                atomicAdd(&c->overflow, 1);
+                if (v.arun[pt].x == -1) atomicAdd(&c->overflow, 1);
             } else if (v.debug_recheck_all && (v.pi[i] != j0 || v.dist[i] != d0)) {
                 atomicAdd(&c->recheck_miss, 1);
             }
-            write_assoc(v, c, i, j0, d0);
+            write_assoc(v, c, i, v.rank2[i], j0, d0);
         }
         __syncthreads();
     }
@@ -705,460 +1003,14 @@ __global__ void __launch_bounds__(256) k_assoc_final_gen(RunView v)
         v.slow[atomicAdd(&c->nslow, 1)] = pt;
         return;
     }
-    write_assoc(v, c, v.Tlist[pt], bj, bd);
+    write_assoc(v, c, v.Tlist[pt], v.rank2[v.Tlist[pt]], bj, bd);
 }
-
-// Few reference directions (w <= ASSOC_SMALL_W, m <= 10): the whole
-// association of a point in one thread, every direction's FP32 unit vector
-// in shared memory (read by all threads of a warp at once).  f' and |f'| in
-// FP64 as k_assoc_prep computes them, the best FP32 cosine over all
-// directions, a second pass over the directions within the band of it (the
-// candidates), their FP64 distances and the lexicographic (d, j) minimum:
-// the same candidates, band and FP64 operations as the pruned path, so the
-// same exact result, in one launch instead of four.
-constexpr int SB_T = 128;
-
-template <int M>
-__global__ void __launch_bounds__(SB_T) k_assoc_small(RunView v)
-{
-    constexpr int M4 = (M + 3) & ~3;
-    extern __shared__ __align__(16) float zs[];  // w x M4 unit directions, original order
-    Ctrl* c = v.ctrl;
-    if (skip_niche(c)) return;
-    const int w = v.w;
-    for (int e = threadIdx.x; e < w * M4; e += SB_T) zs[e] = v.Zh[e];
-    __syncthreads();
-    const int s = blockIdx.x * SB_T + threadIdx.x;
-    if (s >= c->nT) return;
-    const int i = v.Tlist[s];
-    double fp[M];
-    double ss = 0.0;
-#pragma unroll
-    for (int q = 0; q < M; ++q) {
-        const double ft = __dsub_rn((double)v.F[(size_t)i * M + q], c->zstar[q]);
-        fp[q] = __ddiv_rn(ft, c->a[q]);
-        ss = __dadd_rn(ss, __dmul_rn(fp[q], fp[q]));
-    }
-    const double nf = __dsqrt_rn(ss);
-    double bd = 0.0;
-    int bj = 0;
-    if (nf != 0.0 || v.debug_recheck_all) {
-        const double inv = nf > 0.0 ? 1.0 / nf : 0.0;
-        float u[M];
-#pragma unroll
-        for (int q = 0; q < M; ++q) u[q] = __double2float_rn(fp[q] * inv);
-        float best = -1.0f;
-        for (int j = 0; j < w; ++j) {
-            const float* z = zs + j * M4;
-            float dq = 0.0f;
-#pragma unroll
-            for (int q = 0; q < M; ++q) dq = fmaf(u[q], z[q], dq);
-            best = fmaxf(best, dq);
-        }
-        const float band = 2.0f * (float)(M + 4) * 5.9604644775390625e-08f + 1e-12f;
-        bd = CUDART_INF;
-        bj = 0x7fffffff;
-        for (int j = 0; j < w; ++j) {
-            const float* z = zs + j * M4;
-            float dq = 0.0f;
-#pragma unroll
-            for (int q = 0; q < M; ++q) dq = fmaf(u[q], z[q], dq);
-            if (dq >= best - band) {
-                const double d = perp_dist(fp, nf, v.Zd + (size_t)j * M, v.nz[j], M);
-                if (lex_less(d, j, bd, bj)) {
-                    bd = d;
-                    bj = j;
-                }
-            }
-        }
-        if (v.debug_recheck_all) {
-            // every direction in FP64: the band must not have missed the minimum
-            double fd = CUDART_INF;
-            int fj = 0x7fffffff;
-            for (int j = 0; j < w; ++j) {
-                const double d = perp_dist(fp, nf, v.Zd + (size_t)j * M, v.nz[j], M);
-                if (lex_less(d, j, fd, fj)) {
-                    fd = d;
-                    fj = j;
-                }
-            }
-            if (fj != bj || fd != bd) atomicAdd(&c->recheck_miss, 1);
-            bd = fd;
-            bj = fj;
-        }
-    }
-    write_assoc(v, c, i, bj, bd);
-}
-
-// ---------------------------------------------------------------------------
-// Tiled scan (m <= 10, more than ASSOC_SMALL_W directions).  Where the cone
-// bounds prune little (several objectives: a block's cone and a point's
-// distance to its nearest direction are comparable), every cosine is formed,
-// at the FP32 FMA rate: a CTA holds TP = TT x TP_P points in registers and
-// streams the reference blocks of its range through shared memory (each
-// direction read once per CTA by a broadcast load, then TP_P x m FMAs per
-// thread).  A work item is (a tile of TP slots, a range of reference
-// blocks); the ranges are chosen so that the items fill the grid.  Per
-// point and item the scan keeps the largest block maximum (the item's best
-// cosine) and up to ASSOC_K blocks whose maximum is within the band of it
-// (a block is taken when its maximum is within the band of the best so
-// far, replacing a block that has fallen out of the band; none free: the
-// point overflows to the FP64 scan).  The block holding the exact argmin
-// has a maximum within the band of every later best, so it is never
-// replaced.  k_assoc_final_tile takes the best over the items, rescans the
-// blocks within the band of it (FP32, then FP64 for the directions within
-// the band, as the pruned path does) and writes the association.
-constexpr int TT = 128;     // threads per CTA
-constexpr int TP_P = 4;     // points per thread
-constexpr int TP = TT * TP_P;
-constexpr int TCB = 8;      // reference blocks per shared-memory chunk
-constexpr int TOCC = 4;     // CTAs per SM (the grid, and the register bound)
-constexpr int ASSOC_K = 4;  // entries per point and item
-
-// tiles of T slots, items per tile (splits) and blocks per split: the same
-// on the device for both kernels (from nT) and on the host for the maximum.
-// The split count minimises the waves of the grid times the blocks an item
-// scans, over at most twice the count that fills the grid once (so that
-// items <= 2 (grid + ntile)).
-__host__ __device__ __forceinline__ void tile_split(int nT, int nb, int grid, int& ntile, int& S, int& bps)
-{
-    ntile = (nT + TP - 1) / TP;
-    S = 1;
-    bps = nb;
-    if (ntile == 0 || nb == 0) return;
-    const int fill = (grid + ntile - 1) / ntile;
-    const int smax = min(nb, 2 * fill);
-    long long best = -1;
-    for (int t = 1; t <= smax; ++t) {
-        const int b = (nb + t - 1) / t;
-        const int st = (nb + b - 1) / b;
-        const long long cost = (long long)(((long long)ntile * st + grid - 1) / grid) * b;
-        if (best < 0 || cost < best) {
-            best = cost;
-            S = st;
-            bps = b;
-        }
-    }
-}
-
-// Two points' cosines with one direction in one instruction: FP32 pairs
-// (fma.rn.f32x2 rounds each lane once, as fmaf does), the points' unit
-// vectors packed by pairs, each direction component duplicated in shared
-// memory.  Packing and unpacking are register moves.
-__device__ __forceinline__ unsigned long long f2_pack(float lo, float hi)
-{
-    unsigned long long r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-
-__device__ __forceinline__ void f2_unpack(unsigned long long x, float& lo, float& hi)
-{
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(x));
-}
-
-__device__ __forceinline__ unsigned long long f2_fma(unsigned long long a, unsigned long long b,
-                                                     unsigned long long c)
-{
-    unsigned long long d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-
-__device__ __forceinline__ float fmax3f(float a, float b, float c)
-{
-    float d;
-    asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-    return d;
-}
-
-template <int M>
-__global__ void __launch_bounds__(TT, TOCC) k_assoc_tile(RunView v)
-{
-    static_assert(TP_P % 2 == 0, "points are packed by pairs");
-    constexpr int M4 = (M + 3) & ~3;
-    constexpr int ZQ = (M + 1) / 2;  // 16-byte words per staged direction: (z0, z0, z1, z1), ...
-    constexpr int PP = TP_P / 2;
-    __shared__ ulonglong2 zs[TCB * 32 * ZQ];
-    __shared__ float slm[TP_P][ASSOC_K][TT];  // candidate blocks of each point: maximum, block
-    __shared__ int slk[TP_P][ASSOC_K][TT];
-    Ctrl* c = v.ctrl;
-    if (skip_niche(c)) return;
-    const int nT = c->nT;
-    const int nb = v.nblk, w = v.w;
-    int ntile, S, bps;
-    tile_split(nT, nb, gridDim.x, ntile, S, bps);
-    const int items = ntile * S;
-    const float band = 2.0f * (float)(M + 4) * 5.9604644775390625e-08f + 1e-12f;
-    const int tid = threadIdx.x;
-    for (int it = blockIdx.x; it < items; it += gridDim.x) {
-        const int tile = it / S, sp = it - (it / S) * S;
-        const int b0 = sp * bps;
-        const int b1 = min(nb, b0 + bps);
-        unsigned long long u2[PP][M];
-#pragma unroll
-        for (int pp = 0; pp < PP; ++pp) {
-            const int sa = tile * TP + (2 * pp) * TT + tid;
-            const int sb = sa + TT;
-            const float* ra = v.uhat + (size_t)sa * M4;
-            const float* rb = v.uhat + (size_t)sb * M4;
-#pragma unroll
-            for (int t = 0; t < M; ++t)
-                u2[pp][t] = f2_pack(sa < nT ? ra[t] : 0.0f, sb < nT ? rb[t] : 0.0f);
-        }
-        float lbest[TP_P];
-        unsigned ovf = 0u;
-#pragma unroll
-        for (int k = 0; k < TP_P; ++k) {
-            lbest[k] = -4.0f;
-#pragma unroll
-            for (int e = 0; e < ASSOC_K; ++e) {
-                slm[k][e][tid] = -4.0f;
-                slk[k][e][tid] = -1;
-            }
-        }
-        for (int cb = b0; cb < b1; cb += TCB) {
-            const int nbk = min(TCB, b1 - cb);
-            __syncthreads();  // the previous chunk is consumed
-            // padding directions (position >= w) get -1 components: their
-            // cosine with a unit vector of non-negative components is <= -1
-            for (int e = tid; e < nbk * 32 * ZQ; e += TT) {
-                const int r = e / ZQ, q2 = e - r * ZQ;
-                const int pos = cb * 32 + r;
-                float2 a = make_float2(-1.0f, -1.0f);
-                if (pos < w) a = __ldg(reinterpret_cast<const float2*>(v.blk_z + (size_t)pos * M4) + q2);
-                zs[e] = make_ulonglong2(f2_pack(a.x, a.x), f2_pack(a.y, a.y));
-            }
-            __syncthreads();
-            for (int bb = 0; bb < nbk; ++bb) {
-                float bm[TP_P];
-#pragma unroll
-                for (int k = 0; k < TP_P; ++k) bm[k] = -4.0f;
-                const ulonglong2* zb = zs + bb * 32 * ZQ;
-#pragma unroll 2
-                for (int r = 0; r < 32; r += 2) {
-                    ulonglong2 za[ZQ], zc[ZQ];
-#pragma unroll
-                    for (int q2 = 0; q2 < ZQ; ++q2) {
-                        za[q2] = zb[r * ZQ + q2];
-                        zc[q2] = zb[(r + 1) * ZQ + q2];
-                    }
-#pragma unroll
-                    for (int pp = 0; pp < PP; ++pp) {
-                        unsigned long long qa = 0ull, qc = 0ull;
-#pragma unroll
-                        for (int t = 0; t < M; ++t) {
-                            qa = f2_fma(u2[pp][t], (t & 1) ? za[t >> 1].y : za[t >> 1].x, qa);
-                            qc = f2_fma(u2[pp][t], (t & 1) ? zc[t >> 1].y : zc[t >> 1].x, qc);
-                        }
-                        float a0, a1, c0, c1;
-                        f2_unpack(qa, a0, a1);
-                        f2_unpack(qc, c0, c1);
-                        bm[2 * pp] = fmax3f(bm[2 * pp], a0, c0);
-                        bm[2 * pp + 1] = fmax3f(bm[2 * pp + 1], a1, c1);
-                    }
-                }
-#pragma unroll
-                for (int k = 0; k < TP_P; ++k) {
-                    if (bm[k] >= lbest[k] - band) {
-                        const float thr = fmaxf(lbest[k], bm[k]) - band;
-                        int slot = -1;
-#pragma unroll
-                        for (int e = 0; e < ASSOC_K; ++e)
-                            if (slot < 0 && (slk[k][e][tid] < 0 || slm[k][e][tid] < thr)) slot = e;
-                        if (slot < 0) {
-                            ovf |= 1u << k;
-                        } else {
-                            slm[k][slot][tid] = bm[k];
-                            slk[k][slot][tid] = cb + bb;
-                        }
-                    }
-                    lbest[k] = fmaxf(lbest[k], bm[k]);
-                }
-            }
-        }
-        // point k of this thread is T slot tile * TP + k * TT + tid (pairs:
-        // points 2 pp and 2 pp + 1 are TT slots apart)
-#pragma unroll
-        for (int k = 0; k < TP_P; ++k) {
-            const int l = k * TT + tid;
-            if (tile * TP + l >= nT) continue;
-            int4* dst = reinterpret_cast<int4*>(v.aent + ((size_t)it * TP + l) * ASSOC_K);
-            if ((ovf >> k) & 1u) {
-                dst[0] = make_int4(0, -2, 0, -2);
-                dst[1] = make_int4(0, -2, 0, -2);
-            } else {
-                dst[0] = make_int4(__float_as_int(slm[k][0][tid]), slk[k][0][tid],
-                                   __float_as_int(slm[k][1][tid]), slk[k][1][tid]);
-                dst[1] = make_int4(__float_as_int(slm[k][2][tid]), slk[k][2][tid],
-                                   __float_as_int(slm[k][3][tid]), slk[k][3][tid]);
-            }
-        }
-    }
-}
-
-static_assert(ASSOC_K == 4, "the entries of a point are written as two int4");
-
-// per point (a thread per T slot): the best cosine over the items, the
-// blocks within the band of it rescanned in FP32, the FP64 distances of
-// their directions within the band and the lexicographic (d, j) minimum.
-// The blocks and then the candidate directions of each thread are listed
-// first (shared memory, a column per thread), so that a warp runs as many
-// rescans and FP64 evaluations as its busiest thread needs rather than the
-// union of its threads' positions.  A point with more than FT_BLK blocks or
-// FT_CAND candidates takes the FP64 scan over all directions.
-constexpr int FT_BLK = 8;
-constexpr int FT_CAND = 16;
-
-template <int M>
-__global__ void __launch_bounds__(FB) k_assoc_final_tile(RunView v)
-{
-    constexpr int M4 = (M + 3) & ~3;
-    constexpr int Q4 = M4 / 4;
-    // a block's directions in groups of RC, every load of a group in flight
-    // together (a thread's blocks are its own: the loads do not coalesce,
-    // so round trips, not bytes, set the time)
-    constexpr int RC = M4 <= 8 ? 8 : 4;
-    __shared__ int sblk[FT_BLK][FB];
-    __shared__ int scand[FT_CAND][FB];
-    Ctrl* c = v.ctrl;
-    if (skip_niche(c)) return;
-    const int nT = c->nT;
-    const int tid = threadIdx.x;
-    const int s = blockIdx.x * FB + tid;
-    if (s >= nT) return;
-    int ntile, S, bps;
-    tile_split(nT, v.nblk, v.assoc_grid, ntile, S, bps);
-    const int tile = s / TP, l = s - tile * TP;
-    const double nf = v.fnorm[s];
-    double bd = 0.0;
-    int bj = 0;
-    if (nf != 0.0) {
-        const float band = 2.0f * (float)(M + 4) * 5.9604644775390625e-08f + 1e-12f;
-        float gbest = -4.0f;
-        bool ovf = false;
-        for (int sp = 0; sp < S; ++sp) {
-            const int4* e = reinterpret_cast<const int4*>(v.aent + ((size_t)(tile * S + sp) * TP + l) * ASSOC_K);
-            const int4 x0 = e[0], x1 = e[1];
-            const int bk[4] = {x0.y, x0.w, x1.y, x1.w};
-            const int bv[4] = {x0.x, x0.z, x1.x, x1.z};
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                if (bk[k] == -2) ovf = true;
-                if (bk[k] >= 0) gbest = fmaxf(gbest, __int_as_float(bv[k]));
-            }
-        }
-        const float thr = gbest - band;
-        int nblk = 0;
-        for (int sp = 0; sp < S && !ovf; ++sp) {
-            const int4* e = reinterpret_cast<const int4*>(v.aent + ((size_t)(tile * S + sp) * TP + l) * ASSOC_K);
-            const int4 x0 = e[0], x1 = e[1];
-            const int bk[4] = {x0.y, x0.w, x1.y, x1.w};
-            const int bv[4] = {x0.x, x0.z, x1.x, x1.z};
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                if (bk[k] < 0 || __int_as_float(bv[k]) < thr) continue;
-                if (nblk == FT_BLK) {
-                    ovf = true;
-                } else {
-                    sblk[nblk][tid] = bk[k];
-                    ++nblk;
-                }
-            }
-        }
-        float u[M];
-#pragma unroll
-        for (int q = 0; q < M; ++q) u[q] = v.uhat[(size_t)s * M4 + q];
-        int ncand = 0;
-        const float4* bz4 = reinterpret_cast<const float4*>(v.blk_z);
-        for (int i = 0; i < nblk && !ovf; ++i) {
-            const int base = sblk[i][tid] * 32;
-            for (int r0 = 0; r0 < 32; r0 += RC) {
-                float qv[RC];
-#pragma unroll
-                for (int t = 0; t < RC; ++t) {
-                    const int pos = min(base + r0 + t, v.w - 1);
-                    float z[M4];
-#pragma unroll
-                    for (int q4 = 0; q4 < Q4; ++q4) {
-                        const float4 a = __ldg(bz4 + (size_t)pos * Q4 + q4);
-                        z[4 * q4 + 0] = a.x;
-                        z[4 * q4 + 1] = a.y;
-                        z[4 * q4 + 2] = a.z;
-                        z[4 * q4 + 3] = a.w;
-                    }
-                    float q = 0.0f;
-#pragma unroll
-                    for (int t2 = 0; t2 < M; ++t2) q = fmaf(u[t2], z[t2], q);
-                    qv[t] = q;
-                }
-#pragma unroll
-                for (int t = 0; t < RC; ++t) {
-                    const int pos = base + r0 + t;
-                    if (pos >= v.w || qv[t] < thr) continue;
-                    if (ncand == FT_CAND) {
-                        ovf = true;
-                    } else {
-                        scand[ncand][tid] = pos;
-                        ++ncand;
-                    }
-                }
-            }
-        }
-        if (ovf) {
-            v.arun[s] = make_int2(-1, 0);
-            v.slow[atomicAdd(&c->nslow, 1)] = s;
-            return;
-        }
-        double fp[M];
-#pragma unroll
-        for (int q = 0; q < M; ++q) fp[q] = v.fprime[(size_t)s * M + q];
-        bd = CUDART_INF;
-        bj = 0x7fffffff;
-        for (int i = 0; i < ncand; ++i) {
-            const int j = v.blk_j[scand[i][tid]];
-            const double d = perp_dist(fp, nf, v.Zd + (size_t)j * M, v.nz[j], M);
-            if (lex_less(d, j, bd, bj)) {
-                bd = d;
-                bj = j;
-            }
-        }
-    }
-    if (v.debug_recheck_all) {
-        v.dist[v.Tlist[s]] = bd;  // compared by k_assoc_slow
-        v.pi[v.Tlist[s]] = bj;
-        v.arun[s] = make_int2(0, 0);
-        v.slow[atomicAdd(&c->nslow, 1)] = s;
-        return;
-    }
-    write_assoc(v, c, v.Tlist[s], bj, bd);
-}
-
-size_t small_smem(const RunView& v) { return (size_t)v.w * v.M4 * sizeof(float); }
-
-size_t scan_smem(const RunView& v) { return (size_t)v.nblk * (v.M4 + 2 + 8) * 4 + 8 * 2 * LC * 4; }
 
 template <int M>
 cudaError_t launch_m(const RunView& v, cudaStream_t s, int num_sms)
 {
-    if (assoc_small(v)) {
-        k_assoc_small<M><<<(v.n2 + SB_T - 1) / SB_T, SB_T, small_smem(v), s>>>(v);
-        return cudaGetLastError();
-    }
-    if (v.aent) {
-        k_assoc_tile<M><<<v.assoc_grid, TT, 0, s>>>(v);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        k_assoc_final_tile<M><<<(v.n2 + FB - 1) / FB, FB, 0, s>>>(v);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        k_assoc_slow<M><<<num_sms, AB, 0, s>>>(v);
-        return cudaGetLastError();
-    }
-    const size_t sm = scan_smem(v);
-    int blocks = (v.n2 + 7) / 8;
-    if (blocks > num_sms * 8) blocks = num_sms * 8;
-    k_assoc_scan<M><<<blocks, AB, sm, s>>>(v);
+    constexpr int KP = kp_of<M>();
+    k_assoc_mma<KP><<<v.assoc_grid, MT, mma_smem<KP>(), s>>>(v);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_assoc_final<M><<<(v.n2 + FB - 1) / FB, FB, 0, s>>>(v);
@@ -1168,27 +1020,47 @@ cudaError_t launch_m(const RunView& v, cudaStream_t s, int num_sms)
     return cudaGetLastError();
 }
 
-template <int M>
-cudaError_t attr_m(size_t sm)
-{
-    return cudaFuncSetAttribute(k_assoc_scan<M>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-}
-
 }  // namespace
 
-int assoc_tile_grid(int num_sms) { return (num_sms > 0 ? num_sms : 1) * TOCC; }
+int assoc_grid(int num_sms) { return num_sms > 0 ? num_sms : 1; }
 
-size_t assoc_tile_entries(int n2, int num_sms)
+size_t assoc_entries(int n2, int num_sms)
 {
     // items = ntile x S <= ntile x 2 ceil(grid / ntile) <= 2 (grid + ntile)
     // for every nT <= n2
     const size_t ntile = ((size_t)n2 + TP - 1) / TP;
-    return 2 * ((size_t)assoc_tile_grid(num_sms) + ntile) * TP * ASSOC_K;
+    return 2 * ((size_t)assoc_grid(num_sms) + ntile) * TP;
+}
+
+size_t assoc_rows_bytes(int m, int rows)
+{
+    const size_t kp = 3 * m <= 16 ? 16 : 32;
+    return ((size_t)rows + TP - 1) / TP * TP * kp * 2;
+}
+
+// the directions' FP16 rows [zh, zl, zh] in chunks of 128 as k_assoc_mma
+// reads them; z: w x M4 unit vectors in block order.  Rows past w are -1 in
+// every h: their cosines with unit vectors of non-negative components are
+// below -0.9.
+void assoc_pack_refs(int m, int M4, int w, const float* z, unsigned char* out)
+{
+    const int KP = 3 * m <= 16 ? 16 : 32, rows = (w + CHUNK - 1) / CHUNK * CHUNK;
+    for (int j = 0; j < rows; ++j) {
+        __half r[32];
+        for (int e = 0; e < KP; ++e) r[e] = __float2half_rn(0.0f);
+        for (int q = 0; q < m; ++q) {
+            const float x = j < w ? z[(size_t)j * M4 + q] : -1.0f;
+            const __half h = __float2half_rn(x);
+            r[q] = r[2 * m + q] = h;
+            r[m + q] = __float2half_rn(x - __half2float(h));
+        }
+        unsigned char* row = out + (size_t)(j / CHUNK) * (CHUNK * KP * 2) + (j % CHUNK) * 16;
+        for (int k = 0; k < KP / 8; ++k) memcpy(row + k * CHUNK * 16, r + 8 * k, 16);
+    }
 }
 
 cudaError_t launch_assoc_prep(const RunView& v, cudaStream_t s)
 {
-    if (assoc_small(v)) return cudaSuccess;  // k_assoc_small forms f' itself
     const int g = (v.n2 + PB - 1) / PB;
     switch (v.m) {
     case 2: k_assoc_prep<2><<<g, PB, 0, s>>>(v); break;
@@ -1244,31 +1116,11 @@ cudaError_t launch_assoc_scan(const RunView& v, int num_sms, cudaStream_t s)
     return cudaGetLastError();
 }
 
-// The scan's shared-memory opt-in is set once per process, at its maximum,
-// before any launch (changing a kernel's attribute while graphs that launch
-// it run on other streams is avoided); a run only checks that its block
-// tables fit (about 5,000 blocks of 32 references).
-constexpr size_t SCAN_SMEM_MAX = 220 * 1024;
-
-cudaError_t assoc_prepare(const RunView& v)
-{
-    if (v.m < 2 || v.m > NSGA3_MAX_M) return cudaErrorInvalidValue;
-    if (v.m > NSGA3_FAST_M) return cudaSuccess;  // the generic scan keeps no block tables
-    return scan_smem(v) <= SCAN_SMEM_MAX ? cudaSuccess : cudaErrorInvalidValue;
-}
-
 cudaError_t assoc_init_attributes()
 {
-    cudaError_t e = cudaSuccess;
-    if (e == cudaSuccess) e = attr_m<2>(SCAN_SMEM_MAX);
-    if (e == cudaSuccess) e = attr_m<3>(SCAN_SMEM_MAX);
-    if (e == cudaSuccess) e = attr_m<4>(SCAN_SMEM_MAX);
-    if (e == cudaSuccess) e = attr_m<5>(SCAN_SMEM_MAX);
-    if (e == cudaSuccess) e = attr_m<6>(SCAN_SMEM_MAX);
-    if (e == cudaSuccess) e = attr_m<7>(SCAN_SMEM_MAX);
-    if (e == cudaSuccess) e = attr_m<8>(SCAN_SMEM_MAX);
-    if (e == cudaSuccess) e = attr_m<9>(SCAN_SMEM_MAX);
-    if (e == cudaSuccess) e = attr_m<10>(SCAN_SMEM_MAX);
+    cudaError_t e = cudaFuncSetAttribute(k_assoc_mma<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mma_smem<16>());
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_assoc_mma<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mma_smem<32>());
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_assoc_scan_gen, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)scan_gen_smem(NSGA3_MAX_M));

@@ -27,6 +27,13 @@ constexpr int EXACT = 1024; // candidates ranked pairwise in the last select pha
 constexpr int CKCAP = 4096; // level-L* reference keys staged in shared memory
 constexpr int RRCAP = 12288; // references whose (rho, rho') are staged in shared memory
 
+// key of reference j: its priority (k_sort.cu writes them for the generation:
+// one block forming up to 12 Philox values per thread here took 4 us), then j
+__device__ __forceinline__ unsigned long long ref_key_of(const RunView& v, int j)
+{
+    return ((unsigned long long)v.rprio[j] << 32) | (unsigned)j;
+}
+
 // ------------------------------------------------ block-wide helpers -------
 __device__ int block_sum(int x, int* scratch)
 {
@@ -193,7 +200,6 @@ __global__ void __launch_bounds__(LB) k_level(RunView v)
     Ctrl* c = v.ctrl;
     if (skip_niche(c)) return;
     const int w = v.w, K = c->K;
-    const uint32_t gen = c->gen;
     const bool staged = w <= RRCAP;
     if (staged) {
         // all loads of a thread in flight at once (one SM does this work)
@@ -328,7 +334,7 @@ __global__ void __launch_bounds__(LB) k_level(RunView v)
             if (j < w) {
                 const int rp = sh.rr[j].y, lo = sh.rr[j].x;
                 v.take[j] = rp > 0 ? min(rp, max(0, Lstar - lo)) : 0;
-                if (rp > 0 && lo <= Lstar && Lstar < lo + rp) kk[t] = ref_key(v.seed, gen, j);
+                if (rp > 0 && lo <= Lstar && Lstar < lo + rp) kk[t] = ref_key_of(v, j);
             }
         }
         __syncthreads();  // every thread has read `before` from the level table
@@ -389,9 +395,9 @@ __global__ void __launch_bounds__(LB) k_level(RunView v)
             if (threadIdx.x == 0) atomicOr(&c->npath, NPATH_BINOVER);
             auto pred = [&](int j) {
                 const int rp = sh.rr[j].y, lo = sh.rr[j].x;
-                return rp > 0 && lo <= Lstar && Lstar < lo + rp && (int)(ref_key(v.seed, gen, j) >> 52) == b;
+                return rp > 0 && lo <= Lstar && Lstar < lo + rp && (int)(ref_key_of(v, j) >> 52) == b;
             };
-            auto key = [&](int j) { return ref_key(v.seed, gen, j); };
+            auto key = [&](int j) { return ref_key_of(v, j); };
             auto mark = [&](int j) { v.take[j] += 1; };
             block_select_smallest(w, need, key, pred, mark, sh.sel, &c->npath);
         }
@@ -407,7 +413,7 @@ __global__ void __launch_bounds__(LB) k_level(RunView v)
             v.take[j] = rp > 0 ? min(rp, max(0, Lstar - lo)) : 0;
             if (rp > 0 && lo <= Lstar && Lstar < lo + rp) {
                 const int p = atomicAdd(&sh.nck, 1);
-                if (p < CKCAP) sh.ck[p] = ref_key(v.seed, gen, j);
+                if (p < CKCAP) sh.ck[p] = ref_key_of(v, j);
             }
         }
         __syncthreads();
@@ -424,7 +430,7 @@ __global__ void __launch_bounds__(LB) k_level(RunView v)
                 const int lo = rho_of(j);
                 return rp > 0 && lo <= Lstar && Lstar < lo + rp;
             };
-            auto key = [&](int j) { return ref_key(v.seed, gen, j); };
+            auto key = [&](int j) { return ref_key_of(v, j); };
             auto mark = [&](int j) { v.take[j] += 1; };
             block_select_smallest(w, r, key, pred, mark, sh.sel, &c->npath);
         }
@@ -458,22 +464,52 @@ __global__ void __launch_bounds__(LB) k_level(RunView v)
 }
 
 // ----------------------------------------------------------- k_bucket ------
-__global__ void k_bucket(RunView v)
+// Members of F_l into their references' lists.  With few references (at most
+// BK_W) many members share one: a CTA numbers its members of each reference
+// in shared memory and takes their places by one global atomic per reference
+// (one per member, hundreds on one address, took 30 us at 165,000 members of
+// 275 references; 7 now).  Each member's priority and distance go with it:
+// the selections read them in list order.
+constexpr int BK = 1024;
+constexpr int BK_W = 4096;
+
+__global__ void __launch_bounds__(BK) k_bucket(RunView v)
 {
+    extern __shared__ int cnt[];  // w counts, then first places (w <= BK_W)
     Ctrl* c = v.ctrl;
     if (skip_niche(c)) return;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= v.n2 || v.rank2[i] != c->l) return;
-    const int j = v.pi[i];
+    const int i = blockIdx.x * BK + threadIdx.x;
+    const bool in = i < v.n2 && v.rank2[i] == c->l;
+    int j = in ? v.pi[i] : 0;
     if (j < 0 || j >= v.w) {
         set_status(c, DEV_EINTERNAL);
-        return;
+        j = -1;
     }
-    const int p = atomicAdd(&v.cursor[j], 1);
-    if (p < v.rhop[j])
-        v.bucket[v.ref_off[j] + p] = i;
-    else
+    const bool mem = in && j >= 0;
+    int p = 0;
+    const double d = in ? v.dist[i] : 0.0;
+    const uint32_t prio = in ? mem_prio(v.seed, c->gen, i) : 0u;
+    if (v.w <= BK_W) {
+        for (int t = threadIdx.x; t < v.w; t += BK) cnt[t] = 0;
+        __syncthreads();
+        if (mem) p = atomicAdd(&cnt[j], 1);
+        __syncthreads();
+        for (int t = threadIdx.x; t < v.w; t += BK)
+            if (cnt[t]) cnt[t] = atomicAdd(&v.cursor[t], cnt[t]);
+        __syncthreads();
+        if (mem) p += cnt[j];
+    } else if (mem) {
+        p = atomicAdd(&v.cursor[j], 1);
+    }
+    if (!mem) return;
+    if (p < v.rhop[j]) {
+        const int at = v.ref_off[j] + p;
+        v.bucket[at] = i;
+        v.bprio[at] = prio;
+        v.bdist[at] = d;
+    } else {
         set_status(c, DEV_EINTERNAL);
+    }
 }
 
 __device__ __forceinline__ void mark_member(const RunView& v, int i)
@@ -482,67 +518,60 @@ __device__ __forceinline__ void mark_member(const RunView& v, int i)
 }
 
 // ------------------------------------------------------------- k_pick ------
-// one warp per reference
+// one warp per reference; a partial take from more than 32 members goes to a
+// whole CTA (k_pick_large), its nearest member too (a warp walking thousands
+// of members for it took 96 us at 165,000 members of 275 references)
 __global__ void __launch_bounds__(256) k_pick(RunView v)
 {
     Ctrl* c = v.ctrl;
-    if (skip_niche(c)) return;
     const int lane = lane_id();
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nw = (gridDim.x * blockDim.x) >> 5;
-    const uint32_t gen = c->gen;
+    if (skip_niche(c)) return;
     for (int j = gw; j < v.w; j += nw) {
-        const int take = v.take[j];
+        const int take = v.take[j], cnt = v.rhop[j], off = v.ref_off[j], rho = v.rho[j];
         if (take == 0) continue;
-        const int cnt = v.rhop[j], off = v.ref_off[j];
         if (take >= cnt) {
             for (int e = lane; e < cnt; e += 32) mark_member(v, v.bucket[off + e]);
             continue;
         }
+        if (cnt > 32) {
+            if (lane == 0) {
+                const int p = atomicAdd(&c->nlarge, 1);
+                v.large[p] = make_int4(j, take, rho, 0);
+                // more members to take than the nearest: the block-wide selection runs
+                if (take > (rho == 0 ? 1 : 0)) atomicOr(&c->npath, NPATH_LARGE);
+            }
+            continue;
+        }
+        // one member per lane
+        int i = -1;
+        double d = CUDART_INF;
+        unsigned long long k = ~0ull;
+        if (lane < cnt) {
+            i = v.bucket[off + lane];
+            d = v.bdist[off + lane];
+            k = ((unsigned long long)v.bprio[off + lane] << 32) | (unsigned)i;
+        }
         int need = take, excl = -1;
-        if (v.rho[j] == 0) {
-            double bd = CUDART_INF;
-            int bi = 0x7fffffff;
-#pragma unroll 4
-            for (int e = lane; e < cnt; e += 32) {
-                const int i = v.bucket[off + e];
-                if (lex_less(v.dist[i], i, bd, bi)) {
-                    bd = v.dist[i];
-                    bi = i;
-                }
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                double od = __shfl_xor_sync(0xffffffffu, bd, o);
-                int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-                if (lex_less(od, oi, bd, bi)) {
-                    bd = od;
-                    bi = oi;
-                }
-            }
-            if (lane == 0) mark_member(v, bi);
-            excl = bi;
+        if (rho == 0) {
+            // nearest: distances are >= 0 and order like their bits
+            unsigned long long b = lane < cnt ? (unsigned long long)__double_as_longlong(d) : ~0ull;
+            const unsigned hi = __reduce_min_sync(0xffffffffu, (unsigned)(b >> 32));
+            const unsigned lo = __reduce_min_sync(0xffffffffu, (unsigned)(b >> 32) == hi ? (unsigned)b : 0xffffffffu);
+            const bool eq = lane < cnt && b == (((unsigned long long)hi << 32) | lo);
+            excl = (int)__reduce_min_sync(0xffffffffu, eq ? (unsigned)i : 0x7fffffffu);
+            if (lane == 0) mark_member(v, excl);
             need -= 1;
         }
         if (need == 0) continue;
-        if (cnt <= 32) {
-            unsigned long long k = ~0ull;
-            int i = -1;
-            if (lane < cnt) {
-                i = v.bucket[off + lane];
-                if (i != excl) k = ((unsigned long long)mem_prio(v.seed, gen, i) << 32) | (unsigned)i;
-            }
-            int rk = 0;
-            for (int b = 0; b < cnt; ++b) {
-                unsigned long long kb = __shfl_sync(0xffffffffu, k, b);
-                rk += kb < k;
-            }
-            if (lane < cnt && i != excl && rk < need) mark_member(v, i);
-        } else if (lane == 0) {
-            const int p = atomicAdd(&c->nlarge, 1);
-            v.large[p] = make_int4(j, need, excl, 0);
-            atomicOr(&c->npath, NPATH_LARGE);
+        if (i == excl) k = ~0ull;
+        int rk = 0;
+        for (int b = 0; b < cnt; ++b) {
+            unsigned long long kb = __shfl_sync(0xffffffffu, k, b);
+            rk += kb < k;
         }
+        if (lane < cnt && i != excl && rk < need) mark_member(v, i);
     }
 }
 
@@ -550,19 +579,55 @@ __global__ void __launch_bounds__(256) k_pick(RunView v)
 __global__ void __launch_bounds__(512) k_pick_large(RunView v)
 {
     __shared__ SelShared sh;
+    __shared__ double sd[16];
+    __shared__ int si[16];
     Ctrl* c = v.ctrl;
     if (skip_niche(c)) return;
     const int nl = c->nlarge;
-    const uint32_t gen = c->gen;
     for (int t = blockIdx.x; t < nl; t += gridDim.x) {
         const int4 L = v.large[t];
-        const int j = L.x, need = L.y, excl = L.z;
+        const int j = L.x;
+        int need = L.y, excl = -1;
         const int cnt = v.rhop[j], off = v.ref_off[j];
         const int32_t* mem = v.bucket + off;
+        if (L.z == 0) {  // rho = 0: the nearest member first
+            double bd = CUDART_INF;
+            int bi = 0x7fffffff;
+#pragma unroll 4
+            for (int e = threadIdx.x; e < cnt; e += 512) {
+                const int i = mem[e];
+                const double d = v.bdist[off + e];
+                if (lex_less(d, i, bd, bi)) {
+                    bd = d;
+                    bi = i;
+                }
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const double od = __shfl_xor_sync(0xffffffffu, bd, o);
+                const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+                if (lex_less(od, oi, bd, bi)) {
+                    bd = od;
+                    bi = oi;
+                }
+            }
+            if (lane_id() == 0) {
+                sd[threadIdx.x >> 5] = bd;
+                si[threadIdx.x >> 5] = bi;
+            }
+            __syncthreads();
+            for (int w = 0; w < 16; ++w)
+                if (lex_less(sd[w], si[w], bd, bi)) {
+                    bd = sd[w];
+                    bi = si[w];
+                }
+            excl = bi;
+            if (threadIdx.x == 0) mark_member(v, bi);
+            need -= 1;
+        }
         auto pred = [&](int e) { return mem[e] != excl; };
         auto key = [&](int e) {
-            const int i = mem[e];
-            return ((unsigned long long)mem_prio(v.seed, gen, i) << 32) | (unsigned)i;
+            return ((unsigned long long)v.bprio[off + e] << 32) | (unsigned)mem[e];
         };
         auto mark = [&](int e) { mark_member(v, mem[e]); };
         block_select_smallest(cnt, need, key, pred, mark, sh, &c->npath);
@@ -596,7 +661,7 @@ cudaError_t launch_level(const RunView& v, cudaStream_t s)
 
 cudaError_t launch_bucket(const RunView& v, cudaStream_t s)
 {
-    k_bucket<<<(v.n2 + 255) / 256, 256, 0, s>>>(v);
+    k_bucket<<<(v.n2 + BK - 1) / BK, BK, v.w <= BK_W ? (size_t)v.w * sizeof(int) : 0, s>>>(v);
     return cudaGetLastError();
 }
 

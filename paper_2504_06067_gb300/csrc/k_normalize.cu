@@ -101,6 +101,11 @@ __device__ __noinline__ void solve_intercepts(const RunView& v, Ctrl* c, const i
     if (row) {
         if (!ok) a = sf64::is_zero(nad[lane]) ? 1.0 : nad[lane];
         c->a[lane] = a;
+        if (m <= NSGA3_FAST_M) {
+            c->da[lane] = sf64::divisor(a);
+            c->z32[lane] = (float)z;
+            c->ia32[lane] = __frcp_rn((float)a);
+        }
     }
     if (lane == 0) c->fallback = ok ? 0 : 1;
     if (v.norm_history) {

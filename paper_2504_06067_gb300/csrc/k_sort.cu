@@ -145,6 +145,7 @@ __device__ __forceinline__ void sel_reset(const RunView& v, int tid, int stride)
         v.rho[j] = 0;
         v.rhop[j] = 0;
         v.cursor[j] = 0;
+        v.rprio[j] = philox((uint32_t)j, v.ctrl->gen, RNG_REFPRIO, 0u, v.seed).x;
     }
     Ctrl* c = v.ctrl;
     if (tid < v.m) c->zmin[tid] = 0xffffffffu;

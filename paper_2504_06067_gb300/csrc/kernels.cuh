@@ -44,20 +44,17 @@ cudaError_t launch_norm_ideal(const RunView& v, cudaStream_t s);
 cudaError_t launch_norm_extreme(const RunView& v, int num_sms, cudaStream_t s);
 cudaError_t norm_init_attributes();
 cudaError_t launch_assoc_prep(const RunView& v, cudaStream_t s);
-// at most this many reference directions (and m <= 10): the association is
-// one kernel with every direction in shared memory (k_assoc_small)
-#define ASSOC_SMALL_W 512
-inline bool assoc_small(const RunView& v) { return v.m <= NSGA3_FAST_M && v.w <= ASSOC_SMALL_W; }
-// FP32 candidate scan, FP64 distances and per-point argmin, FP64 slow path
-// (three launches; four for m > 10, where the distances are a kernel of
-// their own); f' and |f'| are launch_assoc_prep (one launch, two for m > 10)
+// candidate scan, FP64 distances and per-point argmin, FP64 slow path (three
+// launches; four for m > 10, where the distances are a kernel of their own);
+// the unit vectors are launch_assoc_prep (one launch, two for m > 10)
 cudaError_t launch_assoc_scan(const RunView& v, int num_sms, cudaStream_t s);
-cudaError_t assoc_prepare(const RunView& v);
-// tiled association scan (m <= 10, more than ASSOC_SMALL_W directions):
-// its grid for a device of num_sms SMs and the int2 entries it writes for
-// at most n2 points
-int assoc_tile_grid(int num_sms);
-size_t assoc_tile_entries(int n2, int num_sms);
+// m <= 10: the tensor-core scan's grid for a device of num_sms SMs, the int4
+// entries it writes for at most n2 points, the bytes of `rows` FP16 operand
+// rows, and the directions' rows (host)
+int assoc_grid(int num_sms);
+size_t assoc_entries(int n2, int num_sms);
+size_t assoc_rows_bytes(int m, int rows);
+void assoc_pack_refs(int m, int M4, int w, const float* z, unsigned char* out);
 cudaError_t assoc_init_attributes();
 cudaError_t launch_level(const RunView& v, cudaStream_t s);
 cudaError_t launch_bucket(const RunView& v, cudaStream_t s);
