@@ -7,7 +7,8 @@
 //   F     ld x m  FP32 row-major   merged objectives (parents, then children); rows >= n2
 //                                  are NaN padding (never dominate)
 //   PF    N x m   FP32             the parents' objectives between generations
-//   Fp    ld x m  FP32             F in bucket order of f_0 (perm: position -> index)
+//   Fp    ld x fs FP32             F in key order (perm: position -> index); rows of
+//                                  fs = m rounded up to 4 (m > 10: m) floats
 //   Dom   NW x ld u32              bit (i mod 32) of Dom[i/32][j] = "i dominates j",
 //                                  i, j positions in bucket order
 //   rank2 ld int32                 front index of the merged population, -1 = F_drop
@@ -81,6 +82,9 @@ struct Ctrl {
     uint32_t peel_rows;      // dominator word-rows in the peel's row lists, all passes
     uint32_t npath;          // NPATH_* bits: capacity paths the niching kernels took
     int32_t ntile;           // tiles listed in tlist by k_tile_plan
+    int32_t ntask;           // column blocks of k_dominance_front handed out
+    int32_t nF0;             // |F_1| by k_dominance_front
+    int32_t nrem;            // points left for the matrix (0: the first front holds N)
     unsigned long long domstat[8];  // block pairs of the dominance build by mode (zero, f_0
                                     // one-direction, row-dom-column, column-dom-row, both),
                                     // tiles with nothing to test, (lane, column) pairs
@@ -144,7 +148,22 @@ struct RunView {
     int32_t* perm;     // ld   bucket order position -> original index
     uint32_t* skey;    // ld   sort key of each position (0xffffffff for padding)
     uint32_t* pkey;    // n2   sort key of each point (original order)
-    float* Fp;         // ld x m objectives in bucket order, -0.0 as +0.0, NaN padding
+    float* Fp;         // ld x fs objectives in key order, -0.0 as +0.0, NaN padding rows
+    int fs;            // floats per row of Fp: M4 (m <= 10, zero padded) or m
+    // First front before the matrix (null: off).  domw: NW words, dominated
+    // positions; bmin: m rows of NW block minima; kend: NW ends of the keys of
+    // the blocks' last positions; jpos: NW units of row blocks handed out;
+    // Fp2, skey2, rmap: the dominated points in key order and their positions.
+    // A view with rest = 1 has Fp and skey of those points: its kernels take
+    // their number from Ctrl::nrem and do nothing when it is 0.
+    uint32_t* domw;
+    float* bmin;
+    int32_t* kend;
+    int32_t* jpos;
+    float* Fp2;
+    uint32_t* skey2;
+    int32_t* rmap;
+    int rest;
     int32_t* bcnt;     // nkeys key counts
     int32_t* bcur;     // nkeys points of a key placed so far
     int32_t* bgrp;     // nkeys / 32 counts of groups of keys
@@ -294,6 +313,12 @@ __device__ __forceinline__ void set_status(Ctrl* c, int s)
 __device__ __forceinline__ int read_status(const Ctrl* c)
 {
     return *(volatile const int32_t*)&c->status;
+}
+
+// points of a view: all of them, or those the first front left
+__device__ __forceinline__ int view_n2(const RunView& v)
+{
+    return v.rest ? *(volatile const int32_t*)&v.ctrl->nrem : v.n2;
 }
 
 // niching kernels run unconditionally in the graph and return at once when

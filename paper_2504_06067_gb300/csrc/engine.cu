@@ -95,6 +95,23 @@ bool small_varies(const nsga3_ctx* ctx)
     return ctx->v.problem == 0 && (long long)ctx->N * ctx->d <= 16384;
 }
 
+// The first front before the matrix (k_dominance_front): where one front
+// usually holds N points (two and three objectives, integer objectives and
+// complete rankings have many fronts) and the pair tests outweigh its
+// launches.  Selections (us, p = 3 + 2) without and with it, late / early in
+// a run:
+//   2N       m = 5                    m = 8                    m = 10
+//   50,000   226, 228 / 564, 606      269, 258 / 583, 543      287, 299 / 593, 534
+//   65,536   264, 260 / 805, 831      289, 262 / 836, 740      336, 335 / 832, 699
+//   100,000  335, 314 / 1658, 1621    411, 339 / 1602, 1307    457, 405 / 1548, 1167
+// m = 4 gained nowhere up to 100,000 (1 % lost), m = 6 from 65,536 on
+// (255, 238 / 785, 784).
+bool first_front_wanted(const RunView& v)
+{
+    return v.m >= 5 && v.m <= NSGA3_FAST_M && v.n2 >= 65536 && (long long)v.m * v.n2 >= 6 * 65536 && v.problem == 0 &&
+           !v.full_sort;
+}
+
 // Kernels of one selection / one generation; m > 10: with the ideal point,
 // extreme-point keys and reduction, |f'| and candidate distances, m > 32 the
 // cooperative elimination, and a split dominance build (few tiles) its
@@ -103,7 +120,8 @@ int select_launches(const nsga3_ctx* ctx)
 {
     if (ctx->small) return 1;
     const int m = ctx->m;
-    if (m <= NSGA3_FAST_M) return 19;
+    // (first front: three more)
+    if (m <= NSGA3_FAST_M) return 19 + (ctx->v.domw ? 3 : 0);
     return 24 + (m > NSGA3_WARP_M ? 1 : 0) + (ctx->v.dom_ks > 1 ? 1 : 0);
 }
 // the softmax-simplex objective's dot-product kernel (m > 10)
@@ -206,10 +224,12 @@ nsga3_status record_selection(nsga3_ctx* ctx, const RunView& v, cudaStream_t s,
     CK(launch_sort(v, ctx->num_sms, s));
     nsga3_status st = record_event(ctx, s, EV_RESET, events);
     if (st) return st;
-    CK(launch_dominance(v, s));
+    CK(launch_first_front(v, s));
+    const RunView rest = rest_view(v);
+    CK(launch_dominance(rest, s));
     st = record_event(ctx, s, EV_DOM, events);
     if (st) return st;
-    CK(launch_peel(v, ctx->num_sms, s));
+    CK(launch_peel(rest, ctx->num_sms, s));
     st = record_event(ctx, s, EV_PEEL, events);
     if (st) return st;
     // ranks back to the original order, then (when niching is needed) the
@@ -256,10 +276,12 @@ nsga3_status eager_selection(nsga3_ctx* ctx, const RunView& v, cudaStream_t s, b
     CK(launch_sort(v, ctx->num_sms, s));
     nsga3_status st = record_event(ctx, s, EV_RESET, true);
     if (st) return st;
-    CK(launch_dominance(v, s));
+    CK(launch_first_front(v, s));
+    const RunView rest = rest_view(v);
+    CK(launch_dominance(rest, s));
     st = record_event(ctx, s, EV_DOM, true);
     if (st) return st;
-    CK(launch_peel(v, ctx->num_sms, s));
+    CK(launch_peel(rest, ctx->num_sms, s));
     st = record_event(ctx, s, EV_PEEL, true);
     if (st) return st;
     CK(launch_norm_ideal(v, s));  // also writes the ranks back in the original order
@@ -479,7 +501,17 @@ nsga3_status setup_alloc(nsga3_ctx* ctx)
     AL(v.perm, ld);
     AL(v.skey, ld);
     AL(v.pkey, n2);
-    AL(v.Fp, (size_t)ld * m);
+    v.fs = m <= NSGA3_FAST_M ? M4 : m;
+    AL(v.Fp, (size_t)ld * v.fs);
+    if (first_front_wanted(v)) {
+        AL(v.domw, NW);
+        AL(v.bmin, (size_t)NW * m);
+        AL(v.kend, NW);
+        AL(v.jpos, NW);
+        AL(v.Fp2, (size_t)ld * v.fs);
+        AL(v.skey2, ld);
+        AL(v.rmap, ld);
+    }
     // sort keys (k_sort.cu): m <= 10 interleaves lbits of level per objective
     // (Morton order), truncated to kbits, about n2 / 2 keys; above, 4,096 f_0 buckets
     if (m <= NSGA3_FAST_M) {

@@ -149,12 +149,13 @@ __global__ void __launch_bounds__(256) k_block_box(RunView v)
     __shared__ float slo[8][NSGA3_FAST_M], shi[8][NSGA3_FAST_M];
     __shared__ uint32_t skmin[8], skmax[8];
     if (read_status(v.ctrl)) return;
+    if (v.rest && (int)blockIdx.x * NSGA3_TILE >= view_n2(v)) return;
     const int lane = lane_id(), warp = threadIdx.x >> 5, m = v.m, M4 = v.M4;
     const int b = blockIdx.x * 8 + warp;
     const int p = b * 32 + lane;
     float* box = v.bbox + (size_t)b * 2 * M4;
     for (int q = 0; q < m; ++q) {
-        float lo = v.Fp[(size_t)p * m + q], hi = lo;
+        float lo = v.Fp[(size_t)p * v.fs + q], hi = lo;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
@@ -165,6 +166,27 @@ __global__ void __launch_bounds__(256) k_block_box(RunView v)
             box[M4 + q] = hi;
             slo[warp][q] = lo;
             shi[warp][q] = hi;
+            if (v.bmin && !v.rest) v.bmin[(size_t)q * v.NW + b] = lo;
+        }
+    }
+    if (v.rest && (warp & 3) == 3) {
+        // the row limit of the peel's chunk that ends with this block: the
+        // end of its last column's key (a long run of one key: no limit)
+        const int n = view_n2(v), last = min(p - lane + 32, n) - 1, chunk = b / (NSGA3_PEEL_COLS / 32);
+        const int c0 = chunk * NSGA3_PEEL_COLS;
+        if (c0 < n) {
+            const int e0 = max(last, min(c0 + NSGA3_PEEL_COLS, n) - 1);
+            const uint32_t key = v.skey[e0];
+            int end = n;
+            for (int t = 0; t < 32; ++t) {
+                const int e = e0 + 1 + 32 * t + lane;
+                const unsigned other = __ballot_sync(0xffffffffu, e >= n || v.skey[e] != key);
+                if (other) {
+                    end = e0 + 32 * t + __ffs(other);
+                    break;
+                }
+            }
+            if (lane == 0) v.chunk_lim[chunk] = (uint32_t)((min(end, n) + 31) >> 5);
         }
     }
     const uint32_t k = v.skey[p];
@@ -211,10 +233,13 @@ __global__ void __launch_bounds__(256) k_tile_plan(RunView v)
     Ctrl* c = v.ctrl;
     if (t >= (long long)T * (T + 1) / 2) return;
     if (read_status(c)) return;
+    const int n2 = view_n2(v);
+    if (n2 == 0) return;
     int ti, tj;
     decode_tile(t, T, ti, tj);
+    if (v.rest && tj * NSGA3_TILE >= n2) return;
     bool work = ti == tj;
-    if (!work && tj * NSGA3_TILE < v.n2) {
+    if (!work && tj * NSGA3_TILE < n2) {
         const float* bi = v.tbox + (size_t)ti * 2 * M4;
         const float* bj = v.tbox + (size_t)tj * 2 * M4;
         bool fwd = true, bwd = true;
@@ -226,41 +251,17 @@ __global__ void __launch_bounds__(256) k_tile_plan(RunView v)
         bwd = bwd && !(v.tkey[2 * ti + 1] < v.tkey[2 * tj]);
         work = fwd || bwd;
     }
-    if (work)
-        v.tlist[atomicAdd(&c->ntile, 1)] = (int32_t)t;
-    else
-        atomicAdd(&c->domstat[5], 1ull);
-}
-
-// Mode of block pair (ib, jb) from the blocks' boxes and keys (warp-wide:
-// lane q < M compares objective q).  Row i can dominate column j only if
-// f_iq <= f_jq for every q, so some row of I can dominate some column of J
-// only if min_I q <= max_J q for every q (fwd), and symmetrically (bwd); when
-// a box test fails, some objective separates every pair of the two blocks,
-// so their vectors differ and the other direction's dominance needs no
-// strictness test.  Dominators never have a larger sort key, so every key
-// of I below every key of J also rules out "column dom row".
-template <int M>
-__device__ __forceinline__ int block_pair_mode(const RunView& v, int ib, int jb)
-{
-    if (jb < ib) return BP_SKIP;
-    if (jb == ib) return BP_FULL;
-    if (jb * 32 >= v.n2) return BP_ZERO;  // a column block of padding only
-    constexpr int M4 = (M + 3) & ~3;
-    const int lane = lane_id();
-    const float* bi = v.bbox + (size_t)ib * 2 * M4;
-    const float* bj = v.bbox + (size_t)jb * 2 * M4;
-    const int q = lane < M ? lane : 0;
-    const float imin = bi[q], imax = bi[M4 + q], jmin = bj[q], jmax = bj[M4 + q];
-    // NaN boxes (padding only) fail every comparison: no dominance
-    const bool fwd = __all_sync(0xffffffffu, lane >= M || imin <= jmax);
-    const bool bwd = __all_sync(0xffffffffu, lane >= M || jmin <= imax) && !(v.bkey[2 * ib + 1] < v.bkey[2 * jb]);
-    const bool f0sep = __shfl_sync(0xffffffffu, imax < jmin, 0);  // every row f_0 below every column f_0
-    if (!fwd && !bwd) return BP_ZERO;
-    if (fwd && f0sep) return BP_FAST0;
-    if (fwd && !bwd) return BP_FASTK;
-    if (!fwd) return BP_FASTR;
-    return BP_FULL;
+    // one atomic per warp: tens of thousands on one address took most of this
+    // kernel's 14 us at m = 10, N = 100,000
+    const unsigned act = __activemask(), yes = __ballot_sync(act, work);
+    const int lane = lane_id(), lead = __ffs(act) - 1;
+    int at = 0;
+    if (lane == lead) {
+        if (yes) at = atomicAdd(&c->ntile, __popc(yes));
+        if (yes != act) atomicAdd(&c->domstat[5], (unsigned long long)__popc(act & ~yes));
+    }
+    at = __shfl_sync(act, at, lead);
+    if (work) v.tlist[at + __popc(yes & ((1u << lane) - 1u))] = (int32_t)t;
 }
 
 // Words of Dom block (dominator block of the word row, 32 columns): written
@@ -535,11 +536,6 @@ __device__ __forceinline__ void entry_row_dom_col(const RunView& v, const float*
 
 // Asynchronous copies into shared memory (cp.async: the data lands while
 // the CTA keeps working; wait_all + a barrier make it visible to all).
-__device__ __forceinline__ void cp_async4(void* dst, const void* src)
-{
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
-}
 __device__ __forceinline__ void cp_async8(void* dst, const void* src)
 {
     const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
@@ -600,6 +596,7 @@ __global__ void __launch_bounds__(256, M <= 8 ? 5 : 4) k_dominance(RunView v)
     if (read_status(v.ctrl)) return;
     const int T = v.ld / NSGA3_TILE;
     const int ntile = *(volatile const int32_t*)&v.ctrl->ntile;
+    const int n2 = view_n2(v);
     if ((int)blockIdx.x >= ntile) return;
     const int tid = threadIdx.x, warp = tid >> 5, lane = lane_id();
     auto srow_of = [&](int buf) { return dsm + buf * BUF; };
@@ -613,12 +610,11 @@ __global__ void __launch_bounds__(256, M <= 8 ? 5 : 4) k_dominance(RunView v)
     auto copy_points = [&](int ti, int tj, int buf) {
         float* dr = srow_of(buf);
         float* dc = scol_of(buf);
-        const float* gr = v.Fp + (size_t)ti * NSGA3_TILE * M;
-        const float* gc = v.Fp + (size_t)tj * NSGA3_TILE * M;
-        for (int e = tid; e < NSGA3_TILE * M; e += blockDim.x) {
-            const int p = e / M, q = e - p * M;
-            cp_async4(dr + p * M4 + q, gr + e);
-            cp_async4(dc + p * M4 + q, gc + e);
+        const float* gr = v.Fp + (size_t)ti * NSGA3_TILE * M4;
+        const float* gc = v.Fp + (size_t)tj * NSGA3_TILE * M4;
+        for (int e = 4 * tid; e < NSGA3_TILE * M4; e += 4 * blockDim.x) {
+            cp_async16(dr + e, gr + e);
+            cp_async16(dc + e, gc + e);
         }
         cp_async_commit();
     };
@@ -651,7 +647,7 @@ __global__ void __launch_bounds__(256, M <= 8 ? 5 : 4) k_dominance(RunView v)
                 mode = BP_SKIP;
             else if (jb == ib)
                 mode = BP_FULL;
-            else if (jb * 32 >= v.n2)
+            else if (jb * 32 >= n2)
                 mode = BP_ZERO;  // a column block of padding only
             else {
                 const float* bi = sb + ri * 2 * M4;
@@ -762,7 +758,7 @@ __global__ void __launch_bounds__(256, M <= 8 ? 5 : 4) k_dominance(RunView v)
             // NaN with a clear sign bit), so the bits of padding rows and
             // columns are masked (the two-way test needs no mask: a NaN
             // gives the same sign both ways, hence no bit).
-            const int cv = v.n2 - jb * 32;
+            const int cv = n2 - jb * 32;
             const uint32_t colvalid = cv >= 32 ? 0xffffffffu : (cv > 0 ? (1u << cv) - 1u : 0u);
             if (mode == BP_FAST0 || mode == BP_FASTK) {
                 // "row dominates column" only, one row block or two
@@ -778,7 +774,7 @@ __global__ void __launch_bounds__(256, M <= 8 ? 5 : 4) k_dominance(RunView v)
             uint32_t dij = 0u, dji = 0u;
             if (mode == BP_FASTR) {
                 // column j dominates row i: no f_jq > f_iq (the vectors differ)
-                const bool rowvalid = ib * 32 + lane < v.n2;
+                const bool rowvalid = ib * 32 + lane < n2;
                 uint32_t acc = 0u;
 #pragma unroll 4
                 for (int k = 31; k >= 0; --k) {
@@ -850,6 +846,271 @@ __global__ void __launch_bounds__(256, M <= 8 ? 5 : 4) k_dominance(RunView v)
     if (tid == 0 && stat[0]) {
         atomicAdd(&v.ctrl->domstat[6], 32ull * stat[0]);
         atomicAdd(&v.ctrl->domstat[7], stat[1]);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// The first front alone (m >= 5).  Late in a run it holds N points or more,
+// and the selection needs nothing of the rest: which points are dominated,
+// not by whom.  Once a point is known to be dominated it need be looked at no
+// more, as a column (it is decided) or as a row (whatever dominates it
+// dominates what it dominates).
+//
+// A warp takes a column block J (a lane per column, objectives in registers)
+// and units of row blocks up to the end of the keys of J's last column (a
+// dominator never has a larger key).  Row blocks whose box minimum lies above
+// the live columns' maxima h somewhere are passed over, 32 at a time (a lane
+// per block); of the others the rows not above h anywhere go, from row block
+// after row block, into a buffer, and a full buffer is tested row by row
+// (broadcast loads) by all columns at once: ceil(m / 2) packed subtractions and as
+// many ORs per row.  The OR of the differences f_j - f_i has its sign bit set
+// iff some f_i > f_j and is zero only for equal vectors, so i dominates j iff
+// it is positive.  Dominated columns leave h at once and the other warps'
+// rows through domw.  Column blocks differ by two orders of magnitude (one
+// near the ideal point meets nothing, one far from it most row blocks): a
+// warp without a block of its own joins one that has units left (fixed
+// segments of row blocks left half the time to the tail at m = 6, N = 60,000,
+// short ones cost their set-up; whole tiles staged in shared memory, as the
+// matrix build stages them, cost more instructions than the tests).
+//
+// Bound: instruction issue (per row block met about 45 warp instructions, per
+// row tested 14) at half the issue slots, and the latency of the row blocks'
+// reads from L2.  Measured (the dominance phase with the matrix of all points, and with
+// this kernel and the rest's matrix): generations of m = 10, N = 100,000 1,060 and
+// 660 us, a selection early in that run 5.1 and 3.2 ms, m = 6, N = 60,000 200
+// and 140 us.  Blocks of 32 points interleaved by objective in place of rows, and
+// two or four CTAs per SM in place of three, gave the same times or longer ones.
+// The rest (l > 0) goes through the matrix build and the peel as a
+// smaller population (k_split_front).
+constexpr int FW = 8;        // warps per CTA
+constexpr int RBUF = 64;     // buffered rows per warp
+constexpr int RFULL = 32;    // rows at which a buffer is tested
+constexpr int PROBES = 6;    // looks for units left before a warp ends
+constexpr int JDONE = 1 << 28;
+
+template <int M>
+__global__ void __launch_bounds__(FW * 32, 3) k_dominance_front(RunView v, int UB)
+{
+    constexpr int M4 = (M + 3) & ~3, Q4 = M4 / 4, H = (M + 1) / 2;
+    __shared__ float4 rbuf[FW][RBUF * Q4];
+    Ctrl* c = v.ctrl;
+    if (read_status(c)) return;
+    const int lane = lane_id(), warp = threadIdx.x >> 5;
+    const uint32_t lt = (1u << lane) - 1u;
+    const int nblk = (v.n2 + 31) / 32, nchunk = (nblk + 31) / 32;
+    const float4* Fp4 = reinterpret_cast<const float4*>(v.Fp);
+    volatile uint32_t* domw = v.domw;
+    volatile int32_t* jpos = v.jpos;
+    float4* rb = rbuf[warp];
+    const uint32_t rbase = (uint32_t)__cvta_generic_to_shared(rb);
+    unsigned long long tested = 0ull, livep = 0ull;
+    unsigned entries = 0u;
+    int next = 0;  // (lane 0) the column block after this one, taken ahead
+    if (lane == 0) next = atomicAdd(&c->ntask, 1);
+    unsigned probe = (unsigned)(blockIdx.x * FW + warp) * 40503u;  // where to look for units left
+    int misses = 0;
+    for (;;) {
+        // column blocks in ascending order: low keys are decided first
+        int J = __shfl_sync(0xffffffffu, next, 0);
+        if (J < nblk) {
+            if (lane == 0) next = atomicAdd(&c->ntask, 1);
+        } else {
+            // all are begun: join the one with the most units left of 32
+            if (misses == PROBES) break;
+            const int k = (int)((probe >> 8) % (unsigned)nchunk) * 32 + lane;
+            probe = probe * 1664525u + 1013904223u;
+            const int left = k < nblk ? (v.kend[k] + 32 * UB - 1) / (32 * UB) - jpos[k] : 0;
+            const int most = __reduce_max_sync(0xffffffffu, max(left, 0));
+            if (most == 0) {
+                ++misses;
+                continue;
+            }
+            misses = 0;
+            J = __shfl_sync(0xffffffffu, k, __ffs(__ballot_sync(0xffffffffu, left == most)) - 1);
+        }
+        int unit = 0;  // (lane 0) the next one taken ahead
+        if (lane == 0) unit = atomicAdd(&v.jpos[J], 1);
+        const int I1 = (v.kend[J] + 31) / 32;
+        bool alive = J * 32 + lane < v.n2 && !((domw[J] >> lane) & 1u);
+        unsigned long long pj[2 * Q4];  // (the pads are 0)
+#pragma unroll
+        for (int q4 = 0; q4 < Q4; ++q4) {
+            const float4 x = Fp4[(size_t)(J * 32 + lane) * Q4 + q4];
+            pj[2 * q4] = p2_pack(x.x, x.y);
+            pj[2 * q4 + 1] = p2_pack(x.z, x.w);
+        }
+        float h[M];  // maxima of the live columns
+        auto maxima = [&]() {
+#pragma unroll
+            for (int q = 0; q < M; ++q) {
+                const float f = __uint_as_float((uint32_t)(pj[q / 2] >> (32 * (q & 1))));
+                h[q] = s2f(__reduce_max_sync(0xffffffffu, alive ? f2s(f) : (int)0x80000000));
+            }
+        };
+        bool go = __any_sync(0xffffffffu, alive);
+        if (go) maxima();
+        int nbuf = 0;
+        // tests the buffered rows; false when no column is left
+        auto flush = [&]() -> bool {
+            __syncwarp();
+            int d = 0;  // positive once a row dominates this lane's column
+#pragma unroll 4
+            for (int t = 0; t < nbuf; ++t) {
+                unsigned long long y[M4 / 2];
+                lds_col<M4>(rbase + (uint32_t)(t * M4 * 4), y);
+                uint32_t w[2 * H];
+#pragma unroll
+                for (int k = 0; k < H; ++k) p2_sub(pj[k], y[k], w[2 * k], w[2 * k + 1]);
+                uint32_t acc = w[0];
+#pragma unroll
+                for (int k = 1; k < 2 * H; k += 2) acc = k + 1 < 2 * H ? or3(acc, w[k], w[k + 1]) : (acc | w[k]);
+                d = max(d, (int)acc);
+            }
+            __syncwarp();
+            tested += 32u * (unsigned)nbuf;
+            const unsigned on = __ballot_sync(0xffffffffu, alive);
+            livep += (unsigned)__popc(on) * (unsigned)nbuf;
+            nbuf = 0;
+            const unsigned fresh = __ballot_sync(0xffffffffu, alive && d > 0);
+            if (fresh && lane == 0) atomicOr(&v.domw[J], fresh);
+            const unsigned now = fresh | (domw[J] & on);  // other warps' finds too
+            if (!now) return true;
+            alive = alive && !((now >> lane) & 1u);
+            if (now == on) return false;
+            maxima();
+            return true;
+        };
+        while (go) {
+            const int u0 = __shfl_sync(0xffffffffu, unit, 0) * UB;
+            if (u0 >= I1) break;
+            if (lane == 0) unit = atomicAdd(&v.jpos[J], 1);
+            const int u1 = min(u0 + UB, I1);
+            for (int Ib = u0; Ib < u1 && go; Ib += 32) {
+                const int I = min(Ib + lane, u1 - 1);
+                float nb[M];
+#pragma unroll
+                for (int q = 0; q < M; ++q) nb[q] = __ldg(v.bmin + (size_t)q * v.NW + I);
+                const uint32_t rows = ~domw[I];
+                bool ok = Ib + lane < u1 && rows != 0u;
+#pragma unroll
+                for (int q = 0; q < M; ++q) ok &= nb[q] <= h[q];
+                unsigned msk = __ballot_sync(0xffffffffu, ok);
+                entries += __popc(msk);
+                while (msk && go) {
+                    // two row blocks' loads in flight
+                    const int ba = __ffs(msk) - 1;
+                    msk &= msk - 1u;
+                    const int bb = msk ? __ffs(msk) - 1 : ba;
+                    const bool two = msk != 0u;
+                    msk &= msk - 1u;
+                    const uint32_t ra = __shfl_sync(0xffffffffu, rows, ba), rbits = __shfl_sync(0xffffffffu, rows, bb);
+                    float4 xa[Q4], xb[Q4];
+#pragma unroll
+                    for (int q4 = 0; q4 < Q4; ++q4) xa[q4] = Fp4[(size_t)((Ib + ba) * 32 + lane) * Q4 + q4];
+#pragma unroll
+                    for (int q4 = 0; q4 < Q4; ++q4) xb[q4] = Fp4[(size_t)((Ib + bb) * 32 + lane) * Q4 + q4];
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        if (u == 1 && !two) break;
+                        const float4* x = u ? xb : xa;
+                        bool live = ((u ? rbits : ra) >> lane) & 1u;  // (NaN padding rows fail the comparisons)
+#pragma unroll
+                        for (int q4 = 0; q4 < Q4; ++q4) {
+                            live &= x[q4].x <= h[4 * q4];
+                            if (4 * q4 + 1 < M) live &= x[q4].y <= h[4 * q4 + 1];
+                            if (4 * q4 + 2 < M) live &= x[q4].z <= h[4 * q4 + 2];
+                            if (4 * q4 + 3 < M) live &= x[q4].w <= h[4 * q4 + 3];
+                        }
+                        const unsigned bal = __ballot_sync(0xffffffffu, live);
+                        if (live) {
+                            const int at = nbuf + __popc(bal & lt);
+#pragma unroll
+                            for (int q4 = 0; q4 < Q4; ++q4) rb[at * Q4 + q4] = x[q4];
+                        }
+                        nbuf += __popc(bal);
+                        if (nbuf > RBUF - RFULL) {
+                            go = flush();
+                            if (!go) break;
+                        }
+                    }
+                }
+            }
+        }
+        if (go && nbuf) go = flush();
+        if (!go && lane == 0) jpos[J] = JDONE;
+    }
+    if (lane == 0 && entries) {
+        atomicAdd(&c->domstat[2], (unsigned long long)entries);
+        atomicAdd(&c->domstat[6], tested);
+        atomicAdd(&c->domstat[7], livep);
+    }
+}
+
+// The first front's rank, and whether it is the last one needed: with N
+// points or more in it the selection goes on with l = 0; else the dominated
+// points, in key order, become the matrix build's and the peel's population
+// (Fp2, skey2, rmap; NaN rows up to a whole tile).  A thread per position; a
+// CTA adds up the words itself.
+__global__ void __launch_bounds__(1024) k_split_front(RunView v)
+{
+    __shared__ int s_pre[32], s_tot[32];
+    Ctrl* c = v.ctrl;
+    const int tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
+    const int nw = (v.n2 + 31) / 32, w0 = blockIdx.x * 32;
+    int pre = 0, tot = 0;  // first front: before this CTA's words, all
+    for (int w = tid; w < nw; w += 1024) {
+        const uint32_t valid = w * 32 + 32 <= v.n2 ? 0xffffffffu : (1u << (v.n2 - w * 32)) - 1u;
+        const int x = __popc(~v.domw[w] & valid);
+        tot += x;
+        if (w < w0) pre += x;
+    }
+    if (read_status(c)) return;
+    pre = warp_sum(pre);
+    tot = warp_sum(tot);
+    if (lane == 0) {
+        s_pre[warp] = pre;
+        s_tot[warp] = tot;
+    }
+    __syncthreads();
+    pre = warp_sum(s_pre[lane]);
+    tot = warp_sum(s_tot[lane]);
+    const bool rest = tot < v.N;
+    const int p = (int)blockIdx.x * 1024 + tid;
+    const uint32_t word = w0 + warp < nw ? v.domw[w0 + warp] : 0u;
+    // dominated before this position: all before it but the first front's
+    int own = 0;
+    for (int t = 0; t < warp; ++t)
+        if (w0 + t < nw) own += __popc(~v.domw[w0 + t]);  // (only the last word is ragged)
+    const bool dom = p < v.n2 && ((word >> lane) & 1u);
+    if (p < v.n2 && !dom) v.srank[p] = 0;
+    if (rest && dom) {
+        const int r = p - (pre + own + __popc(~word & ((1u << lane) - 1u)));
+        const int n4 = v.fs / 4;
+        for (int q = 0; q < n4; ++q)
+            reinterpret_cast<float4*>(v.Fp2)[(size_t)r * n4 + q] = reinterpret_cast<const float4*>(v.Fp)[(size_t)p * n4 + q];
+        v.skey2[r] = v.skey[p];
+        v.rmap[r] = p;
+    }
+    if (blockIdx.x != 0) return;
+    const int nr = rest ? v.n2 - tot : 0;
+    const int pad = (nr + NSGA3_TILE - 1) / NSGA3_TILE * NSGA3_TILE;
+    for (int e = nr * v.fs + tid; e < pad * v.fs; e += 1024) v.Fp2[e] = __int_as_float(0x7fc00000);
+    for (int e = nr + tid; e < pad; e += 1024) v.skey2[e] = 0xffffffffu;
+    if (tid == 0) {
+        c->ntile = 0;  // the rest's plan makes its own list
+        c->nF0 = tot;
+        c->nrem = nr;
+        c->cum = tot;
+        c->passes = 1;
+        c->passes_total += 1ull;
+        if (!rest) {
+            c->l = 0;
+            c->nFl = tot;
+            c->nS = 0;
+            c->K = v.N;
+            c->need_niche = v.N < tot ? 1 : 0;
+        }
+        if (tot == 0) set_status(c, DEV_EINTERNAL);
     }
 }
 
@@ -1049,6 +1310,28 @@ __global__ void __launch_bounds__(256) k_dom_finish(RunView v)
 }
 
 template <int M>
+cudaError_t launch_front_m(const RunView& v, cudaStream_t s)
+{
+    k_block_box<<<(unsigned)(v.ld / NSGA3_TILE), 256, 0, s>>>(v);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    static int occ = 0;  // per M; the same value whatever the run
+    if (occ <= 0 &&
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_dominance_front<M>, FW * 32, 0) != cudaSuccess) {
+        cudaGetLastError();
+        occ = 2;
+    }
+    // every resident warp; units of 32 row blocks, more where a column block
+    // has many
+    const int nblk = (v.n2 + 31) / 32, UB = nblk < 4096 ? 32 : 128;
+    k_dominance_front<M><<<(unsigned)((occ > 0 ? occ : 2) * v.num_sms), FW * 32, 0, s>>>(v, UB);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    k_split_front<<<(v.n2 + 1023) / 1024, 1024, 0, s>>>(v);
+    return cudaGetLastError();
+}
+
+template <int M>
 cudaError_t launch_dom_m(const RunView& v, cudaStream_t s)
 {
     long long T = v.ld / NSGA3_TILE;
@@ -1096,6 +1379,31 @@ cudaError_t dom_init_attributes()
     if (e == cudaSuccess) e = dom_attr_m<9>();
     if (e == cudaSuccess) e = dom_attr_m<10>();
     return e;
+}
+
+RunView rest_view(const RunView& v)
+{
+    RunView r = v;
+    if (v.domw) {
+        r.Fp = v.Fp2;
+        r.skey = v.skey2;
+        r.rest = 1;
+    }
+    return r;
+}
+
+cudaError_t launch_first_front(const RunView& v, cudaStream_t s)
+{
+    if (!v.domw) return cudaSuccess;
+    switch (v.m) {
+    case 5: return launch_front_m<5>(v, s);
+    case 6: return launch_front_m<6>(v, s);
+    case 7: return launch_front_m<7>(v, s);
+    case 8: return launch_front_m<8>(v, s);
+    case 9: return launch_front_m<9>(v, s);
+    case 10: return launch_front_m<10>(v, s);
+    default: return cudaErrorInvalidValue;
+    }
 }
 
 cudaError_t launch_dominance(const RunView& v, cudaStream_t s)

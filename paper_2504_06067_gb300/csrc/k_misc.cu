@@ -175,12 +175,10 @@ __global__ void k_slots_init(RunView v)
 
 __global__ void k_nan_pad(RunView v)
 {
-    const long long lo = (long long)v.n2 * v.m, hi = (long long)v.ld * v.m;
-    for (long long e = lo + blockIdx.x * (long long)blockDim.x + threadIdx.x; e < hi;
-         e += (long long)gridDim.x * blockDim.x) {
-        v.F[e] = __int_as_float(0x7fc00000);
+    const long long t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
+    for (long long e = (long long)v.n2 * v.m + t0; e < (long long)v.ld * v.m; e += stride) v.F[e] = __int_as_float(0x7fc00000);
+    for (long long e = (long long)v.n2 * v.fs + t0; e < (long long)v.ld * v.fs; e += stride)
         v.Fp[e] = __int_as_float(0x7fc00000);
-    }
     for (int p = v.n2 + blockIdx.x * blockDim.x + threadIdx.x; p < v.ld; p += gridDim.x * blockDim.x)
         v.skey[p] = 0xffffffffu;
 }

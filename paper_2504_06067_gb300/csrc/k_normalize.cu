@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(NB) k_norm_ideal(RunView v)
     __shared__ uint32_t smin[NB / 32][NSGA3_FAST_M];
     const int warp = threadIdx.x >> 5;
     for (int q = 0; q < v.m; ++q) {
-        uint32_t o = inZ ? f2ord(v.Fp[(size_t)p * v.m + q]) : 0xffffffffu;
+        uint32_t o = inZ ? f2ord(v.Fp[(size_t)p * v.fs + q]) : 0xffffffffu;
         o = __reduce_min_sync(0xffffffffu, o);
         if (lane == 0) smin[warp][q] = o;
     }

@@ -38,24 +38,30 @@ __global__ void __launch_bounds__(PEEL_THREADS, STREAM ? 1 : 2) k_peel(RunView v
     Ctrl* c = v.ctrl;
     const int tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
     if (read_status(c)) return;  // uniform: set only by earlier kernels
-    const int nchunks = v.ld / NSGA3_PEEL_COLS;
+    // the view's points, and the fronts and points before them (rest: the
+    // first front is taken; no rest: it held N points)
+    const int n2 = view_n2(v), before = v.rest ? 1 : 0;
+    if (n2 == 0) return;
+    const int nchunks = v.rest ? (n2 + NSGA3_PEEL_COLS - 1) / NSGA3_PEEL_COLS : v.ld / NSGA3_PEEL_COLS;
     // every CTA follows the same sequence of front sizes, so each keeps the
     // pass state itself; CTA 0 also publishes it in ctrl
-    int cum = 0, l = -1;
+    const int cum0 = v.rest ? *(volatile const int32_t*)&c->nF0 : 0;
+    int cum = cum0, l = -1;
     for (int k = 0;; ++k) {
         if (tid == 0) s_fs = 0u;  // read after the barrier's first __syncthreads
         __syncthreads();
         for (int chunk = blockIdx.x; chunk < nchunks; chunk += gridDim.x) {
             const int j0 = chunk * NSGA3_PEEL_COLS;
             // prefetch this thread's column state (used after the reduction)
-            int my_rank = 0, my_cnt = 0;
-            if (tid < NSGA3_PEEL_COLS && j0 + tid < v.n2) {
-                my_rank = __ldcg(&v.srank[j0 + tid]);
+            int my_rank = 0, my_cnt = 0, my_pos = j0 + tid;  // (srank is by position among all points)
+            if (tid < NSGA3_PEEL_COLS && j0 + tid < n2) {
+                if (v.rest) my_pos = v.rmap[j0 + tid];
+                my_rank = __ldcg(&v.srank[my_pos]);
                 my_cnt = __ldcg(&v.cnt[j0 + tid]);
             }
             // dominators of a column have a sort key <= its key: the chunk's row
             // blocks end with its last column's key (k_sort.cu)
-            const int lim = j0 < v.n2 ? min((int)v.chunk_lim[chunk], v.NW) : 0;
+            const int lim = j0 < n2 ? min((int)v.chunk_lim[chunk], v.NW) : 0;
 
             uint32_t rw = (tid < NSGA3_PEEL_COLS / 32) ? __ldcg(&v.rem[j0 / 32 + tid]) : 0u;
             const int any_rem = __syncthreads_or(rw != 0u);
@@ -76,7 +82,7 @@ __global__ void __launch_bounds__(PEEL_THREADS, STREAM ? 1 : 2) k_peel(RunView v
                 for (int t = 0; t < 4; ++t) {
 #pragma unroll
                     for (int q = 0; q < NSGA3_FAST_M; ++q)
-                        fc[t][q] = q < m ? v.Fp[(size_t)(j0 + lane * 4 + t) * m + q] : 0.0f;
+                        fc[t][q] = q < m ? v.Fp[(size_t)(j0 + lane * 4 + t) * v.fs + q] : 0.0f;
                     cmin = fminf(cmin, fc[t][0]);  // NaN padding columns are ignored by fminf
                 }
 #pragma unroll
@@ -106,7 +112,7 @@ __global__ void __launch_bounds__(PEEL_THREADS, STREAM ? 1 : 2) k_peel(RunView v
                             const size_t p = (size_t)L.x * 32 + lane;
 #pragma unroll
                             for (int q = 0; q < NSGA3_FAST_M; ++q)
-                                if (q < m) rb[lane * NSGA3_FAST_M + q] = __ldg(&v.Fp[p * m + q]);
+                                if (q < m) rb[lane * NSGA3_FAST_M + q] = __ldg(&v.Fp[p * v.fs + q]);
                         }
                         __syncwarp();
                         uint32_t mk = L.y;
@@ -218,11 +224,11 @@ __global__ void __launch_bounds__(PEEL_THREADS, STREAM ? 1 : 2) k_peel(RunView v
                 for (int w = 0; w < PW; ++w) sum += red[w][tid];
                 const int j = j0 + tid;
                 bool nf = false;
-                if (j < v.n2 && my_rank < 0) {
+                if (j < n2 && my_rank < 0) {
                     const int cv = my_cnt - sum;
                     if (k > 0) v.cnt[j] = cv;
                     if (cv == 0) {
-                        v.srank[j] = k;
+                        v.srank[my_pos] = k + before;
                         nf = true;
                     }
                 }
@@ -241,21 +247,21 @@ __global__ void __launch_bounds__(PEEL_THREADS, STREAM ? 1 : 2) k_peel(RunView v
         const unsigned long long tot = grid_sync_sum(c, &c->pbar, &c->prel, (unsigned)k, s_fs, v.wait_ns, &s_cum);
         if (tot == ~0ull) return;
         // close front k (the same decision in every CTA)
-        const int ncum = (int)tot;
+        const int ncum = cum0 + (int)tot;
         const int fs = ncum - cum;
         bool first = false;
         if (l < 0 && ncum >= v.N) {
-            l = k;
+            l = k + before;
             first = true;
         }
         const bool broken = fs == 0 && ncum < v.n2;
         const bool more = !broken && fs > 0 && ncum < v.n2 && (v.full_sort || l < 0);
         if (blockIdx.x == 0 && tid == 0) {
             c->cum = ncum;
-            c->passes = k + 1;
+            c->passes = k + 1 + before;
             c->passes_total += 1ull;
             if (first) {
-                c->l = k;
+                c->l = l;
                 c->nFl = fs;
                 c->nS = cum;
                 c->K = v.N - cum;

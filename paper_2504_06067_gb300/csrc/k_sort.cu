@@ -140,6 +140,10 @@ __device__ __forceinline__ void sel_reset(const RunView& v, int tid, int stride)
             m = (1u << (v.n2 - lo)) - 1u;
         v.rem[wd] = m;
         v.selmask[wd] = 0u;
+        if (v.domw) {
+            v.domw[wd] = 0u;
+            v.jpos[wd] = 0;
+        }
     }
     for (int j = tid; j < v.w; j += stride) {
         v.rho[j] = 0;
@@ -169,6 +173,9 @@ __device__ __forceinline__ void sel_reset(const RunView& v, int tid, int stride)
         c->nlarge = 0;
         c->npath = 0u;
         c->ntile = 0;
+        c->ntask = 0;
+        c->nF0 = 0;
+        c->nrem = 0;
         c->peel_rows = 0u;
         c->ncand = 0;
         c->nslow = 0;
@@ -323,6 +330,7 @@ __device__ __forceinline__ void chunk_limit(const RunView& v, int pos, int end)
 {
     if ((pos & (NSGA3_PEEL_COLS - 1)) == NSGA3_PEEL_COLS - 1 || pos == v.n2 - 1)
         v.chunk_lim[pos / NSGA3_PEEL_COLS] = (uint32_t)((end + 31) >> 5);
+    if (v.kend && ((pos & 31) == 31 || pos == v.n2 - 1)) v.kend[pos / 32] = end;
 }
 
 __global__ void __launch_bounds__(TB) k_sort_scatter(RunView v)
@@ -344,11 +352,17 @@ __global__ void __launch_bounds__(TB) k_sort_scatter(RunView v)
         spos[threadIdx.x] = pos;
     }
     __syncthreads();
-    // rows, consecutive threads on consecutive values
-    const int ne = min(TB, v.n2 - i0) * m;
+    // rows: a thread per 16 bytes
+    const int n4 = v.fs / 4, ne = min(TB, v.n2 - i0) * n4;
     for (int e = threadIdx.x; e < ne; e += TB) {
-        const int r = e / m;
-        v.Fp[(size_t)spos[r] * m + (e - r * m)] = v.F[(size_t)i0 * m + e] + 0.0f;
+        const int r = e / n4, q = 4 * (e - r * n4);
+        const float* f = v.F + (size_t)(i0 + r) * m + q;
+        float4 x;
+        x.x = f[0] + 0.0f;
+        x.y = q + 1 < m ? f[1] + 0.0f : 0.0f;
+        x.z = q + 2 < m ? f[2] + 0.0f : 0.0f;
+        x.w = q + 3 < m ? f[3] + 0.0f : 0.0f;
+        *reinterpret_cast<float4*>(v.Fp + (size_t)spos[r] * v.fs + q) = x;
     }
 }
 

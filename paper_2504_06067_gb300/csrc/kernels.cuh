@@ -32,6 +32,10 @@ cudaError_t launch_front(const RunView& v, int num_sms, bool check, cudaStream_t
 cudaError_t launch_wait_probe(const RunView& v, cudaStream_t s);
 cudaError_t launch_check_finite(const RunView& v, cudaStream_t s);
 cudaError_t launch_sort(const RunView& v, int num_sms, cudaStream_t s);
+// the first front (v.domw set; nothing otherwise); the view of the points it
+// leaves (v itself when there is no first front)
+cudaError_t launch_first_front(const RunView& v, cudaStream_t s);
+RunView rest_view(const RunView& v);
 cudaError_t launch_dominance(const RunView& v, cudaStream_t s);
 cudaError_t dom_init_attributes();
 // every peel pass in one cooperative launch (grid barrier between passes)
