@@ -9,7 +9,7 @@
 //   PF    N x m   FP32             the parents' objectives between generations
 //   Fp    ld x fs FP32             F in key order (perm: position -> index); rows of
 //                                  fs = m rounded up to 4 (m > 10: m) floats
-//   Dom   NW x ld u32              bit (i mod 32) of Dom[i/32][j] = "i dominates j",
+//   Dom   NW x ld u32              bit (i mod 32) of Dom[i/32][j] (dom_at) = "i dominates j",
 //                                  i, j positions in bucket order
 //   rank2 ld int32                 front index of the merged population, -1 = F_drop
 //   pi/dist ld                     association (reference index, FP64 distance)
@@ -26,6 +26,7 @@
 #define NSGA3_WARP_M 32         // largest m whose intercept system one warp solves
 #define NSGA3_TILE 256          // column tile of the dominance build; ld % 256 == 0
 #define NSGA3_PEEL_COLS 128     // columns per peel chunk (4 per lane, 32 lanes)
+#define NSGA3_FRONT_RING 8      // passes whose front masks are kept
 #define SORT_NB 4096            // sort keys of the f_0 bucket order (m > 10)
 #define SORT_LMAX 7             // level thresholds per objective (3 bits of level)
 
@@ -69,8 +70,6 @@ struct Ctrl {
     int32_t fallback;        // normalization used the nadir fallback
     int32_t passes;          // peel passes (kernel launches) in the last selection
     uint32_t sbar;           // arrivals at the barriers of the cooperative elimination
-    unsigned long long pbar; // peel barrier: arrivals << 32 | points ranked so far
-    unsigned long long prel; // peel barrier release: passes closed << 32 | points ranked
     uint32_t never;          // a word nothing sets (the wait self-test polls it)
     int32_t nT;              // |S u F_l| (association set)
     int32_t Lstar;           // niche level threshold L*
@@ -82,6 +81,7 @@ struct Ctrl {
     uint32_t peel_rows;      // dominator word-rows in the peel's row lists, all passes
     uint32_t npath;          // NPATH_* bits: capacity paths the niching kernels took
     int32_t ntile;           // tiles listed in tlist by k_tile_plan
+    uint32_t parr;           // CTAs arrived at the peel's barriers
     int32_t ntask;           // column blocks of k_dominance_front handed out
     int32_t nF0;             // |F_1| by k_dominance_front
     int32_t nrem;            // points left for the matrix (0: the first front holds N)
@@ -141,7 +141,7 @@ struct RunView {
     int32_t* cslot;    // N  row of merged individual N + c (the children of the last variation)
     float* Xtmp;       // N x d staging of get / set calls on pageable host memory
     int32_t* bsum;     // selected individuals per 1,024 merged ones
-    uint32_t* Dom;     // NW x ld
+    uint32_t* Dom;     // NW x ld words (dom_at)
     int32_t* cnt;      // ld   remaining dominator counts
     int32_t* rank2;    // ld   merged ranks (original order)
     int32_t* srank;    // ld   merged ranks in bucket order (peel)
@@ -182,7 +182,8 @@ struct RunView {
                        // server): the cooperative peel takes fewer CTAs, so that it can
                        // start while other runs' kernels hold part of every SM
     uint32_t* rem;     // NW   not-yet-ranked mask
-    uint32_t* front;   // 2 x NW  ping-pong front masks
+    uint32_t* front;    // NSGA3_FRONT_RING x NW front masks of the last passes
+    uint32_t* selword;  // NW selected individuals (k_mark)
     uint32_t* chunk_lim;   // ld / NSGA3_PEEL_COLS dominator row blocks a column chunk reads
     uint32_t* selmask;     // NW picked members of F_l
     int32_t* Tlist;        // n2 members of S u F_l
@@ -315,6 +316,15 @@ __device__ __forceinline__ int read_status(const Ctrl* c)
     return *(volatile const int32_t*)&c->status;
 }
 
+// Word of Dom: dominator block I, column lane of column block J.  The peel's
+// chunks of 128 columns are contiguous (NW rows of 512 bytes: a chunk's rows
+// share a page or two; as rows of ld words each lay in another 100 KB).
+__device__ __forceinline__ size_t dom_at(const RunView& v, int I, int J, int lane)
+{
+    constexpr int B = NSGA3_PEEL_COLS / 32;
+    return ((size_t)(J / B) * v.NW + I) * NSGA3_PEEL_COLS + (J % B) * 32 + lane;
+}
+
 // points of a view: all of them, or those the first front left
 __device__ __forceinline__ int view_n2(const RunView& v)
 {
@@ -353,16 +363,9 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned* p)
     return x;
 }
 
-__device__ __forceinline__ unsigned long long ld_acquire64(const unsigned long long* p)
+__device__ __forceinline__ void red_release(unsigned* p, unsigned x)
 {
-    unsigned long long x;
-    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];\n" : "=l"(x) : "l"(p) : "memory");
-    return x;
-}
-
-__device__ __forceinline__ void st_release64(unsigned long long* p, unsigned long long x)
-{
-    asm volatile("st.release.gpu.global.u64 [%0], %1;\n" ::"l"(p), "l"(x) : "memory");
+    asm volatile("red.release.gpu.global.add.u32 [%0], %1;\n" ::"l"(p), "r"(x) : "memory");
 }
 
 // Polls `done` until it returns true or wait_ns of device time have passed
@@ -381,38 +384,6 @@ __device__ __forceinline__ bool bounded_wait(Ctrl* c, unsigned long long wait_ns
         }
     }
     return true;
-}
-
-// Summing barrier of the peel: pass k's barrier adds (1 << 32) + add (this
-// CTA's new front members) to *bar; the CTA whose addition completes the
-// (k+1) * gridDim.x arrivals holds the running total of every CTA's adds
-// (no CTA can add for pass k+1 before that) and releases it with the pass
-// number in *rel, which the others poll.  Returns the total (< 2^32) or,
-// on a timeout, ~0ull.  *bar and *rel are zero at launch.
-__device__ __forceinline__ unsigned long long grid_sync_sum(Ctrl* c, unsigned long long* bar, unsigned long long* rel,
-                                                           unsigned k, unsigned add, unsigned long long wait_ns,
-                                                           unsigned long long* s_val)
-{
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long val;
-        __threadfence();
-        const unsigned long long inc = (1ull << 32) | add;
-        const unsigned long long now = atomicAdd(bar, inc) + inc;
-        if ((now >> 32) == (unsigned long long)(k + 1) * gridDim.x) {
-            val = now & 0xffffffffull;
-            __threadfence();  // the arrivals' writes before the release
-            st_release64(rel, ((unsigned long long)(k + 1) << 32) | val);
-        } else {
-            unsigned long long r = 0;
-            const bool ok = bounded_wait(c, wait_ns, [&] { return ((r = ld_acquire64(rel)) >> 32) >= k + 1ull; });
-            val = ok ? (r & 0xffffffffull) : ~0ull;
-        }
-        __threadfence();
-        *s_val = val;
-    }
-    __syncthreads();
-    return *s_val;
 }
 
 // Counting barrier: the k-th barrier of a launch waits until *ctr reaches

@@ -538,8 +538,8 @@ nsga3_status setup_alloc(nsga3_ctx* ctx)
         AL(v.tlist, T * (T + 1) / 2);
         if (!v.streaming) AL(v.dnz, (size_t)NW * v.NB8);
     }
-    AL(v.rem, NW);
-    AL(v.front, 2 * NW);
+    AL(v.front, (size_t)NSGA3_FRONT_RING * NW);
+    AL(v.selword, NW);
     AL(v.chunk_lim, ld / NSGA3_PEEL_COLS);
     AL(v.selmask, NW);
     AL(v.Tlist, n2);

@@ -525,10 +525,10 @@ __device__ __forceinline__ void entry_row_dom_col(const RunView& v, const float*
     }
     w0 = mine ? w0 : 0u;
     w1 = mine ? w1 : 0u;
-    put_block(v, (size_t)ib * v.ld + jb * 32 + lane, w0, nz, ri, cb);
+    put_block(v, dom_at(v, ib, jb, lane), w0, nz, ri, cb);
     int cc = __popc(w0);
     if (two) {
-        put_block(v, (size_t)(ib + 1) * v.ld + jb * 32 + lane, w1, nz, ri + 1, cb);
+        put_block(v, dom_at(v, ib + 1, jb, lane), w1, nz, ri + 1, cb);
         cc += __popc(w1);
     }
     if (cc) atomicAdd(&ccnt[cb * 32 + lane], cc);
@@ -787,12 +787,12 @@ __global__ void __launch_bounds__(256, M <= 8 ? 5 : 4) k_dominance(RunView v)
             }
             // column i = ib*32 + lane, dominators j in block jb: Dom block (jb, ib)
             if (jb != ib) {
-                put_block(v, (size_t)jb * v.ld + ib * 32 + lane, dji, nz, 8 + cb, ri);
+                put_block(v, dom_at(v, jb, ib, lane), dji, nz, 8 + cb, ri);
                 const uint32_t tr = warp_transpose32(dij);
-                put_block(v, (size_t)ib * v.ld + jb * 32 + lane, tr, nz, ri, cb);
+                put_block(v, dom_at(v, ib, jb, lane), tr, nz, ri, cb);
                 if (tr) atomicAdd(&ccnt[cb * 32 + lane], __popc(tr));
             } else {
-                put_block(v, (size_t)jb * v.ld + ib * 32 + lane, dji, nz, ri, cb);
+                put_block(v, dom_at(v, jb, ib, lane), dji, nz, ri, cb);
             }
             if (dji) atomicAdd(&rcnt[ri * 32 + lane], __popc(dji));
         }
@@ -1262,14 +1262,14 @@ __global__ void __launch_bounds__(256) k_dominance_gen(RunView v)
             // i dom j: no f_i > f_j and some f_j > f_i (B is implied in a fast block)
             const uint32_t dij = fast ? ~A[cbi][r] : (B[cbi][r] & ~A[cbi][r]);
             const uint32_t dji = fast ? 0u : (A[cbi][r] & ~B[cbi][r]);
-            if (!v.streaming) D[(size_t)jb * v.ld + ib * 32 + lane] = dji;
+            if (!v.streaming) D[dom_at(v, jb, ib, lane)] = dji;
             if (r)
                 rc1 += __popc(dji);
             else
                 rc0 += __popc(dji);
             if (jb != ib) {
                 const uint32_t t = warp_transpose32(dij);
-                if (!v.streaming) D[(size_t)ib * v.ld + jb * 32 + lane] = t;
+                if (!v.streaming) D[dom_at(v, ib, jb, lane)] = t;
                 if (t) atomicAdd(&colcnt[cb * 32 + lane], __popc(t));
             }
         }
@@ -1300,11 +1300,11 @@ __global__ void __launch_bounds__(256) k_dom_finish(RunView v)
     const bool fast = one_direction(v, ib, jb);
     const uint32_t dij = fast ? ~a : (b & ~a);
     const uint32_t dji = fast ? 0u : (a & ~b);
-    v.Dom[at] = dji;
+    v.Dom[dom_at(v, jb, ib, lane)] = dji;
     if (dji) atomicAdd(&v.cnt[ib * 32 + lane], __popc(dji));
     if (jb != ib) {
         const uint32_t tr = warp_transpose32(dij);
-        v.Dom[(size_t)ib * v.ld + jb * 32 + lane] = tr;
+        v.Dom[dom_at(v, ib, jb, lane)] = tr;
         if (tr) atomicAdd(&v.cnt[jb * 32 + lane], __popc(tr));
     }
 }

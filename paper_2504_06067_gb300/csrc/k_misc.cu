@@ -23,7 +23,7 @@ __global__ void k_check_finite(RunView v)
 // of a 5,600 us selection at N = 100,000, 7 of 227 us at N = 10,628).
 __global__ void __launch_bounds__(1024) k_mark(RunView v)
 {
-    uint32_t* words = v.front;  // front masks are dead after the peel: NW words of scratch
+    uint32_t* words = v.selword;
     __shared__ int cnt[32];
     Ctrl* c = v.ctrl;
     const int lane = lane_id(), warp = threadIdx.x >> 5;
@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(GB) k_gather(RunView v, int mode)
     __shared__ int s_pre[GB / 32], s_tot[GB / 32];
     Ctrl* c = v.ctrl;
     const int lane = lane_id(), warp = threadIdx.x >> 5, tid = threadIdx.x;
-    const uint32_t* words = v.front;
+    const uint32_t* words = v.selword;
     const int nb = (v.NW + 31) / 32, b0 = blockIdx.x >> 2, w0 = blockIdx.x * (GB / 32);
     int pre = 0, tot = 0;
     for (int t = tid; t < nb; t += GB) {

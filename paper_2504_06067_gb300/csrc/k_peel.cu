@@ -2,19 +2,33 @@
 // (Alg. 1, the non-dominated sort: fronts F_1, F_2, ... until |F_1| + ... + |F_l| >= N,
 // splitting R_t into S = F_1..F_{l-1}, F_l and F_drop; Sec. II-C).
 //
-// One cooperative launch runs every pass: the CTAs meet at a grid barrier
-// (common.cuh) after each pass and all take the same decision from the
-// front size, so the host never synchronises.
-// Positions are in bucket order of f_0 (k_sort.cu); ranks are written back
-// to the original order by k_norm_ideal.
+// One cooperative launch runs every pass: each CTA writes its columns' words
+// of the front, waits for the others and counts the words itself, so that all
+// take the same decision and the host never synchronises.
+// Positions are in key order (k_sort.cu); ranks are written back to the
+// original order by k_norm_ideal.
 //   cnt[j]    = dominators of j, counted by the dominance build
 //   pass k>0: cnt[j] -= popc(Dom[w][j] & front_{k-1}[w]) over the nonzero
 //             words w of the previous front's mask
 //   front_k   = { j unranked : cnt[j] == 0 }, rank2[j] = k
-// A CTA of 32 warps owns 128 columns (uint4 per lane); its warps split the
+// A CTA of 16 warps owns 128 columns (uint4 per lane); its warps split the
 // dominator rows and meet in shared memory, so the CTA alone updates its
-// columns' counts, ranks them and writes their front-mask words.  Bound:
-// HBM / L2 bandwidth of the Dom reads.
+// columns' counts, ranks them and writes their front words.  A chunk of
+// columns whose smallest count exceeds the points ranked since it was last
+// looked at has no member in this front: it is passed over and later counts
+// those fronts off together (half of the points are never ranked, and most
+// chunks hold a point of a few fronts only).
+//
+// Bound: latency.  A pass is a chain of trips through L2 (Dom rows, arrival
+// with its release, the poll, the front words), 5 us in all however few the
+// points of its front, about 3 of them from the arrival to the words.  So the
+// block bitmap is kept in shared memory (it was a dependent load before every
+// row), four rows are in flight per warp (eight spill and took 10 % longer)
+// and a chunk's counts stay in registers.  Selections of the knapsack (m = 3,
+// N = 12,800, 27 to 48 fronts): 296 us before, 202 now; m = 5, N = 10,628,
+// three fronts: 38 us before, 20 now; the first generation of m = 10,
+// N = 100,000: 342 us before, 128 now.
+#include <limits.h>
 #include <math_constants.h>
 
 #include "kernels.cuh"
@@ -24,6 +38,9 @@ namespace {
 constexpr int PEEL_THREADS = 512;  // threads per CTA
 constexpr int PWMAX = PEEL_THREADS / 32;
 constexpr int LISTCAP = 2048;
+constexpr int RING = NSGA3_FRONT_RING;
+constexpr int PEEL_U = 4;   // Dom rows in flight per warp
+constexpr int MAXC = 64;  // chunks of a CTA whose state is kept between passes
 
 template <bool STREAM>
 __global__ void __launch_bounds__(PEEL_THREADS, STREAM ? 1 : 2) k_peel(RunView v)
@@ -31,9 +48,13 @@ __global__ void __launch_bounds__(PEEL_THREADS, STREAM ? 1 : 2) k_peel(RunView v
     __shared__ int red[PWMAX][NSGA3_PEEL_COLS];
     const int PT = blockDim.x, PW = PT >> 5;
     __shared__ uint2 list[LISTCAP];
-    __shared__ int nlist;
-    __shared__ unsigned s_fs;             // this CTA's members of the front of this pass
-    __shared__ unsigned long long s_cum;  // points ranked, from the barrier
+    __shared__ int wcnt[2][PWMAX];
+    __shared__ uint32_t last[LISTCAP];   // the last pass's front words (the first LISTCAP; own: of all passes not counted off)
+    __shared__ unsigned char nibs[LISTCAP];  // of the CTA's only chunk: column blocks with bits, per dominator block
+    __shared__ int nlist[2];
+    __shared__ unsigned s_fs[3];  // size of a pass's front
+    __shared__ int s_fail;
+    __shared__ int c_min[MAXC], c_eval[MAXC], c_cum[MAXC];  // per chunk: smallest count left, pass of it, points then
     __shared__ float rowbuf[STREAM ? PWMAX : 1][32][NSGA3_FAST_M];  // streaming: members of a front word
     Ctrl* c = v.ctrl;
     const int tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
@@ -43,33 +64,68 @@ __global__ void __launch_bounds__(PEEL_THREADS, STREAM ? 1 : 2) k_peel(RunView v
     const int n2 = view_n2(v), before = v.rest ? 1 : 0;
     if (n2 == 0) return;
     const int nchunks = v.rest ? (n2 + NSGA3_PEEL_COLS - 1) / NSGA3_PEEL_COLS : v.ld / NSGA3_PEEL_COLS;
+    if ((int)blockIdx.x >= nchunks) return;  // owns no columns: nobody waits for it
+    const int nwords = nchunks * (NSGA3_PEEL_COLS / 32);
+    const bool single = nchunks <= (int)gridDim.x;
+    const bool own = single && nwords <= LISTCAP;  // pending words stay in shared memory
+    int lim1 = 0, my_cnt = 0;
+    bool my_open = false;  // not ranked yet
+    unsigned nrows = 0u;   // (per warp) Dom rows read
+    bool evald = true;  // (own) the chunk was evaluated in the pass before
+    if (tid < 2) nlist[tid] = 0;
+    if (tid < 3) s_fs[tid] = 0u;
+    if (tid == 0) s_fail = 0;
+    if (tid < MAXC) c_min[tid] = INT_MAX;
+    __syncthreads();
     // every CTA follows the same sequence of front sizes, so each keeps the
     // pass state itself; CTA 0 also publishes it in ctrl
     const int cum0 = v.rest ? *(volatile const int32_t*)&c->nF0 : 0;
-    int cum = cum0, l = -1;
+    int cum = cum0, l = -1, par = 0;
     for (int k = 0;; ++k) {
-        if (tid == 0) s_fs = 0u;  // read after the barrier's first __syncthreads
-        __syncthreads();
-        for (int chunk = blockIdx.x; chunk < nchunks; chunk += gridDim.x) {
+        // cum: the points ranked before pass k
+        int slot = 0;
+        for (int chunk = blockIdx.x; chunk < nchunks; chunk += gridDim.x, ++slot) {
             const int j0 = chunk * NSGA3_PEEL_COLS;
-            // prefetch this thread's column state (used after the reduction)
-            int my_rank = 0, my_cnt = 0, my_pos = j0 + tid;  // (srank is by position among all points)
-            if (tid < NSGA3_PEEL_COLS && j0 + tid < n2) {
-                if (v.rest) my_pos = v.rmap[j0 + tid];
-                my_rank = __ldcg(&v.srank[my_pos]);
-                my_cnt = __ldcg(&v.cnt[j0 + tid]);
+            // the fronts of passes k0 .. k-1 are not counted off yet
+            int k0 = k - 1;
+            if (k > 0 && slot < MAXC) {
+                k0 = c_eval[slot];
+                const int least = c_min[slot];
+                evald = !(least == INT_MAX || (least > cum - c_cum[slot] && (own || k - k0 < RING - 1)));
+                if (!evald) {
+                    if (tid < NSGA3_PEEL_COLS / 32)
+                        v.front[(size_t)(k % RING) * v.NW + j0 / 32 + tid] = 0u;
+                    continue;
+                }
+            }
+            // the points ranked in passes k0 .. k-1, by word
+            auto pending = [&](int w) {
+                uint32_t x = w < LISTCAP ? last[w] : __ldcg(&v.front[(size_t)((k - 1) % RING) * v.NW + w]);
+                if (own) return x;
+                for (int kk = k0; kk < k - 1; ++kk) x |= __ldcg(&v.front[(size_t)(kk % RING) * v.NW + w]);
+                return x;
+            };
+            // this thread's column: dominators not counted off (0: ranked or
+            // no column); used after the reduction
+            if (tid < NSGA3_PEEL_COLS && !(single && k > 0)) {
+                const bool in = j0 + tid < n2;
+                my_cnt = in ? __ldcg(&v.cnt[j0 + tid]) : 0;
+                my_open = in && (k == 0 || my_cnt > 0);
             }
             // dominators of a column have a sort key <= its key: the chunk's row
             // blocks end with its last column's key (k_sort.cu)
-            const int lim = j0 < n2 ? min((int)v.chunk_lim[chunk], v.NW) : 0;
-
-            uint32_t rw = (tid < NSGA3_PEEL_COLS / 32) ? __ldcg(&v.rem[j0 / 32 + tid]) : 0u;
-            const int any_rem = __syncthreads_or(rw != 0u);
+            const int lim = single && k > 0 ? lim1 : j0 < n2 ? min((int)v.chunk_lim[chunk], v.NW) : 0;
+            lim1 = lim;
+            const int J0 = j0 / 32;
+            const uint8_t* nz = v.dnz ? v.dnz + (J0 >> 3) : nullptr;
+            if (!STREAM && k == 0 && single)
+                for (int w = tid; w < min(lim, LISTCAP); w += PT)
+                    nibs[w] = nz ? (nz[(size_t)w * v.NB8] >> (J0 & 4)) & 15 : 15;
 
             uint32_t a0 = 0, a1 = 0, a2 = 0, a3 = 0;
             // pass 0 needs no words: the dominance build already counted every
             // column's dominators into cnt[]
-            if (STREAM && any_rem && k > 0) {
+            if (STREAM && k > 0) {
                 // no matrix: every member of front k-1 (up to the row limit)
                 // is tested against this lane's four columns lane*4 .. +3,
                 // with the sign-bit test of the dominance build; a member
@@ -88,23 +144,23 @@ __global__ void __launch_bounds__(PEEL_THREADS, STREAM ? 1 : 2) k_peel(RunView v
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) cmin = fminf(cmin, __shfl_xor_sync(0xffffffffu, cmin, o));
                 float* rb = rowbuf[warp][0];
-                const uint32_t* prev = v.front + ((k - 1) & 1) * v.NW;
                 for (int wb = 0; wb < lim; wb += LISTCAP) {
                     const int whe = min(wb + LISTCAP, lim);
-                    if (tid == 0) nlist = 0;
-                    __syncthreads();
+                    int* const nl = &nlist[par];
                     for (int w0 = wb + warp * 32; w0 < whe; w0 += PT) {
                         const int w = w0 + lane;
-                        const uint32_t msk = w < whe ? __ldcg(&prev[w]) : 0u;
+                        const uint32_t msk = w < whe ? pending(w) : 0u;
                         const unsigned bal = __ballot_sync(0xffffffffu, msk != 0u);
                         int at = 0;
-                        if (lane == 0 && bal) at = atomicAdd(&nlist, __popc(bal));
+                        if (lane == 0 && bal) at = atomicAdd(nl, __popc(bal));
                         at = __shfl_sync(0xffffffffu, at, 0);
                         if (msk) list[at + __popc(bal & ((1u << lane) - 1u))] = make_uint2((unsigned)w, msk);
                     }
                     __syncthreads();
-                    const int n = nlist;
-                    if (tid == 0) atomicAdd(&c->peel_rows, (unsigned)n);
+                    const int n = *nl;
+                    par ^= 1;
+                    if (tid == 0) nlist[par] = 0;
+                    if (warp == 0) nrows += (unsigned)n;
                     for (int e = warp; e < n; e += PW) {
                         const uint2 L = list[e];
                         // the word's members, one per lane, into this warp's row buffer
@@ -150,105 +206,134 @@ __global__ void __launch_bounds__(PEEL_THREADS, STREAM ? 1 : 2) k_peel(RunView v
                         }
                         __syncwarp();
                     }
-                    __syncthreads();
+                    __syncthreads();  // list and nlist are reused
                 }
-            } else if (!STREAM && any_rem && k > 0) {
-                const uint4* base = reinterpret_cast<const uint4*>(v.Dom + j0) + lane;
-                const size_t ld4 = (size_t)v.ld / 4;
+            } else if (!STREAM && k > 0) {
+                const uint4* base = reinterpret_cast<const uint4*>(v.Dom + dom_at(v, 0, J0, 0)) + lane;
                 // with the block bitmap (m <= 10) only the Dom blocks whose bit
-                // is set were written this selection: the lane's column block
-                // J = j0 / 32 + lane / 8 is read from dominator block w only if
-                // bit J of dnz[w] is set
-                const int Jb = j0 / 32 + (lane >> 3);
-                const uint8_t* nzrow = v.dnz ? v.dnz + (Jb >> 3) : nullptr;
-                const unsigned nzbit = 1u << (Jb & 7);
-                auto load = [&](unsigned w) -> uint4 {
-                    if (nzrow && !(nzrow[(size_t)w * v.NB8] & nzbit)) return make_uint4(0u, 0u, 0u, 0u);
-                    return __ldg(base + (size_t)w * ld4);
-                };
-                {
-                    const uint32_t* prev = v.front + ((k - 1) & 1) * v.NW;
-                    for (int wb = 0; wb < lim; wb += LISTCAP) {
-                        const int whe = min(wb + LISTCAP, lim);
-                        if (tid == 0) nlist = 0;
-                        __syncthreads();
-                        for (int w0 = wb + warp * 32; w0 < whe; w0 += PT) {
-                            const int w = w0 + lane;
-                            const uint32_t msk = w < whe ? __ldcg(&prev[w]) : 0u;
-                            const unsigned bal = __ballot_sync(0xffffffffu, msk != 0u);
-                            int at = 0;
-                            if (lane == 0 && bal) at = atomicAdd(&nlist, __popc(bal));
-                            at = __shfl_sync(0xffffffffu, at, 0);
-                            if (msk) list[at + __popc(bal & ((1u << lane) - 1u))] = make_uint2((unsigned)w, msk);
-                        }
-                        __syncthreads();
-                        const int n = nlist;
-                        if (tid == 0) atomicAdd(&c->peel_rows, (unsigned)n);
-                        int e = warp;
-                        for (; e + 3 * PW < n; e += 4 * PW) {
-                            uint2 L[4];
-                            uint4 x[4];
+                // is set were written this selection: bit t of an entry's top
+                // nibble says that the chunk's t-th column block is read from
+                // dominator block w.  Known before the first Dom load, so the
+                // loads of PEEL_U entries are in flight at once.
+                const unsigned mybit = 1u << (28 + (lane >> 3));
+                for (int wb = 0; wb < lim; wb += LISTCAP) {
+                    // the words with members that dominate one of the columns,
+                    // a warp's after those of the warps before it (adding up
+                    // in one counter took 1 us)
+                    constexpr int G = LISTCAP / PEEL_THREADS;
+                    unsigned nib[G];
+                    uint32_t msk[G];
+                    int mine = 0;
 #pragma unroll
-                            for (int t = 0; t < 4; ++t) {
-                                L[t] = list[e + PW * t];
-                                x[t] = load(L[t].x);
-                            }
-#pragma unroll
-                            for (int t = 0; t < 4; ++t) {
-                                a0 += __popc(x[t].x & L[t].y);
-                                a1 += __popc(x[t].y & L[t].y);
-                                a2 += __popc(x[t].z & L[t].y);
-                                a3 += __popc(x[t].w & L[t].y);
-                            }
+                    for (int g = 0; g < G; ++g) {
+                        const int w = wb + g * PEEL_THREADS + tid;
+                        nib[g] = 0u;
+                        msk[g] = 0u;
+                        if (w < lim) {
+                            nib[g] = single && w < LISTCAP ? nibs[w] : nz ? ((unsigned)nz[(size_t)w * v.NB8] >> (J0 & 4)) & 15u : 15u;
+                            msk[g] = pending(w);
                         }
-                        for (; e < n; e += PW) {
-                            const uint2 L = list[e];
-                            const uint4 x = load(L.x);
-                            a0 += __popc(x.x & L.y);
-                            a1 += __popc(x.y & L.y);
-                            a2 += __popc(x.z & L.y);
-                            a3 += __popc(x.w & L.y);
-                        }
-                        __syncthreads();
+                        mine += __popc(__ballot_sync(0xffffffffu, msk[g] != 0u && nib[g] != 0u));
                     }
+                    if (lane == 0) wcnt[par][warp] = mine;
+                    __syncthreads();
+                    const int x0 = lane < PWMAX ? wcnt[par][lane] : 0;
+                    const int n = __reduce_add_sync(0xffffffffu, x0);
+                    int at = __reduce_add_sync(0xffffffffu, lane < warp ? x0 : 0);
+                    par ^= 1;
+#pragma unroll
+                    for (int g = 0; g < G; ++g) {
+                        const bool in = msk[g] != 0u && nib[g] != 0u;
+                        const unsigned bal = __ballot_sync(0xffffffffu, in);
+                        if (in)
+                            list[at + __popc(bal & ((1u << lane) - 1u))] =
+                                make_uint2((unsigned)(wb + g * PEEL_THREADS + tid) | nib[g] << 28, msk[g]);
+                        at += __popc(bal);
+                    }
+                    __syncthreads();
+                    if (warp == 0) nrows += (unsigned)n;
+                    for (int e = warp; e < n; e += PEEL_U * PWMAX) {
+                        uint32_t mk[PEEL_U];
+                        uint4 x[PEEL_U];
+#pragma unroll
+                        for (int t = 0; t < PEEL_U; ++t) {
+                            const uint2 L = e + PWMAX * t < n ? list[e + PWMAX * t] : make_uint2(0u, 0u);
+                            mk[t] = L.y;
+                            x[t] = L.x & mybit ? __ldg(base + (size_t)(L.x & 0x0fffffffu) * (NSGA3_PEEL_COLS / 4)) : make_uint4(0u, 0u, 0u, 0u);
+                        }
+#pragma unroll
+                        for (int t = 0; t < PEEL_U; ++t) {
+                            a0 += __popc(x[t].x & mk[t]);
+                            a1 += __popc(x[t].y & mk[t]);
+                            a2 += __popc(x[t].z & mk[t]);
+                            a3 += __popc(x[t].w & mk[t]);
+                        }
+                    }
+                    if (wb + LISTCAP < lim) __syncthreads();  // list is reused
                 }
             }
             red[warp][lane * 4 + 0] = (int)a0;
             red[warp][lane * 4 + 1] = (int)a1;
             red[warp][lane * 4 + 2] = (int)a2;
             red[warp][lane * 4 + 3] = (int)a3;
+            if (tid == 0 && slot < MAXC) c_min[slot] = INT_MAX;
             __syncthreads();
             // this CTA owns its 128 columns: update the counts and rank the new front
             if (tid < NSGA3_PEEL_COLS) {
                 int sum = 0;
-                for (int w = 0; w < PW; ++w) sum += red[w][tid];
+#pragma unroll
+                for (int w = 0; w < PWMAX; ++w) sum += red[w][tid];
                 const int j = j0 + tid;
-                bool nf = false;
-                if (j < n2 && my_rank < 0) {
-                    const int cv = my_cnt - sum;
-                    if (k > 0) v.cnt[j] = cv;
-                    if (cv == 0) {
-                        v.srank[my_pos] = k + before;
-                        nf = true;
+                const int cv = my_cnt - sum;
+                const bool open = my_open, nf = open && cv == 0;
+                const uint32_t word = __ballot_sync(0xffffffffu, nf);
+                if (lane == 0) v.front[(size_t)(k % RING) * v.NW + j0 / 32 + warp] = word;
+                const int left = __reduce_min_sync(0xffffffffu, open && !nf ? cv : INT_MAX);
+                if (slot < MAXC) {
+                    if (lane == 0) atomicMin(&c_min[slot], left);
+                    if (tid == 0) {
+                        c_eval[slot] = k;
+                        c_cum[slot] = cum;
                     }
                 }
-                const uint32_t word = __ballot_sync(0xffffffffu, nf);
-                if (lane == 0) {
-                    const int wd = j0 / 32 + warp;
-                    v.front[(k & 1) * v.NW + wd] = word;
-                    v.rem[wd] = __ldcg(&v.rem[wd]) & ~word;
-                    if (word) atomicAdd(&s_fs, (unsigned)__popc(word));
-                }
+                if (!single && open && k > 0) v.cnt[j] = cv;
+                if (nf) v.srank[v.rest ? v.rmap[j] : j] = k + before;  // (srank is by position among all points)
+                my_cnt = cv;
+                my_open = open && !nf;
             }
-
-            __syncthreads();  // red and list are reused by the next chunk
+            if (!single) __syncthreads();  // red is reused by the next chunk
         }
-        // the barrier returns the points ranked after pass k
-        const unsigned long long tot = grid_sync_sum(c, &c->pbar, &c->prel, (unsigned)k, s_fs, v.wait_ns, &s_cum);
-        if (tot == ~0ull) return;
+        // the pass ends when every CTA has written its front words of it; then
+        // each counts them all (the same total everywhere) and keeps them.
+        // (Words that carry their pass number and are polled themselves save
+        // a trip through L2, but all CTAs polling the same few lines slow
+        // every other load: 252 us for the many fronts of the knapsack
+        // instead of 225.)
+        __syncthreads();
+        if (tid == 0) {
+            red_release(&c->parr, 1u);
+            const unsigned goal = (k + 1u) * (unsigned)min(nchunks, (int)gridDim.x);
+            if (!bounded_wait(c, v.wait_ns, [&] { return (int)(ld_acquire(&c->parr) - goal) >= 0; })) s_fail = 1;
+        }
+        __syncthreads();
+        if (s_fail) return;
+        {
+            unsigned mine = 0u;
+            const uint32_t* words = v.front + (size_t)(k % RING) * v.NW;
+#pragma unroll 4
+            for (int w = tid; w < nwords; w += PT) {
+                const uint32_t x = __ldcg(words + w);
+                if (w < LISTCAP) last[w] = own && !evald ? last[w] | x : x;
+                mine += __popc(x);
+            }
+            mine = __reduce_add_sync(0xffffffffu, mine);
+            if (lane == 0 && mine) atomicAdd(&s_fs[k % 3], mine);
+            if (tid == 0) s_fs[(k + 1) % 3] = 0u;  // read two barriers ago
+        }
+        __syncthreads();
         // close front k (the same decision in every CTA)
-        const int ncum = cum0 + (int)tot;
-        const int fs = ncum - cum;
+        const int fs = (int)s_fs[k % 3];
+        const int ncum = cum + fs;
         bool first = false;
         if (l < 0 && ncum >= v.N) {
             l = k + before;
@@ -272,6 +357,7 @@ __global__ void __launch_bounds__(PEEL_THREADS, STREAM ? 1 : 2) k_peel(RunView v
         cum = ncum;
         if (!more) break;
     }
+    if (lane == 0 && nrows) atomicAdd(&c->peel_rows, nrows);
 }
 
 

@@ -132,13 +132,6 @@ __device__ __forceinline__ void sel_reset(const RunView& v, int tid, int stride)
         for (long long e = tid; e < nb / 8; e += stride) z[e] = make_uint2(0u, 0u);
     }
     for (int wd = tid; wd < v.NW; wd += stride) {
-        const int lo = wd * 32;
-        uint32_t m = 0u;
-        if (lo + 32 <= v.n2)
-            m = 0xffffffffu;
-        else if (lo < v.n2)
-            m = (1u << (v.n2 - lo)) - 1u;
-        v.rem[wd] = m;
         v.selmask[wd] = 0u;
         if (v.domw) {
             v.domw[wd] = 0u;
@@ -156,8 +149,6 @@ __device__ __forceinline__ void sel_reset(const RunView& v, int tid, int stride)
     if (tid < 8) c->domstat[tid] = 0ull;
     if (tid == 0) {
         c->sbar = 0u;
-        c->pbar = 0ull;
-        c->prel = 0ull;
         c->cum = 0;
         c->l = -1;
         c->nS = 0;
@@ -174,6 +165,7 @@ __device__ __forceinline__ void sel_reset(const RunView& v, int tid, int stride)
         c->npath = 0u;
         c->ntile = 0;
         c->ntask = 0;
+        c->parr = 0u;
         c->nF0 = 0;
         c->nrem = 0;
         c->peel_rows = 0u;
