@@ -215,7 +215,7 @@ struct RunView {
     // association scan (m <= 10): references reordered into compact blocks of 32
     const float* blk_z;    // w x M4     zhat in block order
     const int32_t* blk_j;  // w          original reference index in block order
-    const unsigned char* bop;   // their FP16 rows in chunks of 128 (assoc_pack_refs)
+    const unsigned char* bop;   // their FP16 rows in chunks of 128 (k_assoc_pack)
     unsigned char* aop;    // the T slots' FP16 rows, in the same layout
     int2* arun;            // n2         start -1: the slot takes the FP64 scan; m > 10: its
                            //            candidate run (start, count)

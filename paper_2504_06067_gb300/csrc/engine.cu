@@ -706,18 +706,15 @@ nsga3_status setup(nsga3_ctx* ctx)
         CK(cudaStreamSynchronize(s));
         std::vector<float> hz;
         std::vector<int32_t> hj;
-        std::vector<unsigned char> hb;
         build_ref_blocks(m, w, M4, Zh, hz, hj);
         // copies on the context's own stream: no implicit synchronisation with
         // other streams of the process (runs of a server keep executing)
-        if (v.bop) {
-            hb.assign(assoc_rows_bytes(m, w), 0);
-            assoc_pack_refs(m, M4, w, hz.data(), hb.data());
-            CK(cudaMemcpyAsync(const_cast<unsigned char*>(v.bop), hb.data(), hb.size(), cudaMemcpyHostToDevice, s));
-            CK(cudaMemsetAsync(v.aop, 0, assoc_rows_bytes(m, n2), s));  // rows past the points are read, not used
-        }
         CK(cudaMemcpyAsync(bz, hz.data(), hz.size() * sizeof(float), cudaMemcpyHostToDevice, s));
         CK(cudaMemcpyAsync(bj, hj.data(), hj.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+        if (v.bop) {
+            CK(launch_assoc_pack(m, M4, w, bz, const_cast<unsigned char*>(v.bop), s));
+            CK(cudaMemsetAsync(v.aop, 0, assoc_rows_bytes(m, n2), s));  // rows past the points are read, not used
+        }
         CK(cudaStreamSynchronize(s));
     }
     return build_graphs(ctx);

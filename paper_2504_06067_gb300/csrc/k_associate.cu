@@ -1038,25 +1038,36 @@ size_t assoc_rows_bytes(int m, int rows)
     return ((size_t)rows + TP - 1) / TP * TP * kp * 2;
 }
 
-// the directions' FP16 rows [zh, zl, zh] in chunks of 128 as k_assoc_mma
-// reads them; z: w x M4 unit vectors in block order.  Rows past w are -1 in
-// every h: their cosines with unit vectors of non-negative components are
-// below -0.9.
-void assoc_pack_refs(int m, int M4, int w, const float* z, unsigned char* out)
+namespace {
+
+// The directions' FP16 rows [zh, zl, zh] in chunks of 128 as k_assoc_mma
+// reads them, from their w x M4 unit vectors in block order; a thread per
+// row.  Rows past w are -1 in every h: their cosines with unit vectors of
+// non-negative components are below -0.9.
+__global__ void __launch_bounds__(256) k_assoc_pack(int m, int M4, int w, int rows, const float* z, unsigned char* out)
 {
-    const int KP = 3 * m <= 16 ? 16 : 32, rows = (w + CHUNK - 1) / CHUNK * CHUNK;
-    for (int j = 0; j < rows; ++j) {
-        __half r[32];
-        for (int e = 0; e < KP; ++e) r[e] = __float2half_rn(0.0f);
-        for (int q = 0; q < m; ++q) {
-            const float x = j < w ? z[(size_t)j * M4 + q] : -1.0f;
-            const __half h = __float2half_rn(x);
-            r[q] = r[2 * m + q] = h;
-            r[m + q] = __float2half_rn(x - __half2float(h));
-        }
-        unsigned char* row = out + (size_t)(j / CHUNK) * (CHUNK * KP * 2) + (j % CHUNK) * 16;
-        for (int k = 0; k < KP / 8; ++k) memcpy(row + k * CHUNK * 16, r + 8 * k, 16);
+    const int j = blockIdx.x * 256 + threadIdx.x;
+    if (j >= rows) return;
+    const int KP = 3 * m <= 16 ? 16 : 32;
+    __half* row = reinterpret_cast<__half*>(out + (size_t)(j / CHUNK) * (CHUNK * KP * 2) + (j % CHUNK) * 16);
+    auto put = [&](int e, __half h) { row[(e / 8) * CHUNK * 8 + e % 8] = h; };
+    for (int q = 0; q < m; ++q) {
+        const float x = j < w ? z[(size_t)j * M4 + q] : -1.0f;
+        const __half h = __float2half_rn(x);
+        put(q, h);
+        put(2 * m + q, h);
+        put(m + q, __float2half_rn(x - __half2float(h)));
     }
+    for (int e = 3 * m; e < KP; ++e) put(e, __float2half_rn(0.0f));
+}
+
+}  // namespace
+
+cudaError_t launch_assoc_pack(int m, int M4, int w, const float* z, unsigned char* out, cudaStream_t s)
+{
+    const int rows = (w + TP - 1) / TP * TP;  // what assoc_rows_bytes holds
+    k_assoc_pack<<<(rows + 255) / 256, 256, 0, s>>>(m, M4, w, rows, z, out);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_assoc_prep(const RunView& v, cudaStream_t s)

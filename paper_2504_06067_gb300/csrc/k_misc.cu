@@ -131,38 +131,65 @@ __global__ void __launch_bounds__(256) k_gather_rows(RunView v)
     for (int q = lane_id(); q < v.m; q += 32) v.PF[(size_t)p * v.m + q] = v.F[(size_t)i * v.m + q];
 }
 
-// rows between X and a caller's N x d array (warp per row; 16-byte copies
-// when both sides' rows start on 16-byte boundaries)
-__device__ __forceinline__ void copy_row(float* dst, const float* src, int d, bool vec)
+// Rows between X and a caller's N x d array (16-byte words when both sides'
+// rows start on 16-byte boundaries).  A CTA moves RW * 256 consecutive words
+// of the array, a thread RW of them 256 apart with all loads in flight; one
+// 64-bit division per thread finds the CTA's first row.  (A warp per row left
+// most lanes idle at small d and one load in flight at large ones: 11.3 us
+// for 12,800 rows of 500, 8.2 now.)
+constexpr int RW = 4;
+
+template <class T, class F>
+__device__ __forceinline__ void for_row_words(int N, int words, F&& f)
 {
-    if (vec) {
-        const float4* s4 = reinterpret_cast<const float4*>(src);
-        float4* d4 = reinterpret_cast<float4*>(dst);
-        for (int e = lane_id(); e < d / 4; e += 32) d4[e] = s4[e];
-    } else {
-        for (int e = lane_id(); e < d; e += 32) dst[e] = src[e];
+    const long long e0 = (long long)blockIdx.x * (256 * RW);
+    const long long p0 = e0 / words;
+    const int r0 = (int)(e0 - p0 * words);
+    T x[RW];
+    int p[RW], q[RW];
+#pragma unroll
+    for (int t = 0; t < RW; ++t) {
+        const unsigned r = (unsigned)r0 + t * 256 + threadIdx.x;
+        const unsigned n = r / (unsigned)words;
+        p[t] = p0 + n < N ? (int)(p0 + n) : -1;
+        q[t] = (int)(r - n * (unsigned)words);
     }
+    f(x, p, q);
 }
 
-__global__ void __launch_bounds__(256) k_rows_out(RunView v, const int32_t* idx, float* dst, int vec)
+template <class T>
+__global__ void __launch_bounds__(256) k_rows_out(RunView v, const int32_t* idx, T* dst, int words)
 {
-    const int p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (p >= v.N) return;
-    copy_row(dst + (size_t)p * v.d, v.X + (size_t)idx[p] * v.d, v.d, vec != 0);
+    for_row_words<T>(v.N, words, [&](T(&x)[RW], int(&p)[RW], int(&q)[RW]) {
+#pragma unroll
+        for (int t = 0; t < RW; ++t)
+            if (p[t] >= 0) x[t] = reinterpret_cast<const T*>(v.X)[(size_t)idx[p[t]] * words + q[t]];
+#pragma unroll
+        for (int t = 0; t < RW; ++t)
+            if (p[t] >= 0) dst[(size_t)p[t] * words + q[t]] = x[t];
+    });
 }
 
 // new parents take the rows of the last variation's parents, so that its
 // children stay readable; the next children take the last ones' rows
-__global__ void __launch_bounds__(256) k_rows_in(RunView v, const float* src, int vec)
+template <class T>
+__global__ void __launch_bounds__(256) k_rows_in(RunView v, const T* src, int words)
 {
-    const int p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (p >= v.N) return;
-    const int slot = v.pold[p];
-    copy_row(v.X + (size_t)slot * v.d, src + (size_t)p * v.d, v.d, vec != 0);
-    if (lane_id() == 0) {
-        v.pcan[p] = slot;
-        v.fslot[p] = v.cslot[p];
-    }
+    for_row_words<T>(v.N, words, [&](T(&x)[RW], int(&p)[RW], int(&q)[RW]) {
+#pragma unroll
+        for (int t = 0; t < RW; ++t)
+            if (p[t] >= 0) x[t] = src[(size_t)p[t] * words + q[t]];
+#pragma unroll
+        for (int t = 0; t < RW; ++t)
+            if (p[t] >= 0) {
+                const int slot = v.pold[p[t]];
+                reinterpret_cast<T*>(v.X)[(size_t)slot * words + q[t]] = x[t];
+                if (q[t] == 0) {
+                    v.pcan[p[t]] = slot;
+                    v.fslot[p[t]] = v.cslot[p[t]];
+                }
+            }
+    });
 }
 
 __global__ void k_slots_init(RunView v)
@@ -231,17 +258,26 @@ cudaError_t launch_gather(const RunView& v, cudaStream_t s)
     return cudaGetLastError();
 }
 
+static unsigned row_ctas(int N, int words)
+{
+    return (unsigned)(((long long)N * words + 256 * RW - 1) / (256 * RW));
+}
+
 cudaError_t launch_rows_out(const RunView& v, const int32_t* idx, float* dst, cudaStream_t s)
 {
-    const int vec = (v.d & 3) == 0 && (reinterpret_cast<uintptr_t>(dst) & 15) == 0;
-    k_rows_out<<<(unsigned)(((long long)v.N * 32 + 255) / 256), 256, 0, s>>>(v, idx, dst, vec);
+    if ((v.d & 3) == 0 && (reinterpret_cast<uintptr_t>(dst) & 15) == 0)
+        k_rows_out<float4><<<row_ctas(v.N, v.d / 4), 256, 0, s>>>(v, idx, reinterpret_cast<float4*>(dst), v.d / 4);
+    else
+        k_rows_out<float><<<row_ctas(v.N, v.d), 256, 0, s>>>(v, idx, dst, v.d);
     return cudaGetLastError();
 }
 
 cudaError_t launch_rows_in(const RunView& v, const float* src, cudaStream_t s)
 {
-    const int vec = (v.d & 3) == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0;
-    k_rows_in<<<(unsigned)(((long long)v.N * 32 + 255) / 256), 256, 0, s>>>(v, src, vec);
+    if ((v.d & 3) == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0)
+        k_rows_in<float4><<<row_ctas(v.N, v.d / 4), 256, 0, s>>>(v, reinterpret_cast<const float4*>(src), v.d / 4);
+    else
+        k_rows_in<float><<<row_ctas(v.N, v.d), 256, 0, s>>>(v, src, v.d);
     return cudaGetLastError();
 }
 

@@ -54,11 +54,11 @@ cudaError_t launch_assoc_prep(const RunView& v, cudaStream_t s);
 cudaError_t launch_assoc_scan(const RunView& v, int num_sms, cudaStream_t s);
 // m <= 10: the tensor-core scan's grid for a device of num_sms SMs, the int4
 // entries it writes for at most n2 points, the bytes of `rows` FP16 operand
-// rows, and the directions' rows (host)
+// rows, and the directions' rows
 int assoc_grid(int num_sms);
 size_t assoc_entries(int n2, int num_sms);
 size_t assoc_rows_bytes(int m, int rows);
-void assoc_pack_refs(int m, int M4, int w, const float* z, unsigned char* out);
+cudaError_t launch_assoc_pack(int m, int M4, int w, const float* z, unsigned char* out, cudaStream_t s);
 cudaError_t assoc_init_attributes();
 cudaError_t launch_level(const RunView& v, cudaStream_t s);
 cudaError_t launch_bucket(const RunView& v, cudaStream_t s);
