@@ -69,7 +69,6 @@ struct Ctrl {
     int32_t need_niche;      // K < |F_l|
     int32_t fallback;        // normalization used the nadir fallback
     int32_t passes;          // peel passes (kernel launches) in the last selection
-    uint32_t sbar;           // arrivals at the barriers of the cooperative elimination
     uint32_t never;          // a word nothing sets (the wait self-test polls it)
     int32_t nT;              // |S u F_l| (association set)
     int32_t Lstar;           // niche level threshold L*
@@ -233,9 +232,7 @@ struct RunView {
     unsigned long long* ekey;  // (n2 + m) x 2  ASF keys of the largest / second-largest f~
     int32_t* er1;              // n2 + m        objective of the largest f~
     double* nadv;              // m     max f~ per axis (nadir fallback)
-    // m > NSGA3_WARP_M: intercepts by the cooperative elimination
-    double* amat;          // m x (m + 1)  [E - z* | 1], rows in original order
-    float* etmp;           // m x m        new extreme vectors (copied to he at the end)
+    float* etmp;           // m x m  m > NSGA3_WARP_M: new extreme vectors (copied to he at the end)
     // m > NSGA3_FAST_M with few tiles: the objective chunks of a tile are
     // split over dom_ks CTAs, which OR their sign masks into dpa / dpb
     // (NW x ld, laid out like Dom; zero between selections)
@@ -384,23 +381,4 @@ __device__ __forceinline__ bool bounded_wait(Ctrl* c, unsigned long long wait_ns
         }
     }
     return true;
-}
-
-// Counting barrier: the k-th barrier of a launch waits until *ctr reaches
-// k * gridDim.x (*ctr is zero at launch): one atomic on the arrival path and
-// a tight poll, for kernels that meet at a barrier many times per launch.
-__device__ __forceinline__ bool grid_sync_count(Ctrl* c, unsigned* ctr, unsigned target, unsigned long long wait_ns,
-                                                int* s_ok)
-{
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int ok = 1;
-        __threadfence();
-        if (atomicAdd(ctr, 1u) + 1u < target)
-            ok = bounded_wait(c, wait_ns, [&] { return ld_acquire(ctr) >= target; }) ? 1 : 0;
-        __threadfence();
-        *s_ok = ok;
-    }
-    __syncthreads();
-    return *s_ok != 0;
 }

@@ -114,7 +114,7 @@ bool first_front_wanted(const RunView& v)
 
 // Kernels of one selection / one generation; m > 10: with the ideal point,
 // extreme-point keys and reduction, |f'| and candidate distances, m > 32 the
-// cooperative elimination, and a split dominance build (few tiles) its
+// elimination in a cluster, and a split dominance build (few tiles) its
 // finishing kernel.
 int select_launches(const nsga3_ctx* ctx)
 {
@@ -589,10 +589,7 @@ nsga3_status setup_alloc(nsga3_ctx* ctx)
         AL(v.ekey, 2 * (size_t)(n2 + m));
         AL(v.er1, (size_t)(n2 + m));
     }
-    if (m > NSGA3_WARP_M) {
-        AL(v.amat, (size_t)m * (m + 1));
-        AL(v.etmp, (size_t)m * m);
-    }
+    if (m > NSGA3_WARP_M) AL(v.etmp, (size_t)m * m);
     float* bz;
     int32_t* bj;
     AL(bz, (size_t)w * M4);

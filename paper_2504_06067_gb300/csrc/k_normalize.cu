@@ -300,8 +300,8 @@ __global__ void __launch_bounds__(EB) k_norm_extreme(RunView v)
 // ASF_q = max(f~_q, that key) per entry, (min, lowest index) per axis, and
 // the nadir maxima over the members; k_ext_reduce reduces the blocks (a warp
 // per axis) and either solves the intercepts with one warp
-// (m <= NSGA3_WARP_M) or leaves E and the nadir to the cooperative
-// elimination below.
+// (m <= NSGA3_WARP_M) or leaves E and the nadir to the
+// elimination in a cluster below.
 constexpr int GB = 128;  // threads per block of the m > NSGA3_FAST_M kernels
 constexpr int QG = 8;    // axes per block of k_ext_axis
 
@@ -477,7 +477,7 @@ __global__ void __launch_bounds__(GB) k_ext_axis(RunView v)
 
 // per axis (a warp each) the (min, lowest index) over the parts and the
 // nadir maximum; with m <= NSGA3_WARP_M the last CTA solves the intercepts
-// with one warp, else the cooperative elimination follows
+// with one warp, else the elimination in a cluster follows
 __global__ void __launch_bounds__(256) k_ext_reduce(RunView v, int parts)
 {
     __shared__ unsigned s_ticket;
@@ -534,174 +534,241 @@ __global__ void __launch_bounds__(256) k_ext_reduce(RunView v, int parts)
     if (threadIdx.x < 32) solve_intercepts(v, c, f_ext, f_nad, s_A);
 }
 
-// m > NSGA3_WARP_M: the elimination of the warp solver spread over a
-// cooperative grid.  The augmented rows [E - z* | 1] live in amat (original
-// row order); every CTA keeps the same current row order ord[] and takes
-// the same pivot (first maximal |A[.][col]| in that order), so a pivot step
-// needs one grid barrier: a warp per remaining row forms its factor and
-// updates columns col+1 .. m (m = the right-hand side) with the same _rn
-// operations as the serial elimination (column col is not needed again).
-// Reads of amat bypass L1 (other SMs write it between barriers).  The back
-// substitution (the order of the warp solver) runs in CTA 0.
-constexpr int SB = 256;
-static_assert(NSGA3_MAX_M <= 2 * SB, "the back substitution keeps two rows per thread");
-
-__global__ void __launch_bounds__(SB) k_solve_coop(RunView v)
+// The intercepts from the solution b of E b = 1 (one CTA of SB threads):
+// a = 1 / b where all are usable, else the nadir point's components; the
+// history's extreme vectors.
+__device__ __noinline__ void finish_solve(const RunView& v, Ctrl* c, bool ok, bool ext_ok, double* sb)
 {
-    __shared__ int ord[NSGA3_MAX_M];
-    __shared__ double sb[NSGA3_MAX_M];
-    __shared__ double colv[NSGA3_MAX_M];  // column col of the rows, by position
-    __shared__ double red_x[SB / 32];
-    __shared__ int red_p[SB / 32];
-    __shared__ int s_ok, s_piv;
-    Ctrl* c = v.ctrl;
-    if (skip_niche(c)) return;
-    const int m = v.m, ld = m + 1;
-    unsigned nbar = 0;  // barriers passed (c->sbar is zero at launch: k_sel_reset)
-    const int tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
-    // rows go to the CTAs in turn, so that the FP64 work of a step spreads
-    // over every SM of the grid
-    const int gw = warp * gridDim.x + blockIdx.x, nw = gridDim.x * (SB / 32);
-    double* A = v.amat;
-    const int ncand = v.n2 + ((v.norm_history && c->hvalid) ? m : 0);
-    bool bad_ext = false;
-    for (int q = tid; q < m; q += SB) {
-        const int e = c->ext[q];
-        bad_ext |= e < 0 || e >= ncand;
-        ord[q] = q;
-        if (blockIdx.x == 0) c->zstar[q] = zstar_of(c, q);
-    }
-    const bool ext_ok = !__syncthreads_or(bad_ext);
-    bool ok = ext_ok;
-    if (ok) {
-        // rows of the system and the new extreme vectors (warp per row)
-        for (int q = gw; q < m; q += nw) {
-            const int er = c->ext[q];
-            const float* f = er < v.n2 ? v.F + (size_t)er * m : v.he + (size_t)(er - v.n2) * m;
-            for (int k = lane; k < m; k += 32) {
-                const float ev = f[k];
-                v.etmp[(size_t)q * m + k] = ev;
-                A[(size_t)q * ld + k] = __dsub_rn((double)ev, zstar_of(c, k));
-            }
-            if (lane == 0) A[(size_t)q * ld + m] = 1.0;
-        }
-        if (!grid_sync_count(c, &c->sbar, ++nbar * gridDim.x, v.wait_ns, &s_ok)) return;
-        for (int col = 0; col < m; ++col) {
-            // pivot (every CTA): the first position p >= col of maximal
-            // |A[ord[p]][col]|; a NaN never replaces the running maximum
-            // (the column's values stay in colv for the factors below)
-            double bx = -1.0;
-            int bp = 0x7fffffff;
-#pragma unroll 2
-            for (int p = col + tid; p < m; p += SB) {
-                const double val = __ldcg(&A[(size_t)ord[p] * ld + col]);
-                colv[p] = val;
-                const double x = fabs(val);
-                if (p > col && x > bx) {  // positions ascend per thread: the first maximum stays
-                    bx = x;
-                    bp = p;
-                }
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const double ox = __shfl_xor_sync(0xffffffffu, bx, o);
-                const int op = __shfl_xor_sync(0xffffffffu, bp, o);
-                if (ox > bx || (ox == bx && op < bp)) {
-                    bx = ox;
-                    bp = op;
-                }
-            }
-            if (lane == 0) {
-                red_x[warp] = bx;
-                red_p[warp] = bp;
-            }
-            __syncthreads();
-            if (tid == 0) {
-                for (int w = 1; w < SB / 32; ++w)
-                    if (red_x[w] > bx || (red_x[w] == bx && red_p[w] < bp)) {
-                        bx = red_x[w];
-                        bp = red_p[w];
-                    }
-                const double x0 = fabs(colv[col]);
-                int p = col;
-                double best = x0;
-                if (x0 == x0 && bp != 0x7fffffff && bx > x0) {  // x0 NaN: col stays
-                    p = bp;
-                    best = bx;
-                }
-                s_piv = p;
-                s_ok = best == 0.0 ? 0 : 1;
-                if (p != col) {
-                    const int t = ord[col];
-                    ord[col] = ord[p];
-                    ord[p] = t;
-                }
-            }
-            __syncthreads();
-            if (!s_ok) {
-                ok = false;
-                break;
-            }
-            const int P = ord[col], pp = s_piv;
-            const double pv = colv[pp];  // the pivot row's value (read at its old position)
-            for (int pos = col + 1 + gw; pos < m; pos += nw) {
-                const int r = ord[pos];
-                // the row now at pp came from position col
-                const double factor = __ddiv_rn(pos == pp ? colv[col] : colv[pos], pv);
-#pragma unroll 4  // four pairs of loads in flight (L2 round trips dominate a step)
-                for (int k = col + 1 + lane; k <= m; k += 32)
-                    A[(size_t)r * ld + k] = __dsub_rn(__ldcg(&A[(size_t)r * ld + k]),
-                                                      __dmul_rn(factor, __ldcg(&A[(size_t)P * ld + k])));
-            }
-            if (!grid_sync_count(c, &c->sbar, ++nbar * gridDim.x, v.wait_ns, &s_ok)) return;
-        }
-    }
-    if (blockIdx.x != 0) return;
-    // CTA 0: back substitution column by column from the last unknown (as
-    // in the warp solver); thread t keeps the partial sums of positions t
-    // and t + SB and loads the next column's elements a step ahead
-    if (ok) {
-        const int i0 = tid, i1 = tid + SB;
-        const size_t R0 = i0 < m ? (size_t)ord[i0] * ld : 0, R1 = i1 < m ? (size_t)ord[i1] * ld : 0;
-        double s0 = i0 < m ? __ldcg(&A[R0 + m]) : 0.0, s1 = i1 < m ? __ldcg(&A[R1 + m]) : 0.0;
-        const double d0 = i0 < m ? __ldcg(&A[R0 + i0]) : 1.0, d1 = i1 < m ? __ldcg(&A[R1 + i1]) : 1.0;
-        double c0 = i0 < m - 1 ? __ldcg(&A[R0 + m - 1]) : 0.0;
-        double c1 = i1 < m - 1 ? __ldcg(&A[R1 + m - 1]) : 0.0;
-        for (int r = m - 1; r >= 0; --r) {
-            if (i0 == r) sb[r] = __ddiv_rn(s0, d0);
-            if (i1 == r) sb[r] = __ddiv_rn(s1, d1);
-            __syncthreads();
-            const double br = sb[r];
-            const double u0 = c0, u1 = c1;
-            if (r > 0) {
-                c0 = i0 < r - 1 ? __ldcg(&A[R0 + r - 1]) : 0.0;
-                c1 = i1 < r - 1 ? __ldcg(&A[R1 + r - 1]) : 0.0;
-            }
-            if (i0 < r) s0 = __dsub_rn(s0, __dmul_rn(u0, br));
-            if (i1 < r) s1 = __dsub_rn(s1, __dmul_rn(u1, br));
-        }
-    }
+    const int m = v.m, tid = threadIdx.x, NT = blockDim.x;
     __syncthreads();
     bool bad = false;
     if (ok)
-        for (int q = tid; q < m; q += SB) {
+        for (int q = tid; q < m; q += NT) {
             const double a = __ddiv_rn(1.0, sb[q]);
             bad |= !isfinite(a) || a <= 1e-6;
             sb[q] = a;
         }
     ok = ok && !__syncthreads_or(bad);
-    for (int q = tid; q < m; q += SB) {
+    for (int q = tid; q < m; q += NT) {
         const double nq = v.nadv[q];
         c->a[q] = ok ? sb[q] : (nq == 0.0 ? 1.0 : nq);
     }
     if (tid == 0) c->fallback = ok ? 0 : 1;
     if (v.norm_history) {
-        for (int q = tid; q < m; q += SB) c->hz[q] = zstar_of(c, q);
+        for (int q = tid; q < m; q += NT) c->hz[q] = zstar_of(c, q);
         // the staged extreme vectors (zero rows, as in the warp solver, when
         // an extreme index was invalid and nothing was staged)
-        for (int e = tid; e < m * m; e += SB) v.he[e] = ext_ok ? v.etmp[e] : 0.0f;
+        for (int e = tid; e < m * m; e += NT) v.he[e] = ext_ok ? v.etmp[e] : 0.0f;
         if (tid == 0) c->hvalid = 1;
     }
+}
+
+// m > NSGA3_WARP_M: the elimination in the shared memory of one cluster.  CTA r holds columns r, r + C, ... of [E - z* | 1] (rows in their
+// original order; a thread per row in each group of threads, which keeps the
+// row's current position).  The owner of the next column brings it up to
+// date, finds the pivot, forms the factors and stores them into every CTA
+// before it turns to its other columns, so a step waits for one column, one
+// quotient and one cluster barrier (0.8 us; a grid barrier and four trips
+// through L2 before: 1.7 us), and the other columns' updates, one product and
+// one difference on the FP64 pipe each, pass meanwhile.  Same operations, in
+// the same order for every element, as the warp solver.
+//
+// Bound: the chain of a step up to m of about 100, above it the FP64 pipes of
+// C SMs (two operations per element, m^3 / 3 elements).  Regular systems, with
+// the back substitution: m = 40 188 -> 69 us, m = 64 315 -> 106, m = 128
+// 721 -> 240, m = 256 1,680 -> 647, m = 300 2,070 -> 973 (before: a cooperative grid over the rows in
+// global memory with a barrier per step).  Eight CTAs up to m = 96: a step's
+// factors go to half as many.
+constexpr int SC_M = NSGA3_MAX_M;  // rows (a group of threads at least)
+constexpr int SC_T = 512;
+constexpr int SC_PRE = 4;   // back substitution: columns loaded ahead
+
+__device__ __forceinline__ uint32_t sc_peer(const void* p, int r)
+{
+    uint32_t d;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(r));
+    return d;
+}
+__device__ __forceinline__ double sc_load(uint32_t a)
+{
+    double x;
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(x) : "r"(a) : "memory");
+    return x;
+}
+__device__ __forceinline__ void sc_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void sc_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void sc_group(int threads) { asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory"); }
+
+// CTAs, and bytes of columns in each
+inline int sc_ctas(int m) { return m <= 96 ? 8 : 16; }
+inline size_t sc_bytes(int m) { return (size_t)(m / sc_ctas(m) + 1) * m * sizeof(double); }
+
+struct ScShared {
+    double f[3][SC_M];  // factors by row, three steps of them
+    int piv[3][4];      // pivot row, its position before, valid system
+    unsigned long long wk[SC_M / 32];
+    int wp[SC_M / 32];
+    int x0row, x0nan;
+    double b[SC_M];
+};
+
+__global__ void __launch_bounds__(SC_T) k_solve_cluster(RunView v, int C)
+{
+    extern __shared__ double cols[];  // m values of each of the CTA's columns
+    __shared__ ScShared sh;
+    Ctrl* c = v.ctrl;
+    if (skip_niche(c)) return;  // uniform over the cluster
+    const int m = v.m, rank = blockIdx.x, tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
+    const int RP = (m + 31) & ~31, G = SC_T / RP, g = tid / RP, row = tid - g * RP;
+    const bool mine = row < m && g < G;
+    const int ncol = (m - rank) / C + 1;  // columns rank, rank + C, ... <= m
+    const int ncand = v.n2 + ((v.norm_history && c->hvalid) ? m : 0);
+    bool bad_ext = false;
+    if (tid < m) {
+        const int e = c->ext[tid];
+        bad_ext = e < 0 || e >= ncand;
+        if (rank == 0) c->zstar[tid] = zstar_of(c, tid);
+    }
+    const bool ext_ok = !__syncthreads_or(bad_ext);
+    bool ok = ext_ok;
+    int pos = row;
+    if (ok && mine) {
+        const int er = c->ext[row];
+        const float* f = er < v.n2 ? v.F + (size_t)er * m : v.he + (size_t)(er - v.n2) * m;
+        for (int lc = g; lc < ncol; lc += G) {
+            const int k = lc * C + rank;
+            double x = 1.0;
+            if (k < m) {
+                const float ev = f[k];
+                if (v.norm_history) v.etmp[(size_t)row * m + k] = ev;
+                x = __dsub_rn((double)ev, zstar_of(c, k));
+            }
+            cols[lc * m + row] = x;
+        }
+    }
+    __syncthreads();
+    // column cn of this CTA by its first group: brought up to date with step
+    // cn - 1 (pivot row P, factor f), pivot, factors into every CTA
+    auto pivot = [&](int cn, int P, double f) {
+        double* col = cols + (cn / C) * m;
+        double x = row < m ? col[row] : 0.0;
+        const bool cand = row < m && pos >= cn;
+        if (cn > 0 && cand) {
+            x = __dsub_rn(x, __dmul_rn(f, col[P]));
+            col[row] = x;
+        }
+        const unsigned long long k = sf64::bits(x) << 1;  // |x|, twice
+        const bool isnan = k > (0x7ff0000000000000ull << 1);
+        // the first position of maximal |x|; a NaN replaces nothing, and in
+        // the first position is not replaced
+        const bool in = cand && !isnan;
+        const uint32_t hi = __reduce_max_sync(0xffffffffu, in ? (uint32_t)(k >> 32) : 0u);
+        const uint32_t lo = __reduce_max_sync(0xffffffffu, in && (uint32_t)(k >> 32) == hi ? (uint32_t)k : 0u);
+        const unsigned long long best = ((unsigned long long)hi << 32) | lo;
+        const int at = __reduce_min_sync(0xffffffffu, in && k == best ? pos << 16 | row : 0x7fffffff);
+        if (lane == 0) {
+            sh.wk[warp] = best;
+            sh.wp[warp] = at;
+        }
+        if (row < m && pos == cn) {
+            sh.x0row = row;
+            sh.x0nan = isnan ? 1 : 0;
+        }
+        sc_group(RP);
+        unsigned long long bk = 0ull;
+        int bp = 0x7fffffff;
+        for (int w = 0; w < RP / 32; ++w) {
+            const unsigned long long kw = sh.wk[w];
+            const int pw = sh.wp[w];
+            if (kw > bk || (kw == bk && pw < bp)) {
+                bk = kw;
+                bp = pw;
+            }
+        }
+        const bool nan0 = sh.x0nan != 0;
+        const int np = nan0 ? sh.x0row : bp & 0xffff, pp = nan0 ? cn : bp >> 16;
+        const bool good = nan0 || bk != 0ull;
+        double fr = 0.0;
+        if (good && cand && row != np) fr = div_once(x, col[np]);
+        const int buf = cn % 3;
+#pragma unroll 1
+        for (int r = 0; r < C; ++r) {
+            if (row < m)
+                asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(sc_peer(&sh.f[buf][row], r)), "d"(fr) : "memory");
+            if (tid < 3)
+                asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(sc_peer(&sh.piv[buf][tid], r)),
+                             "r"(tid == 0 ? np : tid == 1 ? pp : good ? 1 : 0)
+                             : "memory");
+        }
+    };
+    // every CTA of the cluster has started (its shared memory is written below)
+    sc_arrive();
+    sc_wait();
+    if (ok) {
+        if (rank == 0 && tid < RP) pivot(0, 0, 0.0);
+        __syncwarp();
+        sc_arrive();
+        sc_wait();
+        for (int col = 0; col < m; ++col) {
+            const int buf = col % 3;
+            const int P = sh.piv[buf][0], pp = sh.piv[buf][1];
+            if (!sh.piv[buf][2]) {  // the same in every CTA
+                ok = false;
+                break;
+            }
+            if (row == P)
+                pos = col;
+            else if (pos == col)
+                pos = pp;
+            const bool below = mine && pos > col;
+            const double f = below ? sh.f[buf][row] : 0.0;
+            if (col + 1 < m && rank == (col + 1) % C && tid < RP) pivot(col + 1, P, f);
+            // the factors of the step before last are read no more: a CTA may
+            // be one step ahead, so there are three buffers
+            __syncwarp();
+            sc_arrive();
+            if (below) {
+                for (int lc = g; lc < ncol; lc += G) {
+                    const int k = lc * C + rank;
+                    if (k <= col || (k == col + 1 && k < m)) continue;
+                    double* a = cols + lc * m;
+                    a[row] = __dsub_rn(a[row], __dmul_rn(f, a[P]));
+                }
+            }
+            // the cluster barrier orders the factors; the columns are the
+            // CTA's own, and its threads arrived before they updated them
+            __syncthreads();
+            sc_wait();
+        }
+    }
+    // back substitution column by column from the last unknown (as in the
+    // warp solver) by CTA 0, a thread per row; the columns are read from
+    // their owners SC_PRE steps ahead
+    if (rank == 0 && ok && tid < RP) {
+        auto at = [&](int k) { return sc_peer(cols + (k / C) * m + (row < m ? row : 0), k % C); };
+        double s = sc_load(at(m));
+        const sf64::Divisor dd = sf64::divisor(row < m ? sc_load(at(pos)) : 1.0);
+        double u[SC_PRE];
+#pragma unroll
+        for (int t = 0; t < SC_PRE; ++t) u[t] = m - 1 - t >= 0 ? sc_load(at(m - 1 - t)) : 0.0;
+        for (int r0 = m - 1; r0 >= 0; r0 -= SC_PRE) {
+#pragma unroll
+            for (int t = 0; t < SC_PRE; ++t) {
+                const int r = r0 - t;
+                if (r < 0) break;
+                const double q = sf64::div(s, dd);
+                if (row < m && pos == r) sh.b[r] = q;
+                sc_group(RP);
+                const double br = sh.b[r], ut = u[t];
+                if (r - SC_PRE >= 0) u[t] = sc_load(at(r - SC_PRE));
+                if (pos < r) s = __dsub_rn(s, __dmul_rn(ut, br));
+            }
+        }
+    }
+    __syncwarp();
+    sc_arrive();  // the other CTAs' columns are read no more
+    sc_wait();
+    if (rank == 0) finish_solve(v, c, ok, ext_ok, sh.b);
 }
 
 }  // namespace
@@ -711,8 +778,6 @@ cudaError_t launch_norm_ideal(const RunView& v, cudaStream_t s)
     k_norm_ideal<<<(v.n2 + NB - 1) / NB, NB, 0, s>>>(v);
     return cudaGetLastError();
 }
-
-static int g_solve_occ = 0;  // resident k_solve_coop CTAs per SM, set at start-up
 
 static cudaError_t launch_norm_extreme_gen(const RunView& v, int num_sms, cudaStream_t s)
 {
@@ -736,28 +801,26 @@ static cudaError_t launch_norm_extreme_gen(const RunView& v, int num_sms, cudaSt
     k_ext_reduce<<<(v.m + 7) / 8, 256, 0, s>>>(v, parts);
     e = cudaGetLastError();
     if (e != cudaSuccess || v.m <= NSGA3_WARP_M) return e;
-    // a CTA per SM (the FP64 pipe of every SM), at most a row per CTA at the
-    // first step; every CTA resident
-    int grid = v.m - 1;
-    if (grid > num_sms) grid = num_sms;
-    const int cap = num_sms * (g_solve_occ > 0 ? g_solve_occ : 1);
-    if (grid > cap) grid = cap;
+    const int C = sc_ctas(v.m);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(SB);
-    cfg.dynamicSmemBytes = 0;
+    cfg.gridDim = dim3(C);
+    cfg.blockDim = dim3(SC_T);
+    cfg.dynamicSmemBytes = sc_bytes(v.m);
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = C;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_solve_coop, v);
+    return cudaLaunchKernelEx(&cfg, k_solve_cluster, v, C);
 }
 
 cudaError_t norm_init_attributes()
 {
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_solve_occ, k_solve_coop, SB, 0);
+    const cudaError_t e = cudaFuncSetAttribute(k_solve_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sc_bytes(SC_M));
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(k_solve_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
 }
 
 cudaError_t launch_norm_extreme(const RunView& v, int num_sms, cudaStream_t s)

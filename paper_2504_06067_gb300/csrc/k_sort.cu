@@ -148,7 +148,6 @@ __device__ __forceinline__ void sel_reset(const RunView& v, int tid, int stride)
     if (tid < v.m) c->zmin[tid] = 0xffffffffu;
     if (tid < 8) c->domstat[tid] = 0ull;
     if (tid == 0) {
-        c->sbar = 0u;
         c->cum = 0;
         c->l = -1;
         c->nS = 0;

@@ -38,13 +38,13 @@ cudaError_t launch_first_front(const RunView& v, cudaStream_t s);
 RunView rest_view(const RunView& v);
 cudaError_t launch_dominance(const RunView& v, cudaStream_t s);
 cudaError_t dom_init_attributes();
-// every peel pass in one cooperative launch (grid barrier between passes)
+// every peel pass in one cooperative launch
 cudaError_t launch_peel(const RunView& v, int num_sms, cudaStream_t s);
 cudaError_t peel_init_attributes();
 cudaError_t launch_norm_ideal(const RunView& v, cudaStream_t s);
 // extreme points and intercepts: one launch (m <= 10); above, the ideal
 // point, entry keys, per-axis blocks and their reduction (four launches),
-// plus the cooperative elimination for m > 32
+// plus the elimination in a cluster for m > 32
 cudaError_t launch_norm_extreme(const RunView& v, int num_sms, cudaStream_t s);
 cudaError_t norm_init_attributes();
 cudaError_t launch_assoc_prep(const RunView& v, cudaStream_t s);
