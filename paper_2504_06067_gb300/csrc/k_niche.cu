@@ -59,12 +59,20 @@ __device__ void block_scan_array(const int32_t* a, int32_t* out, int n, int* scr
     const int per = (n + (int)blockDim.x - 1) / (int)blockDim.x;
     const int lo = min(n, (int)threadIdx.x * per), hi = min(n, lo + per);
     int s = 0;
+#pragma unroll 8
     for (int e = lo; e < hi; ++e) s += a[e];
     int total;
     int run = block_excl_scan(s, scratch, &total);
-    for (int e = lo; e < hi; ++e) {
-        out[e] = run;
-        run += a[e];
+    for (int e = lo; e < hi; e += 8) {
+        int x[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) x[t] = a[min(e + t, hi - 1)];
+#pragma unroll
+        for (int t = 0; t < 8; ++t)
+            if (e + t < hi) {
+                out[e + t] = run;
+                run += x[t];
+            }
     }
     if (threadIdx.x == 0) out[n] = total;
 }
@@ -183,7 +191,7 @@ __device__ void block_select_smallest(int n, int need, Key key, Pred pred, Mark 
 
 // ------------------------------------------------------------ k_level ------
 struct LevelShared {
-    int lev[LCAP + 1];
+    int lev[LCAP + 1], lev2[LCAP + 1];  // references whose levels begin, end there
     int scratch[40];
     int Lstar;
     int maxhi;
@@ -219,7 +227,22 @@ __global__ void __launch_bounds__(LB) k_level(RunView v)
     }
     auto rho_of = [&](int j) { return staged ? sh.rr[j].x : v.rho[j]; };
     auto rhop_of = [&](int j) { return staged ? sh.rr[j].y : v.rhop[j]; };
-    for (int t = threadIdx.x; t <= LCAP; t += LB) sh.lev[t] = 0;
+    // f(j, rho_j, rho'_j) for every reference, four pairs of loads in flight
+    auto for_refs = [&](auto f) {
+        for (int j0 = threadIdx.x; j0 < w; j0 += 4 * LB) {
+            int a[4], b[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const int j = min(j0 + t * LB, w - 1);
+                a[t] = rho_of(j);
+                b[t] = rhop_of(j);
+            }
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+                if (j0 + t * LB < w) f(j0 + t * LB, a[t], b[t]);
+        }
+    };
+    for (int t = threadIdx.x; t <= LCAP; t += LB) sh.lev[t] = sh.lev2[t] = 0;
     if (threadIdx.x == 0) {
         sh.Lstar = LCAP;
         sh.maxhi = 0;
@@ -228,31 +251,19 @@ __global__ void __launch_bounds__(LB) k_level(RunView v)
     int mymax = 0;
     {
         // most references share a few level values (rho_j = 0 when S is
-        // empty): lanes with equal values add once per warp (match groups),
-        // so the shared-memory atomics do not serialise on one address
-        const int lane = lane_id();
-        for (int j0 = (threadIdx.x & ~31); j0 < w; j0 += LB) {
-            const int j = j0 + lane;
-            int rp = j < w ? rhop_of(j) : 0;
-            const int lo = j < w ? rho_of(j) : 0;
+        // empty): increments by one, which the shared-memory atomics take
+        // together for the lanes of a warp (groups of equal lanes by
+        // match_any took 4 us for 10,626 references, this 1)
+        for_refs([&](int, int lo, int rp) {
             if (rp > 0 && (lo < 0 || rp > v.n2)) {  // counts out of range: an invariant failed upstream
                 set_status(c, DEV_EINTERNAL);
                 rp = 0;
             }
             const int hi = lo + rp;
-            const bool add_lo = rp > 0 && lo < LCAP, add_hi = rp > 0 && hi < LCAP;
-            const unsigned m_lo = __ballot_sync(0xffffffffu, add_lo);
-            const unsigned m_hi = __ballot_sync(0xffffffffu, add_hi);
-            if (add_lo) {
-                const unsigned g = __match_any_sync(m_lo, lo);
-                if (lane == __ffs(g) - 1) atomicAdd(&sh.lev[lo], __popc(g));
-            }
-            if (add_hi) {
-                const unsigned g = __match_any_sync(m_hi, hi);
-                if (lane == __ffs(g) - 1) atomicAdd(&sh.lev[hi], -__popc(g));
-            }
+            if (rp > 0 && lo < LCAP) atomicAdd(&sh.lev[lo], 1);
+            if (rp > 0 && hi < LCAP) atomicAdd(&sh.lev2[hi], 1);
             if (rp > 0) mymax = max(mymax, hi);
-        }
+        });
     }
     mymax = __reduce_max_sync(0xffffffffu, mymax);
     if ((threadIdx.x & 31) == 0) atomicMax(&sh.maxhi, mymax);
@@ -263,7 +274,7 @@ __global__ void __launch_bounds__(LB) k_level(RunView v)
         int loc[PER];
         int s = 0;
         for (int t = 0; t < PER; ++t) {
-            s += sh.lev[threadIdx.x * PER + t];
+            s += sh.lev[threadIdx.x * PER + t] - sh.lev2[threadIdx.x * PER + t];
             loc[t] = s;
         }
         int total;
@@ -407,15 +418,13 @@ __global__ void __launch_bounds__(LB) k_level(RunView v)
             atomicOr(&c->npath, NPATH_UNSTAGED);
         }
         __syncthreads();
-        for (int j = threadIdx.x; j < w; j += LB) {
-            const int rp = rhop_of(j);
-            const int lo = rho_of(j);
+        for_refs([&](int j, int lo, int rp) {
             v.take[j] = rp > 0 ? min(rp, max(0, Lstar - lo)) : 0;
             if (rp > 0 && lo <= Lstar && Lstar < lo + rp) {
                 const int p = atomicAdd(&sh.nck, 1);
                 if (p < CKCAP) sh.ck[p] = ref_key_of(v, j);
             }
-        }
+        });
         __syncthreads();
         const int nC = sh.nck;
         if (nC <= CKCAP) {
@@ -518,8 +527,8 @@ __device__ __forceinline__ void mark_member(const RunView& v, int i)
 }
 
 // ------------------------------------------------------------- k_pick ------
-// one warp per reference; a partial take from more than 32 members goes to a
-// whole CTA (k_pick_large), its nearest member too (a warp walking thousands
+// one warp per reference; a partial take from more than 32 members, or all of
+// more than 256, goes to a whole CTA (k_pick_large), the nearest member too (a warp walking thousands
 // of members for it took 96 us at 165,000 members of 275 references)
 __global__ void __launch_bounds__(256) k_pick(RunView v)
 {
@@ -531,7 +540,8 @@ __global__ void __launch_bounds__(256) k_pick(RunView v)
     for (int j = gw; j < v.w; j += nw) {
         const int take = v.take[j], cnt = v.rhop[j], off = v.ref_off[j], rho = v.rho[j];
         if (take == 0) continue;
-        if (take >= cnt) {
+        if (take >= cnt && cnt <= 256) {
+#pragma unroll 4
             for (int e = lane; e < cnt; e += 32) mark_member(v, v.bucket[off + e]);
             continue;
         }
@@ -540,7 +550,7 @@ __global__ void __launch_bounds__(256) k_pick(RunView v)
                 const int p = atomicAdd(&c->nlarge, 1);
                 v.large[p] = make_int4(j, take, rho, 0);
                 // more members to take than the nearest: the block-wide selection runs
-                if (take > (rho == 0 ? 1 : 0)) atomicOr(&c->npath, NPATH_LARGE);
+                if (take < cnt && take > (rho == 0 ? 1 : 0)) atomicOr(&c->npath, NPATH_LARGE);
             }
             continue;
         }
@@ -575,12 +585,20 @@ __global__ void __launch_bounds__(256) k_pick(RunView v)
     }
 }
 
-// large buckets with a partial take: one CTA per bucket
-__global__ void __launch_bounds__(512) k_pick_large(RunView v)
+// Large buckets: one CTA per bucket.  Up to PL_CAP members' keys are staged in
+// shared memory while the nearest is found: the passes of the selection then
+// cost what their barriers cost, not a trip through L2 each.  Bound: the
+// latency of the loads and barriers of the largest buckets' CTAs.  119,000
+// members of 462 references: 48 us without the staging, 26 with it.
+constexpr int PL_T = 512;
+constexpr int PL_CAP = 4096;
+
+__global__ void __launch_bounds__(PL_T) k_pick_large(RunView v)
 {
     __shared__ SelShared sh;
-    __shared__ double sd[16];
-    __shared__ int si[16];
+    __shared__ unsigned long long sd[PL_T / 32];
+    __shared__ int si[PL_T / 32];
+    __shared__ unsigned long long keys[PL_CAP];
     Ctrl* c = v.ctrl;
     if (skip_niche(c)) return;
     const int nl = c->nlarge;
@@ -590,47 +608,61 @@ __global__ void __launch_bounds__(512) k_pick_large(RunView v)
         int need = L.y, excl = -1;
         const int cnt = v.rhop[j], off = v.ref_off[j];
         const int32_t* mem = v.bucket + off;
-        if (L.z == 0) {  // rho = 0: the nearest member first
-            double bd = CUDART_INF;
-            int bi = 0x7fffffff;
+        if (need >= cnt) {
+            for (int e = threadIdx.x; e < cnt; e += PL_T) mark_member(v, mem[e]);
+            continue;
+        }
+        const bool staged = cnt <= PL_CAP;
+        // rho = 0: the nearest member first; distances are >= 0 and order like
+        // their bits (an FP64 compare takes 110 cycles, ten of them in a chain)
+        unsigned long long bd = ~0ull;
+        int bi = 0x7fffffff;
+        if (staged || L.z == 0) {
 #pragma unroll 4
-            for (int e = threadIdx.x; e < cnt; e += 512) {
+            for (int e = threadIdx.x; e < cnt; e += PL_T) {
                 const int i = mem[e];
-                const double d = v.bdist[off + e];
-                if (lex_less(d, i, bd, bi)) {
-                    bd = d;
-                    bi = i;
+                if (staged) keys[e] = ((unsigned long long)v.bprio[off + e] << 32) | (unsigned)i;
+                if (L.z == 0) {
+                    const unsigned long long d = (unsigned long long)__double_as_longlong(v.bdist[off + e]);
+                    if (d < bd || (d == bd && i < bi)) {
+                        bd = d;
+                        bi = i;
+                    }
                 }
             }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const double od = __shfl_xor_sync(0xffffffffu, bd, o);
-                const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-                if (lex_less(od, oi, bd, bi)) {
-                    bd = od;
-                    bi = oi;
-                }
-            }
+        }
+        if (L.z == 0) {
+            auto warp_nearest = [&]() {
+                const unsigned hi = __reduce_min_sync(0xffffffffu, (unsigned)(bd >> 32));
+                const unsigned lo = __reduce_min_sync(0xffffffffu, (unsigned)(bd >> 32) == hi ? (unsigned)bd : 0xffffffffu);
+                const unsigned long long b = ((unsigned long long)hi << 32) | lo;
+                bi = __reduce_min_sync(0xffffffffu, bd == b ? bi : 0x7fffffff);
+                bd = b;
+            };
+            warp_nearest();
             if (lane_id() == 0) {
                 sd[threadIdx.x >> 5] = bd;
                 si[threadIdx.x >> 5] = bi;
             }
             __syncthreads();
-            for (int w = 0; w < 16; ++w)
-                if (lex_less(sd[w], si[w], bd, bi)) {
-                    bd = sd[w];
-                    bi = si[w];
-                }
+            bd = sd[lane_id() & (PL_T / 32 - 1)];
+            bi = si[lane_id() & (PL_T / 32 - 1)];
+            warp_nearest();
             excl = bi;
             if (threadIdx.x == 0) mark_member(v, bi);
             need -= 1;
         }
-        auto pred = [&](int e) { return mem[e] != excl; };
-        auto key = [&](int e) {
-            return ((unsigned long long)v.bprio[off + e] << 32) | (unsigned)mem[e];
-        };
         auto mark = [&](int e) { mark_member(v, mem[e]); };
-        block_select_smallest(cnt, need, key, pred, mark, sh, &c->npath);
+        __syncthreads();
+        if (staged) {
+            auto pred = [&](int e) { return (int)(unsigned)keys[e] != excl; };
+            auto key = [&](int e) { return keys[e]; };
+            block_select_smallest(cnt, need, key, pred, mark, sh, &c->npath);
+        } else {
+            auto pred = [&](int e) { return mem[e] != excl; };
+            auto key = [&](int e) { return ((unsigned long long)v.bprio[off + e] << 32) | (unsigned)mem[e]; };
+            block_select_smallest(cnt, need, key, pred, mark, sh, &c->npath);
+        }
         __syncthreads();
     }
 }
@@ -672,11 +704,14 @@ cudaError_t launch_pick(const RunView& v, cudaStream_t s)
     k_pick<<<blocks, 256, 0, s>>>(v);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    // one CTA per reference with a partial take, up to two per SM (how many
-    // there are is known on the device only: CTAs without one exit)
-    int lblocks = v.w < 2 * v.num_sms ? v.w : 2 * v.num_sms;
+    // one CTA per reference listed (how many there are is known on the device
+    // only: CTAs without one exit), up to three per SM, or one where there are
+    // about as many references as individuals and few hold more than 32 (three:
+    // 5.0 us instead of 3.5 at 10,626 references without a large one)
+    int lblocks = (v.n2 >= 16 * v.w ? 3 : 1) * v.num_sms;
+    if (lblocks > v.w) lblocks = v.w;
     if (lblocks < 16) lblocks = 16;
-    k_pick_large<<<lblocks, 512, 0, s>>>(v);
+    k_pick_large<<<lblocks, PL_T, 0, s>>>(v);
     return cudaGetLastError();
 }
 
