@@ -112,9 +112,16 @@ __global__ void __launch_bounds__(DT) k_obj_dot(RunView v, const int32_t* rows_o
     const int m = v.m, d = v.d, k = m - 1;
     const int base = blockIdx.x * RB;
     const int rows = min(RB, n - base);
-    for (int e = threadIdx.x; e < RB * k; e += DT) {
-        const int r = e / k, c = e - r * k;
-        xs[e] = r < rows ? v.X[(size_t)rows_of[base + r] * d + c] : 0.0f;
+    // (the rows' numbers first: four pairs of dependent loads in flight)
+    const float* x[RB];
+#pragma unroll
+    for (int r = 0; r < RB; ++r) x[r] = v.X + (size_t)rows_of[min(base + r, n - 1)] * d;
+    for (int c = threadIdx.x; c < k; c += DT) {
+        float t[RB];
+#pragma unroll
+        for (int r = 0; r < RB; ++r) t[r] = x[r][c];
+#pragma unroll
+        for (int r = 0; r < RB; ++r) xs[r * k + c] = r < rows ? t[r] : 0.0f;
     }
     __syncthreads();
     const int j = blockIdx.y * DT + threadIdx.x;
@@ -231,6 +238,9 @@ __global__ void k_init(RunView v)
 }
 
 // Variation only (m > 10: the objective follows in k_obj_dot + k_objective).
+// A warp per pair while pairs fill the GPU; with fewer, gridDim.y warps share
+// a pair's variables (each repeats its tournament).  400 pairs of 1,000
+// variables: 26 us in one warp each, 9.4 in six.
 __global__ void k_vary(RunView v)
 {
     const int q = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -239,11 +249,14 @@ __global__ void k_vary(RunView v)
     const uint32_t gen = v.ctrl->gen;
     float* x0 = v.X + (size_t)v.fslot[2 * q] * v.d;
     float* x1 = v.X + (size_t)v.fslot[2 * q + 1] * v.d;
-    merge_pair(v, q);
-    vary_pair(v, q, gen, [&](int var, float c1, float c2) {
-        x0[var] = c1;
-        x1[var] = c2;
-    });
+    if (blockIdx.y == 0) merge_pair(v, q);
+    vary_pair(
+        v, q, gen,
+        [&](int var, float c1, float c2) {
+            x0[var] = c1;
+            x1[var] = c2;
+        },
+        32 * blockIdx.y, 32 * gridDim.y);
 }
 
 // Variation fused with the softmax-simplex objective (m <= 10; see
@@ -316,7 +329,10 @@ cudaError_t launch_vary_eval(const RunView& v, cudaStream_t s)
         }
         return cudaGetLastError();
     }
-    k_vary<<<blocks, 256, 0, s>>>(v);
+    // about 16 warps per SM (a quarter of what is resident: issue-bound)
+    const int want = 16 * v.num_sms / (v.N / 2), most = (v.d + 31) / 32;
+    const int parts = want < 1 ? 1 : want < most ? want : most;
+    k_vary<<<dim3(blocks, parts), 256, 0, s>>>(v);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     e = launch_obj_dot(v, v.cslot, v.N, s);

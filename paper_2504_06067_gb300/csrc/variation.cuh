@@ -48,11 +48,12 @@ __device__ __forceinline__ void merge_pair(const RunView& v, int q)
 // Variation of one pair (one warp, lanes over the variables): binary
 // tournament on rank (first drawn wins ties), SBX with per-variable
 // crossover and child swap, polynomial mutation, clip to [0, 1].  Calls
-// out(var, c1, c2) for every variable in lane order var = lane + 32 t.
+// out(var, c1, c2) for every variable in lane order var = lane + 32 t (from
+// v0 on and every `step`-th only, when several warps share the pair).
 // SBX is written c1,2 = (y1 + y2)/2 -/+ (beta/2)(y2 - y1) with one FMA, the
 // same value as ((1 + beta) y1 + (1 - beta) y2)/2 with fewer roundings.
 template <class Out>
-__device__ __forceinline__ void vary_pair(const RunView& v, int q, uint32_t gen, Out out)
+__device__ __forceinline__ void vary_pair(const RunView& v, int q, uint32_t gen, Out out, int v0 = 0, int step = 32)
 {
     const int lane = lane_id();
     const int N = v.N, d = v.d;
@@ -67,7 +68,7 @@ __device__ __forceinline__ void vary_pair(const RunView& v, int q, uint32_t gen,
     const size_t p2 = v.rank[b2] < v.rank[a2] ? rb2 : ra2;
     const bool cross = u01(cx) < v.p_c;
     const float e = 1.0f / (v.eta_c + 1.0f);
-    for (int var = lane; var < d; var += 32) {
+    for (int var = v0 + lane; var < d; var += step) {
         const float y1 = v.X[p1 * d + var], y2 = v.X[p2 * d + var];
         float c1 = y1, c2 = y2;
         const U4 sb = philox((uint32_t)q * (uint32_t)d + (uint32_t)var, gen, RNG_SBX, 0u, v.seed);
