@@ -747,9 +747,11 @@ nsga3_status device_status(nsga3_ctx* ctx, cudaStream_t s, bool clear)
 }
 
 // Whether kernels of this context's device can use p directly: device
-// memory of that device (or, with pinned, page-locked host memory).
+// memory of that device (or, with pinned, page-locked host memory), aligned
+// to its 4-byte elements.
 bool on_device(const nsga3_ctx* ctx, const void* p, bool pinned)
 {
+    if (reinterpret_cast<uintptr_t>(p) & 3) return false;
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
         cudaGetLastError();
@@ -759,17 +761,37 @@ bool on_device(const nsga3_ctx* ctx, const void* p, bool pinned)
     return pinned && a.type == cudaMemoryTypeHost && a.devicePointer == p;
 }
 
-// Rows idx[0..N) of X to dst (any): written by the kernel where it can reach
-// dst, through the staging rows otherwise (the copy to pageable memory
-// returns when it is done, so the staging rows are free again).
-nsga3_status rows_out(nsga3_ctx* ctx, const int32_t* idx, float* dst, cudaStream_t s)
+// n 4-byte elements from src to dst: into c when a kernel can write dst, by a
+// copy of their own otherwise
+nsga3_status copy_out(nsga3_ctx* ctx, PlainCopy* c, const void* src, void* dst, size_t n, cudaStream_t s)
 {
-    if (on_device(ctx, dst, true)) {
-        CK(launch_rows_out(ctx->v, idx, dst, s));
+    *c = PlainCopy{nullptr, nullptr, 0};
+    if (!dst) return NSGA3_OK;
+    if (on_device(ctx, dst, false))
+        *c = PlainCopy{(const uint32_t*)src, (uint32_t*)dst, (int)n};
+    else
+        CK(cudaMemcpyAsync(dst, src, n * 4, cudaMemcpyDefault, s));
+    return NSGA3_OK;
+}
+
+// Rows idx[0..N) of X to X (any, or null), objectives and ranks beside them:
+// written by one launch where it can reach them, X through the staging rows
+// otherwise (the copy to pageable memory returns when it is done, so the
+// staging rows are free again).
+nsga3_status rows_out(nsga3_ctx* ctx, const int32_t* idx, float* X, const float* Fsrc, float* F, const int32_t* rsrc,
+                      int32_t* rank, cudaStream_t s)
+{
+    PlainCopy a, b;
+    nsga3_status st = copy_out(ctx, &a, Fsrc, F, (size_t)ctx->N * ctx->m, s);
+    if (!st) st = copy_out(ctx, &b, rsrc, rank, (size_t)ctx->N, s);
+    if (st) return st;
+    if (!X) {
+        CK(launch_copies(a, b, s));
         return NSGA3_OK;
     }
-    CK(launch_rows_out(ctx->v, idx, ctx->v.Xtmp, s));
-    CK(cudaMemcpyAsync(dst, ctx->v.Xtmp, (size_t)ctx->N * ctx->d * sizeof(float), cudaMemcpyDefault, s));
+    const bool direct = on_device(ctx, X, true);
+    CK(launch_rows_out(ctx->v, idx, direct ? X : ctx->v.Xtmp, a, b, s));
+    if (!direct) CK(cudaMemcpyAsync(X, ctx->v.Xtmp, (size_t)ctx->N * ctx->d * sizeof(float), cudaMemcpyDefault, s));
     return NSGA3_OK;
 }
 
@@ -1078,8 +1100,11 @@ nsga3_status nsga3_select(nsga3_ctx* ctx, const float* objs, int32_t* ranks, int
         CK(cudaGraphLaunch(ctx->gx_select, s));
     }
     ctx->host_launches += select_launches(ctx);
-    CK(cudaMemcpyAsync(ranks, ctx->vs.rank2, (size_t)ctx->n2 * sizeof(int32_t), cudaMemcpyDefault, s));
-    CK(cudaMemcpyAsync(selected, ctx->vs.sel, (size_t)ctx->N * sizeof(int32_t), cudaMemcpyDefault, s));
+    PlainCopy a, b;
+    nsga3_status st = copy_out(ctx, &a, ctx->vs.rank2, ranks, (size_t)ctx->n2, s);
+    if (!st) st = copy_out(ctx, &b, ctx->vs.sel, selected, (size_t)ctx->N, s);
+    if (st) return st;
+    CK(launch_copies(a, b, s));
     ctx->last_kind = 1;
     return NSGA3_OK;
 }
@@ -1193,13 +1218,7 @@ nsga3_status nsga3_get_population(nsga3_ctx* ctx, float* X, float* F, int32_t* r
 {
     if (!ctx) return fail(ctx, NSGA3_EINVAL, "null context");
     cudaStream_t s = (cudaStream_t)stream;
-    if (X) {
-        nsga3_status st = rows_out(ctx, ctx->v.pcan, X, s);
-        if (st) return st;
-    }
-    if (F) CK(cudaMemcpyAsync(F, ctx->v.PF, (size_t)ctx->N * ctx->m * sizeof(float), cudaMemcpyDefault, s));
-    if (rank) CK(cudaMemcpyAsync(rank, ctx->v.rank, (size_t)ctx->N * sizeof(int32_t), cudaMemcpyDefault, s));
-    return NSGA3_OK;
+    return rows_out(ctx, ctx->v.pcan, X, ctx->v.PF, F, ctx->v.rank, rank, s);
 }
 
 nsga3_status nsga3_set_population(nsga3_ctx* ctx, const float* X, const float* F, const int32_t* rank,
@@ -1224,13 +1243,7 @@ nsga3_status nsga3_get_children(nsga3_ctx* ctx, float* X, float* F, void* stream
 {
     if (!ctx) return fail(ctx, NSGA3_EINVAL, "null context");
     cudaStream_t s = (cudaStream_t)stream;
-    const size_t N = ctx->N;
-    if (X) {
-        nsga3_status st = rows_out(ctx, ctx->v.cslot, X, s);
-        if (st) return st;
-    }
-    if (F) CK(cudaMemcpyAsync(F, ctx->v.F + N * ctx->m, N * ctx->m * sizeof(float), cudaMemcpyDefault, s));
-    return NSGA3_OK;
+    return rows_out(ctx, ctx->v.cslot, X, ctx->v.F + (size_t)ctx->N * ctx->m, F, nullptr, nullptr, s);
 }
 
 nsga3_status nsga3_set_counter(nsga3_ctx* ctx, uint64_t gen, void* stream)

@@ -131,41 +131,84 @@ __global__ void __launch_bounds__(256) k_gather_rows(RunView v)
     for (int q = lane_id(); q < v.m; q += 32) v.PF[(size_t)p * v.m + q] = v.F[(size_t)i * v.m + q];
 }
 
-// Rows between X and a caller's N x d array (16-byte words when both sides'
-// rows start on 16-byte boundaries).  A CTA moves RW * 256 consecutive words
-// of the array, a thread RW of them 256 apart with all loads in flight; one
-// 64-bit division per thread finds the CTA's first row.  (A warp per row left
-// most lanes idle at small d and one load in flight at large ones: 11.3 us
-// for 12,800 rows of 500, 8.2 now.)
+// Rows between X and a caller's N x d array, in words of 16, 8 or 4 bytes as
+// both sides' rows allow.  A CTA moves R * 256 consecutive words of the array,
+// a thread R of them 256 apart with all loads in flight; one 64-bit division
+// per thread finds the CTA's first row.  (A warp per row left most lanes idle
+// at small d and one load in flight at large ones: 11.3 us for 12,800 rows of
+// 500, 8.2 now.)  Bound: requests in flight: 50,000 rows of 200 / 202 / 201
+// floats 10 / 15 / 20 us (a plain copy 12.6).
 constexpr int RW = 4;
 
-template <class T, class F>
+// words per thread (eight of 4 bytes leave too few threads at small sizes)
+template <class T>
+__host__ __device__ constexpr int row_words()
+{
+    return sizeof(T) == 8 ? 8 : 4;
+}
+__host__ __device__ inline int plain_ctas(const PlainCopy& p) { return (p.n + 256 * RW - 1) / (256 * RW); }
+
+template <class T, int R, class F>
 __device__ __forceinline__ void for_row_words(int N, int words, F&& f)
 {
-    const long long e0 = (long long)blockIdx.x * (256 * RW);
+    const long long e0 = (long long)blockIdx.x * (256 * R);
     const long long p0 = e0 / words;
     const int r0 = (int)(e0 - p0 * words);
-    T x[RW];
-    int p[RW], q[RW];
+    T x[R];
+    int p[R], q[R];
+    // r / words for r < words + 256 R: exact by the reciprocal for rows below
+    // 2,048 words (r words < 2^24), one wrap at most for longer ones
+    static_assert(R <= 8, "one wrap");
+    const unsigned inv = words < 2048 ? (1u << 24) / (unsigned)words + 1u : 0u;
 #pragma unroll
-    for (int t = 0; t < RW; ++t) {
+    for (int t = 0; t < R; ++t) {
         const unsigned r = (unsigned)r0 + t * 256 + threadIdx.x;
-        const unsigned n = r / (unsigned)words;
+        const unsigned n = words < 2048 ? (unsigned)(((unsigned long long)r * inv) >> 24) : (r >= (unsigned)words ? 1u : 0u);
         p[t] = p0 + n < N ? (int)(p0 + n) : -1;
         q[t] = (int)(r - n * (unsigned)words);
     }
     f(x, p, q);
 }
 
-template <class T>
-__global__ void __launch_bounds__(256) k_rows_out(RunView v, const int32_t* idx, T* dst, int words)
+__device__ __forceinline__ void plain_copy(int c, PlainCopy a, const PlainCopy& b)
 {
-    for_row_words<T>(v.N, words, [&](T(&x)[RW], int(&p)[RW], int(&q)[RW]) {
+    const int na = plain_ctas(a);
+    if (c >= na) {
+        c -= na;
+        a = b;
+    }
+    uint32_t x[RW];
 #pragma unroll
-        for (int t = 0; t < RW; ++t)
+    for (int t = 0; t < RW; ++t) {
+        const int e = (c * RW + t) * 256 + (int)threadIdx.x;
+        x[t] = e < a.n ? a.src[e] : 0u;
+    }
+#pragma unroll
+    for (int t = 0; t < RW; ++t) {
+        const int e = (c * RW + t) * 256 + (int)threadIdx.x;
+        if (e < a.n) a.dst[e] = x[t];
+    }
+}
+
+__global__ void __launch_bounds__(256) k_copies(PlainCopy a, PlainCopy b) { plain_copy((int)blockIdx.x, a, b); }
+
+// (the objectives and ranks that go out with the rows are copied by further
+// CTAs of the same launch: a copy node of their own each took 1.5 us)
+template <class T>
+__global__ void __launch_bounds__(256) k_rows_out(RunView v, const int32_t* idx, T* dst, int words, int ctas, PlainCopy a,
+                                                  PlainCopy b)
+{
+    if ((int)blockIdx.x >= ctas) {
+        plain_copy((int)blockIdx.x - ctas, a, b);
+        return;
+    }
+    constexpr int R = row_words<T>();
+    for_row_words<T, R>(v.N, words, [&](T(&x)[R], int(&p)[R], int(&q)[R]) {
+#pragma unroll
+        for (int t = 0; t < R; ++t)
             if (p[t] >= 0) x[t] = reinterpret_cast<const T*>(v.X)[(size_t)idx[p[t]] * words + q[t]];
 #pragma unroll
-        for (int t = 0; t < RW; ++t)
+        for (int t = 0; t < R; ++t)
             if (p[t] >= 0) dst[(size_t)p[t] * words + q[t]] = x[t];
     });
 }
@@ -175,12 +218,13 @@ __global__ void __launch_bounds__(256) k_rows_out(RunView v, const int32_t* idx,
 template <class T>
 __global__ void __launch_bounds__(256) k_rows_in(RunView v, const T* src, int words)
 {
-    for_row_words<T>(v.N, words, [&](T(&x)[RW], int(&p)[RW], int(&q)[RW]) {
+    constexpr int R = row_words<T>();
+    for_row_words<T, R>(v.N, words, [&](T(&x)[R], int(&p)[R], int(&q)[R]) {
 #pragma unroll
-        for (int t = 0; t < RW; ++t)
+        for (int t = 0; t < R; ++t)
             if (p[t] >= 0) x[t] = src[(size_t)p[t] * words + q[t]];
 #pragma unroll
-        for (int t = 0; t < RW; ++t)
+        for (int t = 0; t < R; ++t)
             if (p[t] >= 0) {
                 const int slot = v.pold[p[t]];
                 reinterpret_cast<T*>(v.X)[(size_t)slot * words + q[t]] = x[t];
@@ -258,27 +302,58 @@ cudaError_t launch_gather(const RunView& v, cudaStream_t s)
     return cudaGetLastError();
 }
 
-static unsigned row_ctas(int N, int words)
+// 16-, 8- or 4-byte words: what the row width and the caller's address allow
+static int word_bytes(int d, const void* p)
 {
-    return (unsigned)(((long long)N * words + 256 * RW - 1) / (256 * RW));
+    const uintptr_t a = reinterpret_cast<uintptr_t>(p) | (uintptr_t)d * 4;
+    return (a & 15) == 0 ? 16 : (a & 7) == 0 ? 8 : 4;
 }
 
-cudaError_t launch_rows_out(const RunView& v, const int32_t* idx, float* dst, cudaStream_t s)
+template <class T>
+static unsigned row_ctas(int N, int words)
 {
-    if ((v.d & 3) == 0 && (reinterpret_cast<uintptr_t>(dst) & 15) == 0)
-        k_rows_out<float4><<<row_ctas(v.N, v.d / 4), 256, 0, s>>>(v, idx, reinterpret_cast<float4*>(dst), v.d / 4);
-    else
-        k_rows_out<float><<<row_ctas(v.N, v.d), 256, 0, s>>>(v, idx, dst, v.d);
+    const int per = 256 * row_words<T>();
+    return (unsigned)(((long long)N * words + per - 1) / per);
+}
+
+template <class T>
+static cudaError_t rows_out(const RunView& v, const int32_t* idx, float* dst, PlainCopy a, PlainCopy b, cudaStream_t s)
+{
+    const int words = v.d * 4 / (int)sizeof(T);
+    const unsigned ctas = row_ctas<T>(v.N, words);
+    k_rows_out<T><<<ctas + plain_ctas(a) + plain_ctas(b), 256, 0, s>>>(v, idx, reinterpret_cast<T*>(dst), words, (int)ctas,
+                                                                       a, b);
+    return cudaGetLastError();
+}
+
+template <class T>
+static cudaError_t rows_in(const RunView& v, const float* src, cudaStream_t s)
+{
+    const int words = v.d * 4 / (int)sizeof(T);
+    k_rows_in<T><<<row_ctas<T>(v.N, words), 256, 0, s>>>(v, reinterpret_cast<const T*>(src), words);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_rows_out(const RunView& v, const int32_t* idx, float* dst, PlainCopy a, PlainCopy b, cudaStream_t s)
+{
+    const int bytes = word_bytes(v.d, dst);
+    if (bytes == 16) return rows_out<float4>(v, idx, dst, a, b, s);
+    return bytes == 8 ? rows_out<float2>(v, idx, dst, a, b, s) : rows_out<float>(v, idx, dst, a, b, s);
+}
+
+cudaError_t launch_copies(PlainCopy a, PlainCopy b, cudaStream_t s)
+{
+    const int g = plain_ctas(a) + plain_ctas(b);
+    if (g == 0) return cudaSuccess;
+    k_copies<<<g, 256, 0, s>>>(a, b);
     return cudaGetLastError();
 }
 
 cudaError_t launch_rows_in(const RunView& v, const float* src, cudaStream_t s)
 {
-    if ((v.d & 3) == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0)
-        k_rows_in<float4><<<row_ctas(v.N, v.d / 4), 256, 0, s>>>(v, reinterpret_cast<const float4*>(src), v.d / 4);
-    else
-        k_rows_in<float><<<row_ctas(v.N, v.d), 256, 0, s>>>(v, src, v.d);
-    return cudaGetLastError();
+    const int bytes = word_bytes(v.d, src);
+    if (bytes == 16) return rows_in<float4>(v, src, s);
+    return bytes == 8 ? rows_in<float2>(v, src, s) : rows_in<float>(v, src, s);
 }
 
 cudaError_t launch_slots_init(const RunView& v, cudaStream_t s)

@@ -250,7 +250,7 @@ __global__ void k_vary(RunView v)
     float* x0 = v.X + (size_t)v.fslot[2 * q] * v.d;
     float* x1 = v.X + (size_t)v.fslot[2 * q + 1] * v.d;
     if (blockIdx.y == 0) merge_pair(v, q);
-    vary_pair(
+    vary_pair<false>(
         v, q, gen,
         [&](int var, float c1, float c2) {
             x0[var] = c1;
@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(256) k_vary_eval(RunView v)
     const int q = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (q >= v.N / 2) return;
     if (read_status(v.ctrl)) return;
-    vary_eval_pair<M>(v, q, v.ctrl->gen);
+    vary_eval_pair<M, false>(v, q, v.ctrl->gen);
 }
 
 cudaError_t launch_obj_dot(const RunView& v, const int32_t* rows_of, int n, cudaStream_t s)

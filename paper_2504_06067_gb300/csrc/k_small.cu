@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(ST, 1) k_small(RunView v, int mode, int C, con
         for (int t = 0; t < 8; ++t) c->domstat[t] = 0ull;
     }
     if (status == 0 && mode == 1) {
-        for (int q = rank * SWARPS + warp; q < N / 2; q += C * SWARPS) vary_eval_pair<M>(v, q, gen);
+        for (int q = rank * SWARPS + warp; q < N / 2; q += C * SWARPS) vary_eval_pair<M, true>(v, q, gen);
         cluster_sync();  // merged objectives and rows
     }
     const float* Fg = mode == 0 ? Fin : v.F;

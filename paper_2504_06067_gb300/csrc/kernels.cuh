@@ -71,8 +71,15 @@ cudaError_t launch_select_probe(const unsigned long long* keys, int n, int need,
 cudaError_t launch_mark(const RunView& v, cudaStream_t s);
 cudaError_t launch_select_out(const RunView& v, cudaStream_t s);
 cudaError_t launch_gather(const RunView& v, cudaStream_t s);
-// rows of X to dst (row r of dst = row idx[r] of X), and back
-cudaError_t launch_rows_out(const RunView& v, const int32_t* idx, float* dst, cudaStream_t s);
+// rows of X to dst (row r of dst = row idx[r] of X) and up to two plain copies
+// (n = 0: none) in the same launch; plain copies alone; rows back
+struct PlainCopy {
+    const uint32_t* src;
+    uint32_t* dst;
+    int n;  // words
+};
+cudaError_t launch_rows_out(const RunView& v, const int32_t* idx, float* dst, PlainCopy a, PlainCopy b, cudaStream_t s);
+cudaError_t launch_copies(PlainCopy a, PlainCopy b, cudaStream_t s);
 cudaError_t launch_rows_in(const RunView& v, const float* src, cudaStream_t s);
 cudaError_t launch_slots_init(const RunView& v, cudaStream_t s);
 

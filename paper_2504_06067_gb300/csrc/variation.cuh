@@ -52,7 +52,10 @@ __device__ __forceinline__ void merge_pair(const RunView& v, int q)
 // v0 on and every `step`-th only, when several warps share the pair).
 // SBX is written c1,2 = (y1 + y2)/2 -/+ (beta/2)(y2 - y1) with one FMA, the
 // same value as ((1 + beta) y1 + (1 - beta) y2)/2 with fewer roundings.
-template <class Out>
+// ROLL: one copy of the mutation's code for both children (a chain that runs
+// once is bound by instruction fetch; a kernel that fills the GPU by issue: 8 %
+// more instructions, 97 us instead of 92 at N = 50,000, d = 200).
+template <bool ROLL, class Out>
 __device__ __forceinline__ void vary_pair(const RunView& v, int q, uint32_t gen, Out out, int v0 = 0, int step = 32)
 {
     const int lane = lane_id();
@@ -91,15 +94,20 @@ __device__ __forceinline__ void vary_pair(const RunView& v, int q, uint32_t gen,
         const bool mut0 = u01(sb.w) < v.p_m;
         const U4 pm = philox((uint32_t)q * (uint32_t)d + (uint32_t)var, gen, RNG_PM, 0u, v.seed);
         const bool mut1 = u01(pm.y) < v.p_m;
+        if constexpr (ROLL) {
 #pragma unroll 1
-        for (int h = 0; h < 2; ++h)  // one copy of the mutation's code
-            if (h ? mut1 : mut0) {
-                const float y = pm_mutate(h ? c2 : c1, u01(h ? pm.z : pm.x), v.eta_m);
-                if (h)
-                    c2 = y;
-                else
-                    c1 = y;
-            }
+            for (int h = 0; h < 2; ++h)
+                if (h ? mut1 : mut0) {
+                    const float y = pm_mutate(h ? c2 : c1, u01(h ? pm.z : pm.x), v.eta_m);
+                    if (h)
+                        c2 = y;
+                    else
+                        c1 = y;
+                }
+        } else {
+            if (mut0) c1 = pm_mutate(c1, u01(pm.x), v.eta_m);
+            if (mut1) c2 = pm_mutate(c2, u01(pm.z), v.eta_m);
+        }
         out(var, c1, c2);
     }
 }
@@ -134,7 +142,7 @@ __device__ __forceinline__ void g_add(float xv, float& sh, float& sl)
 // den and 1 + g as float-float sums; one correctly rounded division.  The
 // result is within about 4 ulp (2.4e-7) of (1 + g) e_j / den: expf's 2 ulp,
 // the division's and the last product's half ulp.
-template <int M>
+template <int M, bool ROLL>
 __device__ __forceinline__ void vary_eval_pair(const RunView& v, int q, uint32_t gen)
 {
     constexpr int K = M - 1;
@@ -145,7 +153,7 @@ __device__ __forceinline__ void vary_eval_pair(const RunView& v, int q, uint32_t
     merge_pair(v, q);
     float gh0 = 0.0f, gl0 = 0.0f, gh1 = 0.0f, gl1 = 0.0f;
     float xk0 = 0.0f, xk1 = 0.0f;
-    vary_pair(v, q, gen, [&](int var, float c1, float c2) {
+    vary_pair<ROLL>(v, q, gen, [&](int var, float c1, float c2) {
         x0[var] = c1;
         x1[var] = c2;
         if (var < K) {

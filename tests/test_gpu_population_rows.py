@@ -64,3 +64,35 @@ def test_population_calls_in_any_order(n, m, d, N):
             r.check(n.nsga3_vary(r.ctx, None))
             Xc, Fc = r.children()
             assert np.array_equal(r.population()[0], Xs)
+
+
+@pytest.mark.parametrize("shape", [(3, 2, 3), (3, 130, 7), (5, 1100, 8), (4, 514, 33), (12, 90, 13)])
+def test_outputs_beside_the_rows(n, shape):
+    """Rows, objectives and ranks written by one launch: device buffers, device
+    buffers of odd addresses, host buffers and each of them left out give the
+    same values, and nothing past their ends."""
+    import torch
+    m, N, d = shape
+    W = wl.objective_weights(m, 3)
+    with Run(n, m, d, N, 1, seed=4, W=W) as r:
+        r.check(n.nsga3_init(r.ctx, None))
+        r.check(n.nsga3_run(r.ctx, 3, None))
+        X, F, rank = r.population()
+        Xc, Fc = r.children()
+        for off in (0, 1, 3):
+            bx = torch.full((N * d + 8,), -7.0, device="cuda")
+            bf = torch.full((N * m + 8,), -7.0, device="cuda")
+            br = torch.full((N + 8,), -7, device="cuda", dtype=torch.int32)
+            torch.cuda.synchronize()
+            for what in (7, 1, 2, 4, 6):
+                p = [t[off:].data_ptr() if what >> k & 1 else None for k, t in enumerate((bx, bf, br))]
+                r.check(n.nsga3_get_population(r.ctx, p[0], p[1], p[2], None))
+                r.check(r.sync())
+            for t, a in ((bx, X), (bf, F), (br, rank)):
+                h = t.cpu().numpy()
+                assert np.array_equal(h[off:off + a.size], a.ravel())
+                assert (h[:off] == -7).all() and (h[off + a.size:] == -7).all()
+            r.check(n.nsga3_get_children(r.ctx, bx[off:].data_ptr(), bf[off:].data_ptr(), None))
+            r.check(r.sync())
+            assert np.array_equal(bx[off:off + N * d].cpu().numpy(), Xc.ravel())
+            assert np.array_equal(bf[off:off + N * m].cpu().numpy(), Fc.ravel())
