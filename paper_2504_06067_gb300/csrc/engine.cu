@@ -57,7 +57,9 @@ struct nsga3_ctx {
     cudaEvent_t ev[EV_COUNT] = {};
     int last_kind = 0;  // 1 = select, 2 = step
     long long host_launches = 0;  // kernels launched by calls (peel passes counted on the device)
-    DeviceArena* arena = nullptr;  // workspace source (nullptr: cudaMalloc per buffer)
+    DeviceArena* arena = nullptr;  // workspace source (nullptr: one cudaMalloc, carved up)
+    char* slab = nullptr;
+    size_t slab_used = 0;
     bool count_only = false;       // sizing pass: count bytes, allocate nothing
     size_t counted = 0;
     bool eager = false; // NSGA3_EAGER=1: no graphs, host-driven peel loop (profiling)
@@ -186,14 +188,11 @@ nsga3_status alloc(nsga3_ctx* ctx, T** p, size_t count)
     if (ctx->arena) {
         q = ctx->arena->alloc(bytes);
         if (!q) return fail(ctx, NSGA3_ENOMEM, "device arena has no free block of %zu bytes", bytes);
+        ctx->allocs.push_back(q);
     } else {
-        cudaError_t e = cudaMalloc(&q, bytes);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            return fail(ctx, NSGA3_ENOMEM, "cudaMalloc of %zu bytes failed: %s", bytes, cudaGetErrorString(e));
-        }
+        q = ctx->slab + ctx->slab_used;  // (setup counted the same buffers)
+        ctx->slab_used += DeviceArena::round_up(bytes);
     }
-    ctx->allocs.push_back(q);
     *p = static_cast<T*>(q);
     return NSGA3_OK;
 }
@@ -636,6 +635,21 @@ nsga3_status setup(nsga3_ctx* ctx)
     // a limit of the interface: m <= 10 took up to 220 KB of block tables
     if (ctx->m <= NSGA3_FAST_M && (size_t)((ctx->w + 31) / 32) * (ctx->M4 + 10) * 4 + 4096 > 220 * 1024)
         return fail(ctx, NSGA3_EINVAL, "%d reference directions exceed the association's limit", ctx->w);
+    if (!ctx->arena) {
+        // one allocation for all buffers (some 70 of them one by one took 0.2 ms)
+        ctx->count_only = true;
+        const nsga3_status cst = setup_alloc(ctx);
+        ctx->count_only = false;
+        if (cst) return cst;
+        void* q = nullptr;
+        const cudaError_t e = cudaMalloc(&q, ctx->counted);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            return fail(ctx, NSGA3_ENOMEM, "cudaMalloc of %zu bytes failed: %s", ctx->counted, cudaGetErrorString(e));
+        }
+        ctx->allocs.push_back(q);
+        ctx->slab = static_cast<char*>(q);
+    }
     nsga3_status ast = setup_alloc(ctx);
     if (ast) return ast;
     const int m = ctx->m, d = ctx->d, N = ctx->N, n2 = ctx->n2, ld = ctx->ld, NW = ctx->NW;
@@ -652,7 +666,8 @@ nsga3_status setup(nsga3_ctx* ctx)
     for (int e = 0; e < EV_COUNT; ++e) CK(cudaEventCreate(&ctx->ev[e]));
     cudaStream_t s = ctx->cap;
     CK(cudaMemsetAsync(v.ctrl, 0, sizeof(Ctrl), s));
-    if (!v.streaming) CK(cudaMemsetAsync(v.Dom, 0, (size_t)NW * ld * sizeof(uint32_t), s));
+    // (m <= 10: blocks whose bit in dnz is clear are never read)
+    if (!v.streaming && !v.dnz) CK(cudaMemsetAsync(v.Dom, 0, (size_t)NW * ld * sizeof(uint32_t), s));
     if (v.dom_ks > 1) {
         CK(cudaMemsetAsync(v.dpa, 0, (size_t)NW * ld * sizeof(uint32_t), s));
         CK(cudaMemsetAsync(v.dpb, 0, (size_t)NW * ld * sizeof(uint32_t), s));

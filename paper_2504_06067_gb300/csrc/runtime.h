@@ -39,7 +39,7 @@ private:
     mutable std::mutex mu_;
 };
 
-// Context creation with optional arena (nullptr: cudaMalloc per buffer).
+// Context creation with optional arena (nullptr: one cudaMalloc).
 // shared_gpu: the run will share the GPU with other runs (its cooperative
 // launches take fewer CTAs).  On failure *err holds the message and *out is
 // nullptr.
