@@ -451,7 +451,7 @@ nsga3_status setup_alloc(nsga3_ctx* ctx)
     v.w = w;
     v.M4 = M4;
     v.num_sms = ctx->num_sms > 0 ? ctx->num_sms : 1;
-    v.shared_gpu = ctx->shared_gpu ? 1 : 0;
+    v.shared_gpu = ctx->shared_gpu ? 4 : 0;
     v.full_sort = ctx->opts.full_sort ? 1 : 0;
     v.debug_recheck_all = ctx->opts.debug_recheck_all ? 1 : 0;
     v.streaming = ctx->opts.streaming ? 1 : 0;
@@ -998,7 +998,7 @@ nsga3_status build_batch_graph(nsga3_ctx* ctx, nsga3_ctx** ctxs, int n, int gens
             }
             // the runs of a batched graph share the GPU
             const int shared = ctxs[r]->v.shared_gpu;
-            ctxs[r]->v.shared_gpu = 1;
+            ctxs[r]->v.shared_gpu = n < 16 ? 2 : 4;  // (see launch_peel)
             for (int k = 0; k < gens && !st; ++k) {
                 nsga3_status rs = record_generation(ctxs[r], br[r], false);
                 if (rs) {

@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(LB) k_level(RunView v)
         // most references share a few level values (rho_j = 0 when S is
         // empty): increments by one, which the shared-memory atomics take
         // together for the lanes of a warp (groups of equal lanes by
-        // match_any took 4 us for 10,626 references, this 1)
+        // match_any: the kernel 14.1 us for 10,626 references, 12.5 so)
         for_refs([&](int, int lo, int rp) {
             if (rp > 0 && (lo < 0 || rp > v.n2)) {  // counts out of range: an invariant failed upstream
                 set_status(c, DEV_EINTERNAL);

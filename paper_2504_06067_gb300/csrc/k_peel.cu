@@ -375,11 +375,13 @@ cudaError_t launch_peel(const RunView& v, int num_sms, cudaStream_t s)
     if (v.peel_ctas > 0 && v.peel_ctas < occ) occ = v.peel_ctas;  // launch-shape option
     int grid = num_sms * occ;
     if (v.shared_gpu) {
-        // a quarter of the chunks per pass at most: every CTA of a cooperative
-        // launch must be resident at once, which a mix of runs rarely allows
-        // for a grid the size of the GPU (64 batched runs: 4.27x -> 4.61x the
-        // plain path)
-        const int g2 = nchunks / 4 > 0 ? nchunks / 4 : 1;
+        // every CTA of a cooperative launch must be resident at once, which a
+        // mix of runs rarely allows for a grid the size of the GPU: a CTA for
+        // four chunks, or for two with fewer than 16 runs.  Batched runs, 40
+        // generations, a CTA for 1, 2, 4, 8 chunks: 6 runs 11.1, 11.0, 11.2,
+        // 11.4 ms; 12 runs 13.2, 13.5, 14.8, 17.2; 16 runs 23.2, 21.9, 21.5,
+        // 22.9; 64 runs 64.9, 61.3, 60.3, 60.3
+        const int g2 = nchunks / v.shared_gpu > 0 ? nchunks / v.shared_gpu : 1;
         if (grid > g2) grid = g2;
     }
     if (grid > nchunks) grid = nchunks;
