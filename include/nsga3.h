@@ -100,7 +100,7 @@ void nsga3_default_opts(nsga3_opts* o);
  * objectives (2 <= m <= 512; the objective sweep of the paper's Table II
  * reaches 512; kernels are specialised for each m <= 10 and take m at run
  * time above; with m > 32 the intercept system is eliminated by a
- * cooperative grid), d variables (d >= m - 1 when W is given) and
+ * thread-block cluster), d variables (d >= m - 1 when W is given) and
  * Das-Dennis divisions ref_divisions >= 1 (Sec. II-C: w points uniform on
  * the unit simplex; opts->p2 > 0 adds an inner layer).  N must be even,
  * 2 <= N and 2N <= 2^21.  Allocates all device workspace (about
@@ -169,7 +169,9 @@ nsga3_status nsga3_vary(nsga3_ctx* ctx, void* stream);
 
 /* One generation (Alg. 1): variation, merge, selection, next population;
  * advances the counter by one.  One CUDA-graph launch of plain kernel nodes
- * (every front is peeled inside one cooperative kernel). Needs opts.W. */
+ * (every front is peeled inside one cooperative kernel), or for small
+ * populations (2N and w up to 2,048, m <= 10) one launch of one thread-block
+ * cluster.  Needs opts.W. */
 nsga3_status nsga3_step(nsga3_ctx* ctx, void* stream);
 
 /* `generations` calls of nsga3_step. */
