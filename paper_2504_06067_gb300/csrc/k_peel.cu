@@ -28,6 +28,12 @@
 // N = 12,800, 27 to 48 fronts): 296 us before, 202 now; m = 5, N = 10,628,
 // three fronts: 38 us before, 20 now; the first generation of m = 10,
 // N = 100,000: 342 us before, 128 now.
+// Several chunks per CTA keep the masks of the last seven passes in global
+// memory; a longer ring (16) gave a total order of 200,000 points 2.9 s in
+// place of 3.1 with all its loads in flight, and the knapsack 225 us.
+// Without the matrix (STREAM) every chunk is tested every pass: putting the
+// tests off piles them up on the CTAs whose chunks are due (8.6 -> 17.5 ms at
+// m = 3, 2N = 120,000, 32 fronts).
 #include <limits.h>
 #include <math_constants.h>
 
@@ -42,6 +48,54 @@ constexpr int RING = NSGA3_FRONT_RING;
 constexpr int PEEL_U = 4;   // Dom rows in flight per warp
 constexpr int MAXC = 64;  // chunks of a CTA whose state is kept between passes
 
+// Streaming: the members mk of a front word (rb: SQ x 16 bytes each) against
+// this lane's four columns, with the sign-bit test of the dominance build; a
+// member whose f_0 is below every f_0 of the chunk (cmin) needs objectives
+// 1 .. m - 1 only (f_0 makes the dominance strict).  Q = ceil(m / 4).
+// (One loop over ten objectives with a predicate each: 4.7 ms for two fronts
+// of m = 3, 2N = 120,000; 1.9 so.)
+constexpr int SQ = (NSGA3_FAST_M + 3) / 4;
+
+__device__ __forceinline__ uint32_t sign_or(const float4& a, const float4& b)
+{
+    return __float_as_uint(a.x - b.x) | __float_as_uint(a.y - b.y) | __float_as_uint(a.z - b.z) |
+           __float_as_uint(a.w - b.w);
+}
+
+template <int Q>
+__device__ __forceinline__ void stream_rows(const float4* rb, uint32_t mk, const float4 (&fc)[4][SQ], float cmin,
+                                            uint32_t (&a)[4])
+{
+    while (mk) {  // warp-uniform: every lane walks the same rows
+        const int b = __ffs(mk) - 1;
+        mk &= mk - 1u;
+        float4 y[Q];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) y[q] = rb[b * SQ + q];
+        if (y[0].x < cmin) {
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                uint32_t oa = __float_as_uint(fc[t][0].y - y[0].y) | __float_as_uint(fc[t][0].z - y[0].z) |
+                              __float_as_uint(fc[t][0].w - y[0].w);
+#pragma unroll
+                for (int q = 1; q < Q; ++q) oa |= sign_or(fc[t][q], y[q]);
+                a[t] += (~oa) >> 31;  // no f_iq > f_jq
+            }
+        } else {
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                uint32_t oa = 0u, ob = 0u;
+#pragma unroll
+                for (int q = 0; q < Q; ++q) {
+                    oa |= sign_or(fc[t][q], y[q]);
+                    ob |= sign_or(y[q], fc[t][q]);
+                }
+                a[t] += (ob & ~oa) >> 31;  // none greater, some smaller
+            }
+        }
+    }
+}
+
 template <bool STREAM>
 __global__ void __launch_bounds__(PEEL_THREADS, STREAM ? 1 : 2) k_peel(RunView v)
 {
@@ -55,7 +109,7 @@ __global__ void __launch_bounds__(PEEL_THREADS, STREAM ? 1 : 2) k_peel(RunView v
     __shared__ unsigned s_fs[3];  // size of a pass's front
     __shared__ int s_fail;
     __shared__ int c_min[MAXC], c_eval[MAXC], c_cum[MAXC];  // per chunk: smallest count left, pass of it, points then
-    __shared__ float rowbuf[STREAM ? PWMAX : 1][32][NSGA3_FAST_M];  // streaming: members of a front word
+    __shared__ float4 rowbuf[STREAM ? PWMAX : 1][32 * SQ];  // streaming: members of a front word
     Ctrl* c = v.ctrl;
     const int tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
     if (read_status(c)) return;  // uniform: set only by earlier kernels
@@ -91,7 +145,7 @@ __global__ void __launch_bounds__(PEEL_THREADS, STREAM ? 1 : 2) k_peel(RunView v
             if (k > 0 && slot < MAXC) {
                 k0 = c_eval[slot];
                 const int least = c_min[slot];
-                evald = !(least == INT_MAX || (least > cum - c_cum[slot] && (own || k - k0 < RING - 1)));
+                evald = !(least == INT_MAX || (!STREAM && least > cum - c_cum[slot] && (own || k - k0 < RING - 1)));
                 if (!evald) {
                     if (tid < NSGA3_PEEL_COLS / 32)
                         v.front[(size_t)(k % RING) * v.NW + j0 / 32 + tid] = 0u;
@@ -101,8 +155,15 @@ __global__ void __launch_bounds__(PEEL_THREADS, STREAM ? 1 : 2) k_peel(RunView v
             // the points ranked in passes k0 .. k-1, by word
             auto pending = [&](int w) {
                 uint32_t x = w < LISTCAP ? last[w] : __ldcg(&v.front[(size_t)((k - 1) % RING) * v.NW + w]);
-                if (own) return x;
-                for (int kk = k0; kk < k - 1; ++kk) x |= __ldcg(&v.front[(size_t)(kk % RING) * v.NW + w]);
+                if (STREAM || own) return x;
+                if (k0 < k - 1) {  // the older ones, their loads in flight together
+                    uint32_t y[RING - 2];
+#pragma unroll
+                    for (int r = 0; r < RING - 2; ++r)
+                        y[r] = __ldcg(&v.front[(size_t)(min(k0 + r, k - 1) % RING) * v.NW + w]);
+#pragma unroll
+                    for (int r = 0; r < RING - 2; ++r) x |= y[r];
+                }
                 return x;
             };
             // this thread's column: dominators not counted off (0: ranked or
@@ -131,19 +192,21 @@ __global__ void __launch_bounds__(PEEL_THREADS, STREAM ? 1 : 2) k_peel(RunView v
                 // with the sign-bit test of the dominance build; a member
                 // whose f_0 is below every f_0 of the chunk needs objectives
                 // 1..m-1 only (f_0 makes the dominance strict)
-                const int m = v.m;
-                float fc[4][NSGA3_FAST_M];
+                const int q4 = v.fs / 4;  // (the pads are 0 in rows and columns)
+                const float4* Fp4 = reinterpret_cast<const float4*>(v.Fp);
+                float4 fc[4][SQ];
                 float cmin = CUDART_INF_F;
 #pragma unroll
                 for (int t = 0; t < 4; ++t) {
 #pragma unroll
-                    for (int q = 0; q < NSGA3_FAST_M; ++q)
-                        fc[t][q] = q < m ? v.Fp[(size_t)(j0 + lane * 4 + t) * v.fs + q] : 0.0f;
-                    cmin = fminf(cmin, fc[t][0]);  // NaN padding columns are ignored by fminf
+                    for (int q = 0; q < SQ; ++q)
+                        fc[t][q] = q < q4 ? Fp4[(size_t)(j0 + lane * 4 + t) * q4 + q] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                    cmin = fminf(cmin, fc[t][0].x);  // NaN padding columns are ignored by fminf
                 }
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) cmin = fminf(cmin, __shfl_xor_sync(0xffffffffu, cmin, o));
-                float* rb = rowbuf[warp][0];
+                float4* rb = rowbuf[warp];
+                uint32_t a[4] = {0u, 0u, 0u, 0u};
                 for (int wb = 0; wb < lim; wb += LISTCAP) {
                     const int whe = min(wb + LISTCAP, lim);
                     int* const nl = &nlist[par];
@@ -165,49 +228,26 @@ __global__ void __launch_bounds__(PEEL_THREADS, STREAM ? 1 : 2) k_peel(RunView v
                         const uint2 L = list[e];
                         // the word's members, one per lane, into this warp's row buffer
                         if ((L.y >> lane) & 1u) {
-                            const size_t p = (size_t)L.x * 32 + lane;
+                            const float4* f = Fp4 + ((size_t)L.x * 32 + lane) * q4;
 #pragma unroll
-                            for (int q = 0; q < NSGA3_FAST_M; ++q)
-                                if (q < m) rb[lane * NSGA3_FAST_M + q] = __ldg(&v.Fp[p * v.fs + q]);
+                            for (int q = 0; q < SQ; ++q)
+                                if (q < q4) rb[lane * SQ + q] = __ldg(f + q);
                         }
                         __syncwarp();
-                        uint32_t mk = L.y;
-                        while (mk) {  // warp-uniform: every lane walks the same rows
-                            const int b = __ffs(mk) - 1;
-                            mk &= mk - 1u;
-                            const float* fi = rb + b * NSGA3_FAST_M;
-                            uint32_t d4[4];
-                            if (fi[0] < cmin) {
-#pragma unroll
-                                for (int t = 0; t < 4; ++t) {
-                                    uint32_t oa = 0u;
-#pragma unroll
-                                    for (int q = 1; q < NSGA3_FAST_M; ++q)
-                                        if (q < m) oa |= __float_as_uint(fc[t][q] - fi[q]);
-                                    d4[t] = (~oa) >> 31;  // no f_iq > f_jq
-                                }
-                            } else {
-#pragma unroll
-                                for (int t = 0; t < 4; ++t) {
-                                    uint32_t oa = 0u, ob = 0u;
-#pragma unroll
-                                    for (int q = 0; q < NSGA3_FAST_M; ++q)
-                                        if (q < m) {
-                                            oa |= __float_as_uint(fc[t][q] - fi[q]);
-                                            ob |= __float_as_uint(fi[q] - fc[t][q]);
-                                        }
-                                    d4[t] = (ob & ~oa) >> 31;  // none greater, some smaller
-                                }
-                            }
-                            a0 += d4[0];
-                            a1 += d4[1];
-                            a2 += d4[2];
-                            a3 += d4[3];
-                        }
+                        if (q4 == 1)
+                            stream_rows<1>(rb, L.y, fc, cmin, a);
+                        else if (q4 == 2)
+                            stream_rows<2>(rb, L.y, fc, cmin, a);
+                        else
+                            stream_rows<3>(rb, L.y, fc, cmin, a);
                         __syncwarp();
                     }
                     __syncthreads();  // list and nlist are reused
                 }
+                a0 = a[0];
+                a1 = a[1];
+                a2 = a[2];
+                a3 = a[3];
             } else if (!STREAM && k > 0) {
                 const uint4* base = reinterpret_cast<const uint4*>(v.Dom + dom_at(v, 0, J0, 0)) + lane;
                 // with the block bitmap (m <= 10) only the Dom blocks whose bit
@@ -323,7 +363,7 @@ __global__ void __launch_bounds__(PEEL_THREADS, STREAM ? 1 : 2) k_peel(RunView v
 #pragma unroll 4
             for (int w = tid; w < nwords; w += PT) {
                 const uint32_t x = __ldcg(words + w);
-                if (w < LISTCAP) last[w] = own && !evald ? last[w] | x : x;
+                if (w < LISTCAP) last[w] = !STREAM && own && !evald ? last[w] | x : x;
                 mine += __popc(x);
             }
             mine = __reduce_add_sync(0xffffffffu, mine);
