@@ -38,10 +38,16 @@ constexpr int SBINS = 512;     // bins of the reference-key histogram (top 9 bit
 constexpr int SKEYS = 64;      // keys of one bin ranked in shared memory
 constexpr int SLEV = (SMALL_N2 + 1 + ST - 1) / ST;  // niche levels per thread
 
-__device__ __forceinline__ void cluster_sync()
+__device__ __forceinline__ void cluster_arrive()
 {
     __syncwarp();
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_sync()
+{
+    cluster_arrive();
+    cluster_wait();
 }
 // address of the same shared variable in CTA r of the cluster, and stores to it
 __device__ __forceinline__ uint32_t peer(const void* p, int r)
@@ -187,6 +193,10 @@ __global__ void __launch_bounds__(ST, 1) k_small(RunView v, int mode, int C, con
     int* pi0 = reinterpret_cast<int*>(dyn + L.pi);
     uint32_t* dom = reinterpret_cast<uint32_t*>(dyn + L.dom);
     float* Fs = reinterpret_cast<float*>(dyn + L.big);
+    // A peer's shared memory may be written once that CTA is known to have
+    // started: without the variation's cluster barrier the CTAs arrive here and
+    // wait before the first front's words, the pair tests in between.
+    if (mode != 1) cluster_arrive();
     const uint32_t gen = c->gen;
     const int status = read_status(c);
     if (rank == 0 && tid == 0) {  // as k_sel_reset leaves it
@@ -222,6 +232,8 @@ __global__ void __launch_bounds__(ST, 1) k_small(RunView v, int mode, int C, con
     }
     for (int i = tid; i < n2; i += ST) pi0[i] = -1;
     if (__syncthreads_or(bad)) {  // the same in every CTA: each reads every objective
+        __syncwarp();
+        if (mode != 1) cluster_wait();
         if (tid < cols) ranks[c0 + tid] = -1;
         if (status == 0 && rank == 0 && tid == 0) set_status(c, DEV_ENONFINITE);
         return;
@@ -233,6 +245,7 @@ __global__ void __launch_bounds__(ST, 1) k_small(RunView v, int mode, int C, con
     else
         dominance_words<M, 2>(Fs, dom, n2, c0, colsP);
     __syncthreads();
+    if (mode != 1) cluster_wait();
 
     // ---- fronts: an unranked column without an unranked dominator is ranked
     int cum = 0, l = -1, passes = 0, nS = 0, nFl = 0;
