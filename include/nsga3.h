@@ -39,7 +39,8 @@ typedef enum {
     NSGA3_EINVAL = 1,     /* bad argument */
     NSGA3_ENOMEM = 2,     /* device allocation failed */
     NSGA3_ECUDA = 3,      /* a CUDA runtime call failed */
-    NSGA3_ENONFINITE = 4, /* NaN or Inf in the objectives given to nsga3_select */
+    NSGA3_ENONFINITE = 4, /* NaN or Inf in the objectives given to nsga3_select, or in a member
+                             that a generation has to normalise (see nsga3_set_population) */
     NSGA3_ETIMEOUT = 5,   /* a bounded device wait expired */
     NSGA3_ESTATE = 6,     /* call not valid in this context state */
     NSGA3_EINTERNAL = 7   /* a device-side invariant failed */
@@ -200,7 +201,11 @@ nsga3_status nsga3_batch_graph_builds(const nsga3_ctx* ctx, int64_t* builds);
 nsga3_status nsga3_get_population(nsga3_ctx* ctx, float* X, float* F, int32_t* rank, void* stream);
 
 /* Replaces the N parents: X (any, N x d), F (any, N x m), rank (any, N).
- * Any pointer may be NULL to keep the current values. */
+ * Any pointer may be NULL to keep the current values.  A parent with an
+ * objective that is not finite has no place among the reference directions: a
+ * generation in which one is in a front up to F_l and niching is needed sets
+ * NSGA3_ENONFINITE (reported by nsga3_sync) and leaves the population and the
+ * counter as they were. */
 nsga3_status nsga3_set_population(nsga3_ctx* ctx, const float* X, const float* F,
                                   const int32_t* rank, void* stream);
 

@@ -446,6 +446,11 @@ __global__ void __launch_bounds__(MT, 1) k_assoc_mma(RunView v)
 
 __device__ __forceinline__ void write_assoc(const RunView& v, Ctrl* c, int i, int rk, int j, double d)
 {
+    // no candidate: f' and the intercepts are finite here (not_finite_key), so an invariant failed
+    if ((unsigned)j >= (unsigned)v.w) {
+        set_status(c, DEV_EINTERNAL);
+        return;
+    }
     v.pi[i] = j;
     v.dist[i] = d;
     if (rk < c->l)

@@ -80,6 +80,10 @@ __device__ __noinline__ void solve_intercepts(const RunView& v, Ctrl* c, const i
     const int m = v.m;
     const int lane = lane_id();
     const bool row = lane < m;
+    if (__any_sync(0xffffffffu, row && not_finite_key(sf64::bits(nad[lane])))) {
+        if (lane == 0) set_status(c, DEV_ENONFINITE);
+        return;
+    }
     const double z = row ? zstar_of(c, lane) : 0.0;
     if (row) {
         c->zstar[lane] = z;
@@ -516,6 +520,7 @@ __global__ void __launch_bounds__(256) k_ext_reduce(RunView v, int parts)
         if (lane == 0) {
             c->ext[q] = bi;
             v.nadv[q] = __longlong_as_double((long long)n);
+            if (m > NSGA3_WARP_M && not_finite_key(n)) set_status(c, DEV_ENONFINITE);  // (else solve_intercepts)
         }
     }
     if (m > NSGA3_WARP_M) return;

@@ -123,7 +123,7 @@ struct SmallShared {
     int ext[NSGA3_FAST_M];
     int scratch[40];
     unsigned long long key[SKEYS];
-    int fs, nc, novf, Lstar, bin, before, nkey, fallback;
+    int fs, nc, novf, Lstar, bin, before, nkey, fallback, bad;
 };
 
 // Dominance words of the owned columns, NC columns (colsP / NC apart) per
@@ -437,6 +437,8 @@ __global__ void __launch_bounds__(ST, 1) k_small(RunView v, int mode, int C, con
                 sh.nad[lane] = __longlong_as_double((long long)n);
             }
             __syncwarp();
+            const bool inf = __any_sync(0xffffffffu, lane < M && not_finite_key(sf64::bits(sh.nad[lane < M ? lane : 0])));
+            if (lane == 0) sh.bad = inf ? 1 : 0;
             const int er = sh.ext[lane < M ? lane : 0];
             bool ok = __all_sync(0xffffffffu, er >= 0 && er < n2 + (hist ? M : 0));
 #pragma unroll 1
@@ -468,6 +470,10 @@ __global__ void __launch_bounds__(ST, 1) k_small(RunView v, int mode, int C, con
             nm += __popc(T);
         }
         __syncthreads();
+        if (sh.bad) {  // the same in every CTA; no store into a peer since the last cluster barrier
+            if (rank == 0 && tid == 0) set_status(c, DEV_ENONFINITE);
+            return;
+        }
         double* fp = reinterpret_cast<double*>(dyn + L.own);  // colsP x M
         double* nf = fp + colsP * M;
         unsigned long long* bd = reinterpret_cast<unsigned long long*>(nf + colsP);
@@ -622,6 +628,10 @@ __global__ void __launch_bounds__(ST, 1) k_small(RunView v, int mode, int C, con
         __syncthreads();
         for (int p = tid; p < nm; p += ST) {
             const int i = c0 + sh.mem[p];
+            if ((unsigned)bj[p] >= (unsigned)w) {  // no candidate: an invariant failed (not expected)
+                set_status(c, DEV_EINTERNAL);
+                bj[p] = 0;
+            }
             v.pi[i] = bj[p];
             v.dist[i] = __longlong_as_double((long long)bd[p]);
             st_peer(peer(&pi0[i], 0), (uint32_t)bj[p]);

@@ -19,6 +19,13 @@ __device__ __forceinline__ bool key_less(unsigned long long a, int ia, unsigned 
     return a < b || (a == b && ia < ib);
 }
 
+// Whether the largest f~ = f - z* of an objective over T (as its key) says that
+// some member of T, or the ideal point, is not finite: an infinity or a NaN
+// there leaves one in f~, whose key is no finite value's.  The cosines of such
+// a member are NaN, so it has no nearest direction: the selection ends with
+// DEV_ENONFINITE before the association.
+__device__ __forceinline__ bool not_finite_key(unsigned long long k) { return k >= 0x7ff0000000000000ull; }
+
 // The quotients of a chain that runs once: one copy of the code (below).
 __device__ __noinline__ double div_once(double a, double b) { return sf64::div(a, b); }
 
