@@ -201,7 +201,8 @@ nsga3_status nsga3_batch_graph_builds(const nsga3_ctx* ctx, int64_t* builds);
 nsga3_status nsga3_get_population(nsga3_ctx* ctx, float* X, float* F, int32_t* rank, void* stream);
 
 /* Replaces the N parents: X (any, N x d), F (any, N x m), rank (any, N).
- * Any pointer may be NULL to keep the current values.  A parent with an
+ * Any pointer may be NULL to keep the current values.  Infinite objectives
+ * (of an individual that failed, say) compare as values.  A parent with an
  * objective that is not finite has no place among the reference directions: a
  * generation in which one is in a front up to F_l and niching is needed sets
  * NSGA3_ENONFINITE (reported by nsga3_sync) and leaves the population and the

@@ -84,6 +84,7 @@ struct Ctrl {
     int32_t ntask;           // column blocks of k_dominance_front handed out
     int32_t nF0;             // |F_1| by k_dominance_front
     int32_t nrem;            // points left for the matrix (0: the first front holds N)
+    int32_t odd;             // some objective is not finite (runs with a first front)
     unsigned long long domstat[8];  // block pairs of the dominance build by mode (zero, f_0
                                     // one-direction, row-dom-column, column-dom-row, both),
                                     // tiles with nothing to test, (lane, column) pairs

@@ -865,8 +865,10 @@ __global__ void __launch_bounds__(256, M <= 8 ? 5 : 4) k_dominance(RunView v)
 // (broadcast loads) by all columns at once: ceil(m / 2) packed subtractions and as
 // many ORs per row.  The OR of the differences f_j - f_i has its sign bit set
 // iff some f_i > f_j and is zero only for equal vectors, so i dominates j iff
-// it is positive.  Dominated columns leave h at once and the other warps'
-// rows through domw.  Column blocks differ by two orders of magnitude (one
+// it is positive (finite objectives; with one that is not, Ctrl::odd, all
+// points go to the matrix, whose two-sided test gives equal infinities no
+// bit).  Dominated columns leave h at once and the other warps' rows through
+// domw.  Column blocks differ by two orders of magnitude (one
 // near the ideal point meets nothing, one far from it most row blocks): a
 // warp without a block of its own joins one that has units left (fixed
 // segments of row blocks left half the time to the tail at m = 6, N = 60,000,
@@ -898,6 +900,11 @@ __global__ void __launch_bounds__(FW * 32, 3) k_dominance_front(RunView v, int U
     const int lane = lane_id(), warp = threadIdx.x >> 5;
     const uint32_t lt = (1u << lane) - 1u;
     const int nblk = (v.n2 + 31) / 32, nchunk = (nblk + 31) / 32;
+    if (*(volatile const int32_t*)&c->odd) {  // no point in the first front: all are left for the matrix
+        for (int w = blockIdx.x * blockDim.x + threadIdx.x; w < nblk; w += gridDim.x * blockDim.x)
+            v.domw[w] = w * 32 + 32 <= v.n2 ? 0xffffffffu : (1u << (v.n2 - w * 32)) - 1u;
+        return;
+    }
     const float4* Fp4 = reinterpret_cast<const float4*>(v.Fp);
     volatile uint32_t* domw = v.domw;
     volatile int32_t* jpos = v.jpos;
@@ -1101,8 +1108,8 @@ __global__ void __launch_bounds__(1024) k_split_front(RunView v)
         c->nF0 = tot;
         c->nrem = nr;
         c->cum = tot;
-        c->passes = 1;
-        c->passes_total += 1ull;
+        c->passes = tot > 0 ? 1 : 0;
+        c->passes_total += tot > 0 ? 1ull : 0ull;
         if (!rest) {
             c->l = 0;
             c->nFl = tot;
@@ -1110,7 +1117,7 @@ __global__ void __launch_bounds__(1024) k_split_front(RunView v)
             c->K = v.N;
             c->need_niche = v.N < tot ? 1 : 0;
         }
-        if (tot == 0) set_status(c, DEV_EINTERNAL);
+        if (tot == 0 && !c->odd) set_status(c, DEV_EINTERNAL);
     }
 }
 

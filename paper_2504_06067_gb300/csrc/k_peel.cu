@@ -114,8 +114,10 @@ __global__ void __launch_bounds__(PEEL_THREADS, STREAM ? 1 : 2) k_peel(RunView v
     const int tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
     if (read_status(c)) return;  // uniform: set only by earlier kernels
     // the view's points, and the fronts and points before them (rest: the
-    // first front is taken; no rest: it held N points)
-    const int n2 = view_n2(v), before = v.rest ? 1 : 0;
+    // first front is taken, or empty where the matrix is of all points; no
+    // rest: it held N points)
+    const int cum0 = v.rest ? *(volatile const int32_t*)&c->nF0 : 0;
+    const int n2 = view_n2(v), before = cum0 > 0 ? 1 : 0;
     if (n2 == 0) return;
     const int nchunks = v.rest ? (n2 + NSGA3_PEEL_COLS - 1) / NSGA3_PEEL_COLS : v.ld / NSGA3_PEEL_COLS;
     if ((int)blockIdx.x >= nchunks) return;  // owns no columns: nobody waits for it
@@ -133,7 +135,6 @@ __global__ void __launch_bounds__(PEEL_THREADS, STREAM ? 1 : 2) k_peel(RunView v
     __syncthreads();
     // every CTA follows the same sequence of front sizes, so each keeps the
     // pass state itself; CTA 0 also publishes it in ctrl
-    const int cum0 = v.rest ? *(volatile const int32_t*)&c->nF0 : 0;
     int cum = cum0, l = -1, par = 0;
     for (int k = 0;; ++k) {
         // cum: the points ranked before pass k

@@ -131,7 +131,7 @@ struct SmallShared {
 // bounds the loop, so one load serves two columns where they come in pairs.
 // The OR of the differences f_j - f_i has its sign bit set iff some f_i > f_j
 // and is zero only for equal vectors (differences are never -0.0): i
-// dominates j iff it is positive.
+// dominates j iff it is positive.  Finite objectives only.
 template <int M, int NC>
 __device__ __forceinline__ void dominance_words(const float* Fs, uint32_t* dom, int n2, int c0, int colsP)
 {
@@ -169,6 +169,28 @@ __device__ __forceinline__ void dominance_words(const float* Fs, uint32_t* dom, 
         }
 #pragma unroll
         for (int u = 0; u < NC; ++u) dom[I * colsP + cl + u * half] = word[u];
+    }
+}
+
+// The same words where some objective is not finite (a caller's parents; equal
+// infinities differ by NaN): i dominates j iff no f_i > f_j and some f_i < f_j.
+__device__ __noinline__ void dominance_words_any(const float* Fs, uint32_t* dom, int m, int n2, int c0, int colsP)
+{
+    const int NWs = (n2 + 31) / 32, MP = (m + 1) & ~1;
+    for (int t = threadIdx.x; t < NWs * colsP; t += ST) {
+        const int I = t / colsP, cl = t - I * colsP;
+        const float* fj = Fs + min(c0 + cl, n2 - 1) * MP;
+        uint32_t word = 0u;
+        for (int k = 0; k < min(32, n2 - I * 32); ++k) {
+            const float* fi = Fs + (I * 32 + k) * MP;
+            bool greater = false, less = false;
+            for (int q = 0; q < m; ++q) {
+                greater |= fi[q] > fj[q];
+                less |= fi[q] < fj[q];
+            }
+            if (less && !greater) word |= 1u << k;
+        }
+        dom[I * colsP + cl] = word;
     }
 }
 
@@ -211,12 +233,12 @@ __global__ void __launch_bounds__(ST, 1) k_small(RunView v, int mode, int C, con
         cluster_sync();  // merged objectives and rows
     }
     const float* Fg = mode == 0 ? Fin : v.F;
-    bool bad = status != 0;
+    bool odd = status != 0;  // or some objective is not finite
     if (status == 0)
         for (int e = tid; e < n2 * M; e += ST) {
             const int p = e / M, q = e - p * M;
             const float x = __ldcg(Fg + e);
-            bad |= mode == 0 && !isfinite(x);
+            odd |= !isfinite(x);
             Fs[p * MP + q] = x + 0.0f;  // -0.0 as +0.0
         }
     if (M & 1)  // the pad of an odd row
@@ -231,7 +253,8 @@ __global__ void __launch_bounds__(ST, 1) k_small(RunView v, int mode, int C, con
         sh.flag[tid] = 0;
     }
     for (int i = tid; i < n2; i += ST) pi0[i] = -1;
-    if (__syncthreads_or(bad)) {  // the same in every CTA: each reads every objective
+    odd = __syncthreads_or(odd);  // the same in every CTA: each reads every objective
+    if (odd && (mode == 0 || status != 0)) {
         __syncwarp();
         if (mode != 1) cluster_wait();
         if (tid < cols) ranks[c0 + tid] = -1;
@@ -240,7 +263,9 @@ __global__ void __launch_bounds__(ST, 1) k_small(RunView v, int mode, int C, con
     }
 
     // ---- dominance: word I of column j = rows 32 I .. 32 I + 31 that dominate j
-    if (wpc & 1)
+    if (odd)
+        dominance_words_any(Fs, dom, M, n2, c0, colsP);
+    else if (wpc & 1)
         dominance_words<M, 1>(Fs, dom, n2, c0, colsP);
     else
         dominance_words<M, 2>(Fs, dom, n2, c0, colsP);

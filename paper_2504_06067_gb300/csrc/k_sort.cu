@@ -167,6 +167,7 @@ __device__ __forceinline__ void sel_reset(const RunView& v, int tid, int stride)
         c->parr = 0u;
         c->nF0 = 0;
         c->nrem = 0;
+        c->odd = 0;
         c->peel_rows = 0u;
         c->ncand = 0;
         c->nslow = 0;
@@ -252,6 +253,12 @@ __global__ void __launch_bounds__(SB) k_sort_hist(RunView v)
     __syncthreads();
     const int i = blockIdx.x * SB + threadIdx.x;
     if (i < v.n2) {
+        if (v.domw) {  // k_dominance_front's pair test is for finite objectives
+            const float* f = v.F + (size_t)i * v.m;
+            bool odd = false;
+            for (int q = 0; q < v.m; ++q) odd |= !isfinite(f[q]);
+            if (odd) c->odd = 1;
+        }
         const uint32_t key = key_of(v, c, thr, i);
         v.pkey[i] = key;
         atomicAdd(&v.bcnt[key], 1);

@@ -54,3 +54,55 @@ def test_member_to_normalise_is_refused(n, m, d, N, p1, opts, bad):
         r.check(n.nsga3_step(r.ctx, None))
         assert r.sync() == 0 and r.counter() == 3
         assert np.isfinite(r.population()[1]).all()
+
+
+def _parents(kind, N, m, F):
+    """Objectives of N parents, N - 3 of them the given finite ones."""
+    G = F.copy()
+    if kind == "above":  # three equal rows that every finite one dominates
+        G[[1, 4, N - 1]] = np.inf
+    else:  # parents below every child and none of them dominated, so that no niching is needed ...
+        G = wl.objectives("simplex", N, m, seed=7) - np.float32(5.0)
+        G[[1, N - 1]] = -20.0  # ... two equal ones with an infinity
+        G[[1, N - 1], 1] = np.inf
+        if kind == "minus":
+            G[[1, N - 1]] = -3.0
+            G[[1, N - 1], 0] = -np.inf
+    return G
+
+
+# (one cluster: odd and even words per CTA, also with the variation outside)
+SAME = [(3, 8, 100, 12, {}, {"phase_timing": 2}), (3, 8, 100, 12, {"full_sort": 1}, {"full_sort": 1, "phase_timing": 2}),
+        (10, 14, 130, 3, {"full_sort": 1}, {"full_sort": 1, "phase_timing": 2}),
+        (7, 40, 1000, 3, {}, {"phase_timing": 2}),
+        # the first front before the matrix, and the matrix of all points
+        (6, 8, 32768, 3, {}, {"full_sort": 1}), (6, 8, 32790, 3, {"streaming": 1}, {"full_sort": 1})]
+
+
+@pytest.mark.parametrize("m,d,N,p1,opts,general", SAME)
+@pytest.mark.parametrize("kind", ["above", "plus", "minus"])
+def test_infinities_compare_as_values(n, m, d, N, p1, opts, general, kind):
+    """Equal infinities do not make one row dominate another, or itself: the
+    paths with the one-sided pair test against those with the two-sided one."""
+    W = wl.objective_weights(m, 1)
+    with Run(n, m, d, N, p1, seed=3, W=W, **opts) as a, Run(n, m, d, N, p1, seed=3, W=W, **general) as b:
+        out = []
+        for r in (a, b):
+            X, F, rank = _start(n, r)
+            G = _parents(kind, N, m, F)
+            r.set_population(X, G, rank)
+            r.check(n.nsga3_step(r.ctx, None))
+            assert r.sync() == 0
+            out.append(r.population() + r.children())
+            if kind == "above":
+                assert np.isfinite(out[-1][1]).all()
+            else:  # the parents stay, all of them in the first front
+                assert np.array_equal(out[-1][1], G) and (out[-1][2] == 0).all()
+        for x, y in zip(*out):
+            assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan])
+@pytest.mark.parametrize("m,d,N,p1", [(3, 8, 100, 12), (10, 14, 130, 3), (4, 300, 600, 9), (6, 8, 32768, 3)])
+def test_member_to_normalise_is_refused_by_the_other_paths(n, m, d, N, p1, bad):
+    test_member_to_normalise_is_refused(n, m, d, N, p1, {}, bad)
