@@ -326,10 +326,8 @@ __global__ void __launch_bounds__(MT, 1) k_assoc_mma(RunView v)
     volatile int* fail = &s_fail;
     auto wait = [&](unsigned long long* bar, uint32_t n) { return mbar_wait(bar, n & 1u, v.wait_ns, fail); };
     // (after a failed wait: the end of what is in flight, or the limit)
-    auto drain = [&](unsigned long long* bar, uint32_t n) {
-        int none = 0;
-        mbar_wait(bar, n & 1u, v.wait_ns, &none);
-    };
+    int over = 0;  // (one limit for all of a thread's)
+    auto drain = [&](unsigned long long* bar, uint32_t n) { return mbar_wait(bar, n & 1u, v.wait_ns, &over); };
     if (warp == TP / 32 + TILES) {  // loads
         if (lane == 0) {
             uint32_t nload = 0, nitem = 0;
@@ -382,9 +380,18 @@ __global__ void __launch_bounds__(MT, 1) k_assoc_mma(RunView v)
                 }
                 if (ok) mma_commit(&bar_afree);
             }
+            // The commits' arrivals on the barriers land before the CTA, and
+            // the barriers with it, is gone: the accumulators' are waited for
+            // by the maxima, those that free slots and tiles here (each
+            // barrier's last phase; the one before it is over, or the load
+            // that this thread waited for would not have been made).
+            const uint32_t s0 = nstep > RING ? nstep - RING : 0u;
+            if (ok) ok = wait(&bar_afree, nitem - 1);
+            for (uint32_t k = s0; k < nstep && ok; ++k) ok = wait(&bar_bfree[k % RING], k / RING);
             if (!ok) {
                 set_status(c, DEV_ETIMEOUT);
                 for (uint32_t k = nstep > SETS ? nstep - SETS : 0u; k < nstep; ++k) drain(&bar_full[k % SETS][t], k / SETS);
+                for (uint32_t k = s0; k < nstep; ++k) drain(&bar_bfree[k % RING], k / RING);
             }
         }
         __syncwarp();
