@@ -123,7 +123,7 @@ struct SmallShared {
     int ext[NSGA3_FAST_M];
     int scratch[40];
     unsigned long long key[SKEYS];
-    int fs, nc, novf, Lstar, bin, before, nkey, fallback, bad;
+    int fs, nc, novf, Lstar, bin, before, nkey, fallback, bad, longest;
 };
 
 // Dominance words of the owned columns, NC columns (colsP / NC apart) per
@@ -191,6 +191,72 @@ __device__ __noinline__ void dominance_words_any(const float* Fs, uint32_t* dom,
             if (less && !greater) word |= 1u << k;
         }
         dom[I * colsP + cl] = word;
+    }
+}
+
+// The members taken where some reference gives a part of a long list: all of
+// F_l sorted by (reference, nearest first where rho = 0, priority, index),
+// so that a member's place in its reference's order is its position.  Arrays
+// as in the kernel; near_d and near_i (w each) are free, keys has a place per
+// merged individual and may be the distances' own.
+// Bound: the barriers of the sort's 66 steps at 2,048 members (about 10 us).
+// Counting the members before each member, a thread per member, walks the
+// list once per member: quicker while the list's length times a thread's
+// members is below about 400 (SWALK), and 330 us for 2,048 members of one
+// direction.  Selections of N = 1,024, m = 3 whose members share 3 directions
+// (spread, all at one) took 147 and 401 us with it alone, 64 and 64 now; N = 300,
+// m = 3, 3 directions 66 us where all are at one, 33 now.
+constexpr int SWALK = 384;
+
+__device__ __noinline__ void pick_sorted(int n, int w, const int* bkt, const uint32_t* prio, const int* pi, const int* rho,
+                                         const int* off, const int* take, const unsigned long long* dist,
+                                         unsigned long long* near_d, int* near_i, unsigned long long* keys, uint32_t* sel)
+{
+    const int tid = threadIdx.x;
+    for (int j = tid; j < w; j += ST) {
+        near_d[j] = ~0ull;
+        near_i[j] = 0x7fffffff;
+    }
+    __syncthreads();
+    for (int e = tid; e < n; e += ST) {
+        const int i = bkt[e], j = pi[i];
+        // (few of the members of a long list find a smaller distance than they read)
+        if (rho[j] == 0 && dist[i] < *(volatile unsigned long long*)&near_d[j]) atomicMin(&near_d[j], dist[i]);
+    }
+    __syncthreads();
+    for (int e = tid; e < n; e += ST) {
+        const int i = bkt[e], j = pi[i];
+        if (rho[j] == 0 && dist[i] == near_d[j]) atomicMin(&near_i[j], i);
+    }
+    __syncthreads();
+    static_assert(SMALL_N2 <= 2048, "an index takes 11 bits of a key");
+    for (int e = tid; e < n; e += ST) {
+        const int i = bkt[e], j = pi[i];
+        keys[e] = (unsigned long long)j << 44 | (near_i[j] == i ? 0ull : 1ull << 43) | (unsigned long long)prio[e] << 11 | (unsigned)i;
+    }
+    __syncthreads();
+    // bitonic merges whose first step compares mirrored places: every exchange
+    // leaves the smaller key at the lower place, so places past n (the largest
+    // keys) need not exist
+    for (int k = 2; (k >> 1) < n; k <<= 1)
+        for (int o = k >> 1; o > 0; o >>= 1) {
+            for (int t = tid; 2 * (t - (t & (o - 1))) < n; t += ST) {
+                const int a = 2 * t - (t & (o - 1));
+                const int b = o == (k >> 1) ? (a ^ (k - 1)) : a + o;
+                if (b < n) {
+                    const unsigned long long x = keys[a], y = keys[b];
+                    if (y < x) {
+                        keys[a] = y;
+                        keys[b] = x;
+                    }
+                }
+            }
+            __syncthreads();
+        }
+    for (int e = tid; e < n; e += ST) {
+        const unsigned long long key = keys[e];
+        const int j = (int)(key >> 44), i = (int)(key & 2047ull);
+        if (e - off[j] < take[j]) atomicOr(&sel[i >> 5], 1u << (i & 31));
     }
 }
 
@@ -693,8 +759,9 @@ __global__ void __launch_bounds__(ST, 1) k_small(RunView v, int mode, int C, con
             for (int t = tid; t < SBINS; t += ST) bins[t] = 0;
             if (tid == 0) {
                 sh.Lstar = 0x7fffffff;
-                sh.nkey = 0;
+                sh.nkey = sh.longest = 0;
             }
+            const int rounds = (nFl + ST - 1) / ST;  // members per thread
             for (int I = tid; I < NWs; I += ST) sh.sel[I] = sh.S[I];
             __syncthreads();
             for (int i = tid; i < n2; i += ST) {
@@ -773,6 +840,7 @@ __global__ void __launch_bounds__(ST, 1) k_small(RunView v, int mode, int C, con
                 for (int j = lo; j < hi; ++j) {
                     off[j] = run;
                     run += rhop[j];
+                    if (rhop[j] * rounds > SWALK) sh.longest = 1;
                 }
             }
             __syncthreads();
@@ -815,9 +883,18 @@ __global__ void __launch_bounds__(ST, 1) k_small(RunView v, int mode, int C, con
                 prio[e] = mem_prio(v.seed, gen, i);
             }
             __syncthreads();
-            // a member is taken when fewer than take_j of its reference's
+            bool part = false;  // a part of a long list is taken
+            if (sh.longest) {
+                for (int j = tid; j < w; j += ST) part |= take[j] > 0 && take[j] < rhop[j] && rhop[j] * rounds > SWALK;
+                part = __syncthreads_or(part);
+            }
+            if (part) {
+                if (tid == 0) atomicOr(&c->npath, NPATH_LARGE);
+                pick_sorted(nFl, w, bkt, prio, pi0, rho, off, take, dist0, rkey, cur, dist0, sh.sel);
+            }
+            // (else) a member is taken when fewer than take_j of its reference's
             // members come before it (nearest first when rho_j = 0)
-            for (int e = tid; e < nFl; e += ST) {
+            for (int e = part ? nFl : tid; e < nFl; e += ST) {
                 const int i = bkt[e], j = pi0[i];
                 const int tk = take[j], cnt = rhop[j];
                 bool in = tk >= cnt;
