@@ -649,6 +649,152 @@ __global__ void __launch_bounds__(FB) k_assoc_final(RunView v)
     write_assoc(v, c, i, rk, bj, bd);
 }
 
+// The points of the slow list where there are many (m <= 10; objectives of a
+// few values tie with directions of many blocks), GP of them per CTA.  A warp
+// forms the FP32 cosines of GT points with every direction at once, for their
+// maxima and then for the directions within the band of them; f' and |f'| take
+// a thread per point and the FP64 distances a thread per candidate, which the
+// FP64 pipe and the fixed-point quotients serve 32 at a time.  A CTA per point
+// (below) repeats f' in every warp.  Niching of objectives of five values at
+// m = 10, 2N = 66,000, 220 directions: 552 us with a CTA per point, 162 here;
+// at 2N = 10,000, 2,002 directions 461 and 180.
+constexpr int GP = 32;
+constexpr int GT = GP / (AB / 32);
+constexpr int GC = 32;  // candidates of a point; with more, the CTA takes it alone
+
+template <int M>
+struct SlowShared {
+    int j[GP][GC];
+    int n[GP], pt[GP], bj[GP];
+    unsigned long long bd[GP];
+    float thr[GP], u[GP][M];
+    double fp[GP][M], nf[GP];
+};
+
+template <int M>
+__device__ __forceinline__ void assoc_groups(const RunView& v, Ctrl* c, int ns, SlowShared<M>& sh)
+{
+    constexpr int M4 = (M + 3) & ~3;
+    const int tid = threadIdx.x, lane = lane_id(), warp = tid >> 5, w = v.w;
+    for (int g0 = blockIdx.x * GP; g0 < ns; g0 += gridDim.x * GP) {
+        const int np = min(GP, ns - g0);
+        __syncthreads();  // the last group is written
+        if (tid < GP) {
+            sh.pt[tid] = v.slow[min(g0 + tid, ns - 1)];
+            sh.n[tid] = 0;
+            sh.bd[tid] = ~0ull;
+            sh.bj[tid] = 0x7fffffff;
+        }
+        __syncthreads();
+        for (int e = tid; e < GP * M; e += AB) {
+            const int p = e / M, q = e - p * M;
+            sh.u[p][q] = v.uhat[(size_t)sh.pt[p] * M4 + q];
+        }
+        __syncthreads();
+        {
+            float u[GT][M], b[GT];
+#pragma unroll
+            for (int t = 0; t < GT; ++t) {
+                b[t] = 0.0f;
+#pragma unroll
+                for (int q = 0; q < M; ++q) u[t][q] = sh.u[warp * GT + t][q];
+            }
+            auto dots = [&](int j, float (&x)[GT]) {
+                const float4* z4 = reinterpret_cast<const float4*>(v.Zh + (size_t)j * M4);
+                float z[M4];
+#pragma unroll
+                for (int q4 = 0; q4 < M4 / 4; ++q4) {
+                    const float4 y = __ldg(z4 + q4);
+                    z[4 * q4 + 0] = y.x;
+                    z[4 * q4 + 1] = y.y;
+                    z[4 * q4 + 2] = y.z;
+                    z[4 * q4 + 3] = y.w;
+                }
+#pragma unroll
+                for (int t = 0; t < GT; ++t) {
+                    float s = 0.0f;
+#pragma unroll
+                    for (int q = 0; q < M; ++q) s = fmaf(u[t][q], z[q], s);
+                    x[t] = s;
+                }
+            };
+#pragma unroll 4
+            for (int j = lane; j < w; j += 32) {
+                float x[GT];
+                dots(j, x);
+#pragma unroll
+                for (int t = 0; t < GT; ++t) b[t] = fmaxf(b[t], x[t]);
+            }
+#pragma unroll
+            for (int t = 0; t < GT; ++t) {  // cosines are >= 0: their bits order like unsigned ints
+                b[t] = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(b[t]))) - cos_band<M>();
+                if (lane == 0) sh.thr[warp * GT + t] = b[t];
+            }
+#pragma unroll 4
+            for (int j = lane; j < w; j += 32) {
+                float x[GT];
+                dots(j, x);
+#pragma unroll
+                for (int t = 0; t < GT; ++t)
+                    if (x[t] >= b[t]) {
+                        const int e = atomicAdd(&sh.n[warp * GT + t], 1);
+                        if (e < GC) sh.j[warp * GT + t][e] = j;
+                    }
+            }
+        }
+        if (tid < np) {
+            double fp[M];
+            sh.nf[tid] = fprime_of<M>(c, v.F + (size_t)v.Tlist[sh.pt[tid]] * M, fp);
+#pragma unroll
+            for (int q = 0; q < M; ++q) sh.fp[tid][q] = fp[q];
+        }
+        __syncthreads();
+        // distances are >= 0 and order like their bits
+        unsigned long long d[GP * GC / AB];
+#pragma unroll
+        for (int k = 0; k < GP * GC / AB; ++k) {
+            const int p = (tid + k * AB) / GC, e = tid % GC;
+            d[k] = ~0ull;
+            if (p < np && sh.n[p] <= GC && e < sh.n[p]) {
+                const int j = sh.j[p][e];
+                d[k] = sf64::bits(perp_dist(sh.fp[p], sh.nf[p], v.Zd + (size_t)j * M, v.nz[j], M));
+                atomicMin(&sh.bd[p], d[k]);
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < GP * GC / AB; ++k) {
+            const int p = (tid + k * AB) / GC;
+            if (d[k] != ~0ull && d[k] == sh.bd[p]) atomicMin(&sh.bj[p], sh.j[p][tid % GC]);
+        }
+        for (int p = 0; p < np; ++p) {
+            if (sh.n[p] <= GC) continue;  // the same for every thread
+            unsigned long long b = ~0ull;
+            int bj = 0x7fffffff;
+            for (int j = tid; j < w; j += AB) {
+                float x = 0.0f;
+#pragma unroll
+                for (int q = 0; q < M; ++q) x = fmaf(sh.u[p][q], __ldg(v.Zh + (size_t)j * M4 + q), x);
+                if (x < sh.thr[p]) continue;
+                const unsigned long long dj = sf64::bits(perp_dist(sh.fp[p], sh.nf[p], v.Zd + (size_t)j * M, v.nz[j], M));
+                if (dj < b) {  // (j ascends)
+                    b = dj;
+                    bj = j;
+                }
+            }
+            atomicMin(&sh.bd[p], b);
+            __syncthreads();
+            if (b != ~0ull && b == sh.bd[p]) atomicMin(&sh.bj[p], bj);
+        }
+        __syncthreads();
+        if (tid < np) {
+            const int i = v.Tlist[sh.pt[tid]];
+            if (v.arun[sh.pt[tid]].x == -1) atomicAdd(&c->overflow, 1);
+            write_assoc(v, c, i, v.rank2[i], sh.bj[tid], sf64::value(sh.bd[tid]));
+        }
+    }
+}
+
 // One point per CTA over all directions: points whose lists overflowed, and
 // in debug mode every point.  m <= 10: the best FP32 cosine, then the FP64
 // distances of the directions within the band of it (in debug mode and for
@@ -662,6 +808,16 @@ __global__ void __launch_bounds__(AB) k_assoc_slow(RunView v)
     Ctrl* c = v.ctrl;
     if (skip_niche(c)) return;
     const int ns = c->nslow;
+    if constexpr (M > 0) {
+        __shared__ SlowShared<M> sh;
+        // waves of either form times a CTA's time in one: 0.24 us per 256
+        // directions and 4 us, 0.18 us per 32 and 6 us
+        const int grid = gridDim.x, single = (ns + grid - 1) / grid, group = (ns + GP * grid - 1) / (GP * grid);
+        if (!v.debug_recheck_all && (long long)group * (6 * v.w + 6400) < (long long)single * (v.w + 4267)) {
+            assoc_groups<M>(v, c, ns, sh);
+            return;
+        }
+    }
     const int m = M > 0 ? M : v.m;
     const int lane = lane_id(), warp = threadIdx.x >> 5;
     for (int t = blockIdx.x; t < ns; t += gridDim.x) {

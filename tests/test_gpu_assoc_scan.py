@@ -101,6 +101,35 @@ def test_every_direction_agrees(n, orc, m):
         assert _check(orc, a, F, Z, 2)["recheck_miss"] == 0
 
 
+# many points that tie with directions of many blocks: objectives of a few
+# values, with few directions and many
+@pytest.mark.parametrize("m,N,p1", [(2, 1500, 300), (3, 2000, 40), (5, 4000, 8), (7, 2000, 4), (10, 5000, 5), (10, 3000, 2)])
+@pytest.mark.parametrize("kind", ["dups", "grid", "signedzero"])
+def test_many_ties(n, orc, m, N, p1, kind):
+    Z = orc.refdirs(m, p1)
+    F = wl.objectives(kind, 2 * N, m, seed=4)
+    with Run(n, m, m, N, p1, seed=4) as r:
+        st, rank, sel = r.select(F, gen=1)
+        ref = orc.select(F, N, Z, seed=4, gen=1)
+        assert st == 0 and np.array_equal(rank, ref["rank"]) and np.array_equal(sel, ref["selected"])
+        if ref["niche"]:
+            _check(orc, r, F, Z, 1)
+
+
+@pytest.mark.parametrize("k", [151, 153, 2000, 2190])
+def test_more_ties_than_slots(n, orc, k):
+    """k points at the centre, as near to 120 directions, among points near
+    directions: whole and ragged groups."""
+    m, N, p1 = 10, 1100, 3
+    Z = orc.refdirs(m, p1)
+    F = _simplex(2 * N, m, 3)
+    F[:m] = np.eye(m)
+    F[m:m + k] = 1.0 / m
+    F = F[np.random.default_rng(k).permutation(2 * N)].astype(np.float32)
+    with Run(n, m, m, N, p1, seed=4) as r:
+        _check(orc, r, F, Z, 2)
+
+
 @pytest.mark.parametrize("kind", ["late", "early"])
 def test_scale_configuration(n, orc, kind):
     cfg = wl.SCALE
