@@ -29,8 +29,11 @@
 // three fronts: 38 us before, 20 now; the first generation of m = 10,
 // N = 100,000: 342 us before, 128 now.
 // Several chunks per CTA keep the masks of the last seven passes in global
-// memory; a longer ring (16) gave a total order of 200,000 points 2.9 s in
-// place of 3.1 with all its loads in flight, and the knapsack 225 us.
+// memory, and in shared memory the words of those passes that have a few
+// (FEW): a chunk whose pending passes all have few takes its rows from those
+// instead of scanning seven masks.  A total order of 200,000 points: 2.97 s
+// before any deferral, 3.06 with the scans, 1.07 so (100,000 points, m = 3: 612
+// and 337 ms before and so).  A longer ring (16) cost the knapsack 20 us.
 // Without the matrix (STREAM) every chunk is tested every pass: putting the
 // tests off piles them up on the CTAs whose chunks are due (8.6 -> 17.5 ms at
 // m = 3, 2N = 120,000, 32 fronts).
@@ -47,6 +50,7 @@ constexpr int LISTCAP = 2048;
 constexpr int RING = NSGA3_FRONT_RING;
 constexpr int PEEL_U = 4;   // Dom rows in flight per warp
 constexpr int MAXC = 64;  // chunks of a CTA whose state is kept between passes
+constexpr int FEW = 32;   // nonzero words of a pass that are kept beside its mask
 
 // Streaming: the members mk of a front word (rb: SQ x 16 bytes each) against
 // this lane's four columns, with the sign-bit test of the dominance build; a
@@ -109,6 +113,8 @@ __global__ void __launch_bounds__(PEEL_THREADS, STREAM ? 1 : 2) k_peel(RunView v
     __shared__ unsigned s_fs[3];  // size of a pass's front
     __shared__ int s_fail;
     __shared__ int c_min[MAXC], c_eval[MAXC], c_cum[MAXC];  // per chunk: smallest count left, pass of it, points then
+    __shared__ uint2 few[STREAM ? 1 : RING][FEW];  // (several chunks per CTA) the last passes' nonzero words ...
+    __shared__ int nfew[RING];                      // ... and how many; more than FEW: only the masks hold them
     __shared__ float4 rowbuf[STREAM ? PWMAX : 1][32 * SQ];  // streaming: members of a front word
     Ctrl* c = v.ctrl;
     const int tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
@@ -132,6 +138,7 @@ __global__ void __launch_bounds__(PEEL_THREADS, STREAM ? 1 : 2) k_peel(RunView v
     if (tid < 3) s_fs[tid] = 0u;
     if (tid == 0) s_fail = 0;
     if (tid < MAXC) c_min[tid] = INT_MAX;
+    if (tid < RING) nfew[tid] = 0;
     __syncthreads();
     // every CTA follows the same sequence of front sizes, so each keeps the
     // pass state itself; CTA 0 also publishes it in ctrl
@@ -257,7 +264,53 @@ __global__ void __launch_bounds__(PEEL_THREADS, STREAM ? 1 : 2) k_peel(RunView v
                 // dominator block w.  Known before the first Dom load, so the
                 // loads of PEEL_U entries are in flight at once.
                 const unsigned mybit = 1u << (28 + (lane >> 3));
-                for (int wb = 0; wb < lim; wb += LISTCAP) {
+                auto rows = [&](int n) {
+                    if (warp == 0) nrows += (unsigned)n;
+                    for (int e = warp; e < n; e += PEEL_U * PWMAX) {
+                        uint32_t mk[PEEL_U];
+                        uint4 x[PEEL_U];
+#pragma unroll
+                        for (int t = 0; t < PEEL_U; ++t) {
+                            const uint2 L = e + PWMAX * t < n ? list[e + PWMAX * t] : make_uint2(0u, 0u);
+                            mk[t] = L.y;
+                            x[t] = L.x & mybit ? __ldg(base + (size_t)(L.x & 0x0fffffffu) * (NSGA3_PEEL_COLS / 4)) : make_uint4(0u, 0u, 0u, 0u);
+                        }
+#pragma unroll
+                        for (int t = 0; t < PEEL_U; ++t) {
+                            a0 += __popc(x[t].x & mk[t]);
+                            a1 += __popc(x[t].y & mk[t]);
+                            a2 += __popc(x[t].z & mk[t]);
+                            a3 += __popc(x[t].w & mk[t]);
+                        }
+                    }
+                };
+                bool sparse = !own;  // every pending pass has few words: no scan of the masks
+                for (int r = k0; r < k; ++r) sparse = sparse && nfew[r % RING] <= FEW;
+                if (sparse) {
+                    static_assert((RING - 1) * FEW <= PEEL_THREADS, "a thread per word");
+                    const int r = k0 + tid / FEW, e = tid % FEW;
+                    uint2 L = make_uint2(0u, 0u);
+                    if (r < k && e < nfew[r % RING]) L = few[r % RING][e];
+                    bool in = L.y != 0u && (int)L.x < lim;
+                    if (in && nz) {
+                        const unsigned nib = ((unsigned)nz[(size_t)L.x * v.NB8] >> (J0 & 4)) & 15u;
+                        in = nib != 0u;
+                        L.x |= nib << 28;
+                    } else {
+                        L.x |= 15u << 28;
+                    }
+                    const unsigned bal = __ballot_sync(0xffffffffu, in);
+                    if (lane == 0) wcnt[par][warp] = __popc(bal);
+                    __syncthreads();
+                    const int x0 = lane < PWMAX ? wcnt[par][lane] : 0;
+                    const int n = __reduce_add_sync(0xffffffffu, x0);
+                    const int at = __reduce_add_sync(0xffffffffu, lane < warp ? x0 : 0);
+                    par ^= 1;
+                    if (in) list[at + __popc(bal & ((1u << lane) - 1u))] = L;
+                    __syncthreads();
+                    rows(n);
+                }
+                for (int wb = 0; !sparse && wb < lim; wb += LISTCAP) {
                     // the words with members that dominate one of the columns,
                     // a warp's after those of the warps before it (adding up
                     // in one counter took 1 us)
@@ -292,24 +345,7 @@ __global__ void __launch_bounds__(PEEL_THREADS, STREAM ? 1 : 2) k_peel(RunView v
                         at += __popc(bal);
                     }
                     __syncthreads();
-                    if (warp == 0) nrows += (unsigned)n;
-                    for (int e = warp; e < n; e += PEEL_U * PWMAX) {
-                        uint32_t mk[PEEL_U];
-                        uint4 x[PEEL_U];
-#pragma unroll
-                        for (int t = 0; t < PEEL_U; ++t) {
-                            const uint2 L = e + PWMAX * t < n ? list[e + PWMAX * t] : make_uint2(0u, 0u);
-                            mk[t] = L.y;
-                            x[t] = L.x & mybit ? __ldg(base + (size_t)(L.x & 0x0fffffffu) * (NSGA3_PEEL_COLS / 4)) : make_uint4(0u, 0u, 0u, 0u);
-                        }
-#pragma unroll
-                        for (int t = 0; t < PEEL_U; ++t) {
-                            a0 += __popc(x[t].x & mk[t]);
-                            a1 += __popc(x[t].y & mk[t]);
-                            a2 += __popc(x[t].z & mk[t]);
-                            a3 += __popc(x[t].w & mk[t]);
-                        }
-                    }
+                    rows(n);
                     if (wb + LISTCAP < lim) __syncthreads();  // list is reused
                 }
             }
@@ -366,10 +402,18 @@ __global__ void __launch_bounds__(PEEL_THREADS, STREAM ? 1 : 2) k_peel(RunView v
                 const uint32_t x = __ldcg(words + w);
                 if (w < LISTCAP) last[w] = !STREAM && own && !evald ? last[w] | x : x;
                 mine += __popc(x);
+                // (once there are more than FEW the count only has to say so)
+                if (!STREAM && !own && x && *(volatile int*)&nfew[k % RING] <= FEW) {
+                    const int e = atomicAdd(&nfew[k % RING], 1);
+                    if (e < FEW) few[k % RING][e] = make_uint2((unsigned)w, x);
+                }
             }
             mine = __reduce_add_sync(0xffffffffu, mine);
             if (lane == 0 && mine) atomicAdd(&s_fs[k % 3], mine);
-            if (tid == 0) s_fs[(k + 1) % 3] = 0u;  // read two barriers ago
+            if (tid == 0) {
+                s_fs[(k + 1) % 3] = 0u;  // read two barriers ago
+                nfew[(k + 1) % RING] = 0;  // of the pass RING - 1 before this one, which nobody waits for
+            }
         }
         __syncthreads();
         // close front k (the same decision in every CTA)
