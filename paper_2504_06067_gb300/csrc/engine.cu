@@ -55,6 +55,7 @@ struct nsga3_ctx {
     cudaGraphExec_t gx_select = nullptr, gx_step = nullptr;
     cudaStream_t cap = nullptr;
     cudaEvent_t ev[EV_COUNT] = {};
+    cudaEvent_t staged = nullptr;  // after the last use of the staging rows (RunView::Xtmp); null before the first
     int last_kind = 0;  // 1 = select, 2 = step
     long long host_launches = 0;  // kernels launched by calls (peel passes counted on the device)
     DeviceArena* arena = nullptr;  // workspace source (nullptr: one cudaMalloc, carved up)
@@ -789,10 +790,34 @@ nsga3_status copy_out(nsga3_ctx* ctx, PlainCopy* c, const void* src, void* dst, 
     return NSGA3_OK;
 }
 
+// The staging rows are one buffer: a use on another stream than the last one's
+// waits for it (get calls on two streams are independent for their caller).
+// A stream that is being captured is left alone: its work runs when and where
+// the graph is launched.
+bool capturing(cudaStream_t s)
+{
+    cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+    if (s && cudaStreamIsCapturing(s, &c) != cudaSuccess) cudaGetLastError();
+    return c != cudaStreamCaptureStatusNone;
+}
+
+nsga3_status stage_begin(nsga3_ctx* ctx, cudaStream_t s)
+{
+    if (ctx->staged && !capturing(s)) CK(cudaStreamWaitEvent(s, ctx->staged, 0));
+    return NSGA3_OK;
+}
+
+nsga3_status stage_end(nsga3_ctx* ctx, cudaStream_t s)
+{
+    if (capturing(s)) return NSGA3_OK;
+    if (!ctx->staged) CK(cudaEventCreateWithFlags(&ctx->staged, cudaEventDisableTiming));
+    CK(cudaEventRecord(ctx->staged, s));
+    return NSGA3_OK;
+}
+
 // Rows idx[0..N) of X to X (any, or null), objectives and ranks beside them:
 // written by one launch where it can reach them, X through the staging rows
-// otherwise (the copy to pageable memory returns when it is done, so the
-// staging rows are free again).
+// otherwise.
 nsga3_status rows_out(nsga3_ctx* ctx, const int32_t* idx, float* X, const float* Fsrc, float* F, const int32_t* rsrc,
                       int32_t* rank, cudaStream_t s)
 {
@@ -804,10 +829,15 @@ nsga3_status rows_out(nsga3_ctx* ctx, const int32_t* idx, float* X, const float*
         CK(launch_copies(a, b, s));
         return NSGA3_OK;
     }
-    const bool direct = on_device(ctx, X, true);
-    CK(launch_rows_out(ctx->v, idx, direct ? X : ctx->v.Xtmp, a, b, s));
-    if (!direct) CK(cudaMemcpyAsync(X, ctx->v.Xtmp, (size_t)ctx->N * ctx->d * sizeof(float), cudaMemcpyDefault, s));
-    return NSGA3_OK;
+    if (on_device(ctx, X, true)) {
+        CK(launch_rows_out(ctx->v, idx, X, a, b, s));
+        return NSGA3_OK;
+    }
+    st = stage_begin(ctx, s);
+    if (st) return st;
+    CK(launch_rows_out(ctx->v, idx, ctx->v.Xtmp, a, b, s));
+    CK(cudaMemcpyAsync(X, ctx->v.Xtmp, (size_t)ctx->N * ctx->d * sizeof(float), cudaMemcpyDefault, s));
+    return stage_end(ctx, s);
 }
 
 // Checks the arguments of a context and fills its sizes (no device work).
@@ -944,6 +974,7 @@ void ctx_destroy(nsga3_ctx* ctx, bool sync_device)
     if (ctx->gx_step) cudaGraphExecDestroy(ctx->gx_step);
     for (int e = 0; e < EV_COUNT; ++e)
         if (ctx->ev[e]) cudaEventDestroy(ctx->ev[e]);
+    if (ctx->staged) cudaEventDestroy(ctx->staged);
     if (ctx->cap) cudaStreamDestroy(ctx->cap);
     for (void* p : ctx->allocs) {
         if (ctx->arena)
@@ -1242,12 +1273,16 @@ nsga3_status nsga3_set_population(nsga3_ctx* ctx, const float* X, const float* F
     if (!ctx) return fail(ctx, NSGA3_EINVAL, "null context");
     cudaStream_t s = (cudaStream_t)stream;
     if (X) {
-        const float* src = X;
-        if (!on_device(ctx, X, false)) {
+        if (on_device(ctx, X, false)) {
+            CK(launch_rows_in(ctx->v, X, s));
+        } else {
+            nsga3_status st = stage_begin(ctx, s);
+            if (st) return st;
             CK(cudaMemcpyAsync(ctx->v.Xtmp, X, (size_t)ctx->N * ctx->d * sizeof(float), cudaMemcpyDefault, s));
-            src = ctx->v.Xtmp;
+            CK(launch_rows_in(ctx->v, ctx->v.Xtmp, s));
+            st = stage_end(ctx, s);
+            if (st) return st;
         }
-        CK(launch_rows_in(ctx->v, src, s));
     }
     if (F) CK(cudaMemcpyAsync(ctx->v.PF, F, (size_t)ctx->N * ctx->m * sizeof(float), cudaMemcpyDefault, s));
     if (rank) CK(cudaMemcpyAsync(ctx->v.rank, rank, (size_t)ctx->N * sizeof(int32_t), cudaMemcpyDefault, s));
