@@ -764,7 +764,10 @@ nsga3_status device_status(nsga3_ctx* ctx, cudaStream_t s, bool clear)
 
 // Whether kernels of this context's device can use p directly: device
 // memory of that device (or, with pinned, page-locked host memory), aligned
-// to its 4-byte elements.
+// to its 4-byte elements.  Page-locked memory is read and written once, at
+// about the rate of a copy (100,000 rows of 200 419 us, a copy 416; 10,628 of
+// 100 27.2 and 24.5), and X, F and rank take one launch in place of three
+// calls (92 rows of 12: 4.3 us, 10.1 with copies for F and rank).
 bool on_device(const nsga3_ctx* ctx, const void* p, bool pinned)
 {
     if (reinterpret_cast<uintptr_t>(p) & 3) return false;
@@ -777,13 +780,14 @@ bool on_device(const nsga3_ctx* ctx, const void* p, bool pinned)
     return pinned && a.type == cudaMemoryTypeHost && a.devicePointer == p;
 }
 
-// n 4-byte elements from src to dst: into c when a kernel can write dst, by a
-// copy of their own otherwise
-nsga3_status copy_out(nsga3_ctx* ctx, PlainCopy* c, const void* src, void* dst, size_t n, cudaStream_t s)
+// n 4-byte elements from src to dst, one of them the caller's (user; null:
+// nothing to do): into c when a kernel can reach it, by a copy of their own
+// otherwise
+nsga3_status copy_plain(nsga3_ctx* ctx, PlainCopy* c, const void* src, void* dst, const void* user, size_t n, cudaStream_t s)
 {
     *c = PlainCopy{nullptr, nullptr, 0};
-    if (!dst) return NSGA3_OK;
-    if (on_device(ctx, dst, false))
+    if (!user) return NSGA3_OK;
+    if (on_device(ctx, user, true))
         *c = PlainCopy{(const uint32_t*)src, (uint32_t*)dst, (int)n};
     else
         CK(cudaMemcpyAsync(dst, src, n * 4, cudaMemcpyDefault, s));
@@ -822,8 +826,8 @@ nsga3_status rows_out(nsga3_ctx* ctx, const int32_t* idx, float* X, const float*
                       int32_t* rank, cudaStream_t s)
 {
     PlainCopy a, b;
-    nsga3_status st = copy_out(ctx, &a, Fsrc, F, (size_t)ctx->N * ctx->m, s);
-    if (!st) st = copy_out(ctx, &b, rsrc, rank, (size_t)ctx->N, s);
+    nsga3_status st = copy_plain(ctx, &a, Fsrc, F, F, (size_t)ctx->N * ctx->m, s);
+    if (!st) st = copy_plain(ctx, &b, rsrc, rank, rank, (size_t)ctx->N, s);
     if (st) return st;
     if (!X) {
         CK(launch_copies(a, b, s));
@@ -1124,8 +1128,8 @@ nsga3_status nsga3_select(nsga3_ctx* ctx, const float* objs, int32_t* ranks, int
     if (!ctx || !objs || !ranks || !selected) return fail(ctx, NSGA3_EINVAL, "null argument");
     cudaStream_t s = (cudaStream_t)stream;
     if (ctx->small) {
-        // device buffers are read and written by the launch itself
-        const bool of = on_device(ctx, objs, false), ok = on_device(ctx, ranks, false), os = on_device(ctx, selected, false);
+        // device buffers are read and written by the launch itself, page-locked ones written
+        const bool of = on_device(ctx, objs, false), ok = on_device(ctx, ranks, true), os = on_device(ctx, selected, true);
         if (!of) CK(cudaMemcpyAsync(ctx->vs.F, objs, (size_t)ctx->n2 * ctx->m * sizeof(float), cudaMemcpyDefault, s));
         CK(launch_small(ctx->vs, 0, of ? objs : ctx->vs.F, ok ? ranks : ctx->vs.rank2, os ? selected : ctx->vs.sel, s));
         if (!ok) CK(cudaMemcpyAsync(ranks, ctx->vs.rank2, (size_t)ctx->n2 * sizeof(int32_t), cudaMemcpyDefault, s));
@@ -1147,8 +1151,8 @@ nsga3_status nsga3_select(nsga3_ctx* ctx, const float* objs, int32_t* ranks, int
     }
     ctx->host_launches += select_launches(ctx);
     PlainCopy a, b;
-    nsga3_status st = copy_out(ctx, &a, ctx->vs.rank2, ranks, (size_t)ctx->n2, s);
-    if (!st) st = copy_out(ctx, &b, ctx->vs.sel, selected, (size_t)ctx->N, s);
+    nsga3_status st = copy_plain(ctx, &a, ctx->vs.rank2, ranks, ranks, (size_t)ctx->n2, s);
+    if (!st) st = copy_plain(ctx, &b, ctx->vs.sel, selected, selected, (size_t)ctx->N, s);
     if (st) return st;
     CK(launch_copies(a, b, s));
     ctx->last_kind = 1;
@@ -1272,21 +1276,23 @@ nsga3_status nsga3_set_population(nsga3_ctx* ctx, const float* X, const float* F
 {
     if (!ctx) return fail(ctx, NSGA3_EINVAL, "null context");
     cudaStream_t s = (cudaStream_t)stream;
-    if (X) {
-        if (on_device(ctx, X, false)) {
-            CK(launch_rows_in(ctx->v, X, s));
-        } else {
-            nsga3_status st = stage_begin(ctx, s);
-            if (st) return st;
-            CK(cudaMemcpyAsync(ctx->v.Xtmp, X, (size_t)ctx->N * ctx->d * sizeof(float), cudaMemcpyDefault, s));
-            CK(launch_rows_in(ctx->v, ctx->v.Xtmp, s));
-            st = stage_end(ctx, s);
-            if (st) return st;
-        }
+    PlainCopy a, b;
+    nsga3_status st = copy_plain(ctx, &a, F, ctx->v.PF, F, (size_t)ctx->N * ctx->m, s);
+    if (!st) st = copy_plain(ctx, &b, rank, ctx->v.rank, rank, (size_t)ctx->N, s);
+    if (st) return st;
+    if (!X) {
+        CK(launch_copies(a, b, s));
+        return NSGA3_OK;
     }
-    if (F) CK(cudaMemcpyAsync(ctx->v.PF, F, (size_t)ctx->N * ctx->m * sizeof(float), cudaMemcpyDefault, s));
-    if (rank) CK(cudaMemcpyAsync(ctx->v.rank, rank, (size_t)ctx->N * sizeof(int32_t), cudaMemcpyDefault, s));
-    return NSGA3_OK;
+    if (on_device(ctx, X, true)) {
+        CK(launch_rows_in(ctx->v, X, a, b, s));
+        return NSGA3_OK;
+    }
+    st = stage_begin(ctx, s);
+    if (st) return st;
+    CK(cudaMemcpyAsync(ctx->v.Xtmp, X, (size_t)ctx->N * ctx->d * sizeof(float), cudaMemcpyDefault, s));
+    CK(launch_rows_in(ctx->v, ctx->v.Xtmp, a, b, s));
+    return stage_end(ctx, s);
 }
 
 nsga3_status nsga3_get_children(nsga3_ctx* ctx, float* X, float* F, void* stream)

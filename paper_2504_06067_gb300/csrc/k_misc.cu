@@ -216,8 +216,12 @@ __global__ void __launch_bounds__(256) k_rows_out(RunView v, const int32_t* idx,
 // new parents take the rows of the last variation's parents, so that its
 // children stay readable; the next children take the last ones' rows
 template <class T>
-__global__ void __launch_bounds__(256) k_rows_in(RunView v, const T* src, int words)
+__global__ void __launch_bounds__(256) k_rows_in(RunView v, const T* src, int words, int ctas, PlainCopy a, PlainCopy b)
 {
+    if ((int)blockIdx.x >= ctas) {
+        plain_copy((int)blockIdx.x - ctas, a, b);
+        return;
+    }
     constexpr int R = row_words<T>();
     for_row_words<T, R>(v.N, words, [&](T(&x)[R], int(&p)[R], int(&q)[R]) {
 #pragma unroll
@@ -327,10 +331,12 @@ static cudaError_t rows_out(const RunView& v, const int32_t* idx, float* dst, Pl
 }
 
 template <class T>
-static cudaError_t rows_in(const RunView& v, const float* src, cudaStream_t s)
+static cudaError_t rows_in(const RunView& v, const float* src, PlainCopy a, PlainCopy b, cudaStream_t s)
 {
     const int words = v.d * 4 / (int)sizeof(T);
-    k_rows_in<T><<<row_ctas<T>(v.N, words), 256, 0, s>>>(v, reinterpret_cast<const T*>(src), words);
+    const unsigned ctas = row_ctas<T>(v.N, words);
+    k_rows_in<T><<<ctas + plain_ctas(a) + plain_ctas(b), 256, 0, s>>>(v, reinterpret_cast<const T*>(src), words, (int)ctas, a,
+                                                                      b);
     return cudaGetLastError();
 }
 
@@ -349,11 +355,11 @@ cudaError_t launch_copies(PlainCopy a, PlainCopy b, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_rows_in(const RunView& v, const float* src, cudaStream_t s)
+cudaError_t launch_rows_in(const RunView& v, const float* src, PlainCopy a, PlainCopy b, cudaStream_t s)
 {
     const int bytes = word_bytes(v.d, src);
-    if (bytes == 16) return rows_in<float4>(v, src, s);
-    return bytes == 8 ? rows_in<float2>(v, src, s) : rows_in<float>(v, src, s);
+    if (bytes == 16) return rows_in<float4>(v, src, a, b, s);
+    return bytes == 8 ? rows_in<float2>(v, src, a, b, s) : rows_in<float>(v, src, a, b, s);
 }
 
 cudaError_t launch_slots_init(const RunView& v, cudaStream_t s)

@@ -72,7 +72,7 @@ cudaError_t launch_mark(const RunView& v, cudaStream_t s);
 cudaError_t launch_select_out(const RunView& v, cudaStream_t s);
 cudaError_t launch_gather(const RunView& v, cudaStream_t s);
 // rows of X to dst (row r of dst = row idx[r] of X) and up to two plain copies
-// (n = 0: none) in the same launch; plain copies alone; rows back
+// (n = 0: none) in the same launch; plain copies alone; rows back, likewise
 struct PlainCopy {
     const uint32_t* src;
     uint32_t* dst;
@@ -80,7 +80,7 @@ struct PlainCopy {
 };
 cudaError_t launch_rows_out(const RunView& v, const int32_t* idx, float* dst, PlainCopy a, PlainCopy b, cudaStream_t s);
 cudaError_t launch_copies(PlainCopy a, PlainCopy b, cudaStream_t s);
-cudaError_t launch_rows_in(const RunView& v, const float* src, cudaStream_t s);
+cudaError_t launch_rows_in(const RunView& v, const float* src, PlainCopy a, PlainCopy b, cudaStream_t s);
 cudaError_t launch_slots_init(const RunView& v, cudaStream_t s);
 
 // issue-rate probe of the dominance test's FADD / LOP3 mix (k_probe.cu)
