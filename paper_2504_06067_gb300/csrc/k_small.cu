@@ -123,7 +123,7 @@ struct SmallShared {
     int ext[NSGA3_FAST_M];
     int scratch[40];
     unsigned long long key[SKEYS];
-    int fs, nc, novf, Lstar, bin, before, nkey, fallback, bad, longest;
+    int fs, nc, novf, Lstar, bin, before, nkey, fallback, longest;
 };
 
 // Dominance words of the owned columns, NC columns (colsP / NC apart) per
@@ -299,14 +299,14 @@ __global__ void __launch_bounds__(ST, 1) k_small(RunView v, int mode, int C, con
         cluster_sync();  // merged objectives and rows
     }
     const float* Fg = mode == 0 ? Fin : v.F;
-    bool odd = status != 0;  // or some objective is not finite
-    if (status == 0)
-        for (int e = tid; e < n2 * M; e += ST) {
-            const int p = e / M, q = e - p * M;
-            const float x = __ldcg(Fg + e);
-            odd |= !isfinite(x);
-            Fs[p * MP + q] = x + 0.0f;  // -0.0 as +0.0
-        }
+    bool odd = false;  // some objective is not finite, or status (whose load these do not wait for)
+    for (int e = tid; e < n2 * M; e += ST) {
+        const int p = e / M, q = e - p * M;
+        const float x = __ldcg(Fg + e);
+        odd |= !isfinite(x);
+        Fs[p * MP + q] = x + 0.0f;  // -0.0 as +0.0
+    }
+    odd |= status != 0;
     if (M & 1)  // the pad of an odd row
         for (int p = tid; p < n2; p += ST) Fs[p * MP + M] = 0.0f;
     if (tid < NWs) {
@@ -329,7 +329,7 @@ __global__ void __launch_bounds__(ST, 1) k_small(RunView v, int mode, int C, con
     }
 
     // ---- dominance: word I of column j = rows 32 I .. 32 I + 31 that dominate j
-    if (odd)
+    if (__builtin_expect(odd, 0))
         dominance_words_any(Fs, dom, M, n2, c0, colsP);
     else if (wpc & 1)
         dominance_words<M, 1>(Fs, dom, n2, c0, colsP);
@@ -358,18 +358,17 @@ __global__ void __launch_bounds__(ST, 1) k_small(RunView v, int mode, int C, con
                 if (lane < C && wd < NWs) st_peer(peer(&sh.front[k & 1][wd], lane), word);
             }
             cluster_sync();
-            if (warp == 0) {
-                int s = 0;
-                for (int I = lane; I < NWs; I += 32) {
-                    const uint32_t f = sh.front[k & 1][I];
-                    sh.rem[I] &= ~f;
-                    s += __popc(f);
-                }
-                s = warp_sum(s);
-                if (lane == 0) sh.fs = s;
+            // every warp counts the front and takes it out of rem for itself
+            // (all write the same words, so none waits for another)
+            int fs = 0;
+            for (int I = lane; I < NWs; I += 32) {
+                const uint32_t f = sh.front[k & 1][I];
+                sh.rem[I] &= ~f;
+                fs += __popc(f);
             }
-            __syncthreads();
-            const int fs = sh.fs, ncum = cum + fs;
+            fs = __reduce_add_sync(0xffffffffu, fs);
+            __syncwarp();  // rem is read by other lanes
+            const int ncum = cum + fs;
             const bool first = l < 0 && ncum >= N;
             if (l < 0) {  // S: fronts before the selecting one, F_l: that one
                 for (int I = tid; I < NWs; I += ST) {
@@ -414,6 +413,21 @@ __global__ void __launch_bounds__(ST, 1) k_small(RunView v, int mode, int C, con
         c->domstat[7] = c->domstat[6];
     }
     if (niche) {
+        if (__builtin_expect(odd, 0)) {
+            // a member of T that is not finite (a NaN anywhere would enter the
+            // running ideal point) ends the selection, as not_finite_key does
+            // on the general path; no store into a peer is under way
+            bool bad = false;
+            for (int e = tid; e < n2 * M; e += ST) {
+                const int p = e / M;
+                const float x = Fs[p * MP + e - p * M];
+                bad |= (((sh.S[p >> 5] | sh.Fl[p >> 5]) >> (p & 31)) & 1u) ? !isfinite(x) : v.norm_history && isnan(x);
+            }
+            if (__syncthreads_or(bad)) {  // the same in every CTA
+                if (rank == 0 && tid == 0) set_status(c, DEV_ENONFINITE);
+                return;
+            }
+        }
         // ---- ideal point: a warp per objective, every CTA for itself
         const bool hist = v.norm_history && c->hvalid;
         if (warp < M) {
@@ -528,8 +542,6 @@ __global__ void __launch_bounds__(ST, 1) k_small(RunView v, int mode, int C, con
                 sh.nad[lane] = __longlong_as_double((long long)n);
             }
             __syncwarp();
-            const bool inf = __any_sync(0xffffffffu, lane < M && not_finite_key(sf64::bits(sh.nad[lane < M ? lane : 0])));
-            if (lane == 0) sh.bad = inf ? 1 : 0;
             const int er = sh.ext[lane < M ? lane : 0];
             bool ok = __all_sync(0xffffffffu, er >= 0 && er < n2 + (hist ? M : 0));
 #pragma unroll 1
@@ -561,10 +573,6 @@ __global__ void __launch_bounds__(ST, 1) k_small(RunView v, int mode, int C, con
             nm += __popc(T);
         }
         __syncthreads();
-        if (sh.bad) {  // the same in every CTA; no store into a peer since the last cluster barrier
-            if (rank == 0 && tid == 0) set_status(c, DEV_ENONFINITE);
-            return;
-        }
         double* fp = reinterpret_cast<double*>(dyn + L.own);  // colsP x M
         double* nf = fp + colsP * M;
         unsigned long long* bd = reinterpret_cast<unsigned long long*>(nf + colsP);
@@ -719,13 +727,11 @@ __global__ void __launch_bounds__(ST, 1) k_small(RunView v, int mode, int C, con
         __syncthreads();
         for (int p = tid; p < nm; p += ST) {
             const int i = c0 + sh.mem[p];
-            if ((unsigned)bj[p] >= (unsigned)w) {  // no candidate: an invariant failed (not expected)
-                set_status(c, DEV_EINTERNAL);
-                bj[p] = 0;
-            }
-            v.pi[i] = bj[p];
+            // (finite members have a candidate; the bound keeps every index in range regardless)
+            const int j = (int)min((unsigned)bj[p], (unsigned)(w - 1));
+            v.pi[i] = j;
             v.dist[i] = __longlong_as_double((long long)bd[p]);
-            st_peer(peer(&pi0[i], 0), (uint32_t)bj[p]);
+            st_peer(peer(&pi0[i], 0), (uint32_t)j);
             st_peer(peer(&dist0[i], 0), bd[p]);
         }
         cluster_sync();
@@ -823,24 +829,25 @@ __global__ void __launch_bounds__(ST, 1) k_small(RunView v, int mode, int C, con
             __syncthreads();
             {
                 static_assert(SBINS == ST, "a bin per thread");
-                const int x = bins[tid];
-                int total;
-                const int run = block_excl_scan(x, sh.scratch, &total);
-                if (run < r && r <= run + x) {
-                    sh.bin = tid;
-                    sh.before = run;
-                }
-            }
-            // offsets of the references' member lists
-            {
+                static_assert(SMALL_W < 65536 && SMALL_N2 < 32768, "both sums in one scan");
+                // and the offsets of the references' member lists
                 const int per = (w + ST - 1) / ST, lo = min(w, tid * per), hi = min(w, lo + per);
-                int s = 0, total;
-                for (int j = lo; j < hi; ++j) s += rhop[j];
-                int run = block_excl_scan(s, sh.scratch, &total);
+                const int x = bins[tid];
+                int s = 0, most = 0, total;
+                for (int j = lo; j < hi; ++j) {
+                    s += rhop[j];
+                    most = max(most, rhop[j]);
+                }
+                if (most * rounds > SWALK) sh.longest = 1;
+                const int sums = block_excl_scan(x | (s << 16), sh.scratch, &total), before = sums & 0xffff;
+                if (before < r && r <= before + x) {
+                    sh.bin = tid;
+                    sh.before = before;
+                }
+                int run = sums >> 16;
                 for (int j = lo; j < hi; ++j) {
                     off[j] = run;
                     run += rhop[j];
-                    if (rhop[j] * rounds > SWALK) sh.longest = 1;
                 }
             }
             __syncthreads();
@@ -884,11 +891,11 @@ __global__ void __launch_bounds__(ST, 1) k_small(RunView v, int mode, int C, con
             }
             __syncthreads();
             bool part = false;  // a part of a long list is taken
-            if (sh.longest) {
+            if (__builtin_expect(sh.longest, 0)) {
                 for (int j = tid; j < w; j += ST) part |= take[j] > 0 && take[j] < rhop[j] && rhop[j] * rounds > SWALK;
                 part = __syncthreads_or(part);
             }
-            if (part) {
+            if (__builtin_expect(part, 0)) {
                 if (tid == 0) atomicOr(&c->npath, NPATH_LARGE);
                 pick_sorted(nFl, w, bkt, prio, pi0, rho, off, take, dist0, rkey, cur, dist0, sh.sel);
             }

@@ -103,6 +103,7 @@ def test_infinities_compare_as_values(n, m, d, N, p1, opts, general, kind):
 
 
 @pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan])
-@pytest.mark.parametrize("m,d,N,p1", [(3, 8, 100, 12), (10, 14, 130, 3), (4, 300, 600, 9), (6, 8, 32768, 3)])
-def test_member_to_normalise_is_refused_by_the_other_paths(n, m, d, N, p1, bad):
-    test_member_to_normalise_is_refused(n, m, d, N, p1, {}, bad)
+@pytest.mark.parametrize("m,d,N,p1,opts", [(3, 8, 100, 12, {}), (10, 14, 130, 3, {"norm_history": 1}), (4, 300, 600, 9, {}),
+                                           (6, 8, 32768, 3, {})])
+def test_member_to_normalise_is_refused_by_the_other_paths(n, m, d, N, p1, opts, bad):
+    test_member_to_normalise_is_refused(n, m, d, N, p1, opts, bad)
