@@ -931,6 +931,12 @@ nsga3_status ctx_create(int m, int d, int N, int ref_divisions, const nsga3_opts
         }
     }
     if (!st) st = init_attributes(ctx);
+    // a device whose SMs are shared out may have no room for a cluster of 16:
+    // small populations then take the general path, and the elimination of
+    // m > 32 has no other form
+    if (!st && ctx->small) ctx->small = small_fits(ctx->m, ctx->n2, ctx->w);
+    if (!st && !solve_fits(ctx->m))
+        st = fail(ctx, NSGA3_ECUDA, "the device has no room for the cluster of CTAs that %d objectives take", ctx->m);
     if (!st) st = setup(ctx);
     ctx->opts.W = nullptr;
     if (st) {

@@ -784,6 +784,22 @@ cudaError_t launch_norm_ideal(const RunView& v, cudaStream_t s)
     return cudaGetLastError();
 }
 
+// the one cluster of the elimination
+static cudaLaunchConfig_t sc_config(int m, cudaLaunchAttribute* attr, cudaStream_t s)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(sc_ctas(m));
+    cfg.blockDim = dim3(SC_T);
+    cfg.dynamicSmemBytes = sc_bytes(m);
+    cfg.stream = s;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = sc_ctas(m);
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
 static cudaError_t launch_norm_extreme_gen(const RunView& v, int num_sms, cudaStream_t s)
 {
     if (v.m <= NSGA3_FAST_M || v.m > NSGA3_MAX_M) return cudaErrorInvalidValue;
@@ -806,19 +822,20 @@ static cudaError_t launch_norm_extreme_gen(const RunView& v, int num_sms, cudaSt
     k_ext_reduce<<<(v.m + 7) / 8, 256, 0, s>>>(v, parts);
     e = cudaGetLastError();
     if (e != cudaSuccess || v.m <= NSGA3_WARP_M) return e;
-    const int C = sc_ctas(v.m);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(C);
-    cfg.blockDim = dim3(SC_T);
-    cfg.dynamicSmemBytes = sc_bytes(v.m);
-    cfg.stream = s;
     cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = C;
-    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_solve_cluster, v, C);
+    const cudaLaunchConfig_t cfg = sc_config(v.m, attr, s);
+    return cudaLaunchKernelEx(&cfg, k_solve_cluster, v, sc_ctas(v.m));
+}
+
+bool solve_fits(int m)
+{
+    if (m <= NSGA3_WARP_M) return true;
+    cudaLaunchAttribute attr[1];
+    const cudaLaunchConfig_t cfg = sc_config(m, attr, nullptr);
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, k_solve_cluster, &cfg) == cudaSuccess) return n > 0;
+    cudaGetLastError();
+    return false;
 }
 
 cudaError_t norm_init_attributes()

@@ -1010,22 +1010,41 @@ int small_ctas(int n2)
     return NWs > 4 ? 8 : NWs > 2 ? 4 : NWs > 1 ? 2 : 1;
 }
 
+// the one cluster of a launch
+template <int M>
+struct SmallConfig {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    const int C;
+    SmallConfig(int n2, int w, cudaStream_t s) : C(small_ctas(n2))
+    {
+        cfg.gridDim = dim3(C);
+        cfg.blockDim = dim3(ST);
+        cfg.dynamicSmemBytes = small_layout<M>(n2, w, C).bytes;
+        cfg.stream = s;
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = C;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+    }
+};
+
 template <int M>
 cudaError_t launch_m(const RunView& v, int mode, const float* F, int32_t* ranks, int32_t* sel, cudaStream_t s)
 {
-    const int C = small_ctas(v.n2);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(C);
-    cfg.blockDim = dim3(ST);
-    cfg.dynamicSmemBytes = small_layout<M>(v.n2, v.w, C).bytes;
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = C;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_small<M>, v, mode, C, F, ranks, sel);
+    const SmallConfig<M> c(v.n2, v.w, s);
+    return cudaLaunchKernelEx(&c.cfg, k_small<M>, v, mode, c.C, F, ranks, sel);
+}
+
+template <int M>
+bool fits_m(int n2, int w)
+{
+    const SmallConfig<M> c(n2, w, nullptr);
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, k_small<M>, &c.cfg) == cudaSuccess) return n > 0;
+    cudaGetLastError();
+    return false;
 }
 
 template <int M>
@@ -1052,6 +1071,22 @@ cudaError_t launch_small(const RunView& v, int mode, const float* F, int32_t* ra
     case 9: return launch_m<9>(v, mode, F, ranks, sel, s);
     case 10: return launch_m<10>(v, mode, F, ranks, sel, s);
     default: return cudaErrorInvalidValue;
+    }
+}
+
+bool small_fits(int m, int n2, int w)
+{
+    switch (m) {
+    case 2: return fits_m<2>(n2, w);
+    case 3: return fits_m<3>(n2, w);
+    case 4: return fits_m<4>(n2, w);
+    case 5: return fits_m<5>(n2, w);
+    case 6: return fits_m<6>(n2, w);
+    case 7: return fits_m<7>(n2, w);
+    case 8: return fits_m<8>(n2, w);
+    case 9: return fits_m<9>(n2, w);
+    case 10: return fits_m<10>(n2, w);
+    default: return false;
     }
 }
 

@@ -21,6 +21,10 @@ cudaError_t launch_vary_eval(const RunView& v, cudaStream_t s);
 #define SMALL_W 2048   // reference directions at most
 cudaError_t launch_small(const RunView& v, int mode, const float* F, int32_t* ranks, int32_t* sel, cudaStream_t s);
 cudaError_t small_init_attributes();
+// whether the device has room for that cluster (after small_init_attributes),
+// and for the one of the elimination (m > 32; after norm_init_attributes)
+bool small_fits(int m, int n2, int w);
+bool solve_fits(int m);
 
 // selection (Alg. 1 sort / Alg. 2)
 // 0-1 knapsack workload (k_knapsack.cu): bits + repair + objectives
