@@ -888,7 +888,11 @@ constexpr int FW = 8;        // warps per CTA
 constexpr int RBUF = 64;     // buffered rows per warp
 constexpr int RFULL = 32;    // rows at which a buffer is tested
 constexpr int PROBES = 6;    // looks for units left before a warp ends
-constexpr int JDONE = 1 << 28;
+constexpr int UB_MAX = 128;       // row blocks per unit at most
+constexpr int JDONE = 1 << 23;    // units handed out of a block that is done
+// no block has JDONE units, and JDONE and the units that joining warps still
+// take after it stay in range as row blocks
+static_assert((1 << 21) / 32 < JDONE && (JDONE + (1 << 20)) <= 0x7fffffff / UB_MAX, "units past the end");
 
 template <int M>
 __global__ void __launch_bounds__(FW * 32, 3) k_dominance_front(RunView v, int UB)
@@ -1330,7 +1334,7 @@ cudaError_t launch_front_m(const RunView& v, cudaStream_t s)
     }
     // every resident warp; units of 32 row blocks, more where a column block
     // has many
-    const int nblk = (v.n2 + 31) / 32, UB = nblk < 4096 ? 32 : 128;
+    const int nblk = (v.n2 + 31) / 32, UB = nblk < 4096 ? 32 : UB_MAX;
     k_dominance_front<M><<<(unsigned)((occ > 0 ? occ : 2) * v.num_sms), FW * 32, 0, s>>>(v, UB);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
