@@ -82,13 +82,12 @@ namespace {
 
 // Small populations take one launch of one cluster (k_small.cu) instead of
 // the 20 kernels of the general path.  Not with options that belong to the
-// general path's kernels: timed phases, launch shapes, the FP64 recheck, a
-// forced association.
+// general path's kernels: timed phases, launch shapes, the FP64 recheck.
 bool small_wanted(const nsga3_ctx* ctx)
 {
     const nsga3_opts& o = ctx->opts;
     return ctx->m <= NSGA3_FAST_M && ctx->n2 <= SMALL_N2 && ctx->w <= SMALL_W && !ctx->eager && ctx->ev_mask == 0u &&
-           !o.debug_recheck_all && o.dom_ctas_per_sm == 0 && o.peel_ctas_per_sm == 0 && !getenv("NSGA3_ASSOC");
+           !o.debug_recheck_all && o.dom_ctas_per_sm == 0 && o.peel_ctas_per_sm == 0;
 }
 
 // ... and the variation inside that launch while its N d / 2 pair-variables
@@ -633,7 +632,10 @@ nsga3_status setup_alloc(nsga3_ctx* ctx)
 
 nsga3_status setup(nsga3_ctx* ctx)
 {
-    // a limit of the interface: m <= 10 took up to 220 KB of block tables
+    // A limit of the interface: with m <= 10 a context took as many directions
+    // as 220 KB of block tables hold.  The association's scan, which has no such
+    // tables, packs block numbers into 16 bits: the limit keeps it in range.
+    static_assert((220 * 1024 - 4096) / ((4 + 10) * 4) <= 65536, "blocks of 32 directions");
     if (ctx->m <= NSGA3_FAST_M && (size_t)((ctx->w + 31) / 32) * (ctx->M4 + 10) * 4 + 4096 > 220 * 1024)
         return fail(ctx, NSGA3_EINVAL, "%d reference directions exceed the association's limit", ctx->w);
     if (!ctx->arena) {

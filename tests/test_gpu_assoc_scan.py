@@ -101,6 +101,27 @@ def test_every_direction_agrees(n, orc, m):
         assert _check(orc, a, F, Z, 2)["recheck_miss"] == 0
 
 
+def test_no_variable_chooses_the_path(n, monkeypatch):
+    import ctypes as C
+    k = C.c_int32()
+    monkeypatch.setenv("NSGA3_ASSOC", "tile")
+    with Run(n, 3, 3, 92, 12, seed=4) as r:
+        r.select(wl.objectives("late", 184, 3, seed=1))
+        r.check(n.nsga3_last_launches(r.ctx, C.byref(k)))
+        assert k.value == 1  # the one cluster of small populations
+
+
+def test_limit_of_directions(n):
+    """m = 2: 126,368 directions are taken, one more is refused."""
+    most = (220 * 1024 - 4096) // ((4 + 10) * 4) * 32
+    with Run(n, 2, 2, 100, most - 1, seed=1, phase_timing=2) as r:
+        assert r.w == most
+        st, rank, sel = r.select(wl.objectives("late", 200, 2, seed=1))
+        assert st == 0
+    with pytest.raises(Exception):
+        Run(n, 2, 2, 100, most, seed=1, phase_timing=2)
+
+
 # many points that tie with directions of many blocks: objectives of a few
 # values, with few directions and many
 @pytest.mark.parametrize("m,N,p1", [(2, 1500, 300), (3, 2000, 40), (5, 4000, 8), (7, 2000, 4), (10, 5000, 5), (10, 3000, 2)])
