@@ -257,7 +257,12 @@ nsga3_status nsga3_get_selection_info(nsga3_ctx* ctx, int32_t* info);
 nsga3_status nsga3_get_selection_paths(nsga3_ctx* ctx, uint32_t* paths);
 
 /* Work of the dominance build in the last selection (synchronous;
- * diagnostics, m <= 10, zeros above): stats[0..7] = block pairs (32 x 32
+ * diagnostics, m <= 10, zeros above).  Populations of one cluster test all
+ * pairs both ways.  Where the first front is found before the matrix (2N from
+ * 65,536 and m from 5 on), the pairs are those of the points it leaves, and
+ * its own work is added: the row blocks it met per column block to stats[2],
+ * its (row, column) tests and those of live columns to stats[6] and [7].
+ * stats[0..7] = block pairs (32 x 32
  * points, upper triangle) ruled out without a test, tested in one direction
  * with objectives 1..m-1 (every row f_0 below every column f_0), tested in
  * the "row dominates column" direction only, in the "column dominates row"

@@ -369,7 +369,12 @@ __device__ __forceinline__ void red_release(unsigned* p, unsigned x)
 // Polls `done` until it returns true or wait_ns of device time have passed
 // (the clock is read every 1,024 polls; the poll count caps the wait too,
 // should the timer not advance); on expiry records DEV_ETIMEOUT and returns
-// false.  Every device-side wait goes through it.
+// false.  The grid barriers and the wait probe go through it; the waits on
+// mbarriers have the same budget (mbar_wait in k_associate.cu).  Two waits of
+// the hardware have no limit and need none: a cluster barrier, whose CTAs run
+// together and none of which leaves between matched barriers, and the
+// allocation of tensor memory, whose holder (another run's CTA on the SM) never
+// waits for the one that waits.
 template <class Done>
 __device__ __forceinline__ bool bounded_wait(Ctrl* c, unsigned long long wait_ns, Done done)
 {

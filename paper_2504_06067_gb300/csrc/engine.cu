@@ -1486,10 +1486,11 @@ nsga3_status nsga3_last_launches(nsga3_ctx* ctx, int32_t* launches)
 {
     if (!ctx || !launches) return fail(ctx, NSGA3_EINVAL, "null argument");
     CK(cudaDeviceSynchronize());
-    // reset, 3 sort, dominance, peel (every pass), 10 niching (the first
-    // also writes the ranks back; the others return at once when no niching
-    // is needed; one or two more for m > 10), mark, gather (+ finite check
-    // for a selection; + variation, objective for a generation)
+    // small populations: the one cluster (+ the variation where it is large);
+    // m <= 10: reset and thresholds, 2 sort, 3 dominance, peel (every pass), 10
+    // niching (the first also writes the ranks back; the others return at once
+    // when no niching is needed), mark, gather (+ 3 for a first front; + the
+    // variation for a generation); m > 10: as select_launches counts them
     *launches = (ctx->last_kind == 1) ? select_launches(ctx) : generation_launches(ctx);
     return NSGA3_OK;
 }

@@ -56,7 +56,7 @@ __global__ void k_kp_vary(RunView v)
     const int f0 = v.fslot[2 * q], f1 = v.fslot[2 * q + 1];
     float* x0 = v.X + (size_t)f0 * d;
     float* x1 = v.X + (size_t)f1 * d;
-    // the pair's share of the merged state (as merge_pair of k_problem.cu)
+    // the pair's share of the merged state (as merge_pair of variation.cuh)
     if (lane < 2) {
         v.pold[2 * q + lane] = v.pcan[2 * q + lane];
         v.cslot[2 * q + lane] = lane ? f1 : f0;
