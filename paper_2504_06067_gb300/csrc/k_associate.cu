@@ -143,8 +143,9 @@ __global__ void __launch_bounds__(PB) k_assoc_prep(RunView v)
 // and a point whose third maximum in some item is within it too (about one
 // in 20,000) takes the FP32 scan over all directions (k_assoc_slow).
 //
-// Bound: the chain of product, load and barrier of a step, then the tensor
-// cores' reads of operands of so small a K.  Measured at m = 8, 38,700 points
+// Bound: the chain of product, load and barrier of a step; the tensor pipe is
+// busy 32 % of the time at m = 8 and 15 % at m = 5 (K is 32 and 16, so an MMA is
+// short against the read of its accumulator).  Measured at m = 8, 38,700 points
 // and 11,440 directions, and m = 5, 21,000 points and 10,626 directions:
 // 36 and 16-22 us.  FP32 FMAs took 173 us at m = 8 (the FMA pipe's time), a
 // scan pruned by cone bounds 42-52 us at m = 5; on the way here: a branch per
