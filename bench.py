@@ -449,7 +449,8 @@ def roofline_of(cfg, avg_ms, peel_rows_per_step, probe, peaks, peak_kind, domsta
             if front:
                 roof["block_pairs"]["note"] = "row_dom_col includes the row blocks that the first front met"
             roof["all_pairs_compare_rate"] = all_ops / sec / 1e12
-            roof["issue_active_ncu"] = ncu_issue_active("k_dominance")
+            if front:  # (the capture is of the first front)
+                roof["issue_active_ncu"] = ncu_issue_active("k_dominance")
             roof["dense_matrix_gbs"] = (n2 * n2 / 8 + n2 * cfg.m * 4) / sec / 1e9
         return roof
     bytes_read = peel_rows_per_step * 128 * 4.0  # row segments of 128 columns

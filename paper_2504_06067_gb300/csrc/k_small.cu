@@ -15,9 +15,10 @@
 // (normalize.cuh, associate.cuh), the same priorities, ties to the lowest
 // index.  What bounds it: the latency of the chain (FP64 divisions and square
 // roots, barriers) and, from N of a few hundred, the pair tests on 8 or 16 SMs.
-// Measured per generation, general path -> here: m = 3, N = 92 101 -> 33 us;
-// m = 5, N = 500 105 -> 42; m = 8, N = 1,000 115 -> 76; m = 10, N = 1,000
-// 122 -> 86 (20 generations and reading the population).  The limits (SMALL_N2,
+// Measured per generation, general path -> here: m = 3, N = 92 91 -> 31 us;
+// m = 5, N = 500 103 -> 44; m = 8, N = 1,000 113 -> 73; m = 10, N = 1,000
+// 122 -> 82 (20 generations and reading the population); selections of
+// N = 1,024 with 2 to 35 directions 108-185 -> 47-89.  The limits (SMALL_N2,
 // SMALL_W) lie where the objectives, the dominance words and the niche arrays
 // still fit one CTA's shared memory.
 #include "associate.cuh"
